@@ -596,8 +596,18 @@ fly_status_t fly_pld_draft(int32_t device, int32_t B, const int32_t* tokens, int
   p.tokens = tokens; p.stride = stride; p.lengths = lengths;
   p.B = B; p.max_ngram = max_ngram; p.min_ngram = min_ngram; p.K = K;
   p.draft = draft; p.count = count; p.match_pos = match_pos; p.match_ngram = match_ngram;
-  fly::pld::pld_draft_kernel<<<(unsigned)B, fly::pld::kThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(p);
-  return cudaGetLastError() == cudaSuccess ? FLY_OK : FLY_ERR_CUDA;
+  // Blocks per sequence: enough that one round covers the longest context (stride bounds every length).
+  int ranks = 1;
+  while (ranks < fly::pld::kMaxCluster && (int64_t)ranks * fly::pld::kRound < stride) ranks *= 2;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  fill_launch(&cfg, attr, (unsigned)B * (unsigned)ranks, fly::pld::kThreads, static_cast<cudaStream_t>(cuda_stream), true);
+  if (ranks > 1) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)ranks; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
+  return cudaLaunchKernelEx(&cfg, fly::pld::pld_draft_kernel, p) == cudaSuccess ? FLY_OK : FLY_ERR_CUDA;
 }
 
 fly_status_t fly_verify_device_status(fly_verify_t* h, void* cuda_stream) {

@@ -75,3 +75,19 @@ def test_lengths_outside_the_row_propose_nothing_and_read_nothing_outside_it():
     for b in (0, 5):
         prop, p, n = oracle_pld(tok[b, :lengths[b]].tolist(), K, 3, 1)
         assert count[b].item() == len(prop) and pos[b].item() == p and draft[b, :len(prop)].tolist() == prop
+
+
+@pytest.mark.parametrize("L", [2, 3, 5, 4095, 4096, 4097, 8193, 32767, 32768, 33000])
+@pytest.mark.parametrize("pad", [0, 1, 2, 3])
+def test_matches_at_the_edges_of_segments_rounds_and_blocks(L, pad):
+    # one 16-byte segment is 4 tokens, one block round 4096, one cluster round 32768; odd strides shift the segments
+    n = min(3, L - 1)
+    ends = sorted({e for e in (n, 4, 5, 4093, 4096, 4097, 4099, 8192, L // 2, L - 2, L - 1) if n <= e < L})
+    seqs = []
+    for e in ends:
+        s = list(range(10, 10 + L))
+        s[e - n:e] = s[L - n:]                        # the last n tokens also end just before position e
+        seqs.append(s)
+    stride = (L + 3) // 4 * 4 + pad
+    for mx, mn in [(n, n), (5, 1)]:
+        run(seqs, 8, mx, mn, pad_to=stride)
