@@ -307,8 +307,9 @@ fly_status_t fly_verify_device_status(fly_verify_t* handle, void* cuda_stream);
 fly_status_t fly_verify_selftest_wait(fly_verify_t* handle, void* cuda_stream);
 
 /* Introspection, host only (no CUDA call): the launch geometry the logits path chooses for `rows` rows of
- * `vocab` logits of `dtype` on a device with sm_count SMs.  vector_path = 1 if base, row stride and row length
- * allow 16-byte loads (a unit is then a 16-byte segment, else one logit).  forced_pieces as FLY_OPT_SPLITS.
+ * `vocab` logits of `dtype` on a device with sm_count SMs.  vector_path = 1 if the rows are read
+ * in 16-byte segments, as any row of at least 32 of them is (a unit is then a 16-byte segment, else one
+ * logit).  forced_pieces as FLY_OPT_SPLITS.
  *   grid             thread blocks
  *   units_per_block  block b reduces the flat unit range [b * units_per_block, (b + 1) * units_per_block)
  *   units_per_row    whole units in a row

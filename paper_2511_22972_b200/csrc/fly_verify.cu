@@ -204,10 +204,10 @@ void ensure_reduce_attrs(int device) {
   (void)cudaGetLastError();
 }
 
+// Rows shorter than one segment per lane of a warp take the element-wise path: there is nothing to stream.
 template <typename T>
-bool vector_path_ok(const void* logits, int64_t row_stride, int V) {
-  return ((reinterpret_cast<uintptr_t>(logits) & 15u) == 0) && ((row_stride * (int64_t)sizeof(T)) % 16 == 0) &&
-         (V >= fly::Seg<T>::kElems * 32);
+bool vector_path_ok(const void* logits, int V) {
+  return reinterpret_cast<uintptr_t>(logits) % sizeof(T) == 0 && V >= fly::Seg<T>::kElems * 32;
 }
 
 // Launches the row reduction.  `tail` carries the acceptance scan's arguments (tickets == NULL: no scan in
@@ -217,7 +217,7 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
                           fly::Partial* partials, cudaStream_t st, fly::ScanParams* tail, float scale,
                           bool inputs_ready) {
   constexpr int kE = fly::Seg<T>::kElems;
-  const bool vec = vector_path_ok<T>(logits, row_stride, V);
+  const bool vec = vector_path_ok<T>(logits, V);
   const int64_t n = vec ? V / kE : V;
   const int64_t min_units = vec ? kMinBlockBytes / 16 : kMinBlockBytes / (int64_t)sizeof(T);
   const int64_t stride_units = (int64_t)fly::kReduceWarps * kReduceUnroll * 32;

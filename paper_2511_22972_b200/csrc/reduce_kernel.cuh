@@ -113,8 +113,14 @@ __device__ __forceinline__ void acc_add2(WarpAcc& a, float x0, float x1, f2 sc2,
 }
 
 // ---------------------------------------------------------------------------
-// Vector path: rows whose base, stride and length are multiples of 16 bytes.
-// A "segment" is one 16-byte load: 8 bf16 or 4 fp32 logits.
+// Vector path: rows of at least a warp's width of 16-byte segments, at any
+// alignment.  A "segment" is one aligned 16-byte copy: 8 bf16 or 4 fp32 logits.
+// A row that does not start on a 16-byte boundary has its first segment up to
+// kElems - 1 logits in (`head`); what the segments leave over at both ends
+// (fewer than 2 * kElems logits) is one element-wise slice of the warp that
+// ends the row, loaded when the piece is opened so that its latency hides
+// behind the first segments.  Rows of 50257 bf16 logits (288 of them, 29 MB,
+// seven of eight off a 16-byte boundary): 14.1 us a step; element by element 29.0.
 // ---------------------------------------------------------------------------
 
 template <typename T> struct Seg;
@@ -239,8 +245,38 @@ __device__ __forceinline__ void slice_sum_f32(WarpAcc& a, const uint32_t (&w)[UN
   }
 }
 
-// Element-wise slice for rows without 16-byte structure and for the ragged
-// tail of a vector row: UNROLL*32 consecutive elements starting at e0.
+// Folds one logit per UNROLL and lane (x, already clamped; the floor where there is none) with the indices idx(j).
+// An index below the ones folded so far wins a tie.
+template <int UNROLL, typename F>
+__device__ __forceinline__ void fold_elements(WarpAcc& a, const float (&x)[UNROLL], F idx) {
+  float lm = kMaskFloor;
+#pragma unroll
+  for (int j = 0; j < UNROLL; ++j) lm = fmaxf(lm, x[j]);
+  const float wm = warp_max_f32(lm);
+  if (wm > kMaskFloor && wm >= a.cur_max) {
+    const bool moved = wm > a.cur_max;
+    if (moved) acc_rebase(a, wm);
+    uint32_t first = 0xffffffffu;
+    if (lm == wm) {
+#pragma unroll
+      for (int j = UNROLL - 1; j >= 0; --j)
+        if (x[j] == wm) first = min(first, (uint32_t)idx(j));
+    }
+    const int wf = (int)warp_min_u32(first);
+    a.best_idx = moved ? wf : min(a.best_idx, wf);
+  }
+  const f2 nr2 = pack2(-a.r, -a.r), sc2 = pack2(a.scale, a.scale);
+  // lanes without a logit hold the floor: 2^(floor*scale - r) = 0 unless the whole
+  // piece is masked, in which case the piece vanishes when merged
+  if constexpr (UNROLL == 1) {
+    acc_add2(a, x[0], kMaskFloor, sc2, nr2);
+  } else {
+#pragma unroll
+    for (int j = 0; j < UNROLL; j += 2) acc_add2(a, x[j], x[j + 1], sc2, nr2);
+  }
+}
+
+// Element-wise slice of short rows: UNROLL*32 consecutive elements starting at e0.
 template <typename T, int UNROLL>
 __device__ __forceinline__ void warp_slice_scalar(WarpAcc& a, const T* __restrict__ row, int e0, int e_end,
                                                   int lane) {
@@ -252,29 +288,18 @@ __device__ __forceinline__ void warp_slice_scalar(WarpAcc& a, const T* __restric
     if (e < e_end) v = (float)row[e];
     x[j] = max_nan_f32(v, kMaskFloor);
   }
-  float lm = kMaskFloor;
-#pragma unroll
-  for (int j = 0; j < UNROLL; ++j) lm = fmaxf(lm, x[j]);
-  const float wm = warp_max_f32(lm);
-  if (wm > a.cur_max) {
-    acc_rebase(a, wm);
-    uint32_t first = 0xffffffffu;
-    if (lm == wm) {
-#pragma unroll
-      for (int j = UNROLL - 1; j >= 0; --j)
-        if (x[j] == wm) first = (uint32_t)(e0 + j * 32 + lane);
-    }
-    a.best_idx = (int)warp_min_u32(first);
-  }
-  const f2 nr2 = pack2(-a.r, -a.r), sc2 = pack2(a.scale, a.scale);
-  // out-of-range lanes hold the floor: 2^(floor*scale - r) = 0 unless the whole
-  // piece is masked, in which case the piece vanishes when merged
-  if constexpr (UNROLL == 1) {
-    acc_add2(a, x[0], kMaskFloor, sc2, nr2);
-  } else {
-#pragma unroll
-    for (int j = 0; j < UNROLL; j += 2) acc_add2(a, x[j], x[j + 1], sc2, nr2);
-  }
+  fold_elements<UNROLL>(a, x, [&](int j) { return e0 + j * 32 + lane; });
+}
+
+// Logits of a row before its first aligned segment.
+template <typename T>
+__device__ __forceinline__ int row_head(const T* row) {
+  return (int)((0u - (uint32_t)reinterpret_cast<uintptr_t>(row)) & 15u) / (int)sizeof(T);
+}
+// Index of the logit of a row that lane `lane` holds of those that its `segs` segments leave over (>= V: none).
+template <typename T>
+__device__ __forceinline__ int leftover_index(int head, int segs, int lane) {
+  return lane < head ? lane : segs * Seg<T>::kElems + lane;
 }
 
 // One piece on the element-wise path: logits [e_begin, e_end) of the row.
@@ -373,7 +398,7 @@ __device__ __forceinline__ void flush_pending(const Pending* pend, int np, int s
   for (int k = 0; k < np; ++k) sequence_tail(tail, pend[k].row, pend[k].units, lane, sm_y);
 }
 
-// grid.x = ceil(total / Q).  VEC: rows are 16-byte structured (a unit is a segment); else any alignment, any V.
+// grid.x = ceil(total / Q).  VEC: a unit is a segment; else a logit (rows too short for the vector path).
 template <typename T, int UNROLL, bool VEC>
 __global__ void __launch_bounds__(kReduceThreads, kReduceBlocksPerSM)
 reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePlan g, Partial* __restrict__ partials,
@@ -385,6 +410,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
   __shared__ Partial sm_part[2][kReduceWarps];
   __shared__ Pending pend[kMaxPend];
   __shared__ int sm_y[kMaxRows];
+  __shared__ float leftover[32];  // VEC: what the segments of the current row leave over (last warp)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   // The grid is launched as a programmatic dependent of the previous kernel in the stream.  Plain
@@ -420,10 +446,20 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
   const uint32_t ring_warp = smem_addr_u32(ring) + (uint32_t)((warp * kDepth * kSlice + lane) * 16);
   const uint4* psrc = nullptr;
   int ps = 0, pend_seg = 0;
+  auto segments = [&](int head) { return ((int)g.V - head) / kE; };  // of a row with this head: n or n - 1
   auto open_piece = [&](int prow, int pu0, int pu1) {
-    psrc = reinterpret_cast<const uint4*>(logits + (int64_t)prow * g.row_stride) + lane;
+    const T* rp = logits + (int64_t)prow * g.row_stride;
+    const int head = row_head(rp);
+    psrc = reinterpret_cast<const uint4*>(rp + head) + lane;
     ps = pu0 + warp * kSlice;
-    pend_seg = pu1;
+    pend_seg = min(pu1, segments(head));
+  };
+  auto fetch_leftover = [&](int prow, int pu1) {  // after the piece's first slices were asked for
+    if (pu1 == (int)g.n && warp == kReduceWarps - 1) {
+      const T* rp = logits + (int64_t)prow * g.row_stride;
+      const int head = row_head(rp), e = leftover_index<T>(head, segments(head), lane);
+      leftover[lane] = e < g.V ? max_nan_f32((float)rp[e], kMaskFloor) : kMaskFloor;
+    }
   };
   auto issue = [&](int stage) {
     if (ps < pend_seg) {
@@ -444,6 +480,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     open_piece(row, u0, u1);
 #pragma unroll
     for (int d = 0; d < kDepth; ++d) issue(d);
+    fetch_leftover(row, u1);
   }
 
   // The acceptance scan at the end of the step reads draft tokens and carried state, which nothing has
@@ -456,13 +493,13 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
 
   int parity = 0, np = 0;
   while (true) {
-    const T* rp = logits + (int64_t)row * g.row_stride;
     WarpAcc a;
     acc_init(a, g.scale);
     left -= take;
     if constexpr (VEC) {
       int stage = 0;
-      for (int s0 = u0 + warp * kSlice; s0 < u1; s0 += kStride) {
+      const int s_end = pend_seg;
+      for (int s0 = u0 + warp * kSlice; s0 < s_end; s0 += kStride) {
         cp_async_wait<kDepth - 1>();  // the oldest slice in flight has landed
         uint32_t w[UNROLL][4];
         const uint4* src = ring + (warp * kDepth + stage) * kSlice + lane;
@@ -472,8 +509,8 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
           w[j][0] = q.x; w[j][1] = q.y; w[j][2] = q.z; w[j][3] = q.w;
         }
         float lm;
-        if constexpr (sizeof(T) == 2) lm = slice_max_bf16<UNROLL>(w, s0, u1, lane);
-        else lm = slice_max_f32<UNROLL>(w, s0, u1, lane);
+        if constexpr (sizeof(T) == 2) lm = slice_max_bf16<UNROLL>(w, s0, s_end, lane);
+        else lm = slice_max_f32<UNROLL>(w, s0, s_end, lane);
         // every register of the slice has been consumed once, so the stage's bytes are out of shared
         // memory: refill it with the slice kDepth ahead
         issue(stage);
@@ -481,18 +518,25 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
         else slice_sum_f32<UNROLL>(a, w, lm, s0, lane);
         stage = stage + 1 == kDepth ? 0 : stage + 1;
       }
+      const T* rp = logits + (int64_t)row * g.row_stride;
+      const int head = row_head(rp);
+      if (a.best_idx != kIdxNone) a.best_idx += head;
+      if (u1 == (int)g.n && warp == kReduceWarps - 1) {
+        const float x[1] = {leftover[lane]};
+        fold_elements<1>(a, x, [&](int) { return leftover_index<T>(head, segments(head), lane); });
+      }
       // This warp's ring is empty now.  If the block goes on into the next row, start that piece's first
       // slices before the block-wide merge below, so that the row boundary costs no memory round trip.
       if (left > 0) {
         cp_async_wait<0>();
-        open_piece(row + 1, 0, (int)min(g.n, left));
+        const int next_u1 = (int)min(g.n, left);
+        open_piece(row + 1, 0, next_u1);
 #pragma unroll
         for (int d = 0; d < kDepth; ++d) issue(d);
+        fetch_leftover(row + 1, next_u1);
       }
-      // ragged tail (fewer than kElems logits): the piece that ends the row, last warp
-      if (u1 == (int)g.n && warp == kReduceWarps - 1 && (int)g.n * kE < g.V) warp_slice_scalar<T, 1>(a, rp, (int)g.n * kE, g.V, lane);
     } else {
-      reduce_piece_scalar<T, UNROLL>(a, rp, u0, u1, lane, warp);
+      reduce_piece_scalar<T, UNROLL>(a, logits + (int64_t)row * g.row_stride, u0, u1, lane, warp);
     }
     const Partial p = block_finish(a, sm_part[parity], lane, warp);
     if (warp == 0 && lane == 0) {

@@ -511,3 +511,27 @@ def test_two_handles_on_two_streams_at_once():
         assert_parity(ob, oracle_step(lb, db, 1.0, 2), "stream b")
     fa.close()
     fb.close()
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 256), ("bf16", 257), ("bf16", 263), ("bf16", 8191), ("bf16", 8193), ("bf16", 65543),
+                                     ("f32", 128), ("f32", 129), ("f32", 4095), ("f32", 32771)])
+@pytest.mark.parametrize("splits", [0, 1, 5])
+def test_rows_at_every_alignment(dtype, V, splits):
+    # rows packed at an odd length start at every offset within a 16-byte segment; the maximum sits in the logits that the
+    # aligned segments leave over at either end, tied with one inside, and the base is off by one element as well
+    w = small(dtype, B=2, K=8, V=V)
+    fv = FlyVerify(w.B, w.K, V, dtype)
+    fv.set_splits(splits)
+    logits, draft = draw(w, step=V, guard=False)
+    rows = logits.view(-1, V)
+    for r in range(rows.shape[0]):
+        top = rows[r].float().max().item() + 1.0
+        rows[r, {0: [0, V // 2], 1: [V - 1], 2: [V // 2, V - 1], 3: [V - 1, 0]}[r % 4]] = top
+        if r % 5 == 4:
+            rows[r, :V // 2] = -math.inf
+    for off in (0, 1, 3):
+        flat = torch.full((off + rows.numel() + 16,), 1e4, dtype=rows.dtype, device=DEV)   # what lies around must not be read in
+        view = flat[off:off + rows.numel()].view(w.B, w.K + 1, V)
+        view.copy_(logits)
+        check(fv, view, draft, 1.0, 2, what=f"{dtype} V={V} splits={splits} off={off}")
+    fv.close()
