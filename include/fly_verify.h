@@ -252,12 +252,11 @@ fly_status_t fly_pld_draft(int32_t device, int32_t B, const int32_t* tokens, int
  * The first call on each device looks up the device address of the built-in
  * array (which also makes the CUDA runtime load the library's device code).
  * Make that first call outside any stream capture; later calls only enqueue
- * work on `cuda_stream` (one memset of the B arrival counters, one kernel).
+ * work on `cuda_stream` (a small kernel that clears the scratch, then the step's kernel).
  *
  * All calls on a device share the one array, and it keeps whatever the last
- * call left there.  The counters are cleared on the stream at the start of
- * every call and the partial states are fully rewritten before they are read,
- * so stale contents never leak into a result.  But two calls whose work
+ * call left there.  Counters and partial states are cleared on the stream at the
+ * start of every call, so stale contents never leak into a result.  But two calls whose work
  * overlaps on the GPU (different streams, or several host threads) write the same
  * scratch and corrupt each other: serialise them, e.g. keep them on one stream. */
 #define FLY_STATIC_MAX_BATCH 1024

@@ -45,15 +45,15 @@ struct fly_verify {
   fly_verify_config_t cfg;
   int sm_count = 148;
   int64_t max_rows = 0;
-  fly::Partial* partials = nullptr;  // [max_rows * kMaxSplits]
-  unsigned int* tickets = nullptr;   // [max_batch], zero between launches
+  fly::Partial* partials = nullptr;  // [max_rows * kMaxSplits], empty (all zero) between launches
+  unsigned int* tickets = nullptr;   // [max_rows] arrival counters of sequences (of rows: shards), zero between launches
   int forced_splits = 0;
   int scan_mode = 0;   // 0: fused tail, 1: separate kernel
   int last_launches = 0;
   int last_cuda_error = 0;
   // fused LM-head path (cfg.hidden > 0)
   fly::Partial* lm_partials = nullptr;  // [max_rows * sm_count]: one partial state per row and CTA
-  fly::Partial* lm_folded = nullptr;    // [max_rows]: partial states folded over CTAs (fused path) or ranks
+  fly::Partial* lm_folded = nullptr;    // [max_rows]: partial states folded over CTAs
   int* lm_status = nullptr;             // device word: first bounded wait that ran out (sticky until read)
   int lm_pairs = 0;                     // CTA pairs that can be resident at once
   int weight_vd = 0;                    // 0: weight [hidden, V]; 1: weight [V, hidden]
@@ -144,7 +144,8 @@ FlatPlan plan_flat(int sm_count, int64_t rows, int64_t n, int64_t min_units, int
     if (s_fill < 1) s_fill = 1;
     const int64_t blocks = rows * s_fill, waves = (blocks + gmax - 1) / gmax;
     const bool could_fill = rows * n / min_units >= gmax;  // enough work for a full grid at all
-    if (could_fill && 4 * blocks < 3 * waves * gmax) {
+    // (so few waves that a block never holds more than a handful of rows)
+    if (could_fill && 4 * blocks < 3 * waves * gmax && (waves + 1) + 2 <= fly::kMaxPend) {
       // the last wave would be mostly empty: pack the rows end to end and cut the range evenly instead
       s = 0;
       const int64_t Qf = (rows * n + gmax - 1) / gmax;
@@ -204,6 +205,14 @@ void ensure_reduce_attrs(int device) {
   (void)cudaGetLastError();
 }
 
+// Lanes (as a power of two) that share a row's parts in the acceptance scan: one per part as far as a block has threads
+// for all rows of a sequence.
+int lanes_for(int64_t parts, int rows) {
+  int k = 0;
+  while (k < 5 && ((int64_t)1 << k) < parts && ((int64_t)rows << (k + 1)) <= fly::kScanThreads) ++k;
+  return k;
+}
+
 // Rows shorter than one segment per lane of a warp take the element-wise path: there is nothing to stream.
 template <typename T>
 bool vector_path_ok(const void* logits, int V) {
@@ -223,23 +232,25 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   const int64_t stride_units = (int64_t)fly::kReduceWarps * kReduceUnroll * 32;
   const FlatPlan pl = plan_flat(sm_count, rows, n, min_units, stride_units, cap, inputs_ready, forced);
   fly::ReducePlan g;
-  g.n = n; g.span = pl.span; g.Q = pl.Q; g.total = rows * pl.span; g.slots = pl.slots;
+  g.n = n; g.span = pl.span; g.Q = pl.Q; g.total = rows * pl.span;
   g.pieces = pl.Q < (1 << 30) ? pl.pieces : 0; g.V = V; g.row_stride = row_stride;
   g.scale = scale; g.wait_first = inputs_ready ? 0 : 1;
   tail->splits = pl.slots;
+  tail->row_pitch = pl.slots;
+  tail->part_pitch = 1;
+  tail->lanes_log2 = lanes_for(pl.slots, tail->K + 1);
+  tail->partials = partials;
   tail->units_per_row = n;
   tail->row_span = pl.span;
-  tail->Q = pl.Q;
+  tail->Q = pl.pieces > 0 ? 0 : pl.Q;  // whole pieces: every row has exactly pl.slots of them
   tail->scale = scale;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_launch(&cfg, attr, (unsigned)pl.grid, fly::kReduceThreads, st, true);
   cfg.dynamicSmemBytes = vec ? kReduceRingBytes : 0;
   if (vec)
-    return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, true>, static_cast<const T*>(logits), g, partials,
-                              *tail);
-  return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, false>, static_cast<const T*>(logits), g, partials,
-                            *tail);
+    return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, true>, static_cast<const T*>(logits), g, *tail);
+  return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, false>, static_cast<const T*>(logits), g, *tail);
 }
 
 // The current device must be the one the pointers belong to (its ordinal is `device`).
@@ -253,11 +264,12 @@ cudaError_t launch_reduce_any(int device, fly_dtype_t dt, int sm_count, const vo
   return launch_reduce<float>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, scale, inputs_ready);
 }
 
-cudaError_t launch_scan(const fly::ScanParams& p, cudaStream_t st) {
+// tagged: the parts are in the self-validating form that the row reduction leaves.
+cudaError_t launch_scan(const fly::ScanParams& p, bool tagged, cudaStream_t st) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  fill_launch(&cfg, attr, (unsigned)((p.B + fly::kScanWarps - 1) / fly::kScanWarps), fly::kScanThreads, st, true);
-  return cudaLaunchKernelEx(&cfg, fly::scan_sequences, p);
+  fill_launch(&cfg, attr, (unsigned)p.B, fly::kScanThreads, st, true);
+  return tagged ? cudaLaunchKernelEx(&cfg, fly::scan_sequences<true>, p) : cudaLaunchKernelEx(&cfg, fly::scan_sequences<false>, p);
 }
 
 fly_status_t check_args(const fly_verify* h, const fly_verify_args_t* a) {
@@ -291,7 +303,7 @@ float exponent_scale(double temperature) {
   return (float)(1.4426950408889634 / T);
 }
 
-fly::ScanParams scan_params(const fly_verify* h, const fly_verify_args_t* a, const fly::Partial* partials, int splits);
+fly::ScanParams scan_params(const fly_verify* h, const fly_verify_args_t* a, fly::Partial* partials, int splits);
 
 // 2-D bf16 tensor map with the 128-byte swizzle: dims {inner, outer}, row pitch in bytes, box {64, box_rows}.
 bool encode_map(fly_verify* h, CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer, uint64_t pitch_bytes,
@@ -352,14 +364,14 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     cudaLaunchAttribute attr[1];
     const unsigned warps = fly::kFoldThreads / 32;
     fill_launch(&cfg, attr, (unsigned)((rows + warps - 1) / warps), fly::kFoldThreads, st, true);
-    e = cudaLaunchKernelEx(&cfg, fly::fold_partials, (const fly::Partial*)h->lm_partials, grid, (int64_t)grid,
-                           (int64_t)1, h->lm_folded, (int)rows, 0, exponent_scale(a->temperature), (int64_t)0, (int64_t)0);
+    e = cudaLaunchKernelEx(&cfg, fly::fold_partials, (const fly::Partial*)h->lm_partials, grid, h->lm_folded, (int)rows,
+                           exponent_scale(a->temperature));
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->last_launches++;
   }
   fly::ScanParams sp = scan_params(h, a, h->lm_folded, 1);
   sp.status = h->lm_status;  // a step whose GEMM kernel gave up is marked row by row, in stream order
-  e = launch_scan(sp, st);
+  e = launch_scan(sp, false, st);
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches++;
   return FLY_OK;
@@ -371,8 +383,11 @@ float theta_to_nats(const fly_verify* h, const fly_verify_args_t* a) {
   return (float)th;
 }
 
-fly::ScanParams scan_params(const fly_verify* h, const fly_verify_args_t* a, const fly::Partial* partials, int splits) {
+fly::ScanParams scan_params(const fly_verify* h, const fly_verify_args_t* a, fly::Partial* partials, int splits) {
   fly::ScanParams p;
+  p.row_pitch = splits; p.part_pitch = 1;
+  p.lanes_log2 = lanes_for(splits, a->K + 1);
+  p.row_out = nullptr; p.idx_offset = 0;
   p.B = a->B; p.K = a->K; p.V = h->cfg.vocab; p.splits = splits;
   p.units_per_row = 0; p.row_span = 0; p.Q = 0;  // every row has exactly `splits` parts unless the row reduction says otherwise
   p.scale = exponent_scale(a->temperature);
@@ -432,8 +447,9 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   h->sm_count = sms > 0 ? sms : 148;
   e = cudaMalloc(&h->partials, (size_t)h->max_rows * kMaxSplits * sizeof(fly::Partial));
   if (e != cudaSuccess) { delete h; return FLY_ERR_CUDA; }
-  e = cudaMalloc(&h->tickets, (size_t)c->max_batch * sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMemset(h->tickets, 0, (size_t)c->max_batch * sizeof(unsigned int));
+  e = cudaMemset(h->partials, 0, (size_t)h->max_rows * kMaxSplits * sizeof(fly::Partial));
+  if (e == cudaSuccess) e = cudaMalloc(&h->tickets, (size_t)h->max_rows * sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMemset(h->tickets, 0, (size_t)h->max_rows * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMalloc(&h->lm_status, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(h->lm_status, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&h->lm_folded, (size_t)h->max_rows * sizeof(fly::Partial));
@@ -536,20 +552,16 @@ fly_status_t fly_verify_reduce_shard(fly_verify_t* h, int32_t rows, const void* 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int64_t stride = row_stride ? row_stride : V;
   const float scale = exponent_scale(temperature);
-  fly::ScanParams none;
-  memset(&none, 0, sizeof(none));  // tickets == NULL: no acceptance scan in this launch
+  fly::ScanParams p;  // the tail of the reduction folds each row's pieces: a "sequence" is one row
+  memset(&p, 0, sizeof(p));
+  p.B = rows;
+  p.tickets = h->tickets;
+  p.row_out = reinterpret_cast<fly::Partial*>(partial_out);
+  p.idx_offset = vocab_offset;
   cudaError_t e = launch_reduce_any(h->cfg.device, h->cfg.logits_dtype, h->sm_count, logits, stride, V, rows, h->forced_splits, kMaxSplits,
-                                    h->partials, st, &none, scale, false);
+                                    h->partials, st, &p, scale, false);
   if (e != cudaSuccess) return cuda_fail(h, e);
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[1];
-  const unsigned warps = fly::kFoldThreads / 32;
-  fill_launch(&cfg, attr, (unsigned)((rows + warps - 1) / warps), fly::kFoldThreads, st, true);
-  e = cudaLaunchKernelEx(&cfg, fly::fold_partials, (const fly::Partial*)h->partials, none.splits, (int64_t)none.splits,
-                         (int64_t)1, reinterpret_cast<fly::Partial*>(partial_out), (int)rows, (int)vocab_offset, scale,
-                         none.row_span, none.Q);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  h->last_launches = 2;
+  h->last_launches = 1;
   return FLY_OK;
 }
 
@@ -565,23 +577,17 @@ fly_status_t fly_verify_run_partials(fly_verify_t* h, const fly_verify_args_t* a
   if (!g.ok) return FLY_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int64_t rows = (int64_t)a->B * (a->K + 1);
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[1];
-  const unsigned warps = fly::kFoldThreads / 32;
-  fill_launch(&cfg, attr, (unsigned)((rows + warps - 1) / warps), fly::kFoldThreads, st, false);
   // all-gather layout: [world, rows]
-  cudaError_t e = cudaLaunchKernelEx(&cfg, fly::fold_partials, reinterpret_cast<const fly::Partial*>(partials), (int)world,
-                                     (int64_t)1, (int64_t)rows, h->lm_folded, (int)rows, 0, exponent_scale(a->temperature),
-                                     (int64_t)0, (int64_t)0);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  fly::ScanParams sp = scan_params(h, a, h->lm_folded, 1);
+  fly::ScanParams sp = scan_params(h, a, const_cast<fly::Partial*>(reinterpret_cast<const fly::Partial*>(partials)), world);
+  sp.row_pitch = 1;
+  sp.part_pitch = rows;
   sp.V = total_vocab;
   double th = a->theta;
   if (a->theta_unit == FLY_THETA_NORMALIZED) th *= std::log((double)total_vocab);
   sp.theta_nats = (float)th;
-  e = launch_scan(sp, st);
+  const cudaError_t e = launch_scan(sp, false, st);
   if (e != cudaSuccess) return cuda_fail(h, e);
-  h->last_launches = 2;
+  h->last_launches = 1;
   return FLY_OK;
 }
 
@@ -685,7 +691,7 @@ fly_status_t fly_verify_run(fly_verify_t* h, const fly_verify_args_t* a, void* c
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches++;
   if (!fused_tail) {
-    e = launch_scan(p, st);
+    e = launch_scan(p, true, st);
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->last_launches++;
   }
@@ -863,8 +869,14 @@ fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t lo
   fly::ScanParams p = scan_params(&h, a, partials, 1);
   p.tickets = tickets;
 
-  // The arrival counters must start at zero, whatever an earlier call left behind.
-  cudaError_t e = cudaMemsetAsync(tickets, 0, (size_t)a->B * 4, st);
+  // Counters and slots must start empty, whatever an earlier call left behind.  A kernel in the stream's chain of
+  // programmatic dependents and not a memset, which would break the chain: the reduction's launch latency stays hidden.
+  const int slot_words = (int)(rows * cap), ticket_words = (a->B + 3) / 4;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  fill_launch(&cfg, attr, (unsigned)((slot_words + fly::kClearThreads - 1) / fly::kClearThreads), fly::kClearThreads, st, true);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, fly::clear_scratch, reinterpret_cast<uint4*>(tickets), ticket_words,
+                                     reinterpret_cast<uint4*>(partials), slot_words);
   if (e != cudaSuccess) return FLY_ERR_CUDA;
   e = launch_reduce_any(device, logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, p.scale,
                         a->inputs_ready != 0);

@@ -43,7 +43,7 @@ constexpr int kReduceThreads = 256;
 constexpr int kReduceWarps = kReduceThreads / 32;
 constexpr int kReduceBlocksPerSM = 4;  // __launch_bounds__ below: <= 64 registers; measured against 3, 5 and 6
 constexpr int kDepth = 2;              // slices in flight per warp (3 and 4 measured: no faster)
-constexpr int kMaxPend = 8;            // finished pieces a block holds back before it writes them out
+constexpr int kMaxPend = 8;            // pieces of a block at most; it holds them back and writes them out at its end
 
 // ---- packed fp32 pairs ------------------------------------------------------------------------
 using f2 = unsigned long long;  // two fp32 values in one 64-bit register: {lo, hi}
@@ -318,7 +318,6 @@ struct ReducePlan {
   int64_t Q;       // units per block
   int64_t total;   // rows * span
   int pieces;      // > 0: span = pieces * Q, block b is piece b % pieces of row b / pieces (32-bit arithmetic)
-  int slots;       // Partial slots per row (>= the largest number of pieces of any row)
   int V;
   int64_t row_stride;  // elements
   float scale;     // log2(e) / temperature
@@ -326,7 +325,7 @@ struct ReducePlan {
                    //    order); 0: the logits are known to be complete, wait only before the first write
 };
 
-// Lanes -> warp -> block; warp 0 / lane 0 ends up with the piece's Partial.  sm: kReduceWarps Partials of
+// Lanes -> warp -> block; warp 0 ends up with the piece's Partial.  sm: kReduceWarps Partials of
 // shared memory; consecutive pieces of a block alternate between two such buffers, so one barrier per
 // piece is enough.
 __device__ __forceinline__ Partial block_finish(const WarpAcc& a, Partial* sm, int lane, int warp) {
@@ -347,12 +346,8 @@ __device__ __forceinline__ Partial block_finish(const WarpAcc& a, Partial* sm, i
   __syncthreads();
   Partial p = empty_partial();
   if (warp == 0) {
-    if (lane < kReduceWarps) p = sm[lane];
-#pragma unroll
-    for (int o = kReduceWarps / 2; o > 0; o >>= 1) {
-      Partial q = shfl_xor_partial(p, o);
-      merge_partial(p, q, a.scale);
-    }
+    static_assert(kReduceWarps == 8, "the fold below is over 8 lanes");
+    p = fold_lanes(sm[lane & (kReduceWarps - 1)], 3, a.scale);
   }
   return p;
 }
@@ -365,59 +360,70 @@ struct __align__(16) Pending {
   int pad;
 };
 
-// Fused tail: the block that completes a sequence verifies it.  A sequence's arrival counter counts the
-// units (segments or logits) of its K+1 rows that have been reduced; the block whose piece brings it to
-// (K+1) * n has seen every other piece's ticket, hence (after the fences) every other Partial.  Called by
-// warp 0 once the piece's Partial is in global memory.
-__device__ __forceinline__ void sequence_tail(const ScanParams& p, int row, unsigned units, int lane, int* sm_y) {
-  const int K1 = p.K + 1;
-  const int b = row / K1;
-  unsigned last = 0;
-  if (lane == 0) {
-    const unsigned t = atomicAdd(p.tickets + b, units);
-    last = (t + units == (unsigned)K1 * (unsigned)p.units_per_row);
-  }
-  last = __shfl_sync(0xffffffffu, last, 0);
-  if (last) {
-    __threadfence();  // every lane reads the other blocks' partials after the ticket was seen
-    scan_one_sequence(p, b, lane, sm_y);
-    if (lane == 0) p.tickets[b] = 0;  // ready for the next launch (ordered by the end of this kernel; off the critical path)
-  }
-}
+struct TailShared {
+  Pending pend[kMaxPend];
+  int done[kMaxPend];  // the sequence that the piece completes, -1: none
+  ScanShared scan;
+};
 
-// Writes the held-back pieces out and takes their tickets (warp 0).
-__device__ __forceinline__ void flush_pending(const Pending* pend, int np, int slots, Partial* __restrict__ partials,
-                                              const ScanParams& tail, int lane, int* sm_y) {
-  if (lane < np) partials[(int64_t)pend[lane].row * slots + pend[lane].slot] = pend[lane].p;
-  if (tail.tickets == nullptr) return;
-  __threadfence();  // the partials written above are visible ...
-  if (np > 1) {     // (one piece: lane 0 wrote it and lane 0 takes its ticket, its own fence is enough)
+// Writes the block's np finished pieces (sm_tail.pend) out, takes their tickets and verifies the sequences they
+// complete.  The newest piece is part `slot` of row `row`.  A sequence's arrival counter counts the
+// units (segments or logits) of its K+1 rows that have been reduced; the piece that brings it to (K+1) * n is its
+// last, and every other piece's state has been issued by then (see the head of scan_kernel.cuh).
+// Only that block reads the sequence's states: asking for them before the counter has answered would save it a round
+// trip, but when all blocks of a step belong to one sequence they then read each other's lines while these are being
+// written, and the states arrive 2 us late (one sequence, 144 blocks: 7.1 us a step instead of 5.0).
+// Called by the whole block.
+__device__ __forceinline__ void flush_pieces(const ScanParams& p, TailShared& sm_tail, int np, int row, int slot) {
+  const int lane = (int)threadIdx.x & 31, warp = (int)threadIdx.x >> 5;
+  const int K1 = p.K + 1;
+  unsigned ticket = 0, units = 0;
+  int seq = -1;
+  if (warp == 0) {
     __syncwarp();
-    __threadfence();  // ... before lane 0 takes any ticket
+    if (lane < np) {
+      const Pending& q = sm_tail.pend[lane];
+      st_part(p.partials + q.row * p.row_pitch + q.slot, tagged(q.p));
+      if (p.tickets != nullptr) {
+        seq = q.row / K1;
+        units = q.units;
+        ticket = atomicAdd(p.tickets + seq, units);
+      }
+    }
   }
-  for (int k = 0; k < np; ++k) sequence_tail(tail, pend[k].row, pend[k].units, lane, sm_y);
+  if (p.tickets == nullptr) return;
+  if (warp == 0 && lane < np) sm_tail.done[lane] = ticket + units == (unsigned)K1 * (unsigned)p.units_per_row ? seq : -1;
+  __syncthreads();
+#pragma unroll 1
+  for (int k = np - 1; k >= 0; --k) {
+    const int b = sm_tail.done[k];
+    if (b < 0) continue;
+    const ScanLoads q = scan_request(p, b);
+    scan_sequence<true>(p, b, q, row, slot, sm_tail.pend[np - 1].p, sm_tail.scan);
+    if (threadIdx.x == 0) p.tickets[b] = 0;  // ready for the next launch (ordered by the end of this kernel)
+    if (np > 1) __syncthreads();  // sm_tail.scan is free again
+  }
 }
 
 // grid.x = ceil(total / Q).  VEC: a unit is a segment; else a logit (rows too short for the vector path).
 template <typename T, int UNROLL, bool VEC>
 __global__ void __launch_bounds__(kReduceThreads, kReduceBlocksPerSM)
-reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePlan g, Partial* __restrict__ partials,
-                 const __grid_constant__ ScanParams tail) {
+reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePlan g, const __grid_constant__ ScanParams tail) {
   constexpr int kE = Seg<T>::kElems;
   constexpr int kSlice = UNROLL * 32;
   constexpr int kStride = kReduceWarps * kSlice;
-  extern __shared__ __align__(16) uint4 ring[];  // VEC: kReduceWarps * kDepth * kSlice segments
+  // VEC: kReduceWarps * kDepth * kSlice segments.  On a 128-byte boundary: a copy of 8 lanes that straddles two lines of
+  // shared memory takes two passes (1088 rows: 60.6 us at an offset of 48 bytes, 54.9 on the boundary).
+  extern __shared__ __align__(128) uint4 ring[];
   __shared__ Partial sm_part[2][kReduceWarps];
-  __shared__ Pending pend[kMaxPend];
-  __shared__ int sm_y[kMaxRows];
+  __shared__ TailShared sm_tail;
   __shared__ float leftover[32];  // VEC: what the segments of the current row leave over (last warp)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   // The grid is launched as a programmatic dependent of the previous kernel in the stream.  Plain
   // stream order: wait for that kernel to complete (and its writes to be visible) before anything is
   // read.  With inputs_ready the reads start at once and the wait comes before the first write.
-  bool waited = g.wait_first != 0;
-  if (waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (g.wait_first != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   // Let the next kernel in the stream get scheduled early if it asks for that; it waits for this
   // grid's completion before it touches anything this grid writes.
   asm volatile("griddepcontrol.launch_dependents;");
@@ -487,7 +493,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
   // touched yet: pull them into L2 now so that the last block does not wait on DRAM for them.
   if (tail.tickets != nullptr && (int)blockIdx.x < tail.B && warp == 1) {
     const int32_t* d = tail.draft + (int64_t)blockIdx.x * tail.K;
-    if (lane * 32 < tail.K) asm volatile("prefetch.global.L2 [%0];" ::"l"(d + lane * 32));
+    if (tail.draft && lane * 32 < tail.K) asm volatile("prefetch.global.L2 [%0];" ::"l"(d + lane * 32));
     if (lane == 31 && tail.state_in) asm volatile("prefetch.global.L2 [%0];" ::"l"(tail.state_in + (int64_t)blockIdx.x * 3));
   }
 
@@ -539,29 +545,14 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
       reduce_piece_scalar<T, UNROLL>(a, logits + (int64_t)row * g.row_stride, u0, u1, lane, warp);
     }
     const Partial p = block_finish(a, sm_part[parity], lane, warp);
-    if (warp == 0 && lane == 0) {
+    if (threadIdx.x == 0) {
       Pending q;
       q.p = p; q.row = row; q.slot = slot; q.units = (unsigned)(u1 - u0); q.pad = 0;
-      pend[np] = q;
+      sm_tail.pend[np] = q;
     }
     ++np;
     parity ^= 1;
-    const bool done = left <= 0;
-    if (np == kMaxPend || done) {
-      // Everything so far only read the logits.  Scratch and outputs are shared with the previous step:
-      // with inputs_ready its kernel may still be running, so wait for it before the first write.
-      if (!waited) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        waited = true;
-      }
-      if (warp == 0) {
-        __syncwarp();
-        flush_pending(pend, np, g.slots, partials, tail, lane, sm_y);
-        __syncwarp();
-      }
-      np = 0;
-    }
-    if (done) break;
+    if (left <= 0) break;
     ++row;
     u0 = 0;
     u1 = (int)min(g.n, left);
@@ -569,6 +560,10 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     slot = 0;
   }
   if constexpr (VEC) cp_async_wait<0>();
+  // Everything so far only read the logits.  Scratch and outputs are shared with the previous step:
+  // with inputs_ready its kernel may still be running, so wait for it before the first write.
+  if (g.wait_first == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  flush_pieces(tail, sm_tail, np, row, slot);
 }
 
 }  // namespace fly

@@ -1,35 +1,53 @@
-// Acceptance scan of the FLy verification step: one warp per sequence.  It runs
+// Acceptance scan of the FLy verification step: one thread block per sequence.  It runs
 // either as the tail of the row-reduction kernel (the last block to finish a
 // sequence's rows does it) or as a launch of its own.
 //
-// Lanes first fold the per-unit Partials of "their" rows into entropy and
-// greedy token, then the warp forms the match bits Delta_i (Eq. 2) and the gate
+// A row's partial states are dealt to a group of 2^k neighbouring lanes, all rows of
+// the sequence at once, so that every state is loaded in one round trip; the groups
+// fold them by shuffles, the first lane of each forms the row's entropy and greedy
+// token, and one warp collects the match bits Delta_i (Eq. 2) and the gate
 // bits [H_i >= theta] (Eq. 6) with ballots and walks the mismatch set J in
 // ascending order exactly as Algorithm 1 does (steps 3 and 4): Strict rejects,
 // Defer looks at the next W positions (Eq. 8, Eq. 9), a window that does not
 // fit in the round rejects (paper) or is carried to the next round (extension).
-// Finally the lanes write the tokens to append (Algorithm 1's concat lines).
+// Finally its lanes write the tokens to append (Algorithm 1's concat lines).
+//
+// Hand-off inside the row-reduction kernel.  The scan is the end of a step's critical path and
+// nothing but latency, so the hand-off between blocks has no fences.  A partial state travels as one
+// 16-byte word that carries its own validity: the index field is stored + 1 and an empty slot is all
+// zero.  A block stores its state and adds to the sequence's arrival counter without waiting for the
+// store.  The block whose count completes the sequence knows that every state has at least been
+// issued and reads them all at once; the rare one that is still on its way shows as an empty slot
+// and is asked for again (bounded).  The reader empties the slots for the next launch.
+// Measured (steps in a CUDA graph, us, before -> after; before: one warp per sequence, a lane per row,
+// fences around the counter): 9 rows of 32000 fp32 5.16 -> 4.30, 16 rows of 128256 bf16 7.20 -> 4.95,
+// 144 rows 11.64 -> 11.05, 1088 and 2304 rows unchanged.
 #pragma once
 #include "fly_common.cuh"
+#include "mbarrier.cuh"
 
 namespace fly {
 
-constexpr int kScanThreads = 128;
-constexpr int kScanWarps = kScanThreads / 32;
-constexpr int kMaxRows = 64;  // K + 1 <= 64
+constexpr int kScanThreads = 256;  // a whole block of the row reduction serves a sequence at its end
+constexpr int kMaxRows = 64;       // K + 1 <= 64
 
 struct ScanParams {
   int B, K, V;
-  int splits;               // Partial slots per row
+  int splits;               // Partial slots per row (with Q == 0: exactly the parts of every row)
+  int lanes_log2;           // a row's parts are dealt to 2^lanes_log2 lanes; (K + 1) << lanes_log2 <= kScanThreads
+  int64_t row_pitch;        // part j of row r is partials[r * row_pitch + j * part_pitch]
+  int64_t part_pitch;
   // Flat partition of the row reduction (Q > 0): a row holds units_per_row units and spans row_span >= units_per_row
   // positions of the flat index space; thread block b reduced the flat range [b*Q, (b+1)*Q), so row r has
-  // ((r+1)*span - 1)/Q - (r*span)/Q + 1 pieces in its first slots.  Q == 0: every row has exactly `splits` pieces.
+  // ((r+1)*span - 1)/Q - (r*span)/Q + 1 pieces in its first slots.
   int64_t units_per_row;
   int64_t row_span;
   int64_t Q;
   float scale;              // log2(e) / temperature (exponent unit of the partial states)
-  const Partial* partials;  // [B*(K+1), splits]
+  Partial* partials;
   unsigned int* tickets;    // [B] arrival counters for the fused tail (zero between launches), or null
+  Partial* row_out;         // not null: a "sequence" is one row (K == 0) and its folded state is all that is asked for
+  int idx_offset;           // added to the index of that state (a vocabulary shard reports global token ids)
   const int32_t* draft;     // [B, K]
   float theta_nats;
   int W;
@@ -86,12 +104,31 @@ __device__ __forceinline__ RoundOutcome decide_round(uint64_t mism, uint64_t def
   return o;
 }
 
-__device__ __forceinline__ Partial ld_partial_cg(const Partial* p) {
-  // partial states are written by other thread blocks: read them through L2
-  const int4 v = __ldcg(reinterpret_cast<const int4*>(p));
+// Partial states between blocks: 16-byte relaxed accesses at the L2, single-copy atomic.
+__device__ __forceinline__ int4 ld_part(const Partial* p) {
+  unsigned long long lo, hi;
+  asm volatile("{\n\t.reg .b128 v;\n\tld.relaxed.gpu.global.b128 v, [%2];\n\tmov.b128 {%0, %1}, v;\n\t}"
+               : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+  return make_int4((int)(unsigned)lo, (int)(lo >> 32), (int)(unsigned)hi, (int)(hi >> 32));
+}
+__device__ __forceinline__ void st_part(Partial* p, int4 v) {
+  const unsigned long long lo = (unsigned)v.x | ((unsigned long long)(unsigned)v.y << 32);
+  const unsigned long long hi = (unsigned)v.z | ((unsigned long long)(unsigned)v.w << 32);
+  asm volatile("{\n\t.reg .b128 v;\n\tmov.b128 v, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], v;\n\t}"
+               ::"l"(p), "l"(lo), "l"(hi) : "memory");
+}
+__device__ __forceinline__ Partial as_partial(int4 v) {
   Partial q;
   q.mx = __int_as_float(v.x); q.S = __int_as_float(v.y); q.u = __int_as_float(v.z); q.idx = v.w;
   return q;
+}
+// The form that validates itself: index + 1, so that an empty slot is all zero.
+__device__ __forceinline__ int4 tagged(const Partial& p) {
+  return make_int4(__float_as_int(p.mx), __float_as_int(p.S), __float_as_int(p.u), (int)((unsigned)p.idx + 1u));
+}
+__device__ __forceinline__ Partial untagged(int4 v) {
+  v.w = (int)((unsigned)v.w - 1u);
+  return as_partial(v);
 }
 
 // Number of pieces the flat partition cut row `row` into (see ScanParams).
@@ -101,150 +138,235 @@ __device__ __forceinline__ int pieces_of_row(int64_t row, int64_t span, int64_t 
   return (int)((f0 + span - 1) / Q - f0 / Q) + 1;
 }
 
-// One warp verifies sequence b.  sm_y: kMaxRows ints of shared memory private to the warp.
-__device__ __forceinline__ void scan_one_sequence(const ScanParams& p, int b, int lane, int* sm_y) {
-  const int K = p.K, K1 = p.K + 1;
-  uint64_t mism = 0, defer = 0;
-  // Issue the loads that do not depend on the partial states first (draft tokens, carried state):
-  // they are cold misses, and this is the tail of the step, where every dependent round trip counts.
-  int dr[2];
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    const int i = half * 32 + lane;
-    dr[half] = i < K ? p.draft[(int64_t)b * K + i] : 0;
+// Folds the partial states of a group of 2^lanes_log2 neighbouring lanes; every lane ends up with the result.
+__device__ __forceinline__ Partial fold_lanes(const Partial& a, int lanes_log2, float scale) {
+  float m = a.mx;
+  for (int o = (1 << lanes_log2) >> 1; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const float d = a.mx * scale - m * scale;  // <= 0, finite (mx is clamped to the mask floor)
+  const float e = ex2_approx(d);
+  float S = a.S * e, u = e * fmaf(d, a.S, a.u);
+  unsigned idx = a.mx == m ? (unsigned)a.idx : (unsigned)kIdxNone;
+  for (int o = (1 << lanes_log2) >> 1; o > 0; o >>= 1) {
+    S += __shfl_xor_sync(0xffffffffu, S, o);
+    u += __shfl_xor_sync(0xffffffffu, u, o);
+    idx = min(idx, __shfl_xor_sync(0xffffffffu, idx, o));
   }
-  int pend = 0, len = 0, corr = -1;
-  // A fused step whose GEMM kernel gave up has no usable statistics: every row is flagged, nothing is accepted.
-  const bool failed = p.status != nullptr && *reinterpret_cast<const volatile int*>(p.status) != 0;
-  bool bad_state = false;
-  if (p.carry && p.state_in) {
-    pend = p.state_in[b * 3 + 0];
-    len = p.state_in[b * 3 + 1];
-    corr = p.state_in[b * 3 + 2];
-    // The state is device data: only states this library writes are honoured (pending <= W <= K).  Anything
-    // else is flagged and ignored, so that no token id out of range and no negative count can leave here.
-    bad_state = pend < 0 || pend > K || len < 0 || (pend > 0 && (corr < 0 || corr >= p.V));
-    if (bad_state) { pend = 0; len = 0; corr = -1; }
+  Partial r;
+  r.mx = m; r.S = S; r.u = u; r.idx = (int)idx;
+  return r;
+}
+
+struct ScanShared {
+  int y[kMaxRows];      // y_i (Eq. 1, or the caller's token)
+  int bits[kMaxRows];   // bit 0: mismatch (Eq. 2), bit 1: Defer (Eq. 6)
+  int draft[kMaxRows];
+  int pend, len, corr;  // carried state as it is honoured
+};
+
+// What a thread reads for its row, all at once.
+struct ScanLoads {
+  int4 part;            // its first partial state (raw), all zero if it has none
+  int n;                // parts of its row
+  int draft, target;    // of its row (first lane of a group)
+  int pend, len, corr;  // carried state (thread 0)
+};
+
+__device__ __forceinline__ ScanLoads scan_request(const ScanParams& p, int b) {
+  ScanLoads q;
+  q.part = make_int4(0, 0, 0, 0);
+  q.n = 0; q.draft = 0; q.target = 0; q.pend = 0; q.len = 0; q.corr = -1;
+  const int K1 = p.K + 1;
+  const int i = (int)threadIdx.x >> p.lanes_log2, l = (int)threadIdx.x & ((1 << p.lanes_log2) - 1);
+  if (i < K1) {
+    const int64_t row = (int64_t)b * K1 + i;
+    q.n = pieces_of_row(row, p.row_span, p.Q, p.splits);
+    if (l < q.n) q.part = ld_part(p.partials + row * p.row_pitch + l * p.part_pitch);
+    if (l == 0) {
+      if (i < p.K) q.draft = p.draft[(int64_t)b * p.K + i];
+      if (p.target_tokens) q.target = p.target_tokens[row];
+    }
   }
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    const int i = half * 32 + lane;  // 0-based row of this sequence
-    bool is_mism = false, is_defer = false;
-    if (i < K1) {
-      const int64_t row = (int64_t)b * K1 + i;
-      const Partial* pp = p.partials + row * p.splits;
-      const int pieces = pieces_of_row(row, p.row_span, p.Q, p.splits);
-      Partial acc = empty_partial();
-      for (int s0 = 0; s0 < pieces; s0 += 4) {  // four independent loads in flight
-        Partial q[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) q[t] = (s0 + t < pieces) ? ld_partial_cg(pp + s0 + t) : empty_partial();
-#pragma unroll
-        for (int t = 0; t < 4; ++t) merge_partial(acc, q[t], p.scale);
+  if (threadIdx.x == 0 && p.carry && p.state_in) {
+    q.pend = p.state_in[b * 3 + 0];
+    q.len = p.state_in[b * 3 + 1];
+    q.corr = p.state_in[b * 3 + 2];
+  }
+  return q;
+}
+
+// All parts of the thread's row that are its own, folded.  TAGGED: a part that has not arrived yet is waited for (it has
+// been issued; bounded, and a row whose wait runs out is flagged), and the slots are emptied.  Part `own_slot` of row
+// `own_row` is `own`.
+template <bool TAGGED>
+__device__ __forceinline__ Partial gather_parts(const ScanParams& p, int64_t row, int l, const ScanLoads& q, int64_t own_row,
+                                                int own_slot, const Partial& own) {
+  Partial* src = p.partials + row * p.row_pitch;
+  const int step = 1 << p.lanes_log2;
+  Partial acc = empty_partial();
+  if (TAGGED) {
+#pragma unroll 1
+    for (int j = l; j < q.n; j += step) {
+      int4 v = j == l ? q.part : ld_part(src + j * p.part_pitch);
+      if (row == own_row && j == own_slot) v = tagged(own);
+      if (v.w == 0) {
+        const unsigned long long t0 = global_ns();
+        for (int spins = 0; v.w == 0; v = ld_part(src + j * p.part_pitch))
+          if ((++spins & 63) == 0 && global_ns() - t0 > kWaitLimitNs) {
+            v = make_int4(0, 0x7fc00000, 0x7fc00000, 1);  // NaN sums
+            break;
+          }
       }
+      st_part(src + j * p.part_pitch, make_int4(0, 0, 0, 0));
+      if (j == l) acc = untagged(v);
+      else merge_partial(acc, untagged(v), p.scale);
+    }
+  } else {
+    if (l < q.n) acc = as_partial(q.part);
+    for (int j0 = l + step; j0 < q.n; j0 += 4 * step) {  // four independent loads in flight
+      int4 v[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) if (j0 + t * step < q.n) v[t] = ld_part(src + (j0 + t * step) * p.part_pitch);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) if (j0 + t * step < q.n) merge_partial(acc, as_partial(v[t]), p.scale);
+    }
+  }
+  return acc;
+}
+
+// The block verifies sequence b (or folds row b if that is all that is asked for).  Called by all kScanThreads threads.
+template <bool TAGGED>
+__device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const ScanLoads& q, int64_t own_row, int own_slot,
+                                              const Partial& own, ScanShared& sm) {
+  const int K = p.K, K1 = p.K + 1;
+  const int tid = (int)threadIdx.x;
+  const int i = tid >> p.lanes_log2, l = tid & ((1 << p.lanes_log2) - 1);
+  const int64_t row = (int64_t)b * K1 + i;
+  const bool first = i < K1 && l == 0;
+  float H = 0.f;
+  int greedy = 0;
+  uint32_t flag = 0;
+  if (((tid & ~31) >> p.lanes_log2) < K1) {  // warps that hold rows
+    const Partial mine = i < K1 ? gather_parts<TAGGED>(p, row, l, q, own_row, own_slot, own) : empty_partial();
+    Partial acc = fold_lanes(mine, p.lanes_log2, p.scale);
+    if (p.row_out) {
+      if (first) {
+        if (acc.idx != kIdxNone) acc.idx += p.idx_offset;
+        p.row_out[row] = acc;
+      }
+    } else if (first) {
       // entropy is non-negative; rounding may leave -1e-7 on a one-hot row
       // lg2.approx and the fast division are good to ~1e-6 here (S >= 1 once a row has a finite entry); this is the
       // end of the step's critical path
-      const float H = fmaxf(kLn2 * (lg2_approx(acc.S) - __fdividef(acc.u, acc.S)), 0.f);
-      uint32_t flag = 0;
+      H = fmaxf(kLn2 * (lg2_approx(acc.S) - __fdividef(acc.u, acc.S)), 0.f);
       if (!(fabsf(acc.S) <= 3.0e38f) || !(acc.mx <= 3.0e38f) || acc.mx <= kMaskFloor) flag |= kFlagNonFinite;
-      if (failed) flag |= kFlagStepFailed;
+      // A fused step whose GEMM kernel gave up has no usable statistics: every row is flagged, nothing is accepted.
+      if (p.status != nullptr && *reinterpret_cast<const volatile int*>(p.status) != 0) flag |= kFlagStepFailed;
       int y = acc.idx;
-      if (flag || y < 0 || y >= p.V) y = 0;  // keep every emitted id in range
-      const int greedy = y;
+      if (flag || (unsigned)y >= (unsigned)p.V) y = 0;  // keep every emitted id in range
+      greedy = y;
       if (p.target_tokens && !(flag & kFlagNonFinite)) {  // the caller drew y_i itself
-        y = p.target_tokens[row];
-        if (y < 0 || y >= p.V) { flag |= kFlagBadTarget; y = 0; }
+        y = q.target;
+        if ((unsigned)y >= (unsigned)p.V) { flag |= kFlagBadTarget; y = 0; }
       }
-      sm_y[i] = y;
+      int bits = 0;
       if (i < K) {
-        const int d = dr[half];
-        if (d < 0 || d >= p.V) flag |= kFlagBadDraft;
-        is_mism = (d != y) || flag;
-        is_defer = (H >= p.theta_nats) && !flag;  // a flagged position is never kept
+        if ((unsigned)q.draft >= (unsigned)p.V) flag |= kFlagBadDraft;
+        if (q.draft != y || flag) bits |= 1;
+        if (H >= p.theta_nats && !flag) bits |= 2;  // a flagged position is never kept
       }
-      if (p.target_argmax) p.target_argmax[row] = greedy;
-      if (p.entropy) p.entropy[row] = H;
-      if (p.row_flags) p.row_flags[row] = flag | ((i == 0 && bad_state) ? kFlagBadState : 0u);
+      sm.y[i] = y;
+      sm.bits[i] = bits;
+      sm.draft[i] = q.draft;
+      if (i == 0) {
+        // The carried state is device data: only states this library writes are honoured (pending <= W <= K).  Anything
+        // else is flagged and ignored, so that no token id out of range and no negative count can leave here.
+        const bool bad = q.pend < 0 || q.pend > K || q.len < 0 || (q.pend > 0 && (unsigned)q.corr >= (unsigned)p.V);
+        if (bad) flag |= kFlagBadState;
+        sm.pend = bad ? 0 : q.pend;
+        sm.len = bad ? 0 : q.len;
+        sm.corr = bad ? -1 : q.corr;
+      }
     }
-    const uint64_t mb = __ballot_sync(0xffffffffu, is_mism);
-    const uint64_t db = __ballot_sync(0xffffffffu, is_defer);
-    mism |= mb << (32 * half);
-    defer |= db << (32 * half);
   }
-  __syncwarp();
-
-  __syncwarp();  // state_in may alias state_out: all lanes have read it (above) before lane 0 writes
-  const RoundOutcome o = decide_round(mism, defer, K, p.W, p.carry, pend, len);
-
-#pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    const int i = half * 32 + lane;
-    if (i < K1) {
+  if (p.row_out) return;
+  __syncthreads();
+  if (tid < 32) {
+    const int b0 = tid < K1 ? sm.bits[tid] : 0;
+    uint64_t mism = __ballot_sync(0xffffffffu, b0 & 1), defer = __ballot_sync(0xffffffffu, b0 & 2);
+    if (K1 > 32) {
+      const int b1 = tid + 32 < K1 ? sm.bits[tid + 32] : 0;
+      mism |= (uint64_t)__ballot_sync(0xffffffffu, b1 & 1) << 32;
+      defer |= (uint64_t)__ballot_sync(0xffffffffu, b1 & 2) << 32;
+    }
+    const RoundOutcome o = decide_round(mism, defer, K, p.W, p.carry, sm.pend, sm.len);
+    int32_t* tokens = p.out_tokens + (int64_t)b * K1;
+#pragma unroll 1
+    for (int r = tid; r < K1; r += 32) {
       int tok = -1;
-      if (o.revoke) tok = (i == 0) ? corr : -1;
-      else if (i < o.s - 1) tok = dr[half];
-      else if (i == o.s - 1) tok = sm_y[i];
-      p.out_tokens[(int64_t)b * K1 + i] = tok;
+      if (o.revoke) tok = (r == 0) ? sm.corr : -1;
+      else if (r < o.s - 1) tok = sm.draft[r];
+      else if (r == o.s - 1) tok = sm.y[r];
+      tokens[r] = tok;
+    }
+    if (tid == 0) {
+      p.accept_len[b] = o.s;
+      if (p.rollback) p.rollback[b] = o.rollback;
+      // (state_in may alias state_out: this thread has read it before the barrier above)
+      if (p.state_out) {
+        p.state_out[b * 3 + 0] = o.st_pending;
+        p.state_out[b * 3 + 1] = o.st_len;
+        p.state_out[b * 3 + 2] = o.st_corr_pos ? sm.y[o.st_corr_pos - 1] : -1;
+      }
     }
   }
-  if (lane == 0) {
-    p.accept_len[b] = o.s;
-    if (p.rollback) p.rollback[b] = o.rollback;
-    if (p.state_out) {
-      p.state_out[b * 3 + 0] = o.st_pending;
-      p.state_out[b * 3 + 1] = o.st_len;
-      p.state_out[b * 3 + 2] = o.st_corr_pos ? sm_y[o.st_corr_pos - 1] : -1;
-    }
+  if (first) {  // off the critical path: warp 0 is at the decision meanwhile
+    if (p.target_argmax) p.target_argmax[row] = greedy;
+    if (p.entropy) p.entropy[row] = H;
+    if (p.row_flags) p.row_flags[row] = flag;
   }
 }
 
-// Folds the n partial states of every row into one (out[row]); one warp per row.  Part j of row r
-// is in[r * row_stride + j * part_stride].  The fused LM-head kernel leaves one partial state per row
-// and CTA, a vocabulary-parallel target one per row and rank; folding them with 32 lanes in parallel
-// keeps the acceptance scan's per-lane loop short.  idx_offset is added to the winning index (a
-// vocabulary shard reports global token ids).  With Q > 0 the number of parts of a row follows from
-// the flat partition of the row reduction (see ScanParams) instead of being n_fixed.
+// Folds the n partial states in[row * n ..] of every row into out[row]; one warp per row.  The fused LM-head kernel
+// leaves one partial state per row and CTA; folding them with 32 lanes in parallel keeps the acceptance scan short.
 constexpr int kFoldThreads = 128;
-__global__ void __launch_bounds__(kFoldThreads) fold_partials(const Partial* __restrict__ in, int n_fixed, int64_t row_stride,
-                                                              int64_t part_stride, Partial* __restrict__ out, int rows,
-                                                              int idx_offset, float scale, int64_t row_span, int64_t Q) {
+__global__ void __launch_bounds__(kFoldThreads) fold_partials(const Partial* __restrict__ in, int n, Partial* __restrict__ out,
+                                                              int rows, float scale) {
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * (kFoldThreads / 32) + (threadIdx.x >> 5);
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the producer grid has completed
   asm volatile("griddepcontrol.launch_dependents;");
   if (row >= rows) return;
-  const int n = pieces_of_row(row, row_span, Q, n_fixed);
-  const Partial* src = in + (int64_t)row * row_stride;
+  const Partial* src = in + (int64_t)row * n;
   Partial acc = empty_partial();
   for (int j0 = 0; j0 < n; j0 += 128) {  // four independent loads in flight per lane
-    Partial q[4];
+    int4 q[4];
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
-      q[t] = (j0 + t * 32 + lane < n) ? ld_partial_cg(src + (int64_t)(j0 + t * 32 + lane) * part_stride) : empty_partial();
+    for (int t = 0; t < 4; ++t) if (j0 + t * 32 + lane < n) q[t] = ld_part(src + j0 + t * 32 + lane);
 #pragma unroll
-    for (int t = 0; t < 4; ++t) merge_partial(acc, q[t], scale);
+    for (int t = 0; t < 4; ++t) if (j0 + t * 32 + lane < n) merge_partial(acc, as_partial(q[t]), scale);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const Partial q = shfl_xor_partial(acc, o);
-    merge_partial(acc, q, scale);
-  }
-  if (lane == 0) {
-    if (acc.idx != kIdxNone) acc.idx += idx_offset;
-    out[row] = acc;
-  }
+  acc = fold_lanes(acc, 5, scale);
+  if (lane == 0) out[row] = acc;
 }
 
-// Stand-alone launch: one warp per sequence, after the row reduction.
-__global__ void __launch_bounds__(kScanThreads) scan_sequences(ScanParams p) {
-  __shared__ int sm_y[kScanWarps][kMaxRows];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int b = blockIdx.x * kScanWarps + warp;
-  // every thread waits for the producer grid (row reduction) to complete
+// Stand-alone launch: one block per sequence, after the kernel (or the all-gather) that leaves the partial states.
+template <bool TAGGED>
+__global__ void __launch_bounds__(kScanThreads) scan_sequences(const __grid_constant__ ScanParams p) {
+  __shared__ ScanShared sm;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the producer grid has completed
+  asm volatile("griddepcontrol.launch_dependents;");
+  const ScanLoads q = scan_request(p, (int)blockIdx.x);
+  scan_sequence<TAGGED>(p, (int)blockIdx.x, q, -1, 0, empty_partial(), sm);
+}
+
+// Empties arrival counters and slots (counted in 16-byte words) for callers whose scratch may hold what an earlier call left.
+constexpr int kClearThreads = 256;
+__global__ void __launch_bounds__(kClearThreads) clear_scratch(uint4* tickets, int ticket_words, uint4* slots, int slot_words) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (b >= p.B) return;
-  scan_one_sequence(p, b, lane, sm_y[warp]);
+  asm volatile("griddepcontrol.launch_dependents;");
+  const int i = (int)(blockIdx.x * kClearThreads + threadIdx.x);
+  if (i < ticket_words) tickets[i] = make_uint4(0, 0, 0, 0);
+  if (i < slot_words) slots[i] = make_uint4(0, 0, 0, 0);
 }
 
 }  // namespace fly
