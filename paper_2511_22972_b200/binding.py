@@ -1,4 +1,5 @@
-"""ctypes binding of the C ABI in include/fly_verify.h.
+"""Binding of the C ABI in include/fly_verify.h: ctypes for what is called once, the native extension
+(csrc/native_binding.cpp) for what is called every step.
 
 Argument marshalling only: every step of the verification runs in the CUDA
 kernels of libfly_verify.so.  There is no CPU fallback; a missing library that
@@ -7,8 +8,7 @@ cannot be built raises ImportError.
 from __future__ import annotations
 
 import ctypes as C
-import math
-from typing import Optional
+import importlib.util
 
 from . import build as _build
 
@@ -61,16 +61,24 @@ class FlyError(RuntimeError):
 
 
 _lib = None
+_native = None
 
 
 def lib() -> C.CDLL:
     """Loads (building first if a source is newer) libfly_verify.so."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     try:
         path = _build.ensure_built()
         L = C.CDLL(path)
+        import torch  # noqa: F401  (the extension resolves its symbols in torch's libraries)
+        spec = importlib.util.spec_from_file_location(__package__ + "._native", _build.NATIVE_PATH)
+        native = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(native)
+        native.init(*[C.cast(getattr(L, f), C.c_void_p).value for f in (
+            "fly_verify_run", "fly_verify_run_host", "fly_verify_reduce_shard", "fly_verify_run_partials",
+            "fly_verify_run_static", "fly_pld_draft")])
     except Exception as e:  # no silent fallback: the CUDA library is the product
         raise ImportError(f"libfly_verify.so is missing and could not be built: {e}") from e
     L.fly_verify_create.argtypes = [C.POINTER(fly_verify_config_t), C.POINTER(C.c_void_p)]
@@ -107,19 +115,13 @@ def lib() -> C.CDLL:
     L.fly_verify_last_cuda_error.restype = C.c_int32
     L.fly_status_string.argtypes = [C.c_int]
     L.fly_status_string.restype = C.c_char_p
+    _native = native
     _lib = L
     return L
 
 
 def status_string(status: int) -> str:
     return lib().fly_status_string(int(status)).decode()
-
-
-def _ptr(t) -> Optional[int]:
-    """Address of a torch tensor's storage (device or host), None for None."""
-    if t is None:
-        return None
-    return int(t.data_ptr())
 
 
 class FlyVerify:
@@ -132,6 +134,7 @@ class FlyVerify:
     def __init__(self, max_batch: int, max_k: int, vocab: int, dtype: str = "bf16", device: int = 0,
                  hidden: int = 0):
         self._h = C.c_void_p()
+        self.weight_vd = False
         self.vocab = int(vocab)
         self.dtype = dtype
         cfg = fly_verify_config_t(int(device), int(max_batch), int(max_k), int(vocab),
@@ -140,6 +143,9 @@ class FlyVerify:
         if st != FLY_OK:
             self._h = C.c_void_p()
             raise FlyError(st, "fly_verify_create")
+
+    def _raise(self, status: int, what: str):
+        raise FlyError(status, what, lib().fly_verify_last_cuda_error(self._h))
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
@@ -175,19 +181,15 @@ class FlyVerify:
     def reduce_shard(self, logits, vocab_offset: int, partial_out, stream: int = 0, temperature: float = 0.0):
         """fly_verify_reduce_shard: logits [rows, vocab_slice] (a strided view is fine) -> partial_out
         [rows, 4] (any 16-byte element type, e.g. float32 x 4)."""
-        rows = logits.shape[0]
-        assert logits.shape[1] == self.vocab and logits.stride(1) == 1
-        st = lib().fly_verify_reduce_shard(self._h, int(rows), _ptr(logits), int(logits.stride(0)), int(vocab_offset),
-                                           float(temperature), _ptr(partial_out), C.c_void_p(stream))
-        if st != FLY_OK:
-            raise FlyError(st, "fly_verify_reduce_shard", lib().fly_verify_last_cuda_error(self._h))
+        st = _native.reduce_shard(self._h.value or 0, self.vocab, logits, vocab_offset, partial_out, stream or 0, temperature)
+        if st:
+            self._raise(st, "fly_verify_reduce_shard")
 
     def run_partials(self, args: fly_verify_args_t, partials, world: int, total_vocab: int, stream: int = 0):
         """fly_verify_run_partials: partials [world, rows, 4] gathered from the ranks."""
-        st = lib().fly_verify_run_partials(self._h, C.byref(args), _ptr(partials), int(world), int(total_vocab),
-                                           C.c_void_p(stream))
-        if st != FLY_OK:
-            raise FlyError(st, "fly_verify_run_partials", lib().fly_verify_last_cuda_error(self._h))
+        st = _native.run_partials(self._h.value or 0, C.addressof(args), partials, world, total_vocab, stream or 0)
+        if st:
+            self._raise(st, "fly_verify_run_partials")
 
     def selftest_wait(self, stream: int = 0) -> int:
         """fly_verify_selftest_wait: makes one bounded device-side wait run out on purpose (no fault)."""
@@ -202,33 +204,22 @@ class FlyVerify:
                   state_out=None, rollback=None, target_argmax=None, entropy=None, row_flags=None,
                   target_tokens=None, temperature=0.0, inputs_ready=False):
         a = fly_verify_args_t()
-        a.B, a.K = int(B), int(K)
-        a.logits, a.row_stride = _ptr(logits), int(row_stride)
-        a.hidden, a.weight = _ptr(hidden), _ptr(weight)
-        a.draft = _ptr(draft)
-        a.theta = float(theta)
-        a.theta_unit = FLY_THETA_NATS if theta_unit == "nats" else FLY_THETA_NORMALIZED
-        a.W = int(W)
-        a.boundary = FLY_BOUNDARY_CARRY if boundary == "carry" else FLY_BOUNDARY_REJECT
-        a.state_in, a.state_out = _ptr(state_in), _ptr(state_out)
-        a.accept_len, a.rollback, a.out_tokens = _ptr(accept_len), _ptr(rollback), _ptr(out_tokens)
-        a.target_argmax, a.entropy, a.row_flags = _ptr(target_argmax), _ptr(entropy), _ptr(row_flags)
-        a.target_tokens = _ptr(target_tokens)
-        a.temperature = float(temperature)
-        a.inputs_ready = 1 if inputs_ready else 0
+        _native.fill(C.addressof(a), B, K, draft, accept_len, out_tokens, logits, row_stride, hidden, weight, theta,
+                     theta_unit, W, boundary, state_in, state_out, rollback, target_argmax, entropy, row_flags,
+                     target_tokens, temperature, inputs_ready)
         return a
 
     def run(self, args: fly_verify_args_t, stream: int = 0):
         """fly_verify_run: device buffers, asynchronous on `stream` (a raw cudaStream_t value)."""
-        st = lib().fly_verify_run(self._h, C.byref(args), C.c_void_p(stream))
-        if st != FLY_OK:
-            raise FlyError(st, "fly_verify_run", lib().fly_verify_last_cuda_error(self._h))
+        st = _native.run(self._h.value or 0, C.addressof(args), stream or 0, False)
+        if st:
+            self._raise(st, "fly_verify_run")
 
     def run_host(self, args: fly_verify_args_t, stream: int = 0):
         """fly_verify_run_host: host buffers, copies in and out, synchronises."""
-        st = lib().fly_verify_run_host(self._h, C.byref(args), C.c_void_p(stream))
-        if st != FLY_OK:
-            raise FlyError(st, "fly_verify_run_host", lib().fly_verify_last_cuda_error(self._h))
+        st = _native.run(self._h.value or 0, C.addressof(args), stream or 0, True)
+        if st:
+            self._raise(st, "fly_verify_run_host")
 
 
 def run_static(args: fly_verify_args_t, vocab: int, dtype: str = "bf16", device: int = 0, stream: int = 0):
@@ -236,29 +227,25 @@ def run_static(args: fly_verify_args_t, vocab: int, dtype: str = "bf16", device:
     device memory (its scratch is a fixed array inside the library).  `args` is the same struct that
     FlyVerify.run takes; `static_args` fills one without needing a handle.  Calls on one device must not
     overlap on the GPU."""
-    st = lib().fly_verify_run_static(int(device), int(vocab), FLY_BF16 if dtype == "bf16" else FLY_F32,
-                                     C.byref(args), C.c_void_p(stream))
-    if st != FLY_OK:
+    lib()  # (no handle has loaded it for the caller)
+    st = _native.run_static(C.addressof(args), vocab, FLY_BF16 if dtype == "bf16" else FLY_F32, device, stream or 0)
+    if st:
         raise FlyError(st, "fly_verify_run_static")
 
 
 def pld_draft(tokens, lengths, K: int, max_ngram: int = 3, min_ngram: int = 1, device: int = 0, stream: int = 0):
     """fly_pld_draft on tokens [B, Lmax] int32 and lengths [B] int32 (device tensors).  Returns
     (draft [B, K], count [B], match_pos [B], match_ngram [B]) as new device tensors."""
-    import torch
-    B = tokens.shape[0]
-    assert tokens.dtype == torch.int32 and lengths.dtype == torch.int32 and tokens.stride(1) == 1
-    draft = torch.empty(B, K, dtype=torch.int32, device=tokens.device)
-    count, pos, ng = (torch.empty(B, dtype=torch.int32, device=tokens.device) for _ in range(3))
-    st = lib().fly_pld_draft(int(device), int(B), _ptr(tokens), int(tokens.stride(0)), _ptr(lengths), int(max_ngram),
-                             int(min_ngram), int(K), _ptr(draft), _ptr(count), _ptr(pos), _ptr(ng), C.c_void_p(stream))
-    if st != FLY_OK:
+    lib()
+    st, draft, count, pos, ng = _native.pld_draft(tokens, lengths, K, max_ngram, min_ngram, device, stream or 0)
+    if st:
         raise FlyError(st, "fly_pld_draft")
     return draft, count, pos, ng
 
 
 def static_args(*a, **kw) -> fly_verify_args_t:
     """Fills a fly_verify_args_t (same parameters as FlyVerify.make_args) without creating a handle."""
+    lib()
     return FlyVerify.make_args(None, *a, **kw)
 
 
@@ -295,15 +282,10 @@ def verify(fv: FlyVerify, logits, draft, out: VerifyBuffers, theta=1.0, W=3, the
            boundary="reject", stream: int = 0, host: bool = False, temperature=0.0, inputs_ready=False):
     """One verification step on logits [B, K+1, V] and draft [B, K] (int32).
     In carry mode out.state is both the carried-in and the carried-out state."""
-    B, K1, V = logits.shape
-    assert V == fv.vocab and logits.stride(2) == 1 and logits.stride(0) == K1 * logits.stride(1)
-    carry = boundary == "carry"
-    a = fv.make_args(B, K1 - 1, draft, out.accept_len, out.out_tokens, logits=logits,
-                     row_stride=logits.stride(1), theta=theta, theta_unit=theta_unit, W=W, boundary=boundary,
-                     state_in=out.state if carry else None, state_out=out.state, rollback=out.rollback,
-                     target_argmax=out.target_argmax, entropy=out.entropy, row_flags=out.row_flags,
-                     temperature=temperature, inputs_ready=inputs_ready)
-    (fv.run_host if host else fv.run)(a, stream)
+    st = _native.verify(fv._h.value or 0, fv.vocab, logits, draft, out, theta, W, theta_unit, boundary, stream or 0, host,
+                        temperature, inputs_ready)
+    if st:
+        fv._raise(st, "fly_verify_run_host" if host else "fly_verify_run")
     return out
 
 
@@ -312,15 +294,8 @@ def verify_fused(fv: FlyVerify, hidden, weight, draft, out: VerifyBuffers, theta
     """One verification step on the fused LM-head path: hidden [B*(K+1), D] bf16 and weight [D, V] bf16
     (device; with host=True hidden, draft and the outputs are host buffers, the weight stays on the device).
     The logits hidden @ weight are formed and reduced inside the kernel and never stored."""
-    B, K = draft.shape
-    rows, D = hidden.shape
-    assert rows == B * (K + 1)
-    assert tuple(weight.shape) == ((fv.vocab, D) if getattr(fv, "weight_vd", False) else (D, fv.vocab))
-    assert hidden.is_contiguous() and weight.is_contiguous()
-    carry = boundary == "carry"
-    a = fv.make_args(B, K, draft, out.accept_len, out.out_tokens, hidden=hidden, weight=weight, theta=theta,
-                     theta_unit=theta_unit, W=W, boundary=boundary, state_in=out.state if carry else None,
-                     state_out=out.state, rollback=out.rollback, target_argmax=out.target_argmax,
-                     entropy=out.entropy, row_flags=out.row_flags, temperature=temperature)
-    (fv.run_host if host else fv.run)(a, stream)
+    st = _native.verify_fused(fv._h.value or 0, fv.vocab, fv.weight_vd, hidden, weight, draft, out, theta, W, theta_unit,
+                              boundary, stream or 0, host, temperature)
+    if st:
+        fv._raise(st, "fly_verify_run_host" if host else "fly_verify_run")
     return out

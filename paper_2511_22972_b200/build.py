@@ -1,8 +1,9 @@
-"""Builds the C-ABI shared library (libfly_verify.so) for sm_100a with nvcc.
+"""Builds the C-ABI shared library (libfly_verify.so) for sm_100a with nvcc,
+and the Python extension that marshals its arguments (_native.so) with g++.
 
-The library is built in-tree, next to this file.  `python -m
-paper_2511_22972_b200.build` rebuilds it; `ensure_built()` rebuilds only when
-a source is newer than the library.
+Both are built in-tree, next to this file.  `python -m
+paper_2511_22972_b200.build` rebuilds them; `ensure_built()` rebuilds only what
+is older than a source.
 """
 from __future__ import annotations
 
@@ -11,12 +12,15 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG_DIR)
 CSRC = os.path.join(PKG_DIR, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB_PATH = os.path.join(PKG_DIR, "libfly_verify.so")
+NATIVE_SRC = os.path.join(CSRC, "native_binding.cpp")
+NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -34,11 +38,23 @@ def _deps():
     return sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
 
 
-def is_stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+def _older(path: str, deps) -> bool:
+    if not os.path.exists(path):
         return True
-    t = os.path.getmtime(LIB_PATH)
-    return any(os.path.getmtime(p) > t for p in _deps())
+    t = os.path.getmtime(path)
+    return any(os.path.getmtime(p) > t for p in deps)
+
+
+def lib_is_stale() -> bool:
+    return _older(LIB_PATH, _deps())
+
+
+def native_is_stale() -> bool:
+    return _older(NATIVE_PATH, [NATIVE_SRC] + glob.glob(os.path.join(INCLUDE, "*.h")))
+
+
+def is_stale() -> bool:
+    return lib_is_stale() or native_is_stale()
 
 
 def nvcc_path() -> str:
@@ -48,21 +64,43 @@ def nvcc_path() -> str:
     return p
 
 
-def build(verbose: bool = False, extra=()) -> str:
-    cmd = [nvcc_path(), *NVCC_FLAGS, *extra, "-I", INCLUDE, "-I", CSRC, "-o", LIB_PATH, *sources()]
+def _run(cmd, what: str, verbose: bool):
     if verbose:
         print(" ".join(cmd), file=sys.stderr)
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + r.stdout + r.stderr)
+        raise RuntimeError(what + " failed:\n" + r.stdout + r.stderr)
     if verbose and (r.stdout or r.stderr):
         print(r.stdout + r.stderr, file=sys.stderr)
+
+
+def build_lib(verbose: bool = False, extra=()) -> str:
+    _run([nvcc_path(), *NVCC_FLAGS, *extra, "-I", INCLUDE, "-I", CSRC, "-o", LIB_PATH, *sources()], "nvcc", verbose)
     return LIB_PATH
 
 
+def build_native(verbose: bool = False) -> str:
+    import torch
+    root = os.path.dirname(torch.__file__)
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], INCLUDE]
+    abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
+    _run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={abi}",
+          *[x for i in inc for x in ("-isystem" if i != INCLUDE else "-I", i)], "-o", NATIVE_PATH, NATIVE_SRC,
+          "-L", os.path.join(root, "lib"), "-lc10", "-ltorch_cpu", "-ltorch_python"], "g++", verbose)
+    return NATIVE_PATH
+
+
+def build(verbose: bool = False, extra=()) -> str:
+    build_native(verbose)
+    return build_lib(verbose, extra)
+
+
 def ensure_built() -> str:
-    if is_stale():
-        build()
+    if native_is_stale():
+        build_native()
+    if lib_is_stale():
+        build_lib()
     return LIB_PATH
 
 
