@@ -182,8 +182,8 @@ void fill_launch(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, unsigned gr
   cfg->numAttrs = 1;
 }
 
-// Shared memory of the row reduction's cp.async rings (vector path), per block.
-constexpr int kReduceRingBytes = fly::kReduceWarps * fly::kDepth * kReduceUnroll * 32 * 16;
+// Shared memory of the row reduction's cp.async rings (vector path) and of the slice that each warp keeps, per block.
+constexpr int kReduceRingBytes = fly::kReduceWarps * (fly::kDepth + 1) * kReduceUnroll * 32 * 16;
 
 // ... and as much more as keeps a small grid spread over all SMs: in plain stream order the blocks of a step become
 // resident while the step before still runs, and the hardware would put up to four of them on the SMs that empty first,
