@@ -88,9 +88,9 @@ struct FlatPlan {
   int slots = 1;
   int pieces = 0;     // > 0: every row is cut into exactly this many pieces (span = pieces * Q)
 };
-// Launch shape.  Measured on the bench workloads (9 .. 2304 rows of 128 - 300 KB): whole pieces of rows, one per
-// block, are at least as fast as packed rows whenever they fill the resident slots reasonably well - a row boundary
-// inside a block drains that block's copy ring once, and the hardware scheduler back-fills a second wave well.
+// Launch shape.  Measured on 9 .. 3000 rows of 16 - 300 KB: whole pieces of rows, one per block, are as fast as or
+// faster than packed rows almost everywhere - a row boundary inside a block drains that block's copy ring and costs a
+// block-wide merge - and the hardware scheduler back-fills a second wave well.
 // A block's warps walk its piece in strides of `stride_units` (one slice per warp), so a piece of 3.1 strides costs
 // its slowest warp 4 slices: among the piece counts that fit, the one with the fewest slices on the busiest SM wins.
 //   plain stream order   the grid fits on the device at once (4 blocks per SM); cost = blocks on the busiest SM x
@@ -98,7 +98,13 @@ struct FlatPlan {
 //                        can then already be resident, waiting); more rows than slots: whole rows, several waves
 //   inputs_ready         throughput, not latency: few large pieces (a quarter of a block per SM and step is
 //                        enough, consecutive steps overlap many deep), the count with the fewest slices per row
-//   packed rows          only where whole pieces would leave more than a quarter of the last wave's slots empty
+//   packed rows          where whole pieces would leave more than a quarter of the last wave's slots empty, the
+//                        rows are long, and there are enough of them that no even number of pieces per SM helps.
+//                        128256 bf16, packed / whole rows, us: 297 rows 19.4 / 21.7, 360 21.9 / 21.9, 594 30.3 / 32.5,
+//                        702 35.9 / 37.9; but 216 rows 16.2 / 13.9 (two pieces per row), 432 rows 24.7 / 21.9, and
+//                        50257 or 32000 bf16: 216 rows 11.5 / 9.4 and 9.5 / 6.8, 360 rows 14.4 / 12.4 and 12.0 / 9.7.
+// Pieces hold at least 16 KB, rows of less than 112 KB are cut into up to seven of at least 7 KB: a block that gets
+// less is all fixed cost (9 rows of 32000 bf16: three pieces 4.55, seven 4.1 us).
 int64_t piece_units(int64_t n, int64_t s) {
   int64_t q = (n + s - 1) / s;
   if (s > 1) q = (q + 7) / 8 * 8;  // pieces start on 128-byte boundaries of the row
@@ -109,6 +115,10 @@ FlatPlan plan_flat(int sm_count, int64_t rows, int64_t n, int64_t min_units, int
   FlatPlan pl;
   const int64_t gmax = (int64_t)sm_count * fly::kReduceBlocksPerSM;
   int64_t smax = n / min_units;  // pieces of at least min_units
+  if (smax < 7) {
+    const int64_t fine = n * 16 / (7 * min_units);
+    smax = fine > 7 ? 7 : fine > smax ? fine : smax;
+  }
   if (smax > cap) smax = cap;
   if (smax < 1) smax = 1;
   auto slices = [&](int64_t s) { return (piece_units(n, s) + stride_units - 1) / stride_units; };
@@ -144,8 +154,10 @@ FlatPlan plan_flat(int sm_count, int64_t rows, int64_t n, int64_t min_units, int
     if (s_fill < 1) s_fill = 1;
     const int64_t blocks = rows * s_fill, waves = (blocks + gmax - 1) / gmax;
     const bool could_fill = rows * n / min_units >= gmax;  // enough work for a full grid at all
+    const bool uneven = rows >= gmax || 100 * rows < 92 * ((rows + sm_count - 1) / sm_count) * sm_count;
+    const bool long_rows = n >= 12 * min_units ? rows > 2 * sm_count : n >= 6 * min_units && 2 * rows > 5 * sm_count;
     // (so few waves that a block never holds more than a handful of rows)
-    if (could_fill && 4 * blocks < 3 * waves * gmax && (waves + 1) + 2 <= fly::kMaxPend) {
+    if (could_fill && 4 * blocks < 3 * waves * gmax && uneven && long_rows && (waves + 1) + 2 <= fly::kMaxPend) {
       // the last wave would be mostly empty: pack the rows end to end and cut the range evenly instead
       s = 0;
       const int64_t Qf = (rows * n + gmax - 1) / gmax;
@@ -248,7 +260,10 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   g.pieces = pl.Q < (1 << 30) ? pl.pieces : 0; g.V = V; g.row_stride = row_stride;
   g.scale = scale; g.wait_first = inputs_ready ? 0 : 1;
   tail->splits = pl.slots;
-  tail->row_pitch = pl.slots;
+  // A row's states start on a 128-byte line (a power of two of them) where the scratch has the room.
+  int pitch = 1;
+  while (pitch < pl.slots) pitch *= 2;
+  tail->row_pitch = pitch <= cap ? pitch : pl.slots;
   tail->part_pitch = 1;
   tail->lanes_log2 = lanes_for(pl.slots, tail->K + 1);
   tail->partials = partials;
