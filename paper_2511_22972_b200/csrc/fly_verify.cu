@@ -359,8 +359,14 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     if (!ok) return FLY_ERR_CUDA;
     h->map_w_ptr = a->weight;
   }
-  if (h->map_h_ptr != a->hidden || h->map_h_rows != rows) {
-    if (!encode_map(h, &h->map_h, a->hidden, (uint64_t)D, (uint64_t)rows, (uint64_t)D * 2, L::kBoxPos)) return FLY_ERR_CUDA;
+  // One accumulator takes up to 144 positions; more are shared evenly between two, so that both issuers have the same to do.
+  auto first_half = [](int positions) {
+    const int r16 = (positions + 15) / 16 * 16;
+    return r16 <= L::kHalfN ? r16 : (r16 / 2 + 15) / 16 * 16;
+  };
+  const int box = rows > L::kMaxPos ? L::kBoxPos : first_half((int)rows) / 2;
+  if (h->map_h_ptr != a->hidden || h->map_h_rows != rows) {  // (the box follows from the rows)
+    if (!encode_map(h, &h->map_h, a->hidden, (uint64_t)D, (uint64_t)rows, (uint64_t)D * 2, (uint32_t)box)) return FLY_ERR_CUDA;
     h->map_h_ptr = a->hidden;
     h->map_h_rows = rows;
   }
@@ -370,8 +376,16 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     L::Params p;
     p.R = (int)(rows - row0 < L::kMaxPos ? rows - row0 : L::kMaxPos);
     const int r16 = (p.R + 15) / 16 * 16;
-    p.n0 = r16 < L::kHalfN ? r16 : L::kHalfN;
-    p.n1 = r16 > L::kHalfN ? r16 - L::kHalfN : 0;
+    p.n0 = first_half(p.R);
+    p.n1 = r16 - p.n0;
+    p.box = box;
+    p.stages = L::kRingBytes / (L::kBytesW + (p.n1 > 0 ? 2 : 1) * box * L::kBytesPos);
+    // A weight stored [D, V] is read 128 bytes of a row at a time, the next stage's 64 rows far away: a deeper ring spreads
+    // the requests over more DRAM pages than it gains (36 positions, D = 4096, V = 50264: 6 / 7 / 8 / 10 stages 79.4 / 79.3 /
+    // 80.8 / 82.8 us).  Stored [V, D] the next stage is the next 128 bytes (80.2 / 79.4 / 78.8 / 77.8; at D = 8192 and
+    // V = 128256 344 / 339 / 335 / 328).
+    const int deepest = h->weight_vd ? L::kMaxStages : 7;
+    if (p.stages > deepest) p.stages = deepest;
     p.V = V; p.D = D;
     p.num_tiles = num_tiles;
     p.num_kb = (D + L::kBlockK - 1) / L::kBlockK;
@@ -380,8 +394,11 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     p.scale = exponent_scale(a->temperature);
     p.partials = h->lm_partials;
     p.status = h->lm_status;
-    L::lmhead_verify_kernel<<<grid, L::kThreads, L::kSmemBytes, st>>>(h->map_w, h->map_h, p);
-    cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    fill_launch(&cfg, attr, (unsigned)grid, L::kThreads, st, true);
+    cfg.dynamicSmemBytes = L::kSmemBytes;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, L::lmhead_verify_kernel, h->map_w, h->map_h, p);
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->last_launches++;
   }

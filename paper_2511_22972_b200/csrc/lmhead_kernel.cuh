@@ -11,11 +11,11 @@
 //       weight is [D, V] with V contiguous, so A is MN-major; TMA lays it down as
 //       two boxes of 64 entries (128 bytes) x 64 dims with the 128-byte swizzle.
 //   B = hidden tile, K-major, 128-byte swizzle.  The pair shares it: each CTA
-//       loads HALF of the positions of each accumulator (2 x 72 rows), the MMA
+//       loads HALF of the positions of each accumulator (2 x up to 72 rows), the MMA
 //       reads both halves.  This halves the hidden-state traffic per SM, which is
 //       what bounds a one-CTA version of this kernel (the hidden tile is
 //       re-fetched from L2 for every vocabulary tile).
-//   D = two accumulators of 144 fp32 columns in each CTA: lane = one of the
+//   D = two accumulators of up to 144 fp32 columns in each CTA: lane = one of the
 //       CTA's 128 vocabulary entries, column = position.  Tensor memory holds
 //       THREE such slots (columns 0.., 144.., 288..; 432 of 512) and the
 //       accumulators of consecutive tiles rotate through them: accumulator 0 of
@@ -65,12 +65,15 @@ constexpr int kBlockK = 64;    // hidden dims per stage: one 128-byte swizzle ro
 constexpr int kMmaK = 16;      // hidden dims per tcgen05.mma (bf16)
 constexpr int kHalfN = 144;    // positions per accumulator (MMA N <= 256, multiple of 16)
 constexpr int kMaxPos = 2 * kHalfN;
-constexpr int kStages = 6;     // operand ring: one stage = one 64-dim slice of the weight tile and of the hidden tile
 constexpr int kBytesW = kBlockK * kBlockV * 2;      // 16 KB per stage
 constexpr int kBytesWBox = kBlockK * 64 * 2;        // one TMA box: 64 entries x 64 dims
-constexpr int kBoxPos = kHalfN / 2;                 // positions per TMA box: this CTA's half of one accumulator
-constexpr int kBytesHHalf = kBoxPos * kBlockK * 2;  // 9 KB
-constexpr int kBytesH = 2 * kBytesHHalf;            // both accumulators
+constexpr int kBoxPos = kHalfN / 2;                 // positions per TMA box at most: this CTA's half of one accumulator
+constexpr int kBytesPos = kBlockK * 2;              // one position's 64 dims
+// Operand ring: one stage = one 64-dim slice of the weight tile and of the hidden tile.  A stage takes as much shared
+// memory as its positions need, and the ring as many stages as fit: 6 at 288 positions, 12 at 16.  With few positions
+// the weight stream is the work, and what is in flight bounds it.
+constexpr int kRingBytes = 6 * (kBytesW + 2 * kBoxPos * kBytesPos);
+constexpr int kMaxStages = 12;
 constexpr int kChunk = 16;                          // positions turned through shared memory at a time
 constexpr int kChunks = kMaxPos / kChunk;           // 18 per tile, dealt alternately to the two epilogue groups
 constexpr int kGroupChunks = kChunks / 2;           // 9 per group: the running states one thread holds
@@ -84,23 +87,23 @@ constexpr int kThreads = (kEpiWarps + 4) * 32;
 constexpr int kTmemCols = 512;
 constexpr int kSlots = 3;                           // accumulator slots of kHalfN columns in tensor memory
 static_assert(kSlots * kHalfN <= kTmemCols, "accumulator slots must fit in tensor memory");
-constexpr int kHalfChunks = kHalfN / kChunk;        // 9 blocks of 16 positions per accumulator
 
-constexpr int kOffW = 0;
-constexpr int kOffH = kOffW + kStages * kBytesW;
-constexpr int kOffTurn = kOffH + kStages * kBytesH;
+constexpr int kOffW = 0;  // (the hidden tiles follow the weight tiles)
+constexpr int kOffTurn = kRingBytes;
 constexpr int kOffBar = kOffTurn + kTurnBytes;
-constexpr int kNumBars = 2 * kStages + 2 * kSlots + 1;
+constexpr int kNumBars = 2 * kMaxStages + 2 * kSlots + 1;
 constexpr int kOffMisc = kOffBar + kNumBars * 8;
 constexpr int kSmemBytes = kOffMisc + 32 + 1024;    // + slack to align the base to 1024 bytes
 static_assert(kSmemBytes <= 232448, "shared memory budget of one CTA");
-static_assert(kMaxPos * 8 * 16 <= kStages * kBytesW, "final merge buffer reuses the weight ring");
+static_assert(kMaxPos * 8 * 16 <= 6 * kBytesW, "final merge buffer reuses the weight ring");
 
 constexpr int kErrTimeoutProducer = 1, kErrTimeoutMma = 2, kErrTimeoutEpilogue = 3;
 
 struct Params {
   int R;          // positions handled by this launch (1..288)
   int n0, n1;     // MMA N of the two accumulators (multiples of 16; n1 may be 0)
+  int box;        // positions per TMA box of the hidden tile: n0 / 2, or more
+  int stages;     // of the operand ring
   int V, D;
   int num_tiles;  // ceil(V / 256): tiles of the CTA pairs
   int num_kb;     // ceil(D / 64)
@@ -248,12 +251,12 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   // arrive with the expected byte counts; every TMA load of the pair reports its bytes here).
   // empty(s), in each CTA: the MMAs that read the stage have completed, the producers may refill it.
   auto full = [&](int s) { return bar0 + 8u * s; };
-  auto empty = [&](int s) { return bar0 + 8u * (kStages + s); };
+  auto empty = [&](int s) { return bar0 + 8u * (kMaxStages + s); };
   // slot_full(i), in each CTA: the accumulator in tensor-memory slot i is complete.  slot_empty(i), in the leader:
   // the epilogue threads of both CTAs have read slot i out, the next accumulator may be formed there.
-  auto slot_full = [&](int i) { return bar0 + 8u * (2 * kStages + i); };
-  auto slot_empty = [&](int i) { return bar0 + 8u * (2 * kStages + kSlots + i); };
-  const uint32_t drain_bar = bar0 + 8u * (2 * kStages + 2 * kSlots);  // used only on the give-up path
+  auto slot_full = [&](int i) { return bar0 + 8u * (2 * kMaxStages + i); };
+  auto slot_empty = [&](int i) { return bar0 + 8u * (2 * kMaxStages + kSlots + i); };
+  const uint32_t drain_bar = bar0 + 8u * (2 * kMaxStages + 2 * kSlots);  // used only on the give-up path
   volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(gbase + kOffMisc);  // [0] tmem base, [1], [2] go flags of the epilogue groups
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -261,8 +264,10 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   const int pair = (int)blockIdx.x >> 1, npairs = (int)gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&map_h) : "memory");
     const uint32_t issuers = p.n1 > 0 ? 2 : 1;  // one MMA-issuing thread per accumulator
-    for (int s = 0; s < kStages; ++s) { mbar_init(full(s), 2); mbar_init(empty(s), issuers); }
+    for (int s = 0; s < p.stages; ++s) { mbar_init(full(s), 2); mbar_init(empty(s), issuers); }
     for (int i = 0; i < kSlots; ++i) {
       mbar_init(slot_full(i), 1);                  // the one issuer that formed the accumulator
       mbar_init(slot_empty(i), 2 * kEpiThreads);   // the epilogue threads of both CTAs arrive on the leader's
@@ -282,18 +287,25 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   tc_fence_after();
   const uint32_t tmem = misc[0];
 
+  // The grid is a programmatic dependent of the kernel before it: everything above ran next to that kernel's end, and
+  // nothing below starts before it has completed.  The kernel that folds this one's states may be scheduled early too.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+
+  const uint32_t half_bytes = (uint32_t)(p.box * kBytesPos);  // one accumulator's hidden tile of this CTA
+  const uint32_t h_bytes = p.n1 > 0 ? 2 * half_bytes : half_bytes;
+  const uint32_t off_h = (uint32_t)(kOffW + p.stages * kBytesW);
   const int my_tiles = pair < p.num_tiles ? (p.num_tiles - 1 - pair) / npairs + 1 : 0;
 
   if (warp == kWarpW) {
     // ---------------- weight producer: this CTA's 128 vocabulary entries ----------------
     if (lane == 0) {
-      int issued = 0;
+      int s = 0;
+      uint32_t ph = 0;
       bool ok = true;
       for (int t = 0; t < my_tiles && ok; ++t) {
         const int v0 = (pair + t * npairs) * kPairV + (int)rank * kBlockV;
-        for (int kb = 0; kb < p.num_kb; ++kb, ++issued) {
-          const int s = issued % kStages;
-          const uint32_t ph = (issued / kStages) & 1;
+        for (int kb = 0; kb < p.num_kb; ++kb) {
           if (!mbar_wait(empty(s), ph ^ 1, p.status, kErrTimeoutProducer)) { ok = false; break; }
           if (rank == 0) mbar_expect_tx(full(s), 2 * kBytesW);  // both CTAs' bytes
           const uint32_t bar = map_to_cta(full(s), 0);
@@ -304,27 +316,27 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
             tma_load_2d(dst, &map_w, v0, kb * kBlockK, bar);
             tma_load_2d(dst + kBytesWBox, &map_w, v0 + 64, kb * kBlockK, bar);
           }
+          if (++s == p.stages) { s = 0; ph ^= 1; }
         }
       }
     }
   } else if (warp == kWarpH) {
     // ---------------- hidden-state producer: this CTA's half of each accumulator's positions ----------------
     if (lane == 0) {
-      int issued = 0;
+      int s = 0;
+      uint32_t ph = 0;
       bool ok = true;
-      const uint32_t bytes = p.n1 > 0 ? kBytesH : kBytesHHalf;
       const int y0 = p.row0 + (int)rank * (p.n0 / 2);
-      const int y1 = p.row0 + kHalfN + (int)rank * (p.n1 / 2);
+      const int y1 = p.row0 + p.n0 + (int)rank * (p.n1 / 2);
       for (int t = 0; t < my_tiles && ok; ++t) {
-        for (int kb = 0; kb < p.num_kb; ++kb, ++issued) {
-          const int s = issued % kStages;
-          const uint32_t ph = (issued / kStages) & 1;
+        for (int kb = 0; kb < p.num_kb; ++kb) {
           if (!mbar_wait(empty(s), ph ^ 1, p.status, kErrTimeoutProducer)) { ok = false; break; }
-          if (rank == 0) mbar_expect_tx(full(s), 2 * bytes);
+          if (rank == 0) mbar_expect_tx(full(s), 2 * h_bytes);
           const uint32_t bar = map_to_cta(full(s), 0);
-          const uint32_t dst = base + kOffH + s * kBytesH;
+          const uint32_t dst = base + off_h + s * h_bytes;
           tma_load_2d(dst, &map_h, kb * kBlockK, y0, bar);
-          if (p.n1 > 0) tma_load_2d(dst + kBytesHHalf, &map_h, kb * kBlockK, y1, bar);
+          if (p.n1 > 0) tma_load_2d(dst + half_bytes, &map_h, kb * kBlockK, y1, bar);
+          if (++s == p.stages) { s = 0; ph ^= 1; }
         }
       }
     }
@@ -344,7 +356,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
       // With the weight stored [V, D] A is K-major like B: 128 rows of 128 bytes, 16 dims further = 32 bytes.
       const uint32_t a_lo0 = p.w_kmajor ? desc_lo(base + kOffW, 16) : desc_lo(base + kOffW, kBytesWBox);
       const uint32_t a_step = p.w_kmajor ? (uint32_t)((kMmaK * 2) >> 4) : (uint32_t)((kMmaK * 128) >> 4);
-      const uint32_t b_lo0 = desc_lo(base + kOffH + half * kBytesHHalf, 16);
+      const uint32_t b_lo0 = desc_lo(base + off_h + half * half_bytes, 16);
       const uint32_t peer_delta = map_to_cta(bar0, 1) - bar0;  // same offset in the partner's shared memory
       int st = 0;
       uint32_t ph = 0;
@@ -361,7 +373,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
           // TMA-written operands need no tcgen05 fence: the barrier wait orders them before the MMAs
           if (!mbar_wait(full(st), ph, p.status, kErrTimeoutMma)) { ok = false; break; }
           const uint32_t a_lo = a_lo0 + (uint32_t)st * (kBytesW >> 4);
-          const uint32_t b_lo = b_lo0 + (uint32_t)st * (kBytesH >> 4);
+          const uint32_t b_lo = b_lo0 + (uint32_t)st * (h_bytes >> 4);
 #pragma unroll
           for (int ks = 0; ks < kBlockK / kMmaK; ++ks) {
             const uint32_t acc = ks == 0 ? (uint32_t)(kb != 0) : 1u;
@@ -371,7 +383,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
           const uint32_t eb = empty(st);
           mma_commit(eb);
           mma_commit(eb + peer_delta);
-          if (++st == kStages) { st = 0; ph ^= 1; }
+          if (++st == p.stages) { st = 0; ph ^= 1; }
         }
         if (ok) {
           mma_commit(slot_full(slot));
@@ -402,11 +414,12 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
     const int my_chunks = nchunks > group ? (nchunks - group + 1) / 2 : 0;  // ... that this group turns
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     const int nh = p.n1 > 0 ? 2 : 1;
+    const int half_chunks = p.n0 / kChunk;  // blocks of accumulator 0
     // the last block of each accumulator that this group turns (-1: none): after reading it the thread hands the
     // accumulator's slot back
     int last0 = -1, last1 = -1;
     for (int k = 0; k < my_chunks; ++k) {
-      if (2 * k + group < kHalfChunks) last0 = k;
+      if (2 * k + group < half_chunks) last0 = k;
       else last1 = k;
     }
     for (int t = 0; t < my_tiles; ++t) {
@@ -430,9 +443,9 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
       for (int k = 0; k < kGroupChunks; ++k) {
         if (k < my_chunks) {
           const int c = 2 * k + group;
-          const int h = c / kHalfChunks;  // which accumulator the block belongs to
+          const int h = c >= half_chunks ? 1 : 0;  // which accumulator the block belongs to
           uint32_t r[16];
-          tmem_ld16(tmem + lane_base + (uint32_t)((h ? slot1 : slot0) * kHalfN + (c - h * kHalfChunks) * kChunk), r);
+          tmem_ld16(tmem + lane_base + (uint32_t)((h ? slot1 : slot0) * kHalfN + (c - h * half_chunks) * kChunk), r);
           if (k == (h ? last1 : last0)) {  // last read of this accumulator by this thread: hand its slot back
             tc_fence_before();
             mbar_arrive_remote(map_to_cta(slot_empty(h ? slot1 : slot0), 0));

@@ -236,3 +236,22 @@ def test_weight_stored_vocabulary_major(D, V):
     verify_fused(fv, hidden, weight, draft, out, stream=st)
     torch.cuda.synchronize()
     assert_parity(out, ref, f"[D, V] weight D={D} V={V}")
+
+
+@pytest.mark.parametrize("vocab_major", [False, True])
+@pytest.mark.parametrize("rows", [(1, 1), (2, 7), (9, 15), (8, 18), (16, 9), (17, 15), (18, 15), (20, 14)])
+def test_position_counts_at_the_edges_of_the_accumulators(rows, vocab_major):
+    # 2, 16, 144, 152, 160, 272, 288 and 300 positions: one accumulator or two of (un)equal halves, every depth of the operand
+    # ring, and a second pass over the weight; D gives the ring several rounds and a ragged last stage
+    B, K = rows
+    w, hidden, weight, draft, logits = fused_case(B, K, 968, 1512, step=B)
+    fv = FlyVerify(B, K, w.V, "bf16", hidden=w.hidden)
+    fv.set_weight_layout(vocab_major)
+    out = VerifyBuffers(B, K, DEV)
+    st = torch.cuda.current_stream().cuda_stream
+    for _ in range(2):
+        verify_fused(fv, hidden, weight.t().contiguous() if vocab_major else weight, draft, out, stream=st)
+    assert fv.device_status(st) == Bd.FLY_OK
+    ref = O.verify_batch(logits.reshape(B, K + 1, w.V), draft.cpu().numpy(), 1.0, 3)
+    assert_parity(out, ref, f"fused rows={B * (K + 1)} vocab_major={vocab_major}")
+    fv.close()
