@@ -55,6 +55,7 @@
 
 #include "fly_common.cuh"
 #include "mbarrier.cuh"
+#include "scan_kernel.cuh"
 
 namespace fly {
 namespace lmhead {
@@ -162,10 +163,32 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint32_t a_lo, uint32_
       ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// Arrives on `bar` (a shared::cluster address, in either CTA of the pair) once every tcgen05.mma issued
-// so far by this thread has completed in both CTAs.
+// Arrives on the barrier at `bar` (an address in this CTA's shared memory) in BOTH CTAs of the pair once every tcgen05.mma
+// issued so far by this thread has completed in both.
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+               "h"((uint16_t)3)
+               : "memory");
+}
+// The same in this CTA only.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// The producers and issuers run as whole warps and hand one lane the instructions that one thread issues: with uniform
+// control flow the descriptors stay in uniform registers, which is where those instructions take them from.  As code of a
+// single diverged lane an issuer took 690 cycles per stage at any N (75 per MMA, 133 for two commits; cycle counters), a
+// producer 360 - 400: more than the weights of a stage take from HBM (~650), so that the issuers bounded every size.
+// us a step, diverged lane -> uniform warp: 36 positions x 512 x 4096 12.8 -> 9.8, x 4096 x 50264 78.5 -> 71.2,
+// x 8192 x 128256 342 -> 318; 144 x 8192 x 128256 444 -> 387; 288: 587 -> 570 (power-capped).
+__device__ __forceinline__ bool elect_lane() {
+  uint32_t one;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+  return one != 0;
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* status, int code) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, code));
 }
 
 // 32 lanes x 16 columns of fp32: thread = lane, register i = column col0 + i.
@@ -259,7 +282,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   const uint32_t drain_bar = bar0 + 8u * (2 * kMaxStages + 2 * kSlots);  // used only on the give-up path
   volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(gbase + kOffMisc);  // [0] tmem base, [1], [2] go flags of the epilogue groups
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();  // 0: leader of the pair (issues the MMAs, owns the "full" barriers)
   const int pair = (int)blockIdx.x >> 1, npairs = (int)gridDim.x >> 1;
 
@@ -292,6 +315,8 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
 
+  bool failed = false;  // a bounded wait of this thread's role ran out
+  const uint32_t full_leader = map_to_cta(full(0), 0);  // the "full" barriers as both CTAs address them
   const uint32_t half_bytes = (uint32_t)(p.box * kBytesPos);  // one accumulator's hidden tile of this CTA
   const uint32_t h_bytes = p.n1 > 0 ? 2 * half_bytes : half_bytes;
   const uint32_t off_h = (uint32_t)(kOffW + p.stages * kBytesW);
@@ -299,57 +324,57 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
 
   if (warp == kWarpW) {
     // ---------------- weight producer: this CTA's 128 vocabulary entries ----------------
-    if (lane == 0) {
-      int s = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int t = 0; t < my_tiles && ok; ++t) {
-        const int v0 = (pair + t * npairs) * kPairV + (int)rank * kBlockV;
-        for (int kb = 0; kb < p.num_kb; ++kb) {
-          if (!mbar_wait(empty(s), ph ^ 1, p.status, kErrTimeoutProducer)) { ok = false; break; }
+    int s = 0;
+    uint32_t ph = 0;
+    const bool lead = elect_lane();
+    for (int t = 0; t < my_tiles && !failed; ++t) {
+      const int v0 = (pair + t * npairs) * kPairV + (int)rank * kBlockV;
+      for (int kb = 0; kb < p.num_kb; ++kb) {
+        if (!mbar_wait_warp(empty(s), ph ^ 1, p.status, kErrTimeoutProducer)) { failed = true; break; }
+        const uint32_t bar = full_leader + 8u * s;
+        const uint32_t dst = base + kOffW + s * kBytesW;
+        if (lead) {
           if (rank == 0) mbar_expect_tx(full(s), 2 * kBytesW);  // both CTAs' bytes
-          const uint32_t bar = map_to_cta(full(s), 0);
-          const uint32_t dst = base + kOffW + s * kBytesW;
           if (p.w_kmajor) {  // [V, D]: one box of 128 entries x 64 dims, each entry's 64 dims contiguous
             tma_load_2d(dst, &map_w, kb * kBlockK, v0, bar);
           } else {           // [D, V]: two boxes of 64 entries x 64 dims, each dim's 64 entries contiguous
             tma_load_2d(dst, &map_w, v0, kb * kBlockK, bar);
             tma_load_2d(dst + kBytesWBox, &map_w, v0 + 64, kb * kBlockK, bar);
           }
-          if (++s == p.stages) { s = 0; ph ^= 1; }
         }
+        __syncwarp();
+        if (++s == p.stages) { s = 0; ph ^= 1; }
       }
     }
   } else if (warp == kWarpH) {
     // ---------------- hidden-state producer: this CTA's half of each accumulator's positions ----------------
-    if (lane == 0) {
-      int s = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      const int y0 = p.row0 + (int)rank * (p.n0 / 2);
-      const int y1 = p.row0 + p.n0 + (int)rank * (p.n1 / 2);
-      for (int t = 0; t < my_tiles && ok; ++t) {
-        for (int kb = 0; kb < p.num_kb; ++kb) {
-          if (!mbar_wait(empty(s), ph ^ 1, p.status, kErrTimeoutProducer)) { ok = false; break; }
+    int s = 0;
+    uint32_t ph = 0;
+    const bool lead = elect_lane();
+    const int y0 = p.row0 + (int)rank * (p.n0 / 2);
+    const int y1 = p.row0 + p.n0 + (int)rank * (p.n1 / 2);
+    for (int t = 0; t < my_tiles && !failed; ++t) {
+      for (int kb = 0; kb < p.num_kb; ++kb) {
+        if (!mbar_wait_warp(empty(s), ph ^ 1, p.status, kErrTimeoutProducer)) { failed = true; break; }
+        const uint32_t bar = full_leader + 8u * s;
+        const uint32_t dst = base + off_h + s * h_bytes;
+        if (lead) {
           if (rank == 0) mbar_expect_tx(full(s), 2 * h_bytes);
-          const uint32_t bar = map_to_cta(full(s), 0);
-          const uint32_t dst = base + off_h + s * h_bytes;
           tma_load_2d(dst, &map_h, kb * kBlockK, y0, bar);
           if (p.n1 > 0) tma_load_2d(dst + half_bytes, &map_h, kb * kBlockK, y1, bar);
-          if (++s == p.stages) { s = 0; ph ^= 1; }
         }
+        __syncwarp();
+        if (++s == p.stages) { s = 0; ph ^= 1; }
       }
     }
   } else if (warp >= kWarpMma) {
-    // ---------------- MMA issuers (leader CTA): warp 6 feeds accumulator 0, warp 7 accumulator 1 ----------------
-    // One thread cannot issue MMAs, commits and barrier waits fast enough to keep the tensor pipe
-    // busy with two 144-column MMAs per 16 hidden dims, so each accumulator has an issuer of its own.
+    // ---------------- MMA issuers (leader CTA), one warp per accumulator ----------------
     const int half = warp - kWarpMma;
-    if (lane == 0 && rank == 0 && (half == 0 || p.n1 > 0)) {
+    if (rank == 0 && (half == 0 || p.n1 > 0)) {
+      const bool lead = elect_lane();
       const uint32_t idesc = instr_desc(half == 0 ? p.n0 : p.n1, p.w_kmajor != 0);
       const int nh = p.n1 > 0 ? 2 : 1;  // accumulators per tile
-      // Everything that changes from one MMA to the next is a 32-bit add: this thread has to issue one
-      // MMA every ~70 cycles, so the loop is kept to a few instructions per MMA.
+      // Everything that changes from one MMA to the next is a 32-bit add.
       // A, MN-major: 64-entry chunks lie kBytesWBox apart (leading offset), groups of 8 hidden dims
       // 1024 bytes apart (stride offset); 16 hidden dims further = 16 rows of 128 bytes.
       // B, K-major: groups of 8 positions 1024 bytes apart; 16 hidden dims further = 32 bytes.
@@ -357,40 +382,37 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
       const uint32_t a_lo0 = p.w_kmajor ? desc_lo(base + kOffW, 16) : desc_lo(base + kOffW, kBytesWBox);
       const uint32_t a_step = p.w_kmajor ? (uint32_t)((kMmaK * 2) >> 4) : (uint32_t)((kMmaK * 128) >> 4);
       const uint32_t b_lo0 = desc_lo(base + off_h + half * half_bytes, 16);
-      const uint32_t peer_delta = map_to_cta(bar0, 1) - bar0;  // same offset in the partner's shared memory
       int st = 0;
       uint32_t ph = 0;
-      bool ok = true;
-      for (int t = 0; t < my_tiles && ok; ++t) {
+      for (int t = 0; t < my_tiles && !failed; ++t) {
         // this accumulator's slot: the (t * nh + half)-th use of the rotation; the epilogue must have read out
         // what the slot held three uses ago
         const int use = t * nh + half;
         const int slot = use % kSlots;
         const uint32_t d_tmem = tmem + (uint32_t)(slot * kHalfN);
-        if (!mbar_wait(slot_empty(slot), ((use / kSlots) & 1) ^ 1, p.status, kErrTimeoutMma)) { ok = false; break; }
+        if (!mbar_wait_warp(slot_empty(slot), ((use / kSlots) & 1) ^ 1, p.status, kErrTimeoutMma)) { failed = true; break; }
         tc_fence_after();
         for (int kb = 0; kb < p.num_kb; ++kb) {
           // TMA-written operands need no tcgen05 fence: the barrier wait orders them before the MMAs
-          if (!mbar_wait(full(st), ph, p.status, kErrTimeoutMma)) { ok = false; break; }
+          if (!mbar_wait_warp(full(st), ph, p.status, kErrTimeoutMma)) { failed = true; break; }
           const uint32_t a_lo = a_lo0 + (uint32_t)st * (kBytesW >> 4);
           const uint32_t b_lo = b_lo0 + (uint32_t)st * (h_bytes >> 4);
+          if (lead) {
 #pragma unroll
-          for (int ks = 0; ks < kBlockK / kMmaK; ++ks) {
-            const uint32_t acc = ks == 0 ? (uint32_t)(kb != 0) : 1u;
-            mma_bf16(d_tmem, a_lo + ks * a_step, b_lo + ks * ((kMmaK * 2) >> 4), kDescHi, idesc, acc);
+            for (int ks = 0; ks < kBlockK / kMmaK; ++ks) {
+              const uint32_t acc = ks == 0 ? (uint32_t)(kb != 0) : 1u;
+              mma_bf16(d_tmem, a_lo + ks * a_step, b_lo + ks * ((kMmaK * 2) >> 4), kDescHi, idesc, acc);
+            }
+            // the stage may be refilled, in both CTAs, once these MMAs have read it
+            mma_commit_pair(empty(st));
           }
-          // the stage may be refilled, in both CTAs, once these MMAs have read it
-          const uint32_t eb = empty(st);
-          mma_commit(eb);
-          mma_commit(eb + peer_delta);
+          __syncwarp();
           if (++st == p.stages) { st = 0; ph ^= 1; }
         }
-        if (ok) {
-          mma_commit(slot_full(slot));
-          mma_commit(slot_full(slot) + peer_delta);
-        }
+        if (lead && !failed) mma_commit_pair(slot_full(slot));
+        __syncwarp();
       }
-      if (!ok) {
+      if (failed && lead) {
         // Give-up path: MMAs issued before the failed wait may still be reading shared memory and writing
         // tensor memory.  One more commit to a barrier of its own, and a (bounded) wait on it, lets them
         // finish before the common exit hands both back.
@@ -432,7 +454,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
       }
       group_bar(group);
       const bool go = misc[1 + group] != 0;  // one thread per group waits, the group takes the same decision
-      if (!go) break;
+      if (!go) { failed = true; break; }
       tc_fence_after();
       const int v0 = (pair + t * npairs) * kPairV + (int)rank * kBlockV + eighth * 16;
       const int limit = p.V - v0;  // entries of this eighth that exist
@@ -476,22 +498,22 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
     Partial* buf = reinterpret_cast<Partial*>(gbase + kOffW);
 #pragma unroll
     for (int k = 0; k < kGroupChunks; ++k) {
+      if (k >= my_chunks) break;
       Partial pq;
       pq.mx = st[k].mx; pq.S = st[k].S; pq.u = st[k].u; pq.idx = st[k].idx;
       buf[((2 * k + group) * kChunk + pos_i) * 8 + eighth] = pq;
     }
     epi_all_bar();
-    for (int pos = threadIdx.x; pos < p.R; pos += kEpiThreads) {
-      Partial a = buf[pos * 8];
-#pragma unroll
-      for (int e = 1; e < 8; ++e) merge_partial(a, buf[pos * 8 + e], p.scale);
-      p.partials[(int64_t)(p.row0 + pos) * gridDim.x + blockIdx.x] = a;
+    for (int i0 = 0; i0 < p.R * 8; i0 += kEpiThreads) {  // a lane per eighth
+      const int i = i0 + (int)threadIdx.x;
+      const Partial a = fold_lanes(i < p.R * 8 ? buf[i] : empty_partial(), 3, p.scale);
+      if (i < p.R * 8 && (i & 7) == 0) p.partials[(int64_t)(p.row0 + (i >> 3)) * gridDim.x + blockIdx.x] = a;
     }
   }
 
   // Common exit.  After a failed wait give stragglers (TMA copies still in flight towards this
   // CTA's shared memory) time to land before the shared memory is handed back.
-  if (*(volatile int*)p.status != 0) {
+  if (__syncthreads_or(failed)) {
     const unsigned long long t0 = global_ns();
     while (global_ns() - t0 < 2000000ull) {}
   }
