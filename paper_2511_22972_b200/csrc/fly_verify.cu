@@ -24,6 +24,7 @@ constexpr int kMaxSplits = 32;   // Partial slots per row in a handle's scratch
 constexpr int kReduceUnroll = 4;
 constexpr int64_t kMinBlockBytes = 16384;   // a block that gets less than this is all fixed cost
 constexpr int kMaxK = 63;
+constexpr size_t kDirectBytes = 5 << 20;    // host logits up to this size are read in place (fly_verify_run_host)
 
 struct DeviceGuard {
   int prev = -1;
@@ -67,8 +68,8 @@ struct fly_verify {
   // staging for fly_verify_run_host (allocated on first use)
   void* st_logits = nullptr;
   size_t st_logits_bytes = 0;
-  int32_t* st_ints = nullptr;  // device: draft | state_in | target tokens || state_out | accept | rollback | tokens | argmax | flags | entropy
-  int32_t* st_host = nullptr;  // page-locked host copy of the same block
+  int32_t* st_host = nullptr;  // page-locked: draft | state_in | target tokens || state_out | accept | rollback | tokens | argmax | flags | entropy
+  int32_t* st_ints = nullptr;  // the same block's device address
 };
 
 namespace {
@@ -555,7 +556,6 @@ fly_status_t fly_verify_destroy(fly_verify_t* h) {
     cudaFree(h->lm_status);
     cudaFree(h->st_hidden);
     cudaFree(h->st_logits);
-    cudaFree(h->st_ints);
     cudaFreeHost(h->st_host);
   }
   delete h;
@@ -754,24 +754,25 @@ fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, vo
   const int64_t K1 = a->K + 1, B = a->B, rows = B * K1;
   const int64_t stride = a->row_stride ? a->row_stride : V;
   cudaError_t e;
-  if (!h->st_ints) {
-    // staging sized once for the largest run this handle allows: the small inputs and all outputs are
-    // packed into one block each way, so that a step costs one small copy in and one out
+  if (!h->st_host) {
+    // sized once for the largest run this handle allows: the small inputs and all outputs, in page-locked memory that the
+    // kernels read and write over the bus.  A copy each way would cost the stream more than these few bytes do
+    // (4 rows of 32000 bf16: 37.0 us a step with the copies, 28.8 without; 144 rows of 128256: 706 and 698).
     const int64_t mb = h->cfg.max_batch, mk1 = h->cfg.max_k + 1;
     const size_t words = (size_t)(mb * (mk1 - 1) + 3 * mb + mb * mk1) + (size_t)(3 * mb + mb + mb + 4 * mb * mk1);
-    int32_t* dev_block = nullptr;
-    int32_t* host_block = nullptr;
-    if ((e = cudaMalloc(&dev_block, words * sizeof(int32_t))) != cudaSuccess) {
+    int32_t* block = nullptr;
+    if ((e = cudaHostAlloc(&block, words * sizeof(int32_t), cudaHostAllocMapped | cudaHostAllocPortable)) != cudaSuccess) {
       (void)cudaGetLastError();
       return cuda_fail(h, e);
     }
-    if ((e = cudaMallocHost(&host_block, words * sizeof(int32_t))) != cudaSuccess) {
+    void* dev = nullptr;
+    if ((e = cudaHostGetDevicePointer(&dev, block, 0)) != cudaSuccess) {
       (void)cudaGetLastError();
-      cudaFree(dev_block);
+      cudaFreeHost(block);
       return cuda_fail(h, e);
     }
-    h->st_ints = dev_block;  // both or neither
-    h->st_host = host_block;
+    h->st_host = block;
+    h->st_ints = static_cast<int32_t*>(dev);
   }
   const size_t hidden_bytes = a->logits ? 0 : (size_t)rows * h->cfg.hidden * 2;
   if (hidden_bytes > h->st_hidden_bytes) {
@@ -781,7 +782,18 @@ fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, vo
     if ((e = cudaMalloc(&h->st_hidden, hidden_bytes)) != cudaSuccess) return cuda_fail(h, e);
     h->st_hidden_bytes = hidden_bytes;
   }
-  const size_t logit_bytes = a->logits ? (size_t)(((rows - 1) * stride + V)) * esz : 0;
+  const size_t logit_span = a->logits ? (size_t)(((rows - 1) * stride + V)) * esz : 0;
+  // Small logits in page-locked memory that the device can address are read over the bus by the reduction itself: it reads
+  // every logit once, as a copy would, needs no copy before it and starts folding with the first of them.  Large ones are
+  // copied: the copy engine moves 55 GB/s, the SMs' reads 50.  Read in place / copied, us a step: 0.26 MB 29 / 34, 0.9 MB
+  // 61 / 68, 4.6 MB 110 / 177, 36.9 MB 740 / 710.
+  const void* direct = nullptr;
+  if (a->logits && logit_span <= kDirectBytes) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, a->logits) != cudaSuccess) (void)cudaGetLastError();
+    else if (at.type == cudaMemoryTypeHost && at.devicePointer) direct = at.devicePointer;
+  }
+  const size_t logit_bytes = direct ? 0 : logit_span;
   if (logit_bytes > h->st_logits_bytes) {
     cudaFree(h->st_logits);
     h->st_logits = nullptr;
@@ -789,25 +801,24 @@ fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, vo
     if ((e = cudaMalloc(&h->st_logits, logit_bytes)) != cudaSuccess) return cuda_fail(h, e);
     h->st_logits_bytes = logit_bytes;
   }
-  // word offsets inside the staging block (same layout on the host and on the device)
+  // word offsets inside the block
   const int64_t o_draft = 0, o_state_in = o_draft + B * a->K, o_target = o_state_in + 3 * B, in_words = o_target + rows;
   const int64_t o_state_out = in_words, o_accept = o_state_out + 3 * B, o_rollback = o_accept + B,
                 o_tokens = o_rollback + B, o_argmax = o_tokens + rows, o_flags = o_argmax + rows,
-                o_entropy = o_flags + rows, all_words = o_entropy + rows;
+                o_entropy = o_flags + rows;
   int32_t* dv = h->st_ints;
   int32_t* hv = h->st_host;
   memcpy(hv + o_draft, a->draft, (size_t)(B * a->K) * 4);
   if (a->state_in) memcpy(hv + o_state_in, a->state_in, (size_t)B * 12);
   if (a->target_tokens) memcpy(hv + o_target, a->target_tokens, (size_t)rows * 4);
 
-  if (a->logits && (e = cudaMemcpyAsync(h->st_logits, a->logits, logit_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
+  if (logit_bytes && (e = cudaMemcpyAsync(h->st_logits, a->logits, logit_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return cuda_fail(h, e);
   if (!a->logits && (e = cudaMemcpyAsync(h->st_hidden, a->hidden, hidden_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return cuda_fail(h, e);
-  if ((e = cudaMemcpyAsync(dv, hv, (size_t)in_words * 4, cudaMemcpyHostToDevice, st)) != cudaSuccess) return cuda_fail(h, e);
 
   fly_verify_args_t d = *a;
-  d.logits = a->logits ? h->st_logits : nullptr;
+  d.logits = direct ? direct : a->logits ? h->st_logits : nullptr;
   d.hidden = a->logits ? nullptr : h->st_hidden;  // the weight stays where it is: device memory
   d.draft = dv + o_draft;
   d.state_in = a->state_in ? reinterpret_cast<const fly_state_t*>(dv + o_state_in) : nullptr;
@@ -822,9 +833,6 @@ fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, vo
   s = fly_verify_run(h, &d, cuda_stream);
   if (s != FLY_OK) return s;
 
-  if ((e = cudaMemcpyAsync(hv + in_words, dv + in_words, (size_t)(all_words - in_words) * 4, cudaMemcpyDeviceToHost, st)) !=
-      cudaSuccess)
-    return cuda_fail(h, e);
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(h, e);
   auto back = [&](void* dst, int64_t off, size_t bytes) {
     if (dst) memcpy(dst, hv + off, bytes);

@@ -535,3 +535,17 @@ def test_rows_at_every_alignment(dtype, V, splits):
         view.copy_(logits)
         check(fv, view, draft, 1.0, 2, what=f"{dtype} V={V} splits={splits} off={off}")
     fv.close()
+
+
+@pytest.mark.parametrize("pinned", [False, True])
+@pytest.mark.parametrize("B,V", [(1, 5001), (20, 14563), (20, 14564), (21, 32000)])
+def test_host_logits_read_in_place_and_copied(B, V, pinned):
+    # on either side of the 5 MB up to which page-locked logits are read in place (2 x 9 x 20 x 14563 = 5242680 bytes is the
+    # last such size with these rows); pageable logits are always copied
+    w = small("bf16", B=B, K=8, V=V)
+    fv = FlyVerify(B, w.K, V, "bf16")
+    for step in range(2):
+        logits, draft = draw(w, step=step)
+        host = [t.cpu().pin_memory() if pinned else t.cpu() for t in (logits, draft)]
+        check(fv, host[0], host[1], 1.0, 2, host=True, what=f"host B={B} V={V} pinned={pinned}")
+    fv.close()
