@@ -403,8 +403,12 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->last_launches++;
   }
+  // A row's states, one per CTA, are folded by the scan itself where its lanes have about ten each, and by a warp per row
+  // before it otherwise: in the chain of launches a kernel more costs 1 us (36 positions x 512 x 4096: 9.6 against 10.3 us).
   cudaError_t e;
-  {
+  fly::Partial* parts = h->lm_partials;
+  int per_row = grid;
+  if (rows > L::kHalfN || (grid >> lanes_for(grid, a->K + 1)) > 10) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     const unsigned warps = fly::kFoldThreads / 32;
@@ -413,8 +417,10 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
                            exponent_scale(a->temperature));
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->last_launches++;
+    parts = h->lm_folded;
+    per_row = 1;
   }
-  fly::ScanParams sp = scan_params(h, a, h->lm_folded, 1);
+  fly::ScanParams sp = scan_params(h, a, parts, per_row);
   sp.status = h->lm_status;  // a step whose GEMM kernel gave up is marked row by row, in stream order
   e = launch_scan(sp, false, st);
   if (e != cudaSuccess) return cuda_fail(h, e);

@@ -222,12 +222,13 @@ __device__ __forceinline__ Partial gather_parts(const ScanParams& p, int64_t row
     }
   } else {
     if (l < q.n) acc = as_partial(q.part);
-    for (int j0 = l + step; j0 < q.n; j0 += 4 * step) {  // four independent loads in flight
-      int4 v[4];
+    constexpr int kBatch = 5;  // independent loads in flight
+    for (int j0 = l + step; j0 < q.n; j0 += kBatch * step) {
+      int4 v[kBatch];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) if (j0 + t * step < q.n) v[t] = ld_part(src + (j0 + t * step) * p.part_pitch);
+      for (int t = 0; t < kBatch; ++t) if (j0 + t * step < q.n) v[t] = ld_part(src + (j0 + t * step) * p.part_pitch);
 #pragma unroll
-      for (int t = 0; t < 4; ++t) if (j0 + t * step < q.n) merge_partial(acc, as_partial(v[t]), p.scale);
+      for (int t = 0; t < kBatch; ++t) if (j0 + t * step < q.n) merge_partial(acc, as_partial(v[t]), p.scale);
     }
   }
   return acc;
