@@ -313,7 +313,7 @@ fly_status_t fly_verify_selftest_wait(fly_verify_t* handle, void* cuda_stream);
  *   units_per_block  block b reduces the flat unit range [b * units_per_block, (b + 1) * units_per_block)
  *   units_per_row    whole units in a row
  *   row_span         units a row takes in that flat range (>= units_per_row; equal when rows are packed
- *                    end to end, a multiple of units_per_block when rows are cut into whole pieces)
+ *                    end to end or several whole rows go to a block, a multiple of units_per_block when rows are cut into whole pieces)
  *   slots            partial-state slots reserved per row (>= the pieces of any row)
  * Returns FLY_ERR_INVALID_ARG for sizes out of range. */
 typedef struct {

@@ -88,6 +88,7 @@ struct FlatPlan {
   int grid = 1;
   int slots = 1;
   int pieces = 0;     // > 0: every row is cut into exactly this many pieces (span = pieces * Q)
+  int rows_log2 = 0;  // > 0: whole rows, 2^rows_log2 of them per block (Q = 2^rows_log2 * n)
 };
 // Launch shape.  Measured on 9 .. 3000 rows of 16 - 300 KB: whole pieces of rows, one per block, are as fast as or
 // faster than packed rows almost everywhere - a row boundary inside a block drains that block's copy ring and costs a
@@ -104,6 +105,12 @@ struct FlatPlan {
 //                        128256 bf16, packed / whole rows, us: 297 rows 19.4 / 21.7, 360 21.9 / 21.9, 594 30.3 / 32.5,
 //                        702 35.9 / 37.9; but 216 rows 16.2 / 13.9 (two pieces per row), 432 rows 24.7 / 21.9, and
 //                        50257 or 32000 bf16: 216 rows 11.5 / 9.4 and 9.5 / 6.8, 360 rows 14.4 / 12.4 and 12.0 / 9.7.
+//   rows per block       many short rows: what a block costs beyond its data (about 3 us of its slot) is shared by 4 or 8
+//                        rows, two warps or one each.  us, a row per block / as chosen: 756 rows of 1000 bf16 6.3 / 5.8,
+//                        1170 rows 8.2 / 5.9, 2400 of 2003 13.1 / 7.6, of 16000 22.5 / 19.2, 7936 of 1000 33.3 / 11.9, of
+//                        4096 41.2 / 19.5, of 16000 61.9 / 46.2; where the lines lie: 756 rows of 4096 6.8 / 7.0, 900 of 8008
+//                        8.8 / 8.8, 900 of 16000 11.4 / 12.0, 1170 13.5 / 12.3, 2400 of 32000 31.9 / 35.0.  With inputs_ready
+//                        neighbouring steps fill the SMs: 756 rows of 16000 8.7 / 5.5, 900 of 50257 17.6 / 14.8.
 // Pieces hold at least 16 KB, rows of less than 112 KB are cut into up to seven of at least 7 KB: a block that gets
 // less is all fixed cost (9 rows of 32000 bf16: three pieces 4.55, seven 4.1 us).
 int64_t piece_units(int64_t n, int64_t s) {
@@ -111,7 +118,15 @@ int64_t piece_units(int64_t n, int64_t s) {
   if (s > 1) q = (q + 7) / 8 * 8;  // pieces start on 128-byte boundaries of the row
   return q;
 }
-FlatPlan plan_flat(int sm_count, int64_t rows, int64_t n, int64_t min_units, int64_t stride_units, int cap,
+int rows_per_block_log2(int sm_count, int64_t rows, int64_t n, bool inputs_ready) {
+  const int64_t gmax = (int64_t)sm_count * fly::kReduceBlocksPerSM;
+  const bool many = inputs_ready ? n <= 8192 && 4 * rows > 5 * gmax
+                                 : (n <= 256 && 4 * rows > 5 * gmax) || (n <= 1024 && 2 * rows > 3 * gmax) ||
+                                       (n <= 2048 && 4 * rows > 7 * gmax);
+  if (!many) return 0;
+  return (rows >= 8 * gmax && n <= 512) || (rows >= 4 * gmax && n <= 128) ? 3 : 2;
+}
+FlatPlan plan_flat(int sm_count, int64_t rows, int64_t n, bool vector, int64_t min_units, int64_t stride_units, int cap,
                    bool inputs_ready, int forced) {
   FlatPlan pl;
   const int64_t gmax = (int64_t)sm_count * fly::kReduceBlocksPerSM;
@@ -175,6 +190,14 @@ FlatPlan plan_flat(int sm_count, int64_t rows, int64_t n, int64_t min_units, int
     pl.span = s * pl.Q;
     pl.pieces = (int)s;
   }
+  if (vector && s == 1 && forced <= 0 && (pl.rows_log2 = rows_per_block_log2(sm_count, rows, n, inputs_ready)) > 0) {
+    pl.span = n;
+    pl.Q = n << pl.rows_log2;
+    pl.pieces = 0;
+    pl.grid = (int)((rows + (1 << pl.rows_log2) - 1) >> pl.rows_log2);
+    pl.slots = 1;
+    return pl;
+  }
   const int64_t total = rows * pl.span;
   pl.grid = (int)((total + pl.Q - 1) / pl.Q);
   const int64_t most = s > 0 ? s : (n + pl.Q - 1) / pl.Q + 1;
@@ -225,8 +248,10 @@ void ensure_reduce_attrs(int device) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kReduceMaxSmem);
     cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
-  set(fly::reduce_rows_flat<__nv_bfloat16, kReduceUnroll, true>);
-  set(fly::reduce_rows_flat<float, kReduceUnroll, true>);
+  set(fly::reduce_rows_flat<__nv_bfloat16, kReduceUnroll, true, false>);
+  set(fly::reduce_rows_flat<float, kReduceUnroll, true, false>);
+  set(fly::reduce_rows_flat<__nv_bfloat16, kReduceUnroll, true, true>);
+  set(fly::reduce_rows_flat<float, kReduceUnroll, true, true>);
   (void)cudaGetLastError();
 }
 
@@ -255,11 +280,14 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   const int64_t n = vec ? V / kE : V;
   const int64_t min_units = vec ? kMinBlockBytes / 16 : kMinBlockBytes / (int64_t)sizeof(T);
   const int64_t stride_units = (int64_t)fly::kReduceWarps * kReduceUnroll * 32;
-  const FlatPlan pl = plan_flat(sm_count, rows, n, min_units, stride_units, cap, inputs_ready, forced);
+  const FlatPlan pl = plan_flat(sm_count, rows, n, vec, min_units, stride_units, cap, inputs_ready, forced);
   fly::ReducePlan g;
   g.n = n; g.span = pl.span; g.Q = pl.Q; g.total = rows * pl.span;
   g.pieces = pl.Q < (1 << 30) ? pl.pieces : 0; g.V = V; g.row_stride = row_stride;
   g.scale = scale; g.wait_first = inputs_ready ? 0 : 1;
+  g.rows = (int)rows;
+  static_assert(fly::kReduceWarps == 8, "rows per block x warps per row");
+  g.warps_log2 = 3 - pl.rows_log2;
   tail->splits = pl.slots;
   // A row's states start on a 128-byte line (a power of two of them) where the scratch has the room.
   int pitch = 1;
@@ -270,15 +298,16 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   tail->partials = partials;
   tail->units_per_row = n;
   tail->row_span = pl.span;
-  tail->Q = pl.pieces > 0 ? 0 : pl.Q;  // whole pieces: every row has exactly pl.slots of them
+  tail->Q = pl.pieces > 0 || pl.rows_log2 > 0 ? 0 : pl.Q;  // whole pieces: every row has exactly pl.slots of them
   tail->scale = scale;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_launch(&cfg, attr, (unsigned)pl.grid, fly::kReduceThreads, st, true);
   cfg.dynamicSmemBytes = vec ? reduce_smem_bytes(pl.grid, sm_count, inputs_ready) : 0;
-  if (vec)
-    return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, true>, static_cast<const T*>(logits), g, *tail);
-  return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, false>, static_cast<const T*>(logits), g, *tail);
+  const T* src = static_cast<const T*>(logits);
+  if (pl.rows_log2 > 0) return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, true, true>, src, g, *tail);
+  if (vec) return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, true, false>, src, g, *tail);
+  return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, false, false>, src, g, *tail);
 }
 
 // The current device must be the one the pointers belong to (its ordinal is `device`).
@@ -704,7 +733,7 @@ fly_status_t fly_verify_plan(int32_t sm_count, int64_t rows, int32_t vocab, fly_
   if (vector_path && vocab < per_seg * 32) return FLY_ERR_INVALID_ARG;
   const int64_t n = vector_path ? vocab / per_seg : vocab;
   const int64_t min_units = vector_path ? kMinBlockBytes / 16 : kMinBlockBytes / esz;
-  const FlatPlan pl = plan_flat(sm_count, rows, n, min_units, (int64_t)fly::kReduceWarps * kReduceUnroll * 32, kMaxSplits,
+  const FlatPlan pl = plan_flat(sm_count, rows, n, vector_path != 0, min_units, (int64_t)fly::kReduceWarps * kReduceUnroll * 32, kMaxSplits,
                                 inputs_ready != 0, forced_pieces);
   out->grid = pl.grid;
   out->slots = pl.slots;

@@ -348,14 +348,17 @@ struct ReducePlan {
   int V;
   int64_t row_stride;  // elements
   float scale;     // log2(e) / temperature
+  int warps_log2;  // SHORT: warps that share a row
+  int rows;        // SHORT: all rows
   int wait_first;  // 1: wait for the previous kernel in the stream before the first read (plain stream
                    //    order); 0: the logits are known to be complete, wait only before the first write
 };
 
-// Lanes -> warp -> block; warp 0 ends up with the piece's Partial.  sm: kReduceWarps Partials of
+// Lanes -> warp -> block; warp 0 ends up with the piece's Partial (lane l with that of warp l's group of 2^warps_log2
+// warps).  sm: kReduceWarps Partials of
 // shared memory; consecutive pieces of a block alternate between two such buffers, so one barrier per
 // piece is enough.
-__device__ __forceinline__ Partial block_finish(const WarpAcc& a, Partial* sm, int lane, int warp) {
+__device__ __forceinline__ Partial block_finish(const WarpAcc& a, Partial* sm, int lane, int warp, int warps_log2 = 3) {
   float S0, S1, u0, u1;
   unpack2(a.S2, S0, S1);
   unpack2(a.u2, u0, u1);
@@ -374,7 +377,7 @@ __device__ __forceinline__ Partial block_finish(const WarpAcc& a, Partial* sm, i
   Partial p = empty_partial();
   if (warp == 0) {
     static_assert(kReduceWarps == 8, "the fold below is over 8 lanes");
-    p = fold_lanes(sm[lane & (kReduceWarps - 1)], 3, a.scale);
+    p = fold_lanes(sm[lane & (kReduceWarps - 1)], warps_log2, a.scale);
   }
   return p;
 }
@@ -433,18 +436,22 @@ __device__ __forceinline__ void flush_pieces(const ScanParams& p, TailShared& sm
 }
 
 // grid.x = ceil(total / Q).  VEC: a unit is a segment; else a logit (rows too short for the vector path).
-template <typename T, int UNROLL, bool VEC>
+// SHORT: many rows that are too short to occupy a block each (what a block costs beyond its data is about 3 us of its slot):
+// whole rows, several per block, a group of 2^warps_log2 warps each.
+template <typename T, int UNROLL, bool VEC, bool SHORT>
 __global__ void __launch_bounds__(kReduceThreads, kReduceBlocksPerSM)
 reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePlan g, const __grid_constant__ ScanParams tail) {
   constexpr int kE = Seg<T>::kElems;
   constexpr int kSlice = UNROLL * 32;
-  constexpr int kStride = kReduceWarps * kSlice;
+  const int kStride = SHORT ? kSlice << g.warps_log2 : kReduceWarps * kSlice;
+  const int gwarp = SHORT ? ((int)threadIdx.x >> 5) & ((1 << g.warps_log2) - 1) : (int)threadIdx.x >> 5;  // in the row's group
+  const int last_gwarp = SHORT ? (1 << g.warps_log2) - 1 : kReduceWarps - 1;
   // VEC: kReduceWarps * kDepth * kSlice segments, and a slice more per warp (bf16: `cand`).  On a 128-byte boundary: a copy of 8 lanes that straddles two lines of
   // shared memory takes two passes (1088 rows: 60.6 us at an offset of 48 bytes, 54.9 on the boundary).
   extern __shared__ __align__(128) uint4 ring[];
   __shared__ Partial sm_part[2][kReduceWarps];
   __shared__ TailShared sm_tail;
-  __shared__ float leftover[32];  // VEC: what the segments of the current row leave over (last warp)
+  __shared__ float leftover[SHORT ? kReduceWarps : 1][32];  // VEC: what the segments of the current row leave over (last warp)
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
 
   // The grid is launched as a programmatic dependent of the previous kernel in the stream.  Plain
@@ -457,7 +464,13 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
 
   int row, u0, u1, slot;  // the current piece: units [u0, u1) of `row`, stored in the row's slot `slot`
   int64_t left, take;     // flat units of this block not yet assigned to a piece; flat units the current piece takes
-  if (g.pieces > 0) {     // whole pieces of rows: one per block, 32-bit arithmetic (the common small-step case)
+  if (SHORT) {
+    row = (int)(blockIdx.x * (unsigned)(kReduceWarps >> g.warps_log2)) + (((int)threadIdx.x >> 5) >> g.warps_log2);
+    slot = 0;
+    u0 = 0;
+    u1 = row < g.rows ? (int)g.n : 0;
+    left = take = 0;
+  } else if (g.pieces > 0) {     // whole pieces of rows: one per block, 32-bit arithmetic (the common small-step case)
     row = (int)blockIdx.x / g.pieces;
     slot = (int)blockIdx.x - row * g.pieces;
     u0 = slot * (int)g.Q;
@@ -487,15 +500,15 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     const T* rp = logits + (int64_t)prow * g.row_stride;
     const int head = row_head(rp);
     pend_seg = min(pu1, segments(head));
-    const int ps = pu0 + warp * kSlice + lane;
+    const int ps = pu0 + gwarp * kSlice + lane;
     psrc = reinterpret_cast<const uint4*>(rp + head) + ps;
     pleft = pend_seg - ps;
   };
   auto fetch_leftover = [&](int prow, int pu1) {  // after the piece's first slices were asked for
-    if (pu1 == (int)g.n && warp == kReduceWarps - 1) {
+    if (pu1 == (int)g.n && gwarp == last_gwarp) {
       const T* rp = logits + (int64_t)prow * g.row_stride;
       const int head = row_head(rp), e = leftover_index<T>(head, segments(head), lane);
-      leftover[lane] = e < g.V ? max_nan_f32((float)rp[e], kMaskFloor) : kMaskFloor;
+      leftover[SHORT ? warp : 0][lane] = e < g.V ? max_nan_f32((float)rp[e], kMaskFloor) : kMaskFloor;
     }
   };
   auto issue = [&](int stage) {
@@ -531,7 +544,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     if constexpr (VEC) {
       int stage = 0;
       const int s_end = pend_seg;
-      for (int s0 = u0 + warp * kSlice; s0 < s_end; s0 += kStride) {
+      for (int s0 = u0 + gwarp * kSlice; s0 < s_end; s0 += kStride) {
         cp_async_wait<kDepth - 1>();  // the oldest slice in flight has landed
         uint32_t w[UNROLL][4];
         const uint4* src = ring + (warp * kDepth + stage) * kSlice + lane;
@@ -554,13 +567,13 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
       const int head = row_head(rp);
       if constexpr (sizeof(T) == 2) find_best<UNROLL>(a, cand, lane);
       if (a.best_idx != kIdxNone) a.best_idx += head;
-      if (u1 == (int)g.n && warp == kReduceWarps - 1) {
-        const float x[1] = {leftover[lane]};
+      if (u1 == (int)g.n && gwarp == last_gwarp) {
+        const float x[1] = {leftover[SHORT ? warp : 0][lane]};
         fold_elements<1>(a, x, [&](int) { return leftover_index<T>(head, segments(head), lane); });
       }
       // This warp's ring is empty now.  If the block goes on into the next row, start that piece's first
       // slices before the block-wide merge below, so that the row boundary costs no memory round trip.
-      if (left > 0) {
+      if (!SHORT && left > 0) {
         cp_async_wait<0>();
         const int next_u1 = (int)min(g.n, left);
         open_piece(row + 1, 0, next_u1);
@@ -570,6 +583,19 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
       }
     } else {
       reduce_piece_scalar<T, UNROLL>(a, logits + (int64_t)row * g.row_stride, u0, u1, lane, warp);
+    }
+    if constexpr (SHORT) {
+      const Partial p = block_finish(a, sm_part[0], lane, warp, g.warps_log2);
+      const int per = kReduceWarps >> g.warps_log2, row0 = (int)blockIdx.x * per, i = lane >> g.warps_log2;
+      np = min(per, g.rows - row0);
+      if (warp == 0 && lane < kReduceWarps && i < np && (lane & ((1 << g.warps_log2) - 1)) == 0) {
+        Pending q;
+        q.p = p; q.row = row0 + i; q.slot = 0; q.units = (unsigned)g.n; q.pad = 0;
+        sm_tail.pend[i] = q;
+      }
+      row = row0 + np - 1;
+      slot = 0;
+      break;
     }
     const Partial p = block_finish(a, sm_part[parity], lane, warp);
     if (threadIdx.x == 0) {

@@ -549,3 +549,34 @@ def test_host_logits_read_in_place_and_copied(B, V, pinned):
         host = [t.cpu().pin_memory() if pinned else t.cpu() for t in (logits, draft)]
         check(fv, host[0], host[1], 1.0, 2, host=True, what=f"host B={B} V={V} pinned={pinned}")
     fv.close()
+
+
+@pytest.mark.parametrize("dtype,B,K,V", [("bf16", 250, 2, 257), ("bf16", 149, 4, 1000), ("bf16", 797, 2, 4097), ("bf16", 400, 5, 1023),
+                                         ("bf16", 1000, 4, 2003), ("f32", 470, 1, 2051), ("f32", 33, 63, 515), ("bf16", 30, 39, 16391)])
+def test_several_rows_per_block(dtype, B, K, V):
+    # many short rows: 4 or 8 of them per block, two warps or one each; row counts that leave the last block partly empty,
+    # sequences that end inside blocks, rows at every alignment, carried state, and the scan as a kernel of its own
+    from paper_2511_22972_b200 import binding as Bd
+    w = small(dtype, B=B, K=K, V=V)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    p = Bd.plan(sms, w.rows, V, dtype)
+    assert p.units_per_block in (4 * p.units_per_row, 8 * p.units_per_row), "this shape is meant to share blocks"
+    fv = FlyVerify(B, K, V, dtype)
+    logits, draft = draw(w, step=K, guard=False)
+    rows = logits.view(-1, V)
+    rows[::7, 0] = rows[::7].float().max(dim=1).values.to(rows.dtype) + 1.0     # in the head of unaligned rows
+    rows[3::7, V - 1] = rows[3::7].float().max(dim=1).values.to(rows.dtype) + 1.0
+    rows[5::11, V // 3:] = -math.inf
+    for separate in (False, True):
+        fv.set_scan_mode(separate)
+        out = gpu_step(fv, logits, draft, 1.0, 1)
+        ref = oracle_step(logits, draft, 1.0, 1)
+        assert np.array_equal(out.target_argmax.cpu().numpy(), ref.target_argmax)
+        far = np.abs(ref.entropy[:, :-1] - 1.0).min(axis=1) > 1e-4     # entropies at the threshold may go either way
+        assert far.mean() > 0.9 and np.abs(out.entropy.cpu().numpy() - ref.entropy).max() < 1e-4
+        assert np.array_equal(out.accept_len.cpu().numpy()[far], ref.accept_len[far])
+        assert np.array_equal(out.out_tokens.cpu().numpy()[far], ref.out_tokens[far])
+    fv.set_scan_mode(False)
+    again = gpu_step(fv, logits, draft, 1.0, 1, inputs_ready=True)
+    assert torch.equal(again.out_tokens, out.out_tokens) and torch.equal(again.entropy, out.entropy)
+    fv.close()
