@@ -525,19 +525,20 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   if (e != cudaSuccess) { delete h; return FLY_ERR_CUDA; }
   h->sm_count = sms > 0 ? sms : 148;
-  e = cudaMalloc(&h->partials, (size_t)h->max_rows * kMaxSplits * sizeof(fly::Partial));
-  if (e != cudaSuccess) { delete h; return FLY_ERR_CUDA; }
-  e = cudaMemset(h->partials, 0, (size_t)h->max_rows * kMaxSplits * sizeof(fly::Partial));
-  if (e == cudaSuccess) e = cudaMalloc(&h->tickets, (size_t)h->max_rows * sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMemset(h->tickets, 0, (size_t)h->max_rows * sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMalloc(&h->lm_status, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(h->lm_status, 0, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&h->lm_folded, (size_t)h->max_rows * sizeof(fly::Partial));
+  // one block, all zero: slots | folded states | arrival counters | status word
+  const size_t slots = (size_t)h->max_rows * kMaxSplits, rows = (size_t)h->max_rows;
+  const size_t bytes = (slots + rows) * sizeof(fly::Partial) + rows * sizeof(unsigned int) + sizeof(int);
+  e = cudaMalloc(&h->partials, bytes);
+  if (e == cudaSuccess) e = cudaMemset(h->partials, 0, bytes);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the first step may run on a stream that does not wait for this one
   if (e != cudaSuccess) {
-    cudaFree(h->partials); cudaFree(h->tickets); cudaFree(h->lm_status); cudaFree(h->lm_folded);
+    cudaFree(h->partials);
     delete h;
     return FLY_ERR_CUDA;
   }
+  h->lm_folded = h->partials + slots;
+  h->tickets = reinterpret_cast<unsigned int*>(h->lm_folded + rows);
+  h->lm_status = reinterpret_cast<int*>(h->tickets + rows);
   if (c->hidden > 0) {
     e = cudaMalloc(&h->lm_partials, (size_t)h->max_rows * h->sm_count * sizeof(fly::Partial));
     if (e == cudaSuccess)
@@ -569,8 +570,7 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
     if (e != cudaSuccess || !fn) {
       fly_status_t st = cuda_fail(h, e);
       (void)st;
-      cudaFree(h->partials); cudaFree(h->tickets); cudaFree(h->lm_partials); cudaFree(h->lm_folded);
-      cudaFree(h->lm_status);
+      cudaFree(h->partials); cudaFree(h->lm_partials);
       delete h;
       return FLY_ERR_CUDA;
     }
@@ -585,10 +585,7 @@ fly_status_t fly_verify_destroy(fly_verify_t* h) {
   DeviceGuard g(h->cfg.device);
   if (g.ok) {
     cudaFree(h->partials);
-    cudaFree(h->tickets);
     cudaFree(h->lm_partials);
-    cudaFree(h->lm_folded);
-    cudaFree(h->lm_status);
     cudaFree(h->st_hidden);
     cudaFree(h->st_logits);
     cudaFreeHost(h->st_host);

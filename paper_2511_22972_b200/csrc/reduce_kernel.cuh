@@ -4,18 +4,14 @@
 //
 // Work decomposition ("flat partition").  The rows of one step are laid end to
 // end; a row holds `n` units (a unit is one 16-byte segment on the vector path,
-// one logit on the element-wise path).  The grid has G thread blocks, all
-// resident at once, and block b reduces the flat unit range [b*Q, (b+1)*Q): the
-// same number of bytes for every block, so that they finish together whatever
-// the number of rows is.  Where the range crosses a row boundary the block closes
+// one logit on the element-wise path), and block b reduces the flat unit range
+// [b*Q, (b+1)*Q).  Where the range crosses a row boundary the block closes
 // the row's piece (one 16-byte Partial) and starts the next row.  In the flat
-// index space a row spans `span` >= n units (units past n do not exist): span = n
-// packs the rows densely (large steps: a block takes a long range, the odd row
-// boundary inside it costs little); span = s*Q cuts every row into exactly s
-// pieces that never cross a row (small steps, where a boundary inside a block
-// would lengthen its critical path by a whole slice).  Row r is covered by the
-// blocks (r*span)/Q .. ((r+1)*span-1)/Q, and piece k of a row is stored at
-// partials[row * slots + k].
+// index space a row spans `span` >= n units (units past n do not exist): span = s*Q
+// cuts every row into exactly s pieces that never cross a row (the rule); span = n
+// packs the rows densely (some counts of long rows) or, with Q = r*n, gives a block
+// r whole rows, each to some of its warps (many short rows).  Row r is covered by the
+// blocks (r*span)/Q .. ((r+1)*span-1)/Q; piece k of a row goes to slot k of the row.
 //
 // Memory pipeline (vector path).  Every warp owns a small ring in shared memory
 // that it fills with asynchronous 16-byte copies (cp.async): kDepth slices of
