@@ -269,11 +269,17 @@ bool vector_path_ok(const void* logits, int V) {
   return reinterpret_cast<uintptr_t>(logits) % sizeof(T) == 0 && V >= fly::Seg<T>::kElems * 32;
 }
 
+// log2(e) / T: turns a logit into the base-2 exponent of its softmax weight at temperature T (0 = 1).
+float exponent_scale(double temperature) {
+  const double T = temperature == 0.0 ? 1.0 : temperature;
+  return (float)(1.4426950408889634 / T);
+}
+
 // Launches the row reduction.  `tail` carries the acceptance scan's arguments (tickets == NULL: no scan in
 // this launch); its geometry fields are filled in here and returned through it for a stand-alone scan.
 template <typename T>
 cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, int V, int64_t rows, int forced, int cap,
-                          fly::Partial* partials, cudaStream_t st, fly::ScanParams* tail, float scale,
+                          fly::Partial* partials, cudaStream_t st, fly::ScanParams* tail, double temperature,
                           bool inputs_ready) {
   constexpr int kE = fly::Seg<T>::kElems;
   const bool vec = vector_path_ok<T>(logits, V);
@@ -284,7 +290,7 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   fly::ReducePlan g;
   g.n = n; g.span = pl.span; g.Q = pl.Q; g.total = rows * pl.span;
   g.pieces = pl.Q < (1 << 30) ? pl.pieces : 0; g.V = V; g.row_stride = row_stride;
-  g.scale = scale; g.wait_first = inputs_ready ? 0 : 1;
+  g.scale = exponent_scale(temperature); g.floor = fly::mask_floor(temperature); g.wait_first = inputs_ready ? 0 : 1;
   g.rows = (int)rows;
   static_assert(fly::kReduceWarps == 8, "rows per block x warps per row");
   g.warps_log2 = 3 - pl.rows_log2;
@@ -299,7 +305,7 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   tail->units_per_row = n;
   tail->row_span = pl.span;
   tail->Q = pl.pieces > 0 || pl.rows_log2 > 0 ? 0 : pl.Q;  // whole pieces: every row has exactly pl.slots of them
-  tail->scale = scale;
+  tail->scale = g.scale;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_launch(&cfg, attr, (unsigned)pl.grid, fly::kReduceThreads, st, true);
@@ -313,12 +319,12 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
 // The current device must be the one the pointers belong to (its ordinal is `device`).
 cudaError_t launch_reduce_any(int device, fly_dtype_t dt, int sm_count, const void* logits, int64_t row_stride, int V,
                               int64_t rows, int forced, int cap, fly::Partial* partials, cudaStream_t st,
-                              fly::ScanParams* tail, float scale, bool inputs_ready) {
+                              fly::ScanParams* tail, double temperature, bool inputs_ready) {
   ensure_reduce_attrs(device);
   if (dt == FLY_BF16)
-    return launch_reduce<__nv_bfloat16>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, scale,
+    return launch_reduce<__nv_bfloat16>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature,
                                         inputs_ready);
-  return launch_reduce<float>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, scale, inputs_ready);
+  return launch_reduce<float>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature, inputs_ready);
 }
 
 // tagged: the parts are in the self-validating form that the row reduction leaves.
@@ -352,12 +358,6 @@ fly_status_t check_args(const fly_verify* h, const fly_verify_args_t* a) {
     return FLY_ERR_INVALID_ARG;  // the paper's rule has no cross-round state
   }
   return FLY_OK;
-}
-
-// log2(e) / T: turns a logit into the base-2 exponent of its softmax weight at temperature T (0 = 1).
-float exponent_scale(double temperature) {
-  const double T = temperature == 0.0 ? 1.0 : temperature;
-  return (float)(1.4426950408889634 / T);
 }
 
 fly::ScanParams scan_params(const fly_verify* h, const fly_verify_args_t* a, fly::Partial* partials, int splits);
@@ -422,6 +422,7 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     p.row0 = (int)row0;
     p.w_kmajor = h->weight_vd;
     p.scale = exponent_scale(a->temperature);
+    p.floor = fly::mask_floor(a->temperature);
     p.partials = h->lm_partials;
     p.status = h->lm_status;
     cudaLaunchConfig_t cfg;
@@ -627,7 +628,6 @@ fly_status_t fly_verify_reduce_shard(fly_verify_t* h, int32_t rows, const void* 
   if (!g.ok) return FLY_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int64_t stride = row_stride ? row_stride : V;
-  const float scale = exponent_scale(temperature);
   fly::ScanParams p;  // the tail of the reduction folds each row's pieces: a "sequence" is one row
   memset(&p, 0, sizeof(p));
   p.B = rows;
@@ -635,7 +635,7 @@ fly_status_t fly_verify_reduce_shard(fly_verify_t* h, int32_t rows, const void* 
   p.row_out = reinterpret_cast<fly::Partial*>(partial_out);
   p.idx_offset = vocab_offset;
   cudaError_t e = launch_reduce_any(h->cfg.device, h->cfg.logits_dtype, h->sm_count, logits, stride, V, rows, h->forced_splits, kMaxSplits,
-                                    h->partials, st, &p, scale, false);
+                                    h->partials, st, &p, temperature, false);
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches = 1;
   return FLY_OK;
@@ -763,7 +763,7 @@ fly_status_t fly_verify_run(fly_verify_t* h, const fly_verify_args_t* a, void* c
   const bool fused_tail = h->scan_mode == 0;
   p.tickets = fused_tail ? h->tickets : nullptr;
   cudaError_t e = launch_reduce_any(h->cfg.device, h->cfg.logits_dtype, h->sm_count, a->logits, stride, V, rows, h->forced_splits,
-                                    kMaxSplits, h->partials, st, &p, p.scale, a->inputs_ready != 0);
+                                    kMaxSplits, h->partials, st, &p, a->temperature, a->inputs_ready != 0);
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches++;
   if (!fused_tail) {
@@ -962,7 +962,7 @@ fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t lo
   cudaError_t e = cudaLaunchKernelEx(&cfg, fly::clear_scratch, reinterpret_cast<uint4*>(tickets), ticket_words,
                                      reinterpret_cast<uint4*>(partials), slot_words);
   if (e != cudaSuccess) return FLY_ERR_CUDA;
-  e = launch_reduce_any(device, logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, p.scale,
+  e = launch_reduce_any(device, logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, a->temperature,
                         a->inputs_ready != 0);
   return e == cudaSuccess ? FLY_OK : FLY_ERR_CUDA;
 }

@@ -111,6 +111,7 @@ struct Params {
   int row0;       // first row of this launch in hidden / partials
   int w_kmajor;   // 0: weight is [D, V] (vocabulary contiguous, MN-major A); 1: weight is [V, D] (K-major A)
   float scale;    // log2(e) / temperature: logit -> base-2 exponent
+  float floor;    // logits at or below it are masked
   Partial* partials;  // [rows, gridDim.x]: one partial state per position and CTA
   int* status;        // 0, or the code of the first wait that ran out
 };
@@ -228,11 +229,11 @@ struct Stream {
 };
 
 // Folds 16 consecutive vocabulary entries x[0..15] (the first one has index v0) into st.
-__device__ __forceinline__ void fold16(Stream& st, float (&x)[16], int v0, float scale) {
-  float lm = kMaskFloor;
+__device__ __forceinline__ void fold16(Stream& st, float (&x)[16], int v0, float scale, float floor) {
+  float lm = floor;
 #pragma unroll
   for (int e = 0; e < 16; ++e) {
-    x[e] = max_nan_f32(x[e], kMaskFloor);  // masked entries stay finite; NaN survives and ends in S
+    x[e] = max_nan_f32(x[e], floor);  // masked entries stay finite; NaN survives and ends in S
     lm = fmaxf(lm, x[e]);
   }
   if (lm > st.mx) {  // the maximum moves: rebase the sums and record the first entry that holds it
@@ -430,7 +431,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
     const int pos_i = gtid & 15, eighth = gtid >> 4;
     Stream st[kGroupChunks];
 #pragma unroll
-    for (int k = 0; k < kGroupChunks; ++k) { st[k].mx = kMaskFloor; st[k].S = 0.f; st[k].u = 0.f; st[k].idx = kIdxNone; }
+    for (int k = 0; k < kGroupChunks; ++k) { st[k].mx = p.floor; st[k].S = 0.f; st[k].u = 0.f; st[k].idx = kIdxNone; }
     float* turn = reinterpret_cast<float*>(gbase + kOffTurn + group * kTurnGroupBytes);
     const int nchunks = (p.R + kChunk - 1) / kChunk;                 // blocks of this launch
     const int my_chunks = nchunks > group ? (nchunks - group + 1) / 2 : 0;  // ... that this group turns
@@ -486,9 +487,9 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
           if (limit < 16) {  // ragged vocabulary: entries past V do not exist
 #pragma unroll
             for (int e = 0; e < 16; ++e)
-              if (e >= limit) x[e] = kMaskFloor;
+              if (e >= limit) x[e] = p.floor;
           }
-          fold16(st[k], x, v0, p.scale);
+          fold16(st[k], x, v0, p.scale, p.floor);
         }
       }
     }

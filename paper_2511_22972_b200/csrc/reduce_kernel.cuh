@@ -79,10 +79,10 @@ struct WarpAcc {
   f2 S2, u2;
 };
 
-__device__ __forceinline__ void acc_init(WarpAcc& a, float scale) {
-  a.cur_max = kMaskFloor;
+__device__ __forceinline__ void acc_init(WarpAcc& a, float scale, float floor) {
+  a.cur_max = floor;
   a.scale = scale;
-  a.r = kMaskFloor * scale;
+  a.r = floor * scale;
   a.best_idx = kIdxNone;
   a.cand_s0 = 0;
   a.cand_hit = 0;
@@ -159,19 +159,19 @@ __device__ __forceinline__ void cp_async_wait() {
 // segments at or past seg_end do not belong to the piece): masks and clamps the data and returns the
 // lane's maximum.  Masked entries are clamped to the floor (NaN survives the clamp and ends in S).
 template <int UNROLL>
-__device__ __forceinline__ float slice_max_bf16(uint32_t (&w)[UNROLL][4], int seg0, int seg_end, int lane) {
-  constexpr uint32_t kFloor2 = 0xc974c974u;  // bf16(kMaskFloor) twice
+__device__ __forceinline__ float slice_max_bf16(uint32_t (&w)[UNROLL][4], int seg0, int seg_end, int lane, float floor) {
+  const uint32_t floor2 = __byte_perm(__float_as_uint(floor), 0, 0x3232);  // bf16(floor) twice (exact: a power of two times 61 * 2^14)
   if (seg0 + UNROLL * 32 > seg_end) {        // ragged slice (warp-uniform)
 #pragma unroll
     for (int j = 0; j < UNROLL; ++j)
       if (seg0 + j * 32 + lane >= seg_end) w[j][0] = w[j][1] = w[j][2] = w[j][3] = kNegInf2;
   }
-  uint32_t lm2 = kFloor2;
+  uint32_t lm2 = floor2;
 #pragma unroll
   for (int j = 0; j < UNROLL; ++j)
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      w[j][c] = bf2_max_nan(w[j][c], kFloor2);
+      w[j][c] = bf2_max_nan(w[j][c], floor2);
       lm2 = bf2_max(lm2, w[j][c]);
     }
   return fmaxf(bf16lo(lm2), bf16hi(lm2));
@@ -228,18 +228,18 @@ __device__ __forceinline__ void slice_sum_bf16(WarpAcc& a, const uint32_t (&w)[U
 
 // The same two halves for fp32 logits: w[j] holds 4 logits as raw bits.
 template <int UNROLL>
-__device__ __forceinline__ float slice_max_f32(uint32_t (&w)[UNROLL][4], int seg0, int seg_end, int lane) {
+__device__ __forceinline__ float slice_max_f32(uint32_t (&w)[UNROLL][4], int seg0, int seg_end, int lane, float floor) {
   if (seg0 + UNROLL * 32 > seg_end) {
 #pragma unroll
     for (int j = 0; j < UNROLL; ++j)
       if (seg0 + j * 32 + lane >= seg_end) w[j][0] = w[j][1] = w[j][2] = w[j][3] = 0xff800000u;
   }
-  float lm = kMaskFloor;
+  float lm = floor;
 #pragma unroll
   for (int j = 0; j < UNROLL; ++j)
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const float x = max_nan_f32(__uint_as_float(w[j][c]), kMaskFloor);
+      const float x = max_nan_f32(__uint_as_float(w[j][c]), floor);
       w[j][c] = __float_as_uint(x);
       lm = fmaxf(lm, x);
     }
@@ -271,12 +271,12 @@ __device__ __forceinline__ void slice_sum_f32(WarpAcc& a, const uint32_t (&w)[UN
 // Folds one logit per UNROLL and lane (x, already clamped; the floor where there is none) with the indices idx(j).
 // An index below the ones folded so far wins a tie.
 template <int UNROLL, typename F>
-__device__ __forceinline__ void fold_elements(WarpAcc& a, const float (&x)[UNROLL], F idx) {
-  float lm = kMaskFloor;
+__device__ __forceinline__ void fold_elements(WarpAcc& a, const float (&x)[UNROLL], float floor, F idx) {
+  float lm = floor;
 #pragma unroll
   for (int j = 0; j < UNROLL; ++j) lm = fmaxf(lm, x[j]);
   const float wm = warp_max_f32(lm);
-  if (wm > kMaskFloor && wm >= a.cur_max) {
+  if (wm > floor && wm >= a.cur_max) {
     const bool moved = wm > a.cur_max;
     if (moved) acc_rebase(a, wm);
     uint32_t first = 0xffffffffu;
@@ -292,7 +292,7 @@ __device__ __forceinline__ void fold_elements(WarpAcc& a, const float (&x)[UNROL
   // lanes without a logit hold the floor: 2^(floor*scale - r) = 0 unless the whole
   // piece is masked, in which case the piece vanishes when merged
   if constexpr (UNROLL == 1) {
-    acc_add2(a, x[0], kMaskFloor, sc2, nr2);
+    acc_add2(a, x[0], floor, sc2, nr2);
   } else {
 #pragma unroll
     for (int j = 0; j < UNROLL; j += 2) acc_add2(a, x[j], x[j + 1], sc2, nr2);
@@ -302,16 +302,16 @@ __device__ __forceinline__ void fold_elements(WarpAcc& a, const float (&x)[UNROL
 // Element-wise slice of short rows: UNROLL*32 consecutive elements starting at e0.
 template <typename T, int UNROLL>
 __device__ __forceinline__ void warp_slice_scalar(WarpAcc& a, const T* __restrict__ row, int e0, int e_end,
-                                                  int lane) {
+                                                  int lane, float floor) {
   float x[UNROLL];
 #pragma unroll
   for (int j = 0; j < UNROLL; ++j) {
     const int e = e0 + j * 32 + lane;
     float v = -INFINITY;
     if (e < e_end) v = (float)row[e];
-    x[j] = max_nan_f32(v, kMaskFloor);
+    x[j] = max_nan_f32(v, floor);
   }
-  fold_elements<UNROLL>(a, x, [&](int j) { return e0 + j * 32 + lane; });
+  fold_elements<UNROLL>(a, x, floor, [&](int j) { return e0 + j * 32 + lane; });
 }
 
 // Logits of a row before its first aligned segment.
@@ -328,10 +328,10 @@ __device__ __forceinline__ int leftover_index(int head, int segs, int lane) {
 // One piece on the element-wise path: logits [e_begin, e_end) of the row.
 template <typename T, int UNROLL>
 __device__ __forceinline__ void reduce_piece_scalar(WarpAcc& a, const T* __restrict__ rp, int e_begin, int e_end, int lane,
-                                                    int warp) {
+                                                    int warp, float floor) {
   constexpr int kSlice = UNROLL * 32;
   for (int e0 = e_begin + warp * kSlice; e0 < e_end; e0 += kReduceWarps * kSlice)
-    warp_slice_scalar<T, UNROLL>(a, rp, e0, e_end, lane);
+    warp_slice_scalar<T, UNROLL>(a, rp, e0, e_end, lane, floor);
 }
 
 // Geometry of one launch (see the head of this file).
@@ -344,6 +344,7 @@ struct ReducePlan {
   int V;
   int64_t row_stride;  // elements
   float scale;     // log2(e) / temperature
+  float floor;     // logits at or below it are masked
   int warps_log2;  // SHORT: warps that share a row
   int rows;        // SHORT: all rows
   int wait_first;  // 1: wait for the previous kernel in the stream before the first read (plain stream
@@ -504,7 +505,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     if (pu1 == (int)g.n && gwarp == last_gwarp) {
       const T* rp = logits + (int64_t)prow * g.row_stride;
       const int head = row_head(rp), e = leftover_index<T>(head, segments(head), lane);
-      leftover[SHORT ? warp : 0][lane] = e < g.V ? max_nan_f32((float)rp[e], kMaskFloor) : kMaskFloor;
+      leftover[SHORT ? warp : 0][lane] = e < g.V ? max_nan_f32((float)rp[e], g.floor) : g.floor;
     }
   };
   auto issue = [&](int stage) {
@@ -535,7 +536,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
   int parity = 0, np = 0;
   while (true) {
     WarpAcc a;
-    acc_init(a, g.scale);
+    acc_init(a, g.scale, g.floor);
     left -= take;
     if constexpr (VEC) {
       int stage = 0;
@@ -550,8 +551,8 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
           w[j][0] = q.x; w[j][1] = q.y; w[j][2] = q.z; w[j][3] = q.w;
         }
         float lm;
-        if constexpr (sizeof(T) == 2) lm = slice_max_bf16<UNROLL>(w, s0, s_end, lane);
-        else lm = slice_max_f32<UNROLL>(w, s0, s_end, lane);
+        if constexpr (sizeof(T) == 2) lm = slice_max_bf16<UNROLL>(w, s0, s_end, lane, g.floor);
+        else lm = slice_max_f32<UNROLL>(w, s0, s_end, lane, g.floor);
         // every register of the slice has been consumed once, so the stage's bytes are out of shared
         // memory: refill it with the slice kDepth ahead
         issue(stage);
@@ -565,7 +566,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
       if (a.best_idx != kIdxNone) a.best_idx += head;
       if (u1 == (int)g.n && gwarp == last_gwarp) {
         const float x[1] = {leftover[SHORT ? warp : 0][lane]};
-        fold_elements<1>(a, x, [&](int) { return leftover_index<T>(head, segments(head), lane); });
+        fold_elements<1>(a, x, g.floor, [&](int) { return leftover_index<T>(head, segments(head), lane); });
       }
       // This warp's ring is empty now.  If the block goes on into the next row, start that piece's first
       // slices before the block-wide merge below, so that the row boundary costs no memory round trip.
@@ -578,7 +579,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
         fetch_leftover(row + 1, next_u1);
       }
     } else {
-      reduce_piece_scalar<T, UNROLL>(a, logits + (int64_t)row * g.row_stride, u0, u1, lane, warp);
+      reduce_piece_scalar<T, UNROLL>(a, logits + (int64_t)row * g.row_stride, u0, u1, lane, warp, g.floor);
     }
     if constexpr (SHORT) {
       const Partial p = block_finish(a, sm_part[0], lane, warp, g.warps_log2);

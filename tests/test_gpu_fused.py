@@ -255,3 +255,9 @@ def test_position_counts_at_the_edges_of_the_accumulators(rows, vocab_major):
     ref = O.verify_batch(logits.reshape(B, K + 1, w.V), draft.cpu().numpy(), 1.0, 3)
     assert_parity(out, ref, f"fused rows={B * (K + 1)} vocab_major={vocab_major}")
     fv.close()
+
+
+@pytest.mark.parametrize("V", [1512, 1000, 2048])
+def test_entries_past_the_vocabulary_weigh_nothing_at_high_temperature(V):
+    # 1000 and 1512 end inside a tile of 256: what the tile holds past them is no logit
+    run_and_check(8, 8, D=256, V=V, theta=1.0, W=2, temperature=1e6, step=6)

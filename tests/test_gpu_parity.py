@@ -580,3 +580,20 @@ def test_several_rows_per_block(dtype, B, K, V):
     again = gpu_step(fv, logits, draft, 1.0, 1, inputs_ready=True)
     assert torch.equal(again.out_tokens, out.out_tokens) and torch.equal(again.entropy, out.entropy)
     fv.close()
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 100), ("bf16", 1000), ("bf16", 32768), ("bf16", 32776), ("f32", 127), ("f32", 32768)])
+@pytest.mark.parametrize("T", [3000.0, 1e5, 1e6])
+def test_masked_logits_weigh_nothing_at_any_temperature(dtype, V, T):
+    # neither do the lanes of a ragged slice that hold no logit: at T = 1e6 a floor of -999424 would count each as e^-1 of an entry
+    w = small(dtype, B=3, K=4, V=V)
+    fv = FlyVerify(w.B, w.K, V, dtype)
+    logits, draft = draw(w, step=5, guard=False)
+    rows = logits.view(-1, V)
+    rows[::3, :V // 2] = -math.inf
+    rows[1::3, V // 3::2] = -math.inf
+    rows[4] = -math.inf                            # nothing finite: flagged at every temperature
+    for splits in (0, 3):
+        fv.set_splits(splits)
+        check(fv, logits, draft, 1.0, 2, temperature=T, what=f"{dtype} V={V} T={T} splits={splits}")
+    fv.close()

@@ -92,3 +92,15 @@ def test_sharded_vocabulary_at_a_temperature(T):
     logits, draft = draw(w, step=5, temperature=T)
     out = sharded_step(w, logits, draft, 4, 1.0, 2, temperature=T)
     assert_parity(out, oracle_step(logits, draft, 1.0, 2, temperature=T), f"tp4 T={T}")
+
+
+@pytest.mark.parametrize("T", [1e5, 1e6])
+def test_masked_slices_weigh_nothing_at_high_temperature(T):
+    # a slice that is masked throughout vanishes in the merge, and so does the empty state of a rank without one
+    w = S.shrink(S.LLAMA3, B=2, K=3, V=4096)
+    logits, draft = draw(w, step=7, guard=False)
+    rows = logits.view(-1, w.V)
+    rows[::2, :2048] = -math.inf
+    rows[3] = -math.inf
+    out = sharded_step(w, logits, draft, 4, 1.0, 2, temperature=T)
+    assert_parity(out, oracle_step(logits, draft, 1.0, 2, temperature=T), f"T={T}")
