@@ -233,26 +233,19 @@ int reduce_smem_bytes(int grid, int sm_count, bool inputs_ready) {
   return n == 1 ? kReduceMaxSmem : n == 2 ? 80 * 1024 : 60 * 1024;
 }
 
-// Function attributes are per device: set them once on every device that launches the row reduction.
-// The rings of all resident blocks only fit on an SM whose L1/shared split favours shared memory.
-constexpr int kMaxDevices = 64;
-void ensure_reduce_attrs(int device) {
-  static std::mutex mu;
-  static bool done[kMaxDevices] = {};
-  if (device >= 0 && device < kMaxDevices) {
-    std::lock_guard<std::mutex> lock(mu);
-    if (done[device]) return;
-    done[device] = true;
-  }
+// Shared memory above 48 KB has to be asked for, per kernel and context: done when a handle (or the static entry point's slot
+// of a device) is made, before any step of it can run.  The rings of all resident blocks only fit on an SM whose L1/shared
+// split favours shared memory.
+cudaError_t set_reduce_attrs() {
   auto set = [](auto kernel) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kReduceMaxSmem);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kReduceMaxSmem);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
-  set(fly::reduce_rows_flat<__nv_bfloat16, kReduceUnroll, true, false>);
-  set(fly::reduce_rows_flat<float, kReduceUnroll, true, false>);
-  set(fly::reduce_rows_flat<__nv_bfloat16, kReduceUnroll, true, true>);
-  set(fly::reduce_rows_flat<float, kReduceUnroll, true, true>);
-  (void)cudaGetLastError();
+  cudaError_t e = set(fly::reduce_rows_flat<__nv_bfloat16, kReduceUnroll, true, false>);
+  if (e == cudaSuccess) e = set(fly::reduce_rows_flat<float, kReduceUnroll, true, false>);
+  if (e == cudaSuccess) e = set(fly::reduce_rows_flat<__nv_bfloat16, kReduceUnroll, true, true>);
+  if (e == cudaSuccess) e = set(fly::reduce_rows_flat<float, kReduceUnroll, true, true>);
+  return e;
 }
 
 // Lanes (as a power of two) that share a row's parts in the acceptance scan: one per part as far as a block has threads
@@ -316,11 +309,10 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, false, false>, src, g, *tail);
 }
 
-// The current device must be the one the pointers belong to (its ordinal is `device`).
-cudaError_t launch_reduce_any(int device, fly_dtype_t dt, int sm_count, const void* logits, int64_t row_stride, int V,
+// The current device must be the one the pointers belong to.
+cudaError_t launch_reduce_any(fly_dtype_t dt, int sm_count, const void* logits, int64_t row_stride, int V,
                               int64_t rows, int forced, int cap, fly::Partial* partials, cudaStream_t st,
                               fly::ScanParams* tail, double temperature, bool inputs_ready) {
-  ensure_reduce_attrs(device);
   if (dt == FLY_BF16)
     return launch_reduce<__nv_bfloat16>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature,
                                         inputs_ready);
@@ -526,6 +518,7 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   if (e != cudaSuccess) { delete h; return FLY_ERR_CUDA; }
   h->sm_count = sms > 0 ? sms : 148;
+  if (set_reduce_attrs() != cudaSuccess) { delete h; return FLY_ERR_CUDA; }
   // one block, all zero: slots | folded states | arrival counters | status word
   const size_t slots = (size_t)h->max_rows * kMaxSplits, rows = (size_t)h->max_rows;
   const size_t bytes = (slots + rows) * sizeof(fly::Partial) + rows * sizeof(unsigned int) + sizeof(int);
@@ -634,7 +627,7 @@ fly_status_t fly_verify_reduce_shard(fly_verify_t* h, int32_t rows, const void* 
   p.tickets = h->tickets;
   p.row_out = reinterpret_cast<fly::Partial*>(partial_out);
   p.idx_offset = vocab_offset;
-  cudaError_t e = launch_reduce_any(h->cfg.device, h->cfg.logits_dtype, h->sm_count, logits, stride, V, rows, h->forced_splits, kMaxSplits,
+  cudaError_t e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, logits, stride, V, rows, h->forced_splits, kMaxSplits,
                                     h->partials, st, &p, temperature, false);
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches = 1;
@@ -762,7 +755,7 @@ fly_status_t fly_verify_run(fly_verify_t* h, const fly_verify_args_t* a, void* c
   // lets consecutive steps overlap (inputs_ready) and keeps a step at one launch.
   const bool fused_tail = h->scan_mode == 0;
   p.tickets = fused_tail ? h->tickets : nullptr;
-  cudaError_t e = launch_reduce_any(h->cfg.device, h->cfg.logits_dtype, h->sm_count, a->logits, stride, V, rows, h->forced_splits,
+  cudaError_t e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, a->logits, stride, V, rows, h->forced_splits,
                                     kMaxSplits, h->partials, st, &p, a->temperature, a->inputs_ready != 0);
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches++;
@@ -910,6 +903,7 @@ cudaError_t static_scratch_for(int device, StaticSlot* out) {
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
     s.sm_count = sms > 0 ? sms : 148;
+    if ((e = set_reduce_attrs()) != cudaSuccess) return e;
     s.base = p;
   }
   *out = s;
@@ -962,7 +956,7 @@ fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t lo
   cudaError_t e = cudaLaunchKernelEx(&cfg, fly::clear_scratch, reinterpret_cast<uint4*>(tickets), ticket_words,
                                      reinterpret_cast<uint4*>(partials), slot_words);
   if (e != cudaSuccess) return FLY_ERR_CUDA;
-  e = launch_reduce_any(device, logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, a->temperature,
+  e = launch_reduce_any(logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, a->temperature,
                         a->inputs_ready != 0);
   return e == cudaSuccess ? FLY_OK : FLY_ERR_CUDA;
 }
