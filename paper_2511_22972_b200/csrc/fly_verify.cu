@@ -241,11 +241,15 @@ cudaError_t set_reduce_attrs() {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kReduceMaxSmem);
     return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
-  cudaError_t e = set(fly::reduce_rows_flat<__nv_bfloat16, kReduceUnroll, true, false>);
-  if (e == cudaSuccess) e = set(fly::reduce_rows_flat<float, kReduceUnroll, true, false>);
-  if (e == cudaSuccess) e = set(fly::reduce_rows_flat<__nv_bfloat16, kReduceUnroll, true, true>);
-  if (e == cudaSuccess) e = set(fly::reduce_rows_flat<float, kReduceUnroll, true, true>);
-  return e;
+  auto set_all = [&](auto zero) {
+    using T = decltype(zero);
+    cudaError_t e = set(fly::reduce_rows_flat<T, kReduceUnroll, true, false, false>);
+    if (e == cudaSuccess) e = set(fly::reduce_rows_flat<T, kReduceUnroll, true, true, false>);
+    if (e == cudaSuccess) e = set(fly::reduce_rows_flat<T, kReduceUnroll, true, false, true>);
+    return e != cudaSuccess ? e : set(fly::reduce_rows_flat<T, kReduceUnroll, true, true, true>);
+  };
+  const cudaError_t e = set_all(__nv_bfloat16());
+  return e != cudaSuccess ? e : set_all(float());
 }
 
 // Lanes (as a power of two) that share a row's parts in the acceptance scan: one per part as far as a block has threads
@@ -304,9 +308,12 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   fill_launch(&cfg, attr, (unsigned)pl.grid, fly::kReduceThreads, st, true);
   cfg.dynamicSmemBytes = vec ? reduce_smem_bytes(pl.grid, sm_count, inputs_ready) : 0;
   const T* src = static_cast<const T*>(logits);
-  if (pl.rows_log2 > 0) return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, true, true>, src, g, *tail);
-  if (vec) return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, true, false>, src, g, *tail);
-  return cudaLaunchKernelEx(&cfg, fly::reduce_rows_flat<T, kReduceUnroll, false, false>, src, g, *tail);
+  auto kernel = fly::reduce_rows_flat<T, kReduceUnroll, false, false, true>;
+  if (vec && g.floor == fly::kMaskFloor)
+    kernel = pl.rows_log2 > 0 ? fly::reduce_rows_flat<T, kReduceUnroll, true, true, false> : fly::reduce_rows_flat<T, kReduceUnroll, true, false, false>;
+  else if (vec)
+    kernel = pl.rows_log2 > 0 ? fly::reduce_rows_flat<T, kReduceUnroll, true, true, true> : fly::reduce_rows_flat<T, kReduceUnroll, true, false, true>;
+  return cudaLaunchKernelEx(&cfg, kernel, src, g, *tail);
 }
 
 // The current device must be the one the pointers belong to.

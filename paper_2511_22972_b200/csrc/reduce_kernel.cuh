@@ -344,7 +344,7 @@ struct ReducePlan {
   int V;
   int64_t row_stride;  // elements
   float scale;     // log2(e) / temperature
-  float floor;     // logits at or below it are masked
+  float floor;     // FLOOR: logits at or below it are masked
   int warps_log2;  // SHORT: warps that share a row
   int rows;        // SHORT: all rows
   int wait_first;  // 1: wait for the previous kernel in the stream before the first read (plain stream
@@ -435,11 +435,14 @@ __device__ __forceinline__ void flush_pieces(const ScanParams& p, TailShared& sm
 // grid.x = ceil(total / Q).  VEC: a unit is a segment; else a logit (rows too short for the vector path).
 // SHORT: many rows that are too short to occupy a block each (what a block costs beyond its data is about 3 us of its slot):
 // whole rows, several per block, a group of 2^warps_log2 warps each.
-template <typename T, int UNROLL, bool VEC, bool SHORT>
+// FLOOR: the mask floor is g.floor and not kMaskFloor.  An operand of every clamp: as a register instead of a constant it costs
+// the plain kernel 1 % (1000 rows of 128256 bf16 47.3 -> 47.9 us a step, 1088 rows 48.8 -> 49.3).
+template <typename T, int UNROLL, bool VEC, bool SHORT, bool FLOOR>
 __global__ void __launch_bounds__(kReduceThreads, kReduceBlocksPerSM)
 reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePlan g, const __grid_constant__ ScanParams tail) {
   constexpr int kE = Seg<T>::kElems;
   constexpr int kSlice = UNROLL * 32;
+  const float floor = FLOOR ? g.floor : kMaskFloor;
   const int kStride = SHORT ? kSlice << g.warps_log2 : kReduceWarps * kSlice;
   const int gwarp = SHORT ? ((int)threadIdx.x >> 5) & ((1 << g.warps_log2) - 1) : (int)threadIdx.x >> 5;  // in the row's group
   const int last_gwarp = SHORT ? (1 << g.warps_log2) - 1 : kReduceWarps - 1;
@@ -505,7 +508,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     if (pu1 == (int)g.n && gwarp == last_gwarp) {
       const T* rp = logits + (int64_t)prow * g.row_stride;
       const int head = row_head(rp), e = leftover_index<T>(head, segments(head), lane);
-      leftover[SHORT ? warp : 0][lane] = e < g.V ? max_nan_f32((float)rp[e], g.floor) : g.floor;
+      leftover[SHORT ? warp : 0][lane] = e < g.V ? max_nan_f32((float)rp[e], floor) : floor;
     }
   };
   auto issue = [&](int stage) {
@@ -536,7 +539,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
   int parity = 0, np = 0;
   while (true) {
     WarpAcc a;
-    acc_init(a, g.scale, g.floor);
+    acc_init(a, g.scale, floor);
     left -= take;
     if constexpr (VEC) {
       int stage = 0;
@@ -551,8 +554,8 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
           w[j][0] = q.x; w[j][1] = q.y; w[j][2] = q.z; w[j][3] = q.w;
         }
         float lm;
-        if constexpr (sizeof(T) == 2) lm = slice_max_bf16<UNROLL>(w, s0, s_end, lane, g.floor);
-        else lm = slice_max_f32<UNROLL>(w, s0, s_end, lane, g.floor);
+        if constexpr (sizeof(T) == 2) lm = slice_max_bf16<UNROLL>(w, s0, s_end, lane, floor);
+        else lm = slice_max_f32<UNROLL>(w, s0, s_end, lane, floor);
         // every register of the slice has been consumed once, so the stage's bytes are out of shared
         // memory: refill it with the slice kDepth ahead
         issue(stage);
@@ -566,7 +569,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
       if (a.best_idx != kIdxNone) a.best_idx += head;
       if (u1 == (int)g.n && gwarp == last_gwarp) {
         const float x[1] = {leftover[SHORT ? warp : 0][lane]};
-        fold_elements<1>(a, x, g.floor, [&](int) { return leftover_index<T>(head, segments(head), lane); });
+        fold_elements<1>(a, x, floor, [&](int) { return leftover_index<T>(head, segments(head), lane); });
       }
       // This warp's ring is empty now.  If the block goes on into the next row, start that piece's first
       // slices before the block-wide merge below, so that the row boundary costs no memory round trip.
@@ -579,7 +582,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
         fetch_leftover(row + 1, next_u1);
       }
     } else {
-      reduce_piece_scalar<T, UNROLL>(a, logits + (int64_t)row * g.row_stride, u0, u1, lane, warp, g.floor);
+      reduce_piece_scalar<T, UNROLL>(a, logits + (int64_t)row * g.row_stride, u0, u1, lane, warp, floor);
     }
     if constexpr (SHORT) {
       const Partial p = block_finish(a, sm_part[0], lane, warp, g.warps_log2);
