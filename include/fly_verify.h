@@ -41,7 +41,7 @@ typedef enum {
   FLY_ERR_INVALID_ARG = 1, /* null pointer, size out of range, inconsistent arguments */
   FLY_ERR_UNSUPPORTED = 2, /* a valid request this build cannot serve (alignment, W > K in carry mode, ...) */
   FLY_ERR_CUDA = 3,        /* a CUDA runtime call failed; see fly_verify_last_cuda_error */
-  FLY_ERR_TIMEOUT = 4,     /* a bounded device-side wait ran out (fused path) */
+  FLY_ERR_TIMEOUT = 4,     /* a bounded device-side wait ran out */
   FLY_ERR_TOO_LARGE = 5    /* fly_verify_run_static only: the step does not fit the built-in scratch area */
 } fly_status_t;
 
@@ -133,9 +133,10 @@ typedef struct {
                                    library writes (pending outside [0, K], negative rollback_len, or a pending
                                    window whose correction token is outside [0, V)): it is ignored, i.e. the
                                    round is verified from the zero state;
-                             bit 4 fused path only: a bounded wait of the GEMM kernel ran out during this step
-                                   (see fly_verify_device_status); set on every row, every position counts as a
-                                   mismatch that is never deferred, so accept_len is 1 and nothing drafted is kept */
+                             bit 4 a bounded wait ran out (see fly_verify_device_status): such a position counts as a
+                                   mismatch that is never deferred.  Fused path: set on every row, so accept_len is 1
+                                   and nothing drafted is kept.  Logits path: set on the rows whose reduction did not
+                                   complete, and on every row of later steps while the record is pending */
 
   /* Optional (NULL = greedy): dev [B, K+1] tokens y_1..y_{K+1} that the caller drew from the target
    * distributions, e.g. by sampling at temperature 1.  The paper's method text defines y_i only as the
@@ -291,18 +292,23 @@ typedef enum {
 fly_status_t fly_verify_set_option(fly_verify_t* handle, fly_option_t option, int32_t value);
 
 /* The fused path's kernel waits on hardware barriers (TMA arrival, tensor-core
- * completion); every such wait is bounded.  If one runs out, the kernel records
- * it and returns without hanging (its outputs are then undefined).  This call
- * synchronises `cuda_stream` and returns FLY_ERR_TIMEOUT if that happened since
- * the last call (the record is cleared), else FLY_OK.  While a record is
- * pending, further fused steps give up early, and every step run in that state
- * marks all of its rows with row_flags bit 4, so the failure is also visible in
- * stream order without a host synchronisation.  Logits-path kernels have no waits. */
+ * completion), and the block of the logits path that completes a sequence waits for
+ * the partial states that other blocks have stored; every such wait is bounded (200 ms).  If
+ * one runs out, the kernel records it and returns without hanging (what it could not
+ * form is marked with row_flags bit 4; a state of fly_verify_reduce_shard then has
+ * max_logit = +inf, NaN sums and argmax 0x7ffffffe, and the merge marks its row).
+ * This call synchronises `cuda_stream` and returns FLY_ERR_TIMEOUT if that happened since
+ * the last call (the record, and with it the handle's scratch where a state was missed, is
+ * cleared), else FLY_OK.  While a record is pending, every further step of the same path
+ * marks all of its rows with row_flags bit 4 (fused steps give up early), so the failure is
+ * also visible in stream order without a host synchronisation.  fly_verify_run_static keeps
+ * no record: bit 4 marks the rows, and every call clears its scratch. */
 fly_status_t fly_verify_device_status(fly_verify_t* handle, void* cuda_stream);
 
 /* Self-test of that mechanism, safe to run anywhere: enqueues a one-thread kernel that waits, with a
- * 2 ms limit, on a barrier nothing will complete.  The wait gives up, the kernel returns normally, and the
- * next fly_verify_device_status reports FLY_ERR_TIMEOUT.  Nothing faults or hangs. */
+ * 2 ms limit, on a barrier nothing will complete, and a scan that waits as long for a partial state nothing will
+ * store.  The waits give up, the kernels return normally, and the next fly_verify_device_status reports
+ * FLY_ERR_TIMEOUT.  Nothing faults or hangs. */
 fly_status_t fly_verify_selftest_wait(fly_verify_t* handle, void* cuda_stream);
 
 /* Introspection, host only (no CUDA call): the launch geometry the logits path chooses for `rows` rows of

@@ -23,6 +23,7 @@ inline float mask_floor(double T) {
   return f;
 }
 constexpr int kIdxNone = 0x7fffffff;
+constexpr int kIdxFailed = 0x7ffffffe;  // with mx = +inf: the state of a reduction whose bounded wait ran out
 
 constexpr uint32_t kFlagNonFinite = 1u;
 constexpr uint32_t kFlagBadDraft = 2u;
@@ -87,6 +88,16 @@ __device__ __forceinline__ Partial empty_partial() {
   p.S = 0.f;
   p.u = 0.f;
   p.idx = kIdxNone;
+  return p;
+}
+
+// Outlives every merge: its maximum wins, and with it its index (an infinite logit of a lower index is flagged for itself).
+__device__ __forceinline__ Partial failed_partial() {
+  Partial p;
+  p.mx = __int_as_float(0x7f800000);
+  p.S = __int_as_float(0x7fc00000);
+  p.u = p.S;
+  p.idx = kIdxFailed;
   return p;
 }
 

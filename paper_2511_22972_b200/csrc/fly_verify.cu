@@ -56,6 +56,8 @@ struct fly_verify {
   fly::Partial* lm_partials = nullptr;  // [max_rows * sm_count]: one partial state per row and CTA
   fly::Partial* lm_folded = nullptr;    // [max_rows]: partial states folded over CTAs
   int* lm_status = nullptr;             // device word: first bounded wait that ran out (sticky until read)
+  int* state_status = nullptr;          // the word after it: the same of the row reduction, a partial state that did not arrive
+  size_t scratch_bytes = 0;             // of the block that starts at `partials` and ends with these two words
   int lm_pairs = 0;                     // CTA pairs that can be resident at once
   int weight_vd = 0;                    // 0: weight [hidden, V]; 1: weight [V, hidden]
   PFN_cuTensorMapEncodeTiled encode_tiled = nullptr;
@@ -303,6 +305,7 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   tail->row_span = pl.span;
   tail->Q = pl.pieces > 0 || pl.rows_log2 > 0 ? 0 : pl.Q;  // whole pieces: every row has exactly pl.slots of them
   tail->scale = g.scale;
+  tail->wait_ns = fly::kWaitLimitNs;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_launch(&cfg, attr, (unsigned)pl.grid, fly::kReduceThreads, st, true);
@@ -487,6 +490,7 @@ fly::ScanParams scan_params(const fly_verify* h, const fly_verify_args_t* a, fly
   p.row_flags = a->row_flags;
   p.target_tokens = a->target_tokens;
   p.status = nullptr;
+  p.wait_ns = fly::kWaitLimitNs;
   return p;
 }
 
@@ -526,9 +530,9 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   if (e != cudaSuccess) { delete h; return FLY_ERR_CUDA; }
   h->sm_count = sms > 0 ? sms : 148;
   if (set_reduce_attrs() != cudaSuccess) { delete h; return FLY_ERR_CUDA; }
-  // one block, all zero: slots | folded states | arrival counters | status word
+  // one block, all zero: slots | folded states | arrival counters | status words
   const size_t slots = (size_t)h->max_rows * kMaxSplits, rows = (size_t)h->max_rows;
-  const size_t bytes = (slots + rows) * sizeof(fly::Partial) + rows * sizeof(unsigned int) + sizeof(int);
+  const size_t bytes = (slots + rows) * sizeof(fly::Partial) + rows * sizeof(unsigned int) + 2 * sizeof(int);
   e = cudaMalloc(&h->partials, bytes);
   if (e == cudaSuccess) e = cudaMemset(h->partials, 0, bytes);
   if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the first step may run on a stream that does not wait for this one
@@ -540,6 +544,8 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   h->lm_folded = h->partials + slots;
   h->tickets = reinterpret_cast<unsigned int*>(h->lm_folded + rows);
   h->lm_status = reinterpret_cast<int*>(h->tickets + rows);
+  h->state_status = h->lm_status + 1;
+  h->scratch_bytes = bytes;
   if (c->hidden > 0) {
     e = cudaMalloc(&h->lm_partials, (size_t)h->max_rows * h->sm_count * sizeof(fly::Partial));
     if (e == cudaSuccess)
@@ -634,6 +640,7 @@ fly_status_t fly_verify_reduce_shard(fly_verify_t* h, int32_t rows, const void* 
   p.tickets = h->tickets;
   p.row_out = reinterpret_cast<fly::Partial*>(partial_out);
   p.idx_offset = vocab_offset;
+  p.status = h->state_status;
   cudaError_t e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, logits, stride, V, rows, h->forced_splits, kMaxSplits,
                                     h->partials, st, &p, temperature, false);
   if (e != cudaSuccess) return cuda_fail(h, e);
@@ -698,25 +705,33 @@ fly_status_t fly_verify_device_status(fly_verify_t* h, void* cuda_stream) {
   if (!g.ok) return FLY_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e;
-  int word = 0;
-  if (h->lm_status) {
-    if ((e = cudaMemcpyAsync(&word, h->lm_status, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess)
-      return cuda_fail(h, e);
-  }
+  int words[2] = {0, 0};  // lm_status, state_status
+  if ((e = cudaMemcpyAsync(words, h->lm_status, sizeof(words), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_fail(h, e);
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(h, e);
-  if (word != 0) {
-    if ((e = cudaMemsetAsync(h->lm_status, 0, sizeof(int), st)) != cudaSuccess) return cuda_fail(h, e);
-    return FLY_ERR_TIMEOUT;
-  }
-  return FLY_OK;
+  if (words[0] == 0 && words[1] == 0) return FLY_OK;
+  // A state that arrived after its wait had run out lies in a slot that the next step takes for empty: clear them all.
+  e = words[1] ? cudaMemsetAsync(h->partials, 0, h->scratch_bytes, st) : cudaMemsetAsync(h->lm_status, 0, sizeof(int), st);
+  return e == cudaSuccess ? FLY_ERR_TIMEOUT : cuda_fail(h, e);
 }
 
 fly_status_t fly_verify_selftest_wait(fly_verify_t* h, void* cuda_stream) {
   if (!h) return FLY_ERR_INVALID_ARG;
   DeviceGuard g(h->cfg.device);
   if (!g.ok) return FLY_ERR_CUDA;
-  fly::lmhead::wait_selftest_kernel<<<1, 1, 0, static_cast<cudaStream_t>(cuda_stream)>>>(h->lm_status, 2000000ull);
-  const cudaError_t e = cudaGetLastError();
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  constexpr unsigned long long kLimitNs = 2000000;
+  fly::lmhead::wait_selftest_kernel<<<1, 1, 0, st>>>(h->lm_status, kLimitNs);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(h, e);
+  // ... and a scan over one row whose only slot is empty, as every slot is between steps
+  fly::ScanParams p;
+  memset(&p, 0, sizeof(p));
+  p.B = 1; p.splits = 1; p.row_pitch = 1; p.part_pitch = 1; p.scale = 1.0f;
+  p.partials = h->partials;
+  p.row_out = h->lm_folded;
+  p.status = h->state_status;
+  p.wait_ns = kLimitNs;
+  e = launch_scan(p, true, st);
   return e == cudaSuccess ? FLY_OK : cuda_fail(h, e);
 }
 
@@ -762,6 +777,7 @@ fly_status_t fly_verify_run(fly_verify_t* h, const fly_verify_args_t* a, void* c
   // lets consecutive steps overlap (inputs_ready) and keeps a step at one launch.
   const bool fused_tail = h->scan_mode == 0;
   p.tickets = fused_tail ? h->tickets : nullptr;
+  p.status = h->state_status;
   cudaError_t e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, a->logits, stride, V, rows, h->forced_splits,
                                     kMaxSplits, h->partials, st, &p, a->temperature, a->inputs_ready != 0);
   if (e != cudaSuccess) return cuda_fail(h, e);

@@ -7,6 +7,8 @@
 
 namespace fly {
 
+constexpr int kErrTimeoutState = 4;  // status word of the row reduction: a partial state did not arrive (see scan_kernel.cuh)
+
 // Far above any legitimate wait (a tile takes ~70 us).  %globaltimer also runs while the context is
 // preempted or time-sliced with another process, so on a shared GPU a wait can in principle run out
 // without a fault in the kernel: the limit is generous for that reason, and a run-out is reported,

@@ -18,7 +18,9 @@
 // zero.  A block stores its state and adds to the sequence's arrival counter without waiting for the
 // store.  The block whose count completes the sequence knows that every state has at least been
 // issued and reads them all at once; the rare one that is still on its way shows as an empty slot
-// and is asked for again (bounded).  The reader empties the slots for the next launch.
+// and is asked for again (bounded).  The reader empties the slots for the next launch.  A wait that runs
+// out is recorded in *status: the state it waited for may still land, in a slot the next launch takes for
+// empty, so every later step marks all of its rows until the host has cleared the scratch.
 // Measured (steps in a CUDA graph, us, before -> after; before: one warp per sequence, a lane per row,
 // fences around the counter): 9 rows of 32000 fp32 5.16 -> 4.30, 16 rows of 128256 bf16 7.20 -> 4.95,
 // 144 rows 11.64 -> 11.05, 1088 and 2304 rows unchanged.
@@ -61,7 +63,8 @@ struct ScanParams {
   float* entropy;           // [B, K+1] or null
   uint32_t* row_flags;      // [B, K+1] or null
   const int32_t* target_tokens;  // [B, K+1] or null: the caller's y_i instead of the argmax
-  const int* status;             // fused path: device word that is non-zero when a bounded wait of the GEMM kernel ran out
+  int* status;                   // device word that is non-zero when a bounded wait of this path ran out, or null
+  unsigned long long wait_ns;    // TAGGED: how long a state that has been issued is waited for
 };
 
 struct RoundOutcome {
@@ -169,12 +172,13 @@ struct ScanLoads {
   int n;                // parts of its row
   int draft, target;    // of its row (first lane of a group)
   int pend, len, corr;  // carried state (thread 0)
+  int failed;           // first lane of a group: a wait ran out, in this step or before it
 };
 
 __device__ __forceinline__ ScanLoads scan_request(const ScanParams& p, int b) {
   ScanLoads q;
   q.part = make_int4(0, 0, 0, 0);
-  q.n = 0; q.draft = 0; q.target = 0; q.pend = 0; q.len = 0; q.corr = -1;
+  q.n = 0; q.draft = 0; q.target = 0; q.pend = 0; q.len = 0; q.corr = -1; q.failed = 0;
   const int K1 = p.K + 1;
   const int i = (int)threadIdx.x >> p.lanes_log2, l = (int)threadIdx.x & ((1 << p.lanes_log2) - 1);
   if (i < K1) {
@@ -184,6 +188,7 @@ __device__ __forceinline__ ScanLoads scan_request(const ScanParams& p, int b) {
     if (l == 0) {
       if (i < p.K) q.draft = p.draft[(int64_t)b * p.K + i];
       if (p.target_tokens) q.target = p.target_tokens[row];
+      if (p.status) q.failed = *reinterpret_cast<const volatile int*>(p.status);
     }
   }
   if (threadIdx.x == 0 && p.carry && p.state_in) {
@@ -194,9 +199,22 @@ __device__ __forceinline__ ScanLoads scan_request(const ScanParams& p, int b) {
   return q;
 }
 
-// All parts of the thread's row that are its own, folded.  TAGGED: a part that has not arrived yet is waited for (it has
-// been issued; bounded, and a row whose wait runs out is flagged), and the slots are emptied.  Part `own_slot` of row
-// `own_row` is `own`.
+// A state that has been issued but did not show yet.
+__device__ __forceinline__ int4 wait_part(const Partial* slot, int* status, unsigned long long limit_ns) {
+  const unsigned long long t0 = global_ns();
+  int4 v = ld_part(slot);
+  for (int spins = 1; v.w == 0; ++spins, v = ld_part(slot)) {
+    if ((spins & 63) != 0 || global_ns() - t0 <= limit_ns) continue;
+    v = ld_part(slot);  // (the clock also runs while the context is off the GPU: the state may have landed since)
+    if (v.w != 0) break;
+    if (status) atomicCAS(status, 0, kErrTimeoutState);
+    return tagged(failed_partial());
+  }
+  return v;
+}
+
+// All parts of the thread's row that are its own, folded.  TAGGED: a part that has not arrived yet is waited for, and the
+// slots are emptied.  Part `own_slot` of row `own_row` is `own`.
 template <bool TAGGED>
 __device__ __forceinline__ Partial gather_parts(const ScanParams& p, int64_t row, int l, const ScanLoads& q, int64_t own_row,
                                                 int own_slot, const Partial& own) {
@@ -208,14 +226,7 @@ __device__ __forceinline__ Partial gather_parts(const ScanParams& p, int64_t row
     for (int j = l; j < q.n; j += step) {
       int4 v = j == l ? q.part : ld_part(src + j * p.part_pitch);
       if (row == own_row && j == own_slot) v = tagged(own);
-      if (v.w == 0) {
-        const unsigned long long t0 = global_ns();
-        for (int spins = 0; v.w == 0; v = ld_part(src + j * p.part_pitch))
-          if ((++spins & 63) == 0 && global_ns() - t0 > kWaitLimitNs) {
-            v = make_int4(0, 0x7fc00000, 0x7fc00000, 1);  // NaN sums
-            break;
-          }
-      }
+      if (v.w == 0) v = wait_part(src + j * p.part_pitch, p.status, p.wait_ns);
       st_part(src + j * p.part_pitch, make_int4(0, 0, 0, 0));
       if (j == l) acc = untagged(v);
       else merge_partial(acc, untagged(v), p.scale);
@@ -251,7 +262,8 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
     Partial acc = fold_lanes(mine, p.lanes_log2, p.scale);
     if (p.row_out) {
       if (first) {
-        if (acc.idx != kIdxNone) acc.idx += p.idx_offset;
+        if (q.failed) acc = failed_partial();
+        else if (acc.idx < kIdxFailed) acc.idx += p.idx_offset;
         p.row_out[row] = acc;
       }
     } else if (first) {
@@ -259,9 +271,10 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
       // lg2.approx and the fast division are good to ~1e-6 here (S >= 1 once a row has a finite entry); this is the
       // end of the step's critical path
       H = fmaxf(kLn2 * (lg2_approx(acc.S) - __fdividef(acc.u, acc.S)), 0.f);
-      if (!(fabsf(acc.S) <= 3.0e38f) || !(acc.mx <= 3.0e38f) || acc.mx <= kMaskFloor) flag |= kFlagNonFinite;
-      // A fused step whose GEMM kernel gave up has no usable statistics: every row is flagged, nothing is accepted.
-      if (p.status != nullptr && *reinterpret_cast<const volatile int*>(p.status) != 0) flag |= kFlagStepFailed;
+      // A step one of whose waits ran out has no usable statistics: its rows are flagged, nothing is accepted.
+      const bool lost = acc.idx == kIdxFailed && acc.mx > 3.0e38f;
+      if (q.failed || lost) flag |= kFlagStepFailed;
+      if (!lost && (!(fabsf(acc.S) <= 3.0e38f) || !(acc.mx <= 3.0e38f) || acc.mx <= kMaskFloor)) flag |= kFlagNonFinite;
       int y = acc.idx;
       if (flag || (unsigned)y >= (unsigned)p.V) y = 0;  // keep every emitted id in range
       greedy = y;
