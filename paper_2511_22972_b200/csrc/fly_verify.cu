@@ -100,6 +100,11 @@ struct FlatPlan {
 //   plain stream order   the grid fits on the device at once (4 blocks per SM); cost = blocks on the busiest SM x
 //                        slices per warp, ties go to the count nearest two blocks per SM (the next step's blocks
 //                        can then already be resident, waiting); more rows than slots: whole rows, several waves
+//   two pieces per row   6 to 7 long bf16 rows per SM: equal blocks of 200 KB and more leave the second wave uneven, some SMs
+//                        with four of them while others have none.  us, whole rows / two pieces: 128256 bf16: 888 rows
+//                        42.3 / 41.3, 960 46.5 / 44.0, 1024 47.5 / 46.2; 152064: 48.6 / 46.7, 52.7 / 50.1, 54.4 / 52.8; 98312:
+//                        34.9 / 34.5, 36.8 / 36.6, 38.5 / 38.4; where the lines lie: 82000 30.1 / 30.8, 31.8 / 32.6, 33.3 / 34.2;
+//                        fp32, twice the bytes per slice's work: 64000 38.3 / 38.4, 39.9 / 40.8, 41.7 / 43.1
 //   inputs_ready         throughput, not latency: few large pieces (a quarter of a block per SM and step is
 //                        enough, consecutive steps overlap many deep), the count with the fewest slices per row
 //   packed rows          where whole pieces would leave more than a quarter of the last wave's slots empty, the
@@ -128,8 +133,8 @@ int rows_per_block_log2(int sm_count, int64_t rows, int64_t n, bool inputs_ready
   if (!many) return 0;
   return (rows >= 8 * gmax && n <= 512) || (rows >= 4 * gmax && n <= 128) ? 3 : 2;
 }
-FlatPlan plan_flat(int sm_count, int64_t rows, int64_t n, bool vector, int64_t min_units, int64_t stride_units, int cap,
-                   bool inputs_ready, int forced) {
+FlatPlan plan_flat(int sm_count, int64_t rows, int64_t n, int elem_bytes, bool vector, int64_t min_units, int64_t stride_units,
+                   int cap, bool inputs_ready, int forced) {
   FlatPlan pl;
   const int64_t gmax = (int64_t)sm_count * fly::kReduceBlocksPerSM;
   int64_t smax = n / min_units;  // pieces of at least min_units
@@ -155,7 +160,7 @@ FlatPlan plan_flat(int sm_count, int64_t rows, int64_t n, bool vector, int64_t m
       if (best < 0 || cost <= best) { best = cost; s = c; }
     }
   } else if (rows >= gmax) {
-    s = 1;
+    s = elem_bytes == 2 && n >= 12 * min_units && 2 * rows >= 3 * gmax && 4 * rows <= 7 * gmax ? 2 : 1;
   } else {
     int64_t best = -1, best_dist = 0;
     for (int64_t c = 1; c <= smax && rows * c <= gmax; ++c) {
@@ -285,7 +290,7 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   const int64_t n = vec ? V / kE : V;
   const int64_t min_units = vec ? kMinBlockBytes / 16 : kMinBlockBytes / (int64_t)sizeof(T);
   const int64_t stride_units = (int64_t)fly::kReduceWarps * kReduceUnroll * 32;
-  const FlatPlan pl = plan_flat(sm_count, rows, n, vec, min_units, stride_units, cap, inputs_ready, forced);
+  const FlatPlan pl = plan_flat(sm_count, rows, n, (int)sizeof(T), vec, min_units, stride_units, cap, inputs_ready, forced);
   fly::ReducePlan g;
   g.n = n; g.span = pl.span; g.Q = pl.Q; g.total = rows * pl.span;
   g.pieces = pl.Q < (1 << 30) ? pl.pieces : 0; g.V = V; g.row_stride = row_stride;
@@ -745,7 +750,7 @@ fly_status_t fly_verify_plan(int32_t sm_count, int64_t rows, int32_t vocab, fly_
   if (vector_path && vocab < per_seg * 32) return FLY_ERR_INVALID_ARG;
   const int64_t n = vector_path ? vocab / per_seg : vocab;
   const int64_t min_units = vector_path ? kMinBlockBytes / 16 : kMinBlockBytes / esz;
-  const FlatPlan pl = plan_flat(sm_count, rows, n, vector_path != 0, min_units, (int64_t)fly::kReduceWarps * kReduceUnroll * 32, kMaxSplits,
+  const FlatPlan pl = plan_flat(sm_count, rows, n, (int)esz, vector_path != 0, min_units, (int64_t)fly::kReduceWarps * kReduceUnroll * 32, kMaxSplits,
                                 inputs_ready != 0, forced_pieces);
   out->grid = pl.grid;
   out->slots = pl.slots;

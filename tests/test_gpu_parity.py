@@ -597,3 +597,34 @@ def test_masked_logits_weigh_nothing_at_any_temperature(dtype, V, T):
         fv.set_splits(splits)
         check(fv, logits, draft, 1.0, 2, temperature=T, what=f"{dtype} V={V} T={T} splits={splits}")
     fv.close()
+
+
+@pytest.mark.parametrize("B,K,V", [(74, 11, 98309), (111, 7, 98304)])
+def test_many_long_rows_cut_in_two(B, K, V):
+    # 888 rows, at every alignment and at none; the scan as a kernel of its own and without a handle as well
+    from paper_2511_22972_b200 import VerifyBuffers, binding as Bd
+    w = small("bf16", B=B, K=K, V=V)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert Bd.plan(sms, w.rows, V).grid == 2 * w.rows, "this shape is meant to cut rows in two"
+    logits, draft = draw(w, step=K, guard=False)
+    rows = logits.view(-1, V)
+    rows[::3, V // 2 + 7] = rows[::3].float().max(dim=1).values.to(rows.dtype) + 1.0     # in the second piece
+    draft[::2, 0] = rows.view(B, K + 1, V)[::2, 0].float().argmax(-1).to(torch.int32)
+    y = torch.stack([r.float().argmax(-1) for r in logits]).to(torch.int32)
+    fv = FlyVerify(B, K, V, "bf16")
+    a = gpu_step(fv, logits, draft, 1.0, 1)
+    assert torch.equal(a.target_argmax, y) and (a.row_flags == 0).all()
+    H = torch.stack([torch.distributions.Categorical(logits=r.double()).entropy() for r in logits[:: B // 4]])
+    assert (a.entropy[:: B // 4].double() - H).abs().max().item() < 1e-4
+    one = FlyVerify(B, K, V, "bf16")
+    one.set_splits(1)
+    fv.set_scan_mode(True)
+    static = VerifyBuffers(B, K, DEV)
+    Bd.run_static(Bd.static_args(B, K, draft, static.accept_len, static.out_tokens, logits=logits, theta=1.0, W=1, state_out=static.state,
+                                 target_argmax=static.target_argmax, entropy=static.entropy, row_flags=static.row_flags), V)
+    for b in (gpu_step(one, logits, draft, 1.0, 1), gpu_step(fv, logits, draft, 1.0, 1), static):
+        assert torch.equal(a.target_argmax, b.target_argmax) and (a.entropy - b.entropy).abs().max().item() < 1e-5
+        far = ((a.entropy[:, :K] - 1.0).abs() > 1e-4).all(dim=1)      # entropies at the threshold may go either way
+        assert far.float().mean() > 0.9 and torch.equal(a.out_tokens[far], b.out_tokens[far])
+    fv.close()
+    one.close()

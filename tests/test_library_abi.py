@@ -134,3 +134,15 @@ def test_launch_geometry_rule():
                         assert p.grid <= max(148 * 4, rows)
                     else:
                         assert p.grid <= max(2 * 148, rows)
+
+
+@pytest.mark.parametrize("rows,vocab,dtype,pieces", [
+    (887, 128256, "bf16", 0), (888, 128256, "bf16", 2), (1036, 152064, "bf16", 2), (1037, 128256, "bf16", 1), (1024, 98304, "bf16", 2),
+    (1024, 98303, "bf16", 1), (1024, 64000, "f32", 1)])
+def test_six_to_seven_long_rows_per_sm_are_cut_in_two(rows, vocab, dtype, pieces):
+    p = Bd.plan(148, rows, vocab, dtype)
+    n = p.units_per_row
+    if pieces == 0:
+        assert p.row_span == n and p.grid <= 592      # packed end to end
+    else:
+        assert p.row_span == pieces * p.units_per_block >= n and p.grid == rows * pieces and p.slots == pieces
