@@ -172,9 +172,10 @@ typedef struct {
 fly_status_t fly_verify_run(fly_verify_t* handle, const fly_verify_args_t* args, void* cuda_stream);
 
 /* Convenience for callers that hold HOST buffers: the same step with every
- * pointer in args a host pointer (state_in/state_out included).  Inputs are
- * copied to device staging buffers owned by the handle, the step runs, results
- * are copied back and the stream is synchronised before returning.  Host
+ * pointer in args a host pointer (state_in/state_out included).  Inputs go through
+ * staging buffers owned by the handle, the step runs, results come back the same
+ * way and the stream is synchronised before returning.  Logits of up to 5 MB that lie
+ * in one page-locked range are read where they are.  Host
  * buffers should be page-locked for full copy bandwidth.  On the fused path
  * hidden is a host pointer; weight (a model parameter, not a per-step input)
  * remains a DEVICE pointer. */

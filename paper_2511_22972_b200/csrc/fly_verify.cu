@@ -12,6 +12,7 @@
 #include <cudaTypedefs.h>
 
 #include "fly_common.cuh"
+#include "host_span.h"
 #include "lmhead_kernel.cuh"
 #include "pld_kernel.cuh"
 #include "reduce_kernel.cuh"
@@ -72,6 +73,7 @@ struct fly_verify {
   size_t st_logits_bytes = 0;
   int32_t* st_host = nullptr;  // page-locked: draft | state_in | target tokens || state_out | accept | rollback | tokens | argmax | flags | entropy
   int32_t* st_ints = nullptr;  // the same block's device address
+  PFN_cuPointerGetAttributes pointer_attributes = nullptr;
 };
 
 namespace {
@@ -79,6 +81,25 @@ namespace {
 fly_status_t cuda_fail(fly_verify* h, cudaError_t e) {
   h->last_cuda_error = (int)e;
   return FLY_ERR_CUDA;
+}
+
+fly::HostSpan host_span(fly_verify* h, const void* p) {
+  fly::HostSpan s = {};
+  if (!h->pointer_attributes) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &found) != cudaSuccess || !fn) {
+      (void)cudaGetLastError();
+      return s;
+    }
+    h->pointer_attributes = reinterpret_cast<PFN_cuPointerGetAttributes>(fn);
+  }
+  CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE,
+                                CU_POINTER_ATTRIBUTE_IS_MANAGED};
+  void* to[] = {&s.type, &s.device, &s.start, &s.size, &s.managed};
+  if (h->pointer_attributes(5, what, to, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return fly::HostSpan{};
+  return s;
 }
 
 // Launch geometry of the row reduction (the flat index space described at the head of reduce_kernel.cuh).
@@ -841,11 +862,7 @@ fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, vo
   // copied: the copy engine moves 55 GB/s, the SMs' reads 50.  Read in place / copied, us a step: 0.26 MB 29 / 34, 0.9 MB
   // 61 / 68, 4.6 MB 110 / 177, 36.9 MB 740 / 710.
   const void* direct = nullptr;
-  if (a->logits && logit_span <= kDirectBytes) {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, a->logits) != cudaSuccess) (void)cudaGetLastError();
-    else if (at.type == cudaMemoryTypeHost && at.devicePointer) direct = at.devicePointer;
-  }
+  if (a->logits && logit_span <= kDirectBytes && fly::readable_in_place(host_span(h, a->logits), a->logits, logit_span)) direct = a->logits;
   const size_t logit_bytes = direct ? 0 : logit_span;
   if (logit_bytes > h->st_logits_bytes) {
     cudaFree(h->st_logits);
