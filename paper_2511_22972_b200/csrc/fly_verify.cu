@@ -862,7 +862,8 @@ fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, vo
   // copied: the copy engine moves 55 GB/s, the SMs' reads 50.  Read in place / copied, us a step: 0.26 MB 29 / 34, 0.9 MB
   // 61 / 68, 4.6 MB 110 / 177, 36.9 MB 740 / 710.
   const void* direct = nullptr;
-  if (a->logits && logit_span <= kDirectBytes && fly::readable_in_place(host_span(h, a->logits), a->logits, logit_span)) direct = a->logits;
+  if (a->logits && logit_span <= kDirectBytes && fly::readable_in_place(host_span(h, a->logits), a->logits, logit_span, esz))
+    direct = a->logits;
   const size_t logit_bytes = direct ? 0 : logit_span;
   if (logit_bytes > h->st_logits_bytes) {
     cudaFree(h->st_logits);

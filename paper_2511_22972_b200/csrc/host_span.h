@@ -15,10 +15,10 @@ struct HostSpan {
 };
 
 // A kernel that leaves the mapping faults, where a copy is refused: the whole buffer has to lie in one page-locked range, and
-// not its first byte alone.
-inline bool readable_in_place(const HostSpan& s, const void* host, size_t bytes) {
+// not its first byte alone.  Nor can a kernel load elements off their own alignment, which a copy moves to an aligned place.
+inline bool readable_in_place(const HostSpan& s, const void* host, size_t bytes, size_t element) {
   const uint64_t p = (uint64_t)(uintptr_t)host;
-  return s.type == 1 && !s.managed && s.device == p && s.start <= p && bytes <= s.size && p - s.start <= s.size - bytes;
+  return p % element == 0 && s.type == 1 && !s.managed && s.device == p && s.start <= p && bytes <= s.size && p - s.start <= s.size - bytes;
 }
 
 }  // namespace fly

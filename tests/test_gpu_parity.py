@@ -628,3 +628,35 @@ def test_many_long_rows_cut_in_two(B, K, V):
         assert far.float().mean() > 0.9 and torch.equal(a.out_tokens[far], b.out_tokens[far])
     fv.close()
     one.close()
+
+
+@pytest.mark.parametrize("dtype,V", [("bf16", 5000), ("bf16", 130), ("f32", 5000)])
+@pytest.mark.parametrize("off", [0, 1, 2, 3, 4, 6])
+def test_host_logits_at_any_byte_offset_and_rewritten_in_place(dtype, V, off):
+    # a page-locked message whose payload starts at any byte: what no kernel can load in place goes through the copy.  The same
+    # buffers are filled anew for every step, which has to see what they hold then
+    from paper_2511_22972_b200 import VerifyBuffers
+    w = small(dtype, B=3, K=4, V=V)
+    size = 2 if dtype == "bf16" else 4
+    fv = FlyVerify(w.B, w.K, V, dtype)
+    raw = torch.empty(w.rows * V * size + 16, dtype=torch.uint8).pin_memory()
+
+    class View:                                   # torch has no tensors off their element's alignment
+        def data_ptr(self):
+            return raw.data_ptr() + off
+    out = VerifyBuffers(w.B, w.K, "cpu", pinned=True)
+    drafts = torch.empty(w.B, w.K, dtype=torch.int32).pin_memory()
+    state = np.array([[0, 0, -1]] * w.B)
+    for step in range(3):
+        logits, draft = draw(w, step=step)
+        host = logits.cpu().contiguous()
+        raw[off:off + host.numel() * size].copy_(host.view(-1).view(torch.uint8))
+        drafts.copy_(draft)
+        a = fv.make_args(w.B, w.K, drafts, out.accept_len, out.out_tokens, logits=View(), theta=1.0, W=2, boundary="carry",
+                         state_in=out.state, state_out=out.state, rollback=out.rollback, target_argmax=out.target_argmax,
+                         entropy=out.entropy, row_flags=out.row_flags)
+        fv.run_host(a, torch.cuda.current_stream().cuda_stream)
+        ref = oracle_step(logits, draft, 1.0, 2, boundary="carry", state=state)
+        assert_parity(out, ref, f"{dtype} V={V} off={off} step={step}")
+        state = ref.state_out
+    fv.close()

@@ -20,17 +20,18 @@ def rule(tmp_path_factory):
     d = tmp_path_factory.mktemp("span")
     (d / "span.cpp").write_text("""
 #include "host_span.h"
-extern "C" int in_place(unsigned type, uint64_t device, uint64_t start, size_t size, unsigned managed, uint64_t host, size_t bytes) {
+extern "C" int in_place(unsigned type, uint64_t device, uint64_t start, size_t size, unsigned managed, uint64_t host, size_t bytes,
+                        size_t element) {
   fly::HostSpan s; s.type = type; s.device = device; s.start = start; s.size = size; s.managed = managed;
-  return fly::readable_in_place(s, (const void*)(uintptr_t)host, bytes);
+  return fly::readable_in_place(s, (const void*)(uintptr_t)host, bytes, element);
 }
 """)
     subprocess.run([cxx, "-std=c++17", "-Wall", "-Wextra", "-Werror", "-shared", "-fPIC", "-I", build.CSRC, "-o", str(d / "span.so"),
                     str(d / "span.cpp")], check=True)
     fn = C.CDLL(str(d / "span.so")).in_place
-    fn.argtypes = [C.c_uint, C.c_uint64, C.c_uint64, C.c_size_t, C.c_uint, C.c_uint64, C.c_size_t]
-    return lambda host, size, start=BASE, type=1, device=None, managed=0, bytes=PAGE: bool(
-        fn(type, host if device is None else device, start, size, managed, host, bytes))
+    fn.argtypes = [C.c_uint, C.c_uint64, C.c_uint64, C.c_size_t, C.c_uint, C.c_uint64, C.c_size_t, C.c_size_t]
+    return lambda host, size, start=BASE, type=1, device=None, managed=0, bytes=PAGE, element=2: bool(
+        fn(type, host if device is None else device, start, size, managed, host, bytes, element))
 
 
 def test_the_whole_buffer_has_to_lie_in_one_page_locked_range(rule):
@@ -47,3 +48,9 @@ def test_other_memory_is_copied(rule):
     assert not rule(BASE, 16 * PAGE, type=2)                     # device memory
     assert not rule(BASE, 16 * PAGE, managed=1)
     assert not rule(BASE, 16 * PAGE, device=BASE + 2 ** 40)      # registered under another address
+
+
+@pytest.mark.parametrize("element", [2, 4])
+def test_elements_off_their_alignment_are_copied(rule, element):
+    for off in range(1, 9):
+        assert rule(BASE + off, 16 * PAGE, element=element) == (off % element == 0)
