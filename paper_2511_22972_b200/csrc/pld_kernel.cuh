@@ -74,6 +74,8 @@ __global__ void __launch_bounds__(kThreads) pld_draft_kernel(const Params p) {
     const int n_tok = L - 1;  // candidates t = 0 .. L-2 (the continuation starts at t + 1 <= L - 1)
     const int n_seg = (head + n_tok + 3) / 4;
     constexpr int kStep = kThreads * kVecs;
+    // (Ordinary loads: the kernel before may have been writing the tokens while this one was already resident, so they are
+    // not read-only for its life, which the non-coherent path would require.)
     for (int s0 = rank * kStep; s0 < n_seg && seen < p.max_ngram; s0 += ranks * kStep) {
       int4 v[kVecs];
 #pragma unroll
@@ -82,12 +84,12 @@ __global__ void __launch_bounds__(kThreads) pld_draft_kernel(const Params p) {
         const int t = s * 4 - head;
         v[j] = make_int4(~last, ~last, ~last, ~last);
         if (t >= 0 && t + 3 < n_tok) {
-          v[j] = __ldg(seg + s);
+          v[j] = seg[s];
         } else if (s < n_seg) {
-          if (t >= 0 && t < n_tok) v[j].x = __ldg(tok + t);
-          if (t + 1 >= 0 && t + 1 < n_tok) v[j].y = __ldg(tok + t + 1);
-          if (t + 2 >= 0 && t + 2 < n_tok) v[j].z = __ldg(tok + t + 2);
-          if (t + 3 >= 0 && t + 3 < n_tok) v[j].w = __ldg(tok + t + 3);
+          if (t >= 0 && t < n_tok) v[j].x = tok[t];
+          if (t + 1 >= 0 && t + 1 < n_tok) v[j].y = tok[t + 1];
+          if (t + 2 >= 0 && t + 2 < n_tok) v[j].z = tok[t + 2];
+          if (t + 3 >= 0 && t + 3 < n_tok) v[j].w = tok[t + 3];
         }
       }
 #pragma unroll

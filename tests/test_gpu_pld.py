@@ -91,3 +91,30 @@ def test_matches_at_the_edges_of_segments_rounds_and_blocks(L, pad):
     stride = (L + 3) // 4 * 4 + pad
     for mx, mn in [(n, n), (5, 1)]:
         run(seqs, 8, mx, mn, pad_to=stride)
+
+
+def test_contexts_written_by_the_kernel_before_in_the_stream():
+    # the drafter is launched while the step before it still runs, and reads what that step writes: its out_tokens [B, K+1]
+    from paper_2511_22972_b200 import FlyVerify, VerifyBuffers, verify
+    B, K, V = 24, 31, 1000
+    fv = FlyVerify(B, K, V, "f32")
+    st = torch.cuda.current_stream().cuda_stream
+    g = torch.Generator().manual_seed(5)
+    steps = []
+    for i in range(8):                            # tokens of a small alphabet, so that n-grams recur; every position is accepted
+        y = torch.randint(0, 6, (B, K + 1), generator=g)
+        logits = torch.zeros(B, K + 1, V)
+        logits.scatter_(2, y[..., None], 30.0)
+        steps.append((y, logits.to(DEV), y[:, :K].to(torch.int32).contiguous().to(DEV)))
+    out, lengths, got = VerifyBuffers(B, K, DEV), torch.full((B,), K + 1, dtype=torch.int32, device=DEV), []
+    torch.cuda.synchronize()
+    for i in range(200):
+        y, logits, draft = steps[i % len(steps)]
+        verify(fv, logits, draft, out, theta=1.0, W=1, stream=st)
+        got.append(Bd.pld_draft(out.out_tokens, lengths, 5, 4, 1, stream=st))
+    torch.cuda.synchronize()
+    want = [[oracle_pld(row.tolist(), 5, 4, 1) for row in y] for y, _, _ in steps]
+    for i, (draft, count, pos, ng) in enumerate(got):
+        for b, (prop, p, n) in enumerate(want[i % len(steps)]):
+            assert (count[b].item(), pos[b].item(), ng[b].item()) == (len(prop), p, n) and draft[b, :len(prop)].tolist() == prop, (i, b)
+    fv.close()
