@@ -17,9 +17,9 @@ constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kMaskFloor = -999424.0f;
 // The floor at temperature T.  Masked logits, and the lanes of a ragged slice that hold none, weigh 2^(floor * log2(e) / T - r):
 // nothing as long as the exponent is far below -126, which the plain floor is up to T = 1024 (-1408).  Above, it doubles with T.
-inline float mask_floor(double T) {
+__host__ __device__ inline float mask_floor(float T) {
   float f = kMaskFloor;
-  for (; T > 1024.0; T *= 0.5) f *= 2.0f;
+  for (; T > 1024.0f; T *= 0.5f) f *= 2.0f;
   return f;
 }
 constexpr int kIdxNone = 0x7fffffff;

@@ -58,7 +58,7 @@ struct fly_verify {
   fly::Partial* lm_folded = nullptr;    // [max_rows]: partial states folded over CTAs
   int* lm_status = nullptr;             // device word: first bounded wait that ran out (sticky until read)
   int* state_status = nullptr;          // the word after it: the same of the row reduction, a partial state that did not arrive
-  size_t scratch_bytes = 0;             // of the block that starts at `partials` and ends with these two words
+  size_t scratch_bytes = 0;             // of the block that starts at `partials` and holds these two words
   int lm_pairs = 0;                     // CTA pairs that can be resident at once
   int weight_vd = 0;                    // 0: weight [hidden, V]; 1: weight [V, hidden]
   PFN_cuTensorMapEncodeTiled encode_tiled = nullptr;
@@ -315,7 +315,7 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   fly::ReducePlan g;
   g.n = n; g.span = pl.span; g.Q = pl.Q; g.total = rows * pl.span;
   g.pieces = pl.Q < (1 << 30) ? pl.pieces : 0; g.V = V; g.row_stride = row_stride;
-  g.scale = exponent_scale(temperature); g.floor = fly::mask_floor(temperature); g.wait_first = inputs_ready ? 0 : 1;
+  g.scale = exponent_scale(temperature); g.wait_first = inputs_ready ? 0 : 1;
   g.rows = (int)rows;
   static_assert(fly::kReduceWarps == 8, "rows per block x warps per row");
   g.warps_log2 = 3 - pl.rows_log2;
@@ -338,7 +338,7 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   cfg.dynamicSmemBytes = vec ? reduce_smem_bytes(pl.grid, sm_count, inputs_ready) : 0;
   const T* src = static_cast<const T*>(logits);
   auto kernel = fly::reduce_rows_flat<T, kReduceUnroll, false, false, true>;
-  if (vec && g.floor == fly::kMaskFloor)
+  if (vec && fly::mask_floor((float)temperature) == fly::kMaskFloor)
     kernel = pl.rows_log2 > 0 ? fly::reduce_rows_flat<T, kReduceUnroll, true, true, false> : fly::reduce_rows_flat<T, kReduceUnroll, true, false, false>;
   else if (vec)
     kernel = pl.rows_log2 > 0 ? fly::reduce_rows_flat<T, kReduceUnroll, true, true, true> : fly::reduce_rows_flat<T, kReduceUnroll, true, false, true>;
@@ -450,7 +450,7 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     p.row0 = (int)row0;
     p.w_kmajor = h->weight_vd;
     p.scale = exponent_scale(a->temperature);
-    p.floor = fly::mask_floor(a->temperature);
+    p.floor = fly::mask_floor((float)a->temperature);
     p.partials = h->lm_partials;
     p.status = h->lm_status;
     cudaLaunchConfig_t cfg;
@@ -556,9 +556,9 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   if (e != cudaSuccess) { delete h; return FLY_ERR_CUDA; }
   h->sm_count = sms > 0 ? sms : 148;
   if (set_reduce_attrs() != cudaSuccess) { delete h; return FLY_ERR_CUDA; }
-  // one block, all zero: slots | folded states | arrival counters | status words
+  // one block, all zero: slots | folded states | arrival counters | status words, on a line of their own
   const size_t slots = (size_t)h->max_rows * kMaxSplits, rows = (size_t)h->max_rows;
-  const size_t bytes = (slots + rows) * sizeof(fly::Partial) + rows * sizeof(unsigned int) + 2 * sizeof(int);
+  const size_t bytes = (slots + rows) * sizeof(fly::Partial) + (rows + 128) * sizeof(unsigned int);
   e = cudaMalloc(&h->partials, bytes);
   if (e == cudaSuccess) e = cudaMemset(h->partials, 0, bytes);
   if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the first step may run on a stream that does not wait for this one
@@ -569,7 +569,7 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   }
   h->lm_folded = h->partials + slots;
   h->tickets = reinterpret_cast<unsigned int*>(h->lm_folded + rows);
-  h->lm_status = reinterpret_cast<int*>(h->tickets + rows);
+  h->lm_status = reinterpret_cast<int*>(h->tickets + rows + 64);
   h->state_status = h->lm_status + 1;
   h->scratch_bytes = bytes;
   if (c->hidden > 0) {

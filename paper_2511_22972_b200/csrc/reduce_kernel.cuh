@@ -344,7 +344,6 @@ struct ReducePlan {
   int V;
   int64_t row_stride;  // elements
   float scale;     // log2(e) / temperature
-  float floor;     // FLOOR: logits at or below it are masked
   int warps_log2;  // SHORT: warps that share a row
   int rows;        // SHORT: all rows
   int wait_first;  // 1: wait for the previous kernel in the stream before the first read (plain stream
@@ -435,14 +434,14 @@ __device__ __forceinline__ void flush_pieces(const ScanParams& p, TailShared& sm
 // grid.x = ceil(total / Q).  VEC: a unit is a segment; else a logit (rows too short for the vector path).
 // SHORT: many rows that are too short to occupy a block each (what a block costs beyond its data is about 3 us of its slot):
 // whole rows, several per block, a group of 2^warps_log2 warps each.
-// FLOOR: the mask floor is g.floor and not kMaskFloor.  An operand of every clamp: as a register instead of a constant it costs
+// FLOOR: the mask floor is that of the temperature and not kMaskFloor.  An operand of every clamp: as a register instead of a constant it costs
 // the plain kernel 1 % (1000 rows of 128256 bf16 47.3 -> 47.9 us a step, 1088 rows 48.8 -> 49.3).
 template <typename T, int UNROLL, bool VEC, bool SHORT, bool FLOOR>
 __global__ void __launch_bounds__(kReduceThreads, kReduceBlocksPerSM)
 reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePlan g, const __grid_constant__ ScanParams tail) {
   constexpr int kE = Seg<T>::kElems;
   constexpr int kSlice = UNROLL * 32;
-  const float floor = FLOOR ? g.floor : kMaskFloor;
+  const float floor = FLOOR ? mask_floor(kLog2e / g.scale) : kMaskFloor;
   const int kStride = SHORT ? kSlice << g.warps_log2 : kReduceWarps * kSlice;
   const int gwarp = SHORT ? ((int)threadIdx.x >> 5) & ((1 << g.warps_log2) - 1) : (int)threadIdx.x >> 5;  // in the row's group
   const int last_gwarp = SHORT ? (1 << g.warps_log2) - 1 : kReduceWarps - 1;

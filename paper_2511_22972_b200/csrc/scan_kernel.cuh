@@ -164,6 +164,7 @@ struct ScanShared {
   int bits[kMaxRows];   // bit 0: mismatch (Eq. 2), bit 1: Defer (Eq. 6)
   int draft[kMaxRows];
   int pend, len, corr;  // carried state as it is honoured
+  int failed;           // a wait ran out before
 };
 
 // What a thread reads for its row, all at once.
@@ -172,7 +173,7 @@ struct ScanLoads {
   int n;                // parts of its row
   int draft, target;    // of its row (first lane of a group)
   int pend, len, corr;  // carried state (thread 0)
-  int failed;           // first lane of a group: a wait ran out, in this step or before it
+  int failed;           // last thread (row_out: first): a wait ran out before
 };
 
 __device__ __forceinline__ ScanLoads scan_request(const ScanParams& p, int b) {
@@ -188,9 +189,12 @@ __device__ __forceinline__ ScanLoads scan_request(const ScanParams& p, int b) {
     if (l == 0) {
       if (i < p.K) q.draft = p.draft[(int64_t)b * p.K + i];
       if (p.target_tokens) q.target = p.target_tokens[row];
-      if (p.status) q.failed = *reinterpret_cast<const volatile int*>(p.status);
     }
   }
+  // By one thread, for use behind the barrier: as a load of every row's first lane the record cost small steps 0.1 us, and 0.2
+  // on a line it shared with the arrival counters (9 rows of 32000 fp32: 3.92, 3.99 and 4.17 us a step in a CUDA graph).
+  if ((int)threadIdx.x == (p.row_out ? 0 : kScanThreads - 1) && p.status)
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(q.failed) : "l"(p.status) : "memory");
   if (threadIdx.x == 0 && p.carry && p.state_in) {
     q.pend = p.state_in[b * 3 + 0];
     q.len = p.state_in[b * 3 + 1];
@@ -271,9 +275,8 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
       // lg2.approx and the fast division are good to ~1e-6 here (S >= 1 once a row has a finite entry); this is the
       // end of the step's critical path
       H = fmaxf(kLn2 * (lg2_approx(acc.S) - __fdividef(acc.u, acc.S)), 0.f);
-      // A step one of whose waits ran out has no usable statistics: its rows are flagged, nothing is accepted.
       const bool lost = acc.idx == kIdxFailed && acc.mx > 3.0e38f;
-      if (q.failed || lost) flag |= kFlagStepFailed;
+      if (lost) flag |= kFlagStepFailed;
       if (!lost && (!(fabsf(acc.S) <= 3.0e38f) || !(acc.mx <= 3.0e38f) || acc.mx <= kMaskFloor)) flag |= kFlagNonFinite;
       int y = acc.idx;
       if (flag || (unsigned)y >= (unsigned)p.V) y = 0;  // keep every emitted id in range
@@ -303,7 +306,10 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
     }
   }
   if (p.row_out) return;
+  if (tid == kScanThreads - 1) sm.failed = q.failed;
   __syncthreads();
+  // A step that runs while a wait's run-out is on record has no usable statistics: its rows are flagged, nothing is accepted.
+  const bool failed = sm.failed != 0;
   if (tid < 32) {
     const int b0 = tid < K1 ? sm.bits[tid] : 0;
     uint64_t mism = __ballot_sync(0xffffffffu, b0 & 1), defer = __ballot_sync(0xffffffffu, b0 & 2);
@@ -311,6 +317,12 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
       const int b1 = tid + 32 < K1 ? sm.bits[tid + 32] : 0;
       mism |= (uint64_t)__ballot_sync(0xffffffffu, b1 & 1) << 32;
       defer |= (uint64_t)__ballot_sync(0xffffffffu, b1 & 2) << 32;
+    }
+    if (failed) {
+      mism = ~0ull;
+      defer = 0;
+      if (!p.target_tokens && tid == 0) sm.y[0] = 0;
+      __syncwarp();
     }
     const RoundOutcome o = decide_round(mism, defer, K, p.W, p.carry, sm.pend, sm.len);
     int32_t* tokens = p.out_tokens + (int64_t)b * K1;
@@ -332,6 +344,10 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
         p.state_out[b * 3 + 2] = o.st_corr_pos ? sm.y[o.st_corr_pos - 1] : -1;
       }
     }
+  }
+  if (failed) {
+    greedy = 0;
+    flag |= kFlagStepFailed;
   }
   if (first) {  // off the critical path: warp 0 is at the decision meanwhile
     if (p.target_argmax) p.target_argmax[row] = greedy;
