@@ -5,8 +5,12 @@
 // tensors in place, fill the struct on the stack and call the library (0.5 us on top of the launch).  They keep
 // nothing: no pointer, shape or check outlives the call.
 //
+// Reading a tensor may throw (a nested or sparse one has no strides or storage, a functorch wrapper no data): every
+// function runs inside guarded(), which turns that into the Python exception that the same access raises there.
+//
 // The library itself stays free of torch types; its entry points are handed in by address (init), so that there is
 // one copy of it in the process.
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ops/empty.h>
 
@@ -28,12 +32,7 @@ bool address(PyObject* o, void** p) {
   *p = nullptr;
   if (o == Py_None) return true;
   if (THPVariable_Check(o)) {
-    try {
-      *p = THPVariable_Unpack(o).data_ptr();
-    } catch (const std::exception& e) {
-      PyErr_SetString(PyExc_RuntimeError, e.what());
-      return false;
-    }
+    *p = THPVariable_Unpack(o).data_ptr();
     return true;
   }
   PyObject* r = PyObject_CallMethod(o, "data_ptr", nullptr);
@@ -44,11 +43,11 @@ bool address(PyObject* o, void** p) {
 }
 
 bool attribute(PyObject* o, PyObject* name, void** p) {
-  PyObject* v = PyObject_GetAttr(o, name);
-  if (!v) return false;
-  const bool ok = address(v, p);
-  Py_DECREF(v);
-  return ok;
+  struct Owned {
+    PyObject* v;
+    ~Owned() { Py_XDECREF(v); }
+  } owned{PyObject_GetAttr(o, name)};
+  return owned.v && address(owned.v, p);
 }
 
 bool as_text(PyObject* o, const char* what) { return PyUnicode_Check(o) && PyUnicode_CompareWithASCIIString(o, what) == 0; }
@@ -107,6 +106,12 @@ bool enough(Py_ssize_t n, Py_ssize_t want) {
   if (n != want) PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, n);
   return n == want;
 }
+
+// Other threads run while this lives (taken back on every way out, an exception among them).
+struct Unlocked {
+  PyThreadState* state = PyEval_SaveThread();
+  ~Unlocked() { PyEval_RestoreThread(state); }
+};
 
 PyObject* status(fly_status_t s) { return PyLong_FromLong((long)s); }
 
@@ -176,9 +181,10 @@ PyObject* py_verify(PyObject*, PyObject* const* v, Py_ssize_t n) {
   if (PyErr_Occurred()) return nullptr;
   a.inputs_ready = ready;
   fly_status_t s;
-  Py_BEGIN_ALLOW_THREADS
-  s = host ? api.run_host(h, &a, stream) : api.run(h, &a, stream);
-  Py_END_ALLOW_THREADS
+  {
+    Unlocked unlocked;
+    s = host ? api.run_host(h, &a, stream) : api.run(h, &a, stream);
+  }
   return status(s);
 }
 
@@ -214,9 +220,10 @@ PyObject* py_verify_fused(PyObject*, PyObject* const* v, Py_ssize_t n) {
   const int host = PyObject_IsTrue(v[12]);
   if (PyErr_Occurred()) return nullptr;
   fly_status_t s;
-  Py_BEGIN_ALLOW_THREADS
-  s = host ? api.run_host(h, &a, stream) : api.run(h, &a, stream);
-  Py_END_ALLOW_THREADS
+  {
+    Unlocked unlocked;
+    s = host ? api.run_host(h, &a, stream) : api.run(h, &a, stream);
+  }
   return status(s);
 }
 
@@ -236,9 +243,10 @@ PyObject* py_reduce_shard(PyObject*, PyObject* const* v, Py_ssize_t n) {
   if (PyErr_Occurred()) return nullptr;
   const int64_t rows = logits.size(0), stride = logits.stride(0);
   fly_status_t s;
-  Py_BEGIN_ALLOW_THREADS
-  s = api.reduce_shard(h, (int32_t)rows, src, stride, (int32_t)offset, temperature, (fly_partial_t*)dst, stream);
-  Py_END_ALLOW_THREADS
+  {
+    Unlocked unlocked;
+    s = api.reduce_shard(h, (int32_t)rows, src, stride, (int32_t)offset, temperature, (fly_partial_t*)dst, stream);
+  }
   return status(s);
 }
 
@@ -251,9 +259,10 @@ PyObject* py_run(PyObject*, PyObject* const* v, Py_ssize_t n) {
   const int host = PyObject_IsTrue(v[3]);
   if (PyErr_Occurred()) return nullptr;
   fly_status_t s;
-  Py_BEGIN_ALLOW_THREADS
-  s = host ? api.run_host(h, a, stream) : api.run(h, a, stream);
-  Py_END_ALLOW_THREADS
+  {
+    Unlocked unlocked;
+    s = host ? api.run_host(h, a, stream) : api.run(h, a, stream);
+  }
   return status(s);
 }
 
@@ -268,9 +277,10 @@ PyObject* py_run_partials(PyObject*, PyObject* const* v, Py_ssize_t n) {
   void* stream = PyLong_AsVoidPtr(v[5]);
   if (PyErr_Occurred()) return nullptr;
   fly_status_t s;
-  Py_BEGIN_ALLOW_THREADS
-  s = api.run_partials(h, a, (const fly_partial_t*)partials, world, total, stream);
-  Py_END_ALLOW_THREADS
+  {
+    Unlocked unlocked;
+    s = api.run_partials(h, a, (const fly_partial_t*)partials, world, total, stream);
+  }
   return status(s);
 }
 
@@ -283,9 +293,10 @@ PyObject* py_run_static(PyObject*, PyObject* const* v, Py_ssize_t n) {
   void* stream = PyLong_AsVoidPtr(v[4]);
   if (PyErr_Occurred()) return nullptr;
   fly_status_t s;
-  Py_BEGIN_ALLOW_THREADS
-  s = api.run_static(device, vocab, (fly_dtype_t)dtype, a, stream);
-  Py_END_ALLOW_THREADS
+  {
+    Unlocked unlocked;
+    s = api.run_static(device, vocab, (fly_dtype_t)dtype, a, stream);
+  }
   return status(s);
 }
 
@@ -301,29 +312,33 @@ PyObject* py_pld_draft(PyObject*, PyObject* const* v, Py_ssize_t n) {
   if (!integer_as(v[2], &K) || !integer_as(v[3], &mx) || !integer_as(v[4], &mn) || !integer_as(v[5], &device)) return nullptr;
   void* stream = PyLong_AsVoidPtr(v[6]);
   if (PyErr_Occurred()) return nullptr;
-  fly_status_t s = FLY_OK;
+  fly_status_t s;
   at::Tensor draft, count, pos, ngram;
-  try {
+  {
+    Unlocked unlocked;
     const int64_t B = tokens.size(0);
     const auto opt = tokens.options().requires_grad(false);
     draft = at::empty({B, K}, opt);
     count = at::empty({B}, opt);
     pos = at::empty({B}, opt);
     ngram = at::empty({B}, opt);
-    Py_BEGIN_ALLOW_THREADS
     s = api.pld_draft(device, (int32_t)B, (const int32_t*)tokens.data_ptr(), tokens.stride(0), (const int32_t*)lengths.data_ptr(), mx,
                       mn, K, (int32_t*)draft.data_ptr(), (int32_t*)count.data_ptr(), (int32_t*)pos.data_ptr(),
                       (int32_t*)ngram.data_ptr(), stream);
-    Py_END_ALLOW_THREADS
-  } catch (const std::exception& e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
-    return nullptr;
   }
   return Py_BuildValue("(iNNNN)", (int)s, THPVariable_Wrap(draft), THPVariable_Wrap(count), THPVariable_Wrap(pos),
                        THPVariable_Wrap(ngram));
 }
 
-#define FAST(name) {#name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, nullptr}
+// A C++ exception must not leave a function that Python calls.
+template <PyObject* (*F)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* v, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  return F(self, v, n);
+  END_HANDLE_TH_ERRORS
+}
+
+#define FAST(name) {#name, (PyCFunction)(void (*)(void))guarded<py_##name>, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {FAST(init),         FAST(fill), FAST(verify),       FAST(verify_fused), FAST(reduce_shard),
                          FAST(run_partials), FAST(run),  FAST(run_static), FAST(pld_draft),    {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", "Native argument marshalling of the C ABI.", -1, methods};
