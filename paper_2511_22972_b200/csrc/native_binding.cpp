@@ -53,8 +53,15 @@ bool attribute(PyObject* o, PyObject* name, void** p) {
 bool as_text(PyObject* o, const char* what) { return PyUnicode_Check(o) && PyUnicode_CompareWithASCIIString(o, what) == 0; }
 
 bool number(PyObject* o, double* v) {
-  *v = PyFloat_AsDouble(o);
-  return !(*v == -1.0 && PyErr_Occurred());
+  if (PyFloat_CheckExact(o)) {
+    *v = PyFloat_AS_DOUBLE(o);
+    return true;
+  }
+  PyObject* f = PyNumber_Float(o);  // as float(o) does
+  if (!f) return false;
+  *v = PyFloat_AS_DOUBLE(f);
+  Py_DECREF(f);
+  return true;
 }
 bool integer(PyObject* o, long long* v) {
   if (PyLong_CheckExact(o)) {

@@ -47,3 +47,9 @@ def test_tensors_without_strides_or_data_raise():
                                     for i, c in enumerate(CALLS)) + "print('alive', sum(range(4)))\n")
     lines = out.splitlines()
     assert [line.split()[:2] for line in lines] == [[str(i), "raised"] for i in range(len(CALLS))] + [["alive", "6"]], out
+
+
+def test_numbers_are_taken_as_float_and_int_take_them():
+    out = run("a = B.static_args(1, True, draft, draft, draft, theta='inf', W=torch.tensor(2), temperature=torch.tensor(0.5))\n"
+              "print(a.theta, a.K, a.W, a.temperature)\n")
+    assert out.split() == ["inf", "1", "2", "0.5"]
