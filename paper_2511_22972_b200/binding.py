@@ -203,6 +203,8 @@ class FlyVerify:
                   weight=None, theta=1.0, theta_unit="nats", W=3, boundary="reject", state_in=None,
                   state_out=None, rollback=None, target_argmax=None, entropy=None, row_flags=None,
                   target_tokens=None, temperature=0.0, inputs_ready=False):
+        if _native is None:
+            lib()  # (called without a handle)
         a = fly_verify_args_t()
         _native.fill(C.addressof(a), B, K, draft, accept_len, out_tokens, logits, row_stride, hidden, weight, theta,
                      theta_unit, W, boundary, state_in, state_out, rollback, target_argmax, entropy, row_flags,
@@ -245,7 +247,6 @@ def pld_draft(tokens, lengths, K: int, max_ngram: int = 3, min_ngram: int = 1, d
 
 def static_args(*a, **kw) -> fly_verify_args_t:
     """Fills a fly_verify_args_t (same parameters as FlyVerify.make_args) without creating a handle."""
-    lib()
     return FlyVerify.make_args(None, *a, **kw)
 
 

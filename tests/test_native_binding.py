@@ -53,3 +53,8 @@ def test_numbers_are_taken_as_float_and_int_take_them():
     out = run("a = B.static_args(1, True, draft, draft, draft, theta='inf', W=torch.tensor(2), temperature=torch.tensor(0.5))\n"
               "print(a.theta, a.K, a.W, a.temperature)\n")
     assert out.split() == ["inf", "1", "2", "0.5"]
+
+
+def test_arguments_can_be_filled_before_anything_has_loaded_the_library():
+    out = run("print(FlyVerify.make_args(None, 2, 3, draft, draft, draft, theta=0.5).K)\n")
+    assert out.split() == ["3"]
