@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes as C
 import importlib.util
+import os
 
 from . import build as _build
 
@@ -69,9 +70,12 @@ def lib() -> C.CDLL:
     global _lib, _native
     if _lib is not None:
         return _lib
+    what = "libfly_verify.so is missing and could not be built"
     try:
         path = _build.ensure_built()
+        what = "libfly_verify.so could not be loaded"
         L = C.CDLL(path)
+        what = os.path.basename(_build.NATIVE_PATH) + " could not be loaded"
         import torch  # noqa: F401  (the extension resolves its symbols in torch's libraries)
         spec = importlib.util.spec_from_file_location(__package__ + "._native", _build.NATIVE_PATH)
         native = importlib.util.module_from_spec(spec)
@@ -80,7 +84,7 @@ def lib() -> C.CDLL:
             "fly_verify_run", "fly_verify_run_host", "fly_verify_reduce_shard", "fly_verify_run_partials",
             "fly_verify_run_static", "fly_pld_draft")])
     except Exception as e:  # no silent fallback: the CUDA library is the product
-        raise ImportError(f"libfly_verify.so is missing and could not be built: {e}") from e
+        raise ImportError(f"{what}: {e}") from e
     L.fly_verify_create.argtypes = [C.POINTER(fly_verify_config_t), C.POINTER(C.c_void_p)]
     L.fly_verify_create.restype = C.c_int
     L.fly_verify_destroy.argtypes = [C.c_void_p]

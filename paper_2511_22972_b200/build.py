@@ -1,5 +1,5 @@
 """Builds the C-ABI shared library (libfly_verify.so) for sm_100a with nvcc,
-and the Python extension that marshals its arguments (_native.so) with g++.
+and the Python extension that marshals its arguments (_native.*.so) with g++.
 
 Both are built in-tree, next to this file.  `python -m
 paper_2511_22972_b200.build` rebuilds them; `ensure_built()` rebuilds only what
@@ -8,6 +8,7 @@ is older than a source.
 from __future__ import annotations
 
 import glob
+import importlib.metadata
 import os
 import shutil
 import subprocess
@@ -20,7 +21,18 @@ CSRC = os.path.join(PKG_DIR, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB_PATH = os.path.join(PKG_DIR, "libfly_verify.so")
 NATIVE_SRC = os.path.join(CSRC, "native_binding.cpp")
-NATIVE_PATH = os.path.join(PKG_DIR, "_native.so")
+
+
+def _torch_version() -> str:
+    try:
+        return importlib.metadata.version("torch")
+    except importlib.metadata.PackageNotFoundError:  # a source tree on the path
+        import torch
+        return torch.__version__
+
+
+# The extension is bound to one Python and one torch: the name says which, so that another one builds its own.
+NATIVE_PATH = os.path.join(PKG_DIR, "_native.%s.torch-%s.so" % (sysconfig.get_config_var("SOABI"), _torch_version()))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
