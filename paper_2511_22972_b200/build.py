@@ -76,18 +76,25 @@ def nvcc_path() -> str:
     return p
 
 
-def _run(cmd, what: str, verbose: bool):
+def _run(cmd, path: str, what: str, verbose: bool):
+    """Builds `path` beside its place and moves it there, so that processes that build or load it meanwhile see whole files."""
+    new = "%s.%d.so" % (path[:-3], os.getpid())
     if verbose:
-        print(" ".join(cmd), file=sys.stderr)
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    if r.returncode != 0:
-        raise RuntimeError(what + " failed:\n" + r.stdout + r.stderr)
+        print(" ".join([*cmd, "-o", path]), file=sys.stderr)
+    try:
+        r = subprocess.run([*cmd, "-o", new], capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(what + " failed:\n" + r.stdout + r.stderr)
+        os.replace(new, path)
+    finally:
+        if os.path.exists(new):
+            os.remove(new)
     if verbose and (r.stdout or r.stderr):
         print(r.stdout + r.stderr, file=sys.stderr)
 
 
 def build_lib(verbose: bool = False, extra=()) -> str:
-    _run([nvcc_path(), *NVCC_FLAGS, *extra, "-I", INCLUDE, "-I", CSRC, "-o", LIB_PATH, *sources()], "nvcc", verbose)
+    _run([nvcc_path(), *NVCC_FLAGS, *extra, "-I", INCLUDE, "-I", CSRC, *sources()], LIB_PATH, "nvcc", verbose)
     return LIB_PATH
 
 
@@ -98,8 +105,8 @@ def build_native(verbose: bool = False) -> str:
            sysconfig.get_paths()["include"], INCLUDE]
     abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
     _run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={abi}",
-          *[x for i in inc for x in ("-isystem" if i != INCLUDE else "-I", i)], "-o", NATIVE_PATH, NATIVE_SRC,
-          "-L", os.path.join(root, "lib"), "-lc10", "-ltorch_cpu", "-ltorch_python"], "g++", verbose)
+          *[x for i in inc for x in ("-isystem" if i != INCLUDE else "-I", i)], NATIVE_SRC,
+          "-L", os.path.join(root, "lib"), "-lc10", "-ltorch_cpu", "-ltorch_python"], NATIVE_PATH, "g++", verbose)
     return NATIVE_PATH
 
 

@@ -27,3 +27,37 @@ def test_a_failing_extension_is_named(monkeypatch):
     monkeypatch.setattr(binding._build, "ensure_built", lambda: build.LIB_PATH)
     with pytest.raises(ImportError, match="_native.other.so could not be loaded"):
         binding.lib()
+
+
+def test_a_build_replaces_its_file_only_when_it_is_whole(monkeypatch, tmp_path):
+    # ranks that start together each build what is out of date, while others load it
+    import os
+    import subprocess
+    import pytest
+    target = tmp_path / "lib.so"
+    target.write_text("old")
+    written = []
+
+    class Result:
+        returncode, stdout, stderr = 0, "", ""
+
+    def compiler(cmd, **kw):
+        out = cmd[cmd.index("-o") + 1]
+        written.append(out)
+        open(out, "w").write("half")
+        assert target.read_text() == "old" and os.path.dirname(out) == str(tmp_path)
+        open(out, "w").write("new")
+        return Result
+    monkeypatch.setattr(subprocess, "run", compiler)
+    monkeypatch.setattr(build, "LIB_PATH", str(target))
+    monkeypatch.setattr(build, "NATIVE_PATH", str(target))
+    for make in (build.build_lib, build.build_native):
+        target.write_text("old")
+        Result.returncode = 1
+        with pytest.raises(RuntimeError):
+            make()
+        assert target.read_text() == "old" and os.listdir(tmp_path) == ["lib.so"]
+        Result.returncode = 0
+        make()
+        assert target.read_text() == "new" and os.listdir(tmp_path) == ["lib.so"]
+    assert str(target) not in written
