@@ -101,13 +101,4 @@ __device__ __forceinline__ Partial failed_partial() {
   return p;
 }
 
-__device__ __forceinline__ Partial shfl_xor_partial(const Partial& p, int lane_mask) {
-  Partial q;
-  q.mx = __shfl_xor_sync(0xffffffffu, p.mx, lane_mask);
-  q.S = __shfl_xor_sync(0xffffffffu, p.S, lane_mask);
-  q.u = __shfl_xor_sync(0xffffffffu, p.u, lane_mask);
-  q.idx = __shfl_xor_sync(0xffffffffu, p.idx, lane_mask);
-  return q;
-}
-
 }  // namespace fly
