@@ -264,10 +264,14 @@ int reduce_smem_bytes(int grid, int sm_count, bool inputs_ready) {
 // Shared memory above 48 KB has to be asked for, per kernel and context: done when a handle (or the static entry point's slot
 // of a device) is made, before any step of it can run.  The rings of all resident blocks only fit on an SM whose L1/shared
 // split favours shared memory.
+// A call per attribute takes 10 us; whether this context has had them is asked of the kernel that gets them last.
 cudaError_t set_reduce_attrs() {
+  cudaFuncAttributes have;
+  cudaError_t e = cudaFuncGetAttributes(&have, fly::reduce_rows_flat<float, kReduceUnroll, true, true, true>);
+  if (e != cudaSuccess || have.maxDynamicSharedSizeBytes >= kReduceMaxSmem) return e;
   auto set = [](auto kernel) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kReduceMaxSmem);
-    return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kReduceMaxSmem);
   };
   auto set_all = [&](auto zero) {
     using T = decltype(zero);
@@ -276,7 +280,7 @@ cudaError_t set_reduce_attrs() {
     if (e == cudaSuccess) e = set(fly::reduce_rows_flat<T, kReduceUnroll, true, false, true>);
     return e != cudaSuccess ? e : set(fly::reduce_rows_flat<T, kReduceUnroll, true, true, true>);
   };
-  const cudaError_t e = set_all(__nv_bfloat16());
+  e = set_all(__nv_bfloat16());
   return e != cudaSuccess ? e : set_all(float());
 }
 
