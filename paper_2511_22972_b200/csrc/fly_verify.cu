@@ -564,8 +564,13 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   const size_t slots = (size_t)h->max_rows * kMaxSplits, rows = (size_t)h->max_rows;
   const size_t bytes = (slots + rows) * sizeof(fly::Partial) + (rows + 128) * sizeof(unsigned int);
   e = cudaMalloc(&h->partials, bytes);
-  if (e == cudaSuccess) e = cudaMemset(h->partials, 0, bytes);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the first step may run on a stream that does not wait for this one
+  // Cleared and waited for, as the first step may run on any stream.  Where the default stream has work queued, which it would
+  // finish first, on a stream made for it (0.2 - 0.6 ms, and 0.02 on an idle default stream).
+  cudaStream_t own = nullptr;
+  if (e == cudaSuccess && cudaStreamQuery(nullptr) == cudaErrorNotReady) e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->partials, 0, bytes, own);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(own);
+  if (own) cudaStreamDestroy(own);
   if (e != cudaSuccess) {
     cudaFree(h->partials);
     delete h;

@@ -65,3 +65,29 @@ threads = [threading.Thread(target=go, args=(i,)) for i in range(16)]
 [t.join() for t in threads]
 assert not failed, failed
 """)
+
+
+def test_making_a_handle_does_not_wait_for_work_that_is_queued():
+    # a server makes handles while the model runs; and the first step on a stream of its own finds the scratch clear
+    run("""
+logits = torch.randn(4, 4, 32000, device="cuda").to(torch.bfloat16)
+draft = logits[:, :3].float().argmax(-1).to(torch.int32)
+a = torch.randn(8192, 8192, device="cuda", dtype=torch.bfloat16)
+FlyVerify(4, 3, 32000).close()
+torch.mm(a, a)
+side = torch.cuda.Stream()
+torch.cuda.synchronize()
+for _ in range(3):
+    for _ in range(60):
+        torch.mm(a, a)                      # some 40 ms on the default stream
+    queued = torch.cuda.Event()
+    queued.record()
+    fv = FlyVerify(4, 3, 32000)
+    assert not queued.query(), "the handle was made only after the queue had run dry"
+    out = VerifyBuffers(4, 3, "cuda")
+    side.wait_stream(torch.cuda.current_stream())
+    verify(fv, logits, draft, out, theta=1.0, W=0, stream=side.cuda_stream)
+    torch.cuda.synchronize()
+    assert torch.equal(out.target_argmax.long(), logits.float().argmax(-1)) and (out.row_flags == 0).all()
+    fv.close()
+""")
