@@ -25,7 +25,7 @@ constexpr int kMaxSplits = 32;   // Partial slots per row in a handle's scratch
 constexpr int kReduceUnroll = 4;
 constexpr int64_t kMinBlockBytes = 16384;   // a block that gets less than this is all fixed cost
 constexpr int kMaxK = 63;
-constexpr size_t kDirectBytes = 5 << 20;    // host logits up to this size are read in place (fly_verify_run_host)
+constexpr size_t kDirectBytes = 5 << 20;    // host logits up to this size are read in place (fly_verify_run_host, with the figures)
 
 struct DeviceGuard {
   int prev = -1;
@@ -119,8 +119,9 @@ struct FlatPlan {
 // A block's warps walk its piece in strides of `stride_units` (one slice per warp), so a piece of 3.1 strides costs
 // its slowest warp 4 slices: among the piece counts that fit, the one with the fewest slices on the busiest SM wins.
 //   plain stream order   the grid fits on the device at once (4 blocks per SM); cost = blocks on the busiest SM x
-//                        slices per warp, ties go to the count nearest two blocks per SM (the next step's blocks
-//                        can then already be resident, waiting); more rows than slots: whole rows, several waves
+//                        slices per warp, ties go to the count nearest two blocks per SM: one has fewer bytes in flight, four
+//                        more ends (144 rows of 128256 bf16: one, two, four pieces 11.1, 10.6, 11.2 us; 72 rows: two, four,
+//                        eight 8.0, 8.1, 8.5); more rows than slots: whole rows, several waves
 //   two pieces per row   6 to 7 long bf16 rows per SM: equal blocks of 200 KB and more leave the second wave uneven, some SMs
 //                        with four of them while others have none.  us, whole rows / two pieces: 128256 bf16: 888 rows
 //                        42.3 / 41.3, 960 46.5 / 44.0, 1024 47.5 / 46.2; 152064: 48.6 / 46.7, 52.7 / 50.1, 54.4 / 52.8; 98312:
@@ -869,7 +870,8 @@ fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, vo
   // Small logits in page-locked memory that the device can address are read over the bus by the reduction itself: it reads
   // every logit once, as a copy would, needs no copy before it and starts folding with the first of them.  Large ones are
   // copied: the copy engine moves 55 GB/s, the SMs' reads 50.  Read in place / copied, us a step: 0.26 MB 29 / 34, 0.9 MB
-  // 61 / 68, 4.6 MB 110 / 177, 36.9 MB 740 / 710.
+  // 61 / 68, 4.6 MB 110 / 177, 36.9 MB 740 / 710.  The two cross somewhere between the last two; the line lies at the last
+  // size where reading in place is known to win, and nothing between has been timed.
   const void* direct = nullptr;
   if (a->logits && logit_span <= kDirectBytes && fly::readable_in_place(host_span(h, a->logits), a->logits, logit_span, esz))
     direct = a->logits;

@@ -181,7 +181,8 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
 // single diverged lane an issuer took 690 cycles per stage at any N (75 per MMA, 133 for two commits; cycle counters), a
 // producer 360 - 400: more than the weights of a stage take from HBM (~650), so that the issuers bounded every size.
 // us a step, diverged lane -> uniform warp: 36 positions x 512 x 4096 12.8 -> 9.8, x 4096 x 50264 78.5 -> 71.2,
-// x 8192 x 128256 342 -> 318; 144 x 8192 x 128256 444 -> 387; 288: 587 -> 570 (power-capped).
+// x 8192 x 128256 342 -> 318; 144 x 8192 x 128256 444 -> 387.  At 288 positions power bounds it: 589 -> 586, within what two
+// runs of one side differ by.
 __device__ __forceinline__ bool elect_lane() {
   uint32_t one;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
@@ -222,7 +223,7 @@ __host__ __device__ constexpr uint32_t instr_desc(int n, bool a_kmajor) {
          ((uint32_t)(kPairV >> 4) << 24);
 }
 
-// Running statistics of one (position, vocabulary quarter) stream.
+// Running statistics of one (position, vocabulary eighth) stream.
 struct Stream {
   float mx, S, u;
   int idx;

@@ -16,8 +16,9 @@
 // Memory pipeline (vector path).  Every warp owns a small ring in shared memory
 // that it fills with asynchronous 16-byte copies (cp.async): kDepth slices of
 // UNROLL*32 segments (2 KB each) are in flight per warp while it folds the oldest
-// one, 4 blocks x 8 warps per SM (128 KB in flight per SM, none of it in
-// registers).  A lane reads back exactly the bytes it copied, so the ring needs
+// one, none of it in registers.  An SM holds up to 4 blocks of 8 warps (128 KB
+// in flight); in plain stream order a grid of fewer blocks is spread evenly, one
+// to three per SM.  A lane reads back exactly the bytes it copied, so the ring needs
 // no barrier.  The whole grid issues its first 2 x 2 KB per warp at once, and a
 // block that goes on into the next row starts that row's first slices before it
 // merges the finished piece: a grid that runs alone (one step of a decode loop)
