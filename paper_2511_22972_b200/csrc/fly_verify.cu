@@ -59,6 +59,8 @@ struct fly_verify {
   int* lm_status = nullptr;             // device word: first bounded wait that ran out (sticky until read)
   int* state_status = nullptr;          // the word after it: the same of the row reduction, a partial state that did not arrive
   size_t scratch_bytes = 0;             // of the block that starts at `partials` and holds these two words
+  cudaEvent_t cleared = nullptr;        // the block has been cleared ...
+  bool scratch_clear = false;           // ... and that has been seen
   int lm_pairs = 0;                     // CTA pairs that can be resident at once
   int weight_vd = 0;                    // 0: weight [hidden, V]; 1: weight [V, hidden]
   PFN_cuTensorMapEncodeTiled encode_tiled = nullptr;
@@ -81,6 +83,26 @@ namespace {
 fly_status_t cuda_fail(fly_verify* h, cudaError_t e) {
   h->last_cuda_error = (int)e;
   return FLY_ERR_CUDA;
+}
+
+// A handle's scratch is cleared in the order of the default stream, and nobody waits for what is queued there: a step that comes
+// before the clearing is done waits for it on its own stream.  (One that is being captured cannot: there the host waits.)
+cudaError_t scratch_ready(fly_verify* h, cudaStream_t st) {
+  if (h->scratch_clear || st == nullptr || st == cudaStreamLegacy) return cudaSuccess;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // none of this belongs into a capture
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return e;
+  e = cudaEventQuery(h->cleared);
+  if (e == cudaErrorNotReady) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(st, &capture);
+    if (e == cudaSuccess && capture == cudaStreamCaptureStatusNone) e = cudaStreamWaitEvent(st, h->cleared, 0);
+    else if (e == cudaSuccess && (e = cudaEventSynchronize(h->cleared)) == cudaSuccess) h->scratch_clear = true;
+  } else if (e == cudaSuccess) {
+    h->scratch_clear = true;
+  }
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  return e;
 }
 
 fly::HostSpan host_span(fly_verify* h, const void* p) {
@@ -565,15 +587,13 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   const size_t slots = (size_t)h->max_rows * kMaxSplits, rows = (size_t)h->max_rows;
   const size_t bytes = (slots + rows) * sizeof(fly::Partial) + (rows + 128) * sizeof(unsigned int);
   e = cudaMalloc(&h->partials, bytes);
-  // Cleared and waited for, as the first step may run on any stream.  Where the default stream has work queued, which it would
-  // finish first, on a stream made for it (0.2 - 0.6 ms, and 0.02 on an idle default stream).
-  cudaStream_t own = nullptr;
-  if (e == cudaSuccess && cudaStreamQuery(nullptr) == cudaErrorNotReady) e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->partials, 0, bytes, own);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(own);
-  if (own) cudaStreamDestroy(own);
+  // Cleared in the order of the default stream, which the first step may not run on: see scratch_ready.
+  if (e == cudaSuccess) e = cudaMemsetAsync(h->partials, 0, bytes, nullptr);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->cleared, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(h->cleared, nullptr);
   if (e != cudaSuccess) {
     cudaFree(h->partials);
+    if (h->cleared) cudaEventDestroy(h->cleared);
     delete h;
     return FLY_ERR_CUDA;
   }
@@ -614,6 +634,7 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
       fly_status_t st = cuda_fail(h, e);
       (void)st;
       cudaFree(h->partials); cudaFree(h->lm_partials);
+      cudaEventDestroy(h->cleared);
       delete h;
       return FLY_ERR_CUDA;
     }
@@ -632,6 +653,7 @@ fly_status_t fly_verify_destroy(fly_verify_t* h) {
     cudaFree(h->st_hidden);
     cudaFree(h->st_logits);
     cudaFreeHost(h->st_host);
+    cudaEventDestroy(h->cleared);
   }
   delete h;
   return FLY_OK;
@@ -670,6 +692,8 @@ fly_status_t fly_verify_reduce_shard(fly_verify_t* h, int32_t rows, const void* 
   if (!g.ok) return FLY_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int64_t stride = row_stride ? row_stride : V;
+  cudaError_t e = scratch_ready(h, st);
+  if (e != cudaSuccess) return cuda_fail(h, e);
   fly::ScanParams p;  // the tail of the reduction folds each row's pieces: a "sequence" is one row
   memset(&p, 0, sizeof(p));
   p.B = rows;
@@ -677,8 +701,8 @@ fly_status_t fly_verify_reduce_shard(fly_verify_t* h, int32_t rows, const void* 
   p.row_out = reinterpret_cast<fly::Partial*>(partial_out);
   p.idx_offset = vocab_offset;
   p.status = h->state_status;
-  cudaError_t e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, logits, stride, V, rows, h->forced_splits, kMaxSplits,
-                                    h->partials, st, &p, temperature, false);
+  e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, logits, stride, V, rows, h->forced_splits, kMaxSplits, h->partials, st, &p,
+                        temperature, false);
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches = 1;
   return FLY_OK;
@@ -740,7 +764,8 @@ fly_status_t fly_verify_device_status(fly_verify_t* h, void* cuda_stream) {
   DeviceGuard g(h->cfg.device);
   if (!g.ok) return FLY_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  cudaError_t e;
+  cudaError_t e = scratch_ready(h, st);
+  if (e != cudaSuccess) return cuda_fail(h, e);
   int words[2] = {0, 0};  // lm_status, state_status
   if ((e = cudaMemcpyAsync(words, h->lm_status, sizeof(words), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return cuda_fail(h, e);
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(h, e);
@@ -756,8 +781,10 @@ fly_status_t fly_verify_selftest_wait(fly_verify_t* h, void* cuda_stream) {
   if (!g.ok) return FLY_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   constexpr unsigned long long kLimitNs = 2000000;
+  cudaError_t e = scratch_ready(h, st);
+  if (e != cudaSuccess) return cuda_fail(h, e);
   fly::lmhead::wait_selftest_kernel<<<1, 1, 0, st>>>(h->lm_status, kLimitNs);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e);
   // ... and a scan over one row whose only slot is empty, as every slot is between steps
   fly::ScanParams p;
@@ -805,6 +832,8 @@ fly_status_t fly_verify_run(fly_verify_t* h, const fly_verify_args_t* a, void* c
   const int64_t rows = (int64_t)a->B * (a->K + 1);
   const int64_t stride = a->row_stride ? a->row_stride : V;
   h->last_launches = 0;
+  cudaError_t e = scratch_ready(h, st);
+  if (e != cudaSuccess) return cuda_fail(h, e);
   if (!a->logits) return run_fused(h, a, st);
 
   fly::ScanParams p = scan_params(h, a, h->partials, 1);
@@ -814,7 +843,7 @@ fly_status_t fly_verify_run(fly_verify_t* h, const fly_verify_args_t* a, void* c
   const bool fused_tail = h->scan_mode == 0;
   p.tickets = fused_tail ? h->tickets : nullptr;
   p.status = h->state_status;
-  cudaError_t e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, a->logits, stride, V, rows, h->forced_splits,
+  e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, a->logits, stride, V, rows, h->forced_splits,
                                     kMaxSplits, h->partials, st, &p, a->temperature, a->inputs_ready != 0);
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches++;

@@ -75,19 +75,28 @@ draft = logits[:, :3].float().argmax(-1).to(torch.int32)
 a = torch.randn(8192, 8192, device="cuda", dtype=torch.bfloat16)
 FlyVerify(4, 3, 32000).close()
 torch.mm(a, a)
-side = torch.cuda.Stream()
+side, out, out2 = torch.cuda.Stream(), VerifyBuffers(4, 3, "cuda"), VerifyBuffers(4, 3, "cuda")
 torch.cuda.synchronize()
-for _ in range(3):
+for mode in ("global", "thread_local", "relaxed"):
     for _ in range(60):
         torch.mm(a, a)                      # some 40 ms on the default stream
     queued = torch.cuda.Event()
     queued.record()
     fv = FlyVerify(4, 3, 32000)
     assert not queued.query(), "the handle was made only after the queue had run dry"
-    out = VerifyBuffers(4, 3, "cuda")
-    side.wait_stream(torch.cuda.current_stream())
-    verify(fv, logits, draft, out, theta=1.0, W=0, stream=side.cuda_stream)
+    for step in range(2):                   # neither waits for the default stream by itself
+        verify(fv, logits, draft, out, theta=1.0, W=0, stream=side.cuda_stream)
+    captured = FlyVerify(4, 3, 32000)       # ... nor can a first step that is captured
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(side):
+        assert not queued.query()
+        graph.capture_begin(capture_error_mode=mode)
+        verify(captured, logits, draft, out2, theta=1.0, W=0, stream=side.cuda_stream)
+        graph.capture_end()
+        graph.replay()
     torch.cuda.synchronize()
-    assert torch.equal(out.target_argmax.long(), logits.float().argmax(-1)) and (out.row_flags == 0).all()
+    for o in (out, out2):
+        assert torch.equal(o.target_argmax.long(), logits.float().argmax(-1)) and (o.row_flags == 0).all()
+    captured.close()
     fv.close()
 """)
