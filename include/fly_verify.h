@@ -273,7 +273,8 @@ fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t lo
  * FLY_OPT_SPLITS          How the row reduction cuts rows into thread-block ranges.  0 (default): every row is cut
  *                         into the same number of whole pieces (at least 7 KB each) - in plain stream order the
  *                         count that keeps the grid on the device at once with the least work on the busiest SM,
- *                         with inputs_ready few large pieces, so that consecutive steps overlap many deep; where
+ *                         with inputs_ready few large pieces, so that consecutive steps overlap many deep; more rows than
+ *                         fit at once stay whole, or are cut in two where that evens out a second wave; where
  *                         whole pieces of long rows would leave much of the last wave of blocks empty, the rows are laid end
  *                         to end and that range is cut evenly instead (a block may then cover the end of one row
  *                         and the start of the next).
