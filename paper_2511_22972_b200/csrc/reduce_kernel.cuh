@@ -374,7 +374,23 @@ __device__ __forceinline__ Partial block_finish(const WarpAcc& a, Partial* sm, i
   Partial p = empty_partial();
   if (warp == 0) {
     static_assert(kReduceWarps == 8, "the fold below is over 8 lanes");
-    p = fold_lanes(sm[lane & (kReduceWarps - 1)], warps_log2, a.scale);
+    p = sm[lane & (kReduceWarps - 1)];
+    // One row: its maximum and index are those of the whole warp, one instruction each instead of three shuffles (9 rows of 32000
+    // fp32 3.97 -> 3.93 us a step, 16 rows of 128256 bf16 4.65 -> 4.61, 160 rows 12.35 -> 12.25).
+    if (warps_log2 == 3) {
+      const float m = warp_max_f32(p.mx), d = p.mx * a.scale - m * a.scale, e = ex2_approx(d);
+      p.idx = (int)warp_min_u32(p.mx == m ? (unsigned)p.idx : (unsigned)kIdxNone);
+      p.mx = m;
+      p.u = e * fmaf(d, p.S, p.u);
+      p.S *= e;
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        p.S += __shfl_xor_sync(0xffffffffu, p.S, o);
+        p.u += __shfl_xor_sync(0xffffffffu, p.u, o);
+      }
+    } else {
+      p = fold_lanes(p, warps_log2, a.scale);
+    }
   }
   return p;
 }
