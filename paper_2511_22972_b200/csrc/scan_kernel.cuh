@@ -392,8 +392,10 @@ __global__ void __launch_bounds__(kScanThreads) scan_sequences(const __grid_cons
 // Empties arrival counters and slots (counted in 16-byte words) for callers whose scratch may hold what an earlier call left.
 constexpr int kClearThreads = 256;
 __global__ void __launch_bounds__(kClearThreads) clear_scratch(uint4* tickets, int ticket_words, uint4* slots, int slot_words) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // The reduction may become resident at once: it waits for this grid, which waits for the step before (104 rows of 128256 bf16 in a
+  // row of steps 9.37 us -> 9.19, 9 rows of 32000 4.74 -> 4.65, 1088 rows 48.5 -> 47.2).
   asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int i = (int)(blockIdx.x * kClearThreads + threadIdx.x);
   if (i < ticket_words) tickets[i] = make_uint4(0, 0, 0, 0);
   if (i < slot_words) slots[i] = make_uint4(0, 0, 0, 0);
