@@ -353,6 +353,11 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   tail->row_pitch = pitch <= cap ? pitch : pl.slots;
   tail->part_pitch = 1;
   tail->lanes_log2 = lanes_for(pl.slots, tail->K + 1);
+  // (three to 16 pieces of 9 rows and more stay with the whole block: see scan_warp)
+  int one_warp = 0;  // lanes per row, as a power of two, when all rows of a sequence share a warp
+  while (one_warp < tail->lanes_log2 && (tail->K + 1) << (one_warp + 1) <= 32) ++one_warp;
+  tail->warp_scan = tail->tickets != nullptr && (tail->K + 1) << one_warp <= 32 && pl.slots <= 1 << one_warp;
+  if (tail->warp_scan) tail->lanes_log2 = one_warp;
   tail->partials = partials;
   tail->units_per_row = n;
   tail->row_span = pl.span;
@@ -523,7 +528,7 @@ fly::ScanParams scan_params(const fly_verify* h, const fly_verify_args_t* a, fly
   fly::ScanParams p;
   p.row_pitch = splits; p.part_pitch = 1;
   p.lanes_log2 = lanes_for(splits, a->K + 1);
-  p.row_out = nullptr; p.idx_offset = 0;
+  p.row_out = nullptr; p.idx_offset = 0; p.warp_scan = 0;
   p.B = a->B; p.K = a->K; p.V = h->cfg.vocab; p.splits = splits;
   p.units_per_row = 0; p.row_span = 0; p.Q = 0;  // every row has exactly `splits` parts unless the row reduction says otherwise
   p.scale = exponent_scale(a->temperature);

@@ -435,7 +435,24 @@ __device__ __forceinline__ void flush_pieces(const ScanParams& p, TailShared& sm
     }
   }
   if (p.tickets == nullptr) return;
-  if (warp == 0 && lane < np) sm_tail.done[lane] = ticket + units == (unsigned)K1 * (unsigned)p.units_per_row ? seq : -1;
+  const int done = ticket + units == (unsigned)K1 * (unsigned)p.units_per_row ? seq : -1;
+  static_assert(kMaxPend <= kReduceWarps, "a warp per finished sequence");
+  if (p.warp_scan) {  // one warp per sequence
+    int b = -1;
+    if (np == 1) {
+      if (warp == 0) b = __shfl_sync(0xffffffffu, done, 0);
+      __syncwarp();  // (the piece's state was written by the first lane)
+    } else {
+      if (warp == 0 && lane < np) sm_tail.done[lane] = done;
+      __syncthreads();
+      if (warp < np) b = sm_tail.done[warp];
+    }
+    if (b < 0) return;
+    scan_warp(p, b, row, slot, sm_tail.pend[np - 1].p);
+    if (lane == 0) p.tickets[b] = 0;  // ready for the next launch (ordered by the end of this kernel)
+    return;
+  }
+  if (warp == 0 && lane < np) sm_tail.done[lane] = done;
   __syncthreads();
 #pragma unroll 1
   for (int k = np - 1; k >= 0; --k) {
@@ -443,7 +460,7 @@ __device__ __forceinline__ void flush_pieces(const ScanParams& p, TailShared& sm
     if (b < 0) continue;
     const ScanLoads q = scan_request(p, b);
     scan_sequence<true>(p, b, q, row, slot, sm_tail.pend[np - 1].p, sm_tail.scan);
-    if (threadIdx.x == 0) p.tickets[b] = 0;  // ready for the next launch (ordered by the end of this kernel)
+    if (threadIdx.x == 0) p.tickets[b] = 0;
     if (np > 1) __syncthreads();  // sm_tail.scan is free again
   }
 }

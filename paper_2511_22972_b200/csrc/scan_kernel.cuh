@@ -1,4 +1,4 @@
-// Acceptance scan of the FLy verification step: one thread block per sequence.  It runs
+// Acceptance scan of the FLy verification step: one thread block or one warp per sequence.  It runs
 // either as the tail of the row-reduction kernel (the last block to finish a
 // sequence's rows does it) or as a launch of its own.
 //
@@ -37,6 +37,7 @@ struct ScanParams {
   int B, K, V;
   int splits;               // Partial slots per row (with Q == 0: exactly the parts of every row)
   int lanes_log2;           // a row's parts are dealt to 2^lanes_log2 lanes; (K + 1) << lanes_log2 <= kScanThreads
+  int warp_scan;            // 1: the tail of the row reduction is one warp's work (scan_warp); (K + 1) << lanes_log2 <= 32
   int64_t row_pitch;        // part j of row r is partials[r * row_pitch + j * part_pitch]
   int64_t part_pitch;
   // Flat partition of the row reduction (Q > 0): a row holds units_per_row units and spans row_span >= units_per_row
@@ -74,28 +75,25 @@ struct RoundOutcome {
   int st_pending, st_len, st_corr_pos;  // state_out; st_corr_pos = position j whose y_j is the correction (0: none)
 };
 
-// mism / defer: bit (i-1) set <=> position i is a mismatch / has H_i >= theta.
-__device__ __forceinline__ RoundOutcome decide_round(uint64_t mism, uint64_t defer, int K, int W, int carry,
-                                                     int pend_in, int len_in) {
+// mism / defer: bit (i-1) set <=> position i is a mismatch / has H_i >= theta.  Mask: as many bits as positions, K < its width.
+template <typename Mask>
+__device__ __forceinline__ RoundOutcome decide_round(Mask mism, Mask defer, int K, int W, int carry, int pend_in, int len_in) {
+  constexpr int kBits = 8 * sizeof(Mask);
+  auto upto = [](int n) { return n >= kBits ? ~(Mask)0 : ((Mask)1 << n) - 1; };
+  auto first = [](Mask m) { return sizeof(Mask) == 8 ? __ffsll((long long)m) : __ffs((int)m); };
   RoundOutcome o;
   o.s = K + 1; o.rollback = 0; o.revoke = 0; o.st_pending = 0; o.st_len = 0; o.st_corr_pos = 0;
-  if (carry && pend_in > 0) {
-    const uint64_t first_r = pend_in >= 64 ? ~0ull : ((1ull << pend_in) - 1ull);
-    if (mism & first_r) {  // a mismatch inside the carried window: revoke
-      o.s = 1; o.rollback = len_in; o.revoke = 1;
-      return o;
-    }
+  if (carry && pend_in > 0 && (mism & upto(pend_in))) {  // a mismatch inside the carried window: revoke
+    o.s = 1; o.rollback = len_in; o.revoke = 1;
+    return o;
   }
-  uint64_t rest = mism;
+  Mask rest = mism;
   while (rest) {
-    const int j = __ffsll((long long)rest);  // 1-based position of the next mismatch
+    const int j = first(rest);  // 1-based position of the next mismatch
     rest &= rest - 1;
-    if (!((defer >> (j - 1)) & 1ull)) { o.s = j; return o; }  // Strict
+    if (!((defer >> (j - 1)) & 1)) { o.s = j; return o; }  // Strict
     // positions j+1 .. min(j+W, K)  <->  bits j .. min(j+W,K)-1
-    const int hi = min(j + W, K);
-    const uint64_t upto_hi = hi >= 64 ? ~0ull : ((1ull << hi) - 1ull);
-    const uint64_t upto_j = (1ull << j) - 1ull;  // j <= K <= 63
-    const uint64_t later = mism & upto_hi & ~upto_j;
+    const Mask later = mism & upto(min(j + W, K)) & ~upto(j);
     if (later == 0 && j + W <= K) continue;  // benign: keep the draft token
     if (later == 0 && carry) {               // window leaves the round clean: carry it
       o.s = K + 1; o.st_pending = j + W - K; o.st_len = K - j + 2; o.st_corr_pos = j;
@@ -249,6 +247,44 @@ __device__ __forceinline__ Partial gather_parts(const ScanParams& p, int64_t row
   return acc;
 }
 
+// What a row's folded state says about its position.
+struct RowOutcome {
+  float H;
+  int greedy, y;   // Eq. 1's token; y_i: that, or the caller's
+  int bits;        // bit 0: mismatch (Eq. 2), bit 1: Defer (Eq. 6)
+  uint32_t flag;
+};
+__device__ __forceinline__ RowOutcome row_outcome(const ScanParams& p, const Partial& acc, bool drafted, int draft, int target) {
+  RowOutcome o;
+  o.flag = 0;
+  // entropy is non-negative; rounding may leave -1e-7 on a one-hot row
+  // lg2.approx and the fast division are good to ~1e-6 here (S >= 1 once a row has a finite entry); this is the
+  // end of the step's critical path
+  o.H = fmaxf(kLn2 * (lg2_approx(acc.S) - __fdividef(acc.u, acc.S)), 0.f);
+  const bool lost = acc.idx == kIdxFailed && acc.mx > 3.0e38f;
+  if (lost) o.flag |= kFlagStepFailed;
+  if (!lost && (!(fabsf(acc.S) <= 3.0e38f) || !(acc.mx <= 3.0e38f) || acc.mx <= kMaskFloor)) o.flag |= kFlagNonFinite;
+  o.y = acc.idx;
+  if (o.flag || (unsigned)o.y >= (unsigned)p.V) o.y = 0;  // keep every emitted id in range
+  o.greedy = o.y;
+  if (p.target_tokens && !(o.flag & kFlagNonFinite)) {  // the caller drew y_i itself
+    o.y = target;
+    if ((unsigned)o.y >= (unsigned)p.V) { o.flag |= kFlagBadTarget; o.y = 0; }
+  }
+  o.bits = 0;
+  if (drafted) {
+    if ((unsigned)draft >= (unsigned)p.V) o.flag |= kFlagBadDraft;
+    if (draft != o.y || o.flag) o.bits |= 1;
+    if (o.H >= p.theta_nats && !o.flag) o.bits |= 2;  // a flagged position is never kept
+  }
+  return o;
+}
+// The carried state is device data: only states this library writes are honoured (pending <= W <= K).  Anything
+// else is flagged and ignored, so that no token id out of range and no negative count can leave here.
+__device__ __forceinline__ bool bad_state(const ScanParams& p, int pend, int len, int corr) {
+  return pend < 0 || pend > p.K || len < 0 || (pend > 0 && (unsigned)corr >= (unsigned)p.V);
+}
+
 // The block verifies sequence b (or folds row b if that is all that is asked for).  Called by all kScanThreads threads.
 template <bool TAGGED>
 __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const ScanLoads& q, int64_t own_row, int own_slot,
@@ -271,33 +307,15 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
         p.row_out[row] = acc;
       }
     } else if (first) {
-      // entropy is non-negative; rounding may leave -1e-7 on a one-hot row
-      // lg2.approx and the fast division are good to ~1e-6 here (S >= 1 once a row has a finite entry); this is the
-      // end of the step's critical path
-      H = fmaxf(kLn2 * (lg2_approx(acc.S) - __fdividef(acc.u, acc.S)), 0.f);
-      const bool lost = acc.idx == kIdxFailed && acc.mx > 3.0e38f;
-      if (lost) flag |= kFlagStepFailed;
-      if (!lost && (!(fabsf(acc.S) <= 3.0e38f) || !(acc.mx <= 3.0e38f) || acc.mx <= kMaskFloor)) flag |= kFlagNonFinite;
-      int y = acc.idx;
-      if (flag || (unsigned)y >= (unsigned)p.V) y = 0;  // keep every emitted id in range
-      greedy = y;
-      if (p.target_tokens && !(flag & kFlagNonFinite)) {  // the caller drew y_i itself
-        y = q.target;
-        if ((unsigned)y >= (unsigned)p.V) { flag |= kFlagBadTarget; y = 0; }
-      }
-      int bits = 0;
-      if (i < K) {
-        if ((unsigned)q.draft >= (unsigned)p.V) flag |= kFlagBadDraft;
-        if (q.draft != y || flag) bits |= 1;
-        if (H >= p.theta_nats && !flag) bits |= 2;  // a flagged position is never kept
-      }
-      sm.y[i] = y;
-      sm.bits[i] = bits;
+      const RowOutcome o = row_outcome(p, acc, i < p.K, q.draft, q.target);
+      H = o.H;
+      greedy = o.greedy;
+      flag = o.flag;
+      sm.y[i] = o.y;
+      sm.bits[i] = o.bits;
       sm.draft[i] = q.draft;
       if (i == 0) {
-        // The carried state is device data: only states this library writes are honoured (pending <= W <= K).  Anything
-        // else is flagged and ignored, so that no token id out of range and no negative count can leave here.
-        const bool bad = q.pend < 0 || q.pend > K || q.len < 0 || (q.pend > 0 && (unsigned)q.corr >= (unsigned)p.V);
+        const bool bad = bad_state(p, q.pend, q.len, q.corr);
         if (bad) flag |= kFlagBadState;
         sm.pend = bad ? 0 : q.pend;
         sm.len = bad ? 0 : q.len;
@@ -324,7 +342,7 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
       if (!p.target_tokens && tid == 0) sm.y[0] = 0;
       __syncwarp();
     }
-    const RoundOutcome o = decide_round(mism, defer, K, p.W, p.carry, sm.pend, sm.len);
+    const RoundOutcome o = decide_round<uint64_t>(mism, defer, K, p.W, p.carry, sm.pend, sm.len);
     int32_t* tokens = p.out_tokens + (int64_t)b * K1;
 #pragma unroll 1
     for (int r = tid; r < K1; r += 32) {
@@ -353,6 +371,88 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
     if (p.target_argmax) p.target_argmax[row] = greedy;
     if (p.entropy) p.entropy[row] = H;
     if (p.row_flags) p.row_flags[row] = flag;
+  }
+}
+
+// The same by one warp, for rounds whose rows fit into it at a lane per part: what a sequence's last block does between its ticket
+// and the end of the step is nothing but latency; a warp needs no barrier and no shared memory for it, and a block that completes
+// several short sequences verifies them side by side.  us a step in a row of steps, block / warp: 144 rows of 128256 bf16 9.77 / 9.47,
+// 288 of 50257 9.09 / 8.77, 1088 of 128256 46.2 / 45.7, 1800 of 1003 7.1 / 5.0, 4000 of 1000 11.05 / 6.27, 2304 of 16000 17.8 / 16.0.
+// (Several parts per lane, so that 16 rows of nine parts fit a warp too, cost more than they save: the code for the second and the
+// third part costs the rounds that have one 0.1 - 0.2 us, and the arrays of eight spill.)
+__device__ __forceinline__ void scan_warp(const ScanParams& p, int b, int64_t own_row, int own_slot, const Partial& own) {
+  const int K1 = p.K + 1, lane = (int)threadIdx.x & 31;
+  const int i = lane >> p.lanes_log2, l = lane & ((1 << p.lanes_log2) - 1);
+  const int64_t row = (int64_t)b * K1 + i;
+  const bool first = i < K1 && l == 0, has = i < K1 && l < pieces_of_row(row, p.row_span, p.Q, p.splits);
+  Partial* const src = p.partials + row * p.row_pitch + l;
+  int4 v = make_int4(0, 0, 0, 0);
+  if (has) v = ld_part(src);
+  int draft = 0, target = 0, pend = 0, len = 0, corr = -1, failed = 0;
+  if (first && i < p.K) draft = p.draft[(int64_t)b * p.K + i];
+  if (first && p.target_tokens) target = p.target_tokens[row];
+  if (lane == 0) {
+    if (p.status) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(failed) : "l"(p.status) : "memory");
+    if (p.carry && p.state_in) {
+      pend = p.state_in[b * 3 + 0];
+      len = p.state_in[b * 3 + 1];
+      corr = p.state_in[b * 3 + 2];
+    }
+  }
+  Partial acc = empty_partial();
+  if (has) {
+    if (row == own_row && l == own_slot) v = tagged(own);
+    if (v.w == 0) v = wait_part(src, p.status, p.wait_ns);
+    st_part(src, make_int4(0, 0, 0, 0));
+    acc = untagged(v);
+  }
+  acc = fold_lanes(acc, p.lanes_log2, p.scale);
+  // A step that runs while a wait's run-out is on record has no usable statistics: its rows are flagged, nothing is accepted.
+  const bool lost = __shfl_sync(0xffffffffu, failed, 0) != 0;
+  if (p.row_out) {
+    if (first) {
+      if (lost) acc = failed_partial();
+      else if (acc.idx < kIdxFailed) acc.idx += p.idx_offset;
+      p.row_out[row] = acc;
+    }
+    return;
+  }
+  RowOutcome o = row_outcome(p, acc, i < p.K, draft, target);
+  const bool bad = bad_state(p, pend, len, corr);
+  if (lane == 0 && bad) o.flag |= kFlagBadState;
+  if (lost) {
+    if (!p.target_tokens) o.y = 0;
+    o.greedy = 0;
+    o.bits = 1;
+    o.flag |= kFlagStepFailed;
+  }
+  // lane r: position r + 1
+  const int from = min(lane << p.lanes_log2, 31);
+  const int bits = __shfl_sync(0xffffffffu, o.bits, from), y = __shfl_sync(0xffffffffu, o.y, from);
+  draft = __shfl_sync(0xffffffffu, draft, from);
+  pend = __shfl_sync(0xffffffffu, bad ? 0 : pend, 0);
+  len = __shfl_sync(0xffffffffu, bad ? 0 : len, 0);
+  corr = __shfl_sync(0xffffffffu, bad ? -1 : corr, 0);
+  const uint32_t mism = __ballot_sync(0xffffffffu, lane < p.K && (bits & 1)), defer = __ballot_sync(0xffffffffu, bits & 2);
+  const RoundOutcome r = decide_round<uint32_t>(mism, defer, p.K, p.W, p.carry, pend, len);
+  int tok = lane < r.s - 1 ? draft : lane == r.s - 1 ? y : -1;
+  if (r.revoke) tok = lane == 0 ? corr : -1;
+  if (lane < K1) p.out_tokens[(int64_t)b * K1 + lane] = tok;
+  const int correction = __shfl_sync(0xffffffffu, y, (r.st_corr_pos - 1) & 31);
+  if (lane == 0) {
+    p.accept_len[b] = r.s;
+    if (p.rollback) p.rollback[b] = r.rollback;
+    // (state_in may alias state_out: this lane has read it)
+    if (p.state_out) {
+      p.state_out[b * 3 + 0] = r.st_pending;
+      p.state_out[b * 3 + 1] = r.st_len;
+      p.state_out[b * 3 + 2] = r.st_corr_pos ? correction : -1;
+    }
+  }
+  if (first) {
+    if (p.target_argmax) p.target_argmax[row] = o.greedy;
+    if (p.entropy) p.entropy[row] = o.H;
+    if (p.row_flags) p.row_flags[row] = o.flag;
   }
 }
 
