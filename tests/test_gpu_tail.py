@@ -13,7 +13,7 @@ DEV = "cuda"
 
 
 @pytest.mark.parametrize("B,K,V,pieces", [
-    (3, 31, 2000, 1), (3, 32, 2000, 1),        # 32 rows are a warp's, 33 are not
+    (3, 31, 2000, 1), (3, 32, 2000, 1), (40, 50, 600, 1),   # 32 rows are a warp's, 33 are not
     (3, 15, 4096, 2), (3, 16, 4096, 2),        # two lanes a row
     (3, 7, 8704, 4), (3, 7, 8704, 5),          # four
     (2, 1, 8704, 16), (2, 1, 8704, 17),        # sixteen
