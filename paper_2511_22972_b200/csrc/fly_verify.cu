@@ -476,6 +476,11 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     // V = 128256 344 / 339 / 335 / 328).
     const int deepest = h->weight_vd ? L::kMaxStages : 7;
     if (p.stages > deepest) p.stages = deepest;
+    // The ring's worth of the first weight tile is asked for in L2 before the wait for the previous kernel.  us a step in a row of
+    // steps, without / with: 12 positions, D = 1024, V = 32000 17.54 / 17.11; 2 x 640 x 128256 31.66 / 31.2; 4 x 4096 x 32000 49.7 /
+    // 49.0; 32 x 2752 x 50264 47.3 / 46.6.  Only where the weight's rows are whole lines: others gain nothing or lose
+    // (32 x 2760 x 50264 51.5 / 51.5 - 52.5, x 2752 x 50000, stored [D, V], 46.4 / 46.6).
+    p.ahead = (h->weight_vd ? D : V) % 64 == 0 ? p.stages : 0;
     p.V = V; p.D = D;
     p.num_tiles = num_tiles;
     p.num_kb = (D + L::kBlockK - 1) / L::kBlockK;

@@ -109,6 +109,7 @@ struct Params {
   int num_tiles;  // ceil(V / 256): tiles of the CTA pairs
   int num_kb;     // ceil(D / 64)
   int row0;       // first row of this launch in hidden / partials
+  int ahead;      // stages of the first weight tile asked for in L2 before the wait for the previous kernel
   int w_kmajor;   // 0: weight is [D, V] (vocabulary contiguous, MN-major A); 1: weight is [V, D] (K-major A)
   float scale;    // log2(e) / temperature: logit -> base-2 exponent
   float floor;    // logits at or below it are masked
@@ -144,6 +145,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
       : "memory");
+}
+
+// The same box, asked for in L2.
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, int y) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(map), "r"(x), "r"(y) : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -312,6 +318,20 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   tc_fence_after();
   const uint32_t tmem = misc[0];
 
+  const int my_tiles = pair < p.num_tiles ? (p.num_tiles - 1 - pair) / npairs + 1 : 0;
+  // A prefetch reads nothing for the program: the kernel before may still be writing the weight.
+  if (warp == kWarpW && my_tiles > 0 && elect_lane()) {
+    const int v0 = pair * kPairV + (int)rank * kBlockV;
+    for (int kb = 0; kb < min(p.ahead, p.num_kb); ++kb) {
+      if (p.w_kmajor) {
+        tma_prefetch_2d(&map_w, kb * kBlockK, v0);
+      } else {
+        tma_prefetch_2d(&map_w, v0, kb * kBlockK);
+        tma_prefetch_2d(&map_w, v0 + 64, kb * kBlockK);
+      }
+    }
+  }
+  __syncwarp();
   // The grid is a programmatic dependent of the kernel before it: everything above ran next to that kernel's end, and
   // nothing below starts before it has completed.  The kernel that folds this one's states may be scheduled early too.
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -322,7 +342,6 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   const uint32_t half_bytes = (uint32_t)(p.box * kBytesPos);  // one accumulator's hidden tile of this CTA
   const uint32_t h_bytes = p.n1 > 0 ? 2 * half_bytes : half_bytes;
   const uint32_t off_h = (uint32_t)(kOffW + p.stages * kBytesW);
-  const int my_tiles = pair < p.num_tiles ? (p.num_tiles - 1 - pair) / npairs + 1 : 0;
 
   if (warp == kWarpW) {
     // ---------------- weight producer: this CTA's 128 vocabulary entries ----------------
