@@ -513,7 +513,9 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
         }
       }
     }
-    // Merge the eight vocabulary eighths of every position and write the CTA's partial state.
+    // Merge the eight vocabulary eighths of every position and write the CTA's partial state: a thread per position, the eight at
+    // once (a lane per eighth and a fold by shuffles for every 32 positions took 3.3 us of the end of a step of 288; us a step,
+    // before / after: 288 positions x 1024 x 50264 38.5 / 36.2, x 2048 x 10000 25.3 / 23.0, 36 x 512 x 4096 8.0 / 7.55).
     // The weight ring is free by now: every MMA that read it has completed (slot_full of the last tile).
     epi_all_bar();
     Partial* buf = reinterpret_cast<Partial*>(gbase + kOffW);
@@ -522,13 +524,15 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
       if (k >= my_chunks) break;
       Partial pq;
       pq.mx = st[k].mx; pq.S = st[k].S; pq.u = st[k].u; pq.idx = st[k].idx;
-      buf[((2 * k + group) * kChunk + pos_i) * 8 + eighth] = pq;
+      buf[eighth * kMaxPos + (2 * k + group) * kChunk + pos_i] = pq;
     }
     epi_all_bar();
-    for (int i0 = 0; i0 < p.R * 8; i0 += kEpiThreads) {  // a lane per eighth
-      const int i = i0 + (int)threadIdx.x;
-      const Partial a = fold_lanes(i < p.R * 8 ? buf[i] : empty_partial(), 3, p.scale);
-      if (i < p.R * 8 && (i & 7) == 0) p.partials[(int64_t)(p.row0 + (i >> 3)) * gridDim.x + blockIdx.x] = a;
+    for (int pos = (int)threadIdx.x; pos < p.R; pos += kEpiThreads) {
+      Partial e[8], a;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) e[i] = buf[i * kMaxPos + pos];
+      fold_array(e, a, p.scale);
+      p.partials[(int64_t)(p.row0 + pos) * gridDim.x + blockIdx.x] = a;
     }
   }
 

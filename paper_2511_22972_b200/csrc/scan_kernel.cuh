@@ -157,6 +157,24 @@ __device__ __forceinline__ Partial fold_lanes(const Partial& a, int lanes_log2, 
   return r;
 }
 
+// Folds N partial states that one thread holds: the maximum first, then exponentials that do not wait for one another.
+template <int N>
+__device__ __forceinline__ void fold_array(const Partial (&a)[N], Partial& r, float scale) {
+  r = a[0];
+#pragma unroll
+  for (int i = 1; i < N; ++i) r.mx = fmaxf(r.mx, a[i].mx);
+  r.S = r.u = 0.f;
+  unsigned idx = (unsigned)kIdxNone;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float d = a[i].mx * scale - r.mx * scale, e = ex2_approx(d);  // d <= 0, finite (mx is clamped to the mask floor)
+    r.S = fmaf(e, a[i].S, r.S);
+    r.u = fmaf(e, fmaf(d, a[i].S, a[i].u), r.u);
+    if (a[i].mx == r.mx) idx = min(idx, (unsigned)a[i].idx);
+  }
+  r.idx = (int)idx;
+}
+
 struct ScanShared {
   int y[kMaxRows];      // y_i (Eq. 1, or the caller's token)
   int bits[kMaxRows];   // bit 0: mismatch (Eq. 2), bit 1: Defer (Eq. 6)
