@@ -498,26 +498,28 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->last_launches++;
   }
-  // A row's states, one per CTA, are folded by the scan itself where its lanes have about ten each, and by a warp per row
-  // before it otherwise: in the chain of launches a kernel more costs 1 us (36 positions x 512 x 4096: 9.6 against 10.3 us).
-  cudaError_t e;
-  fly::Partial* parts = h->lm_partials;
-  int per_row = grid;
-  if (rows > L::kHalfN || (grid >> lanes_for(grid, a->K + 1)) > 10) {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[1];
+  // Up to 144 positions the scan folds a row's states itself, a warp per row; more go through a kernel that folds all rows at once.
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  const bool wide = rows <= L::kHalfN;
+  if (!wide) {
     const unsigned warps = fly::kFoldThreads / 32;
     fill_launch(&cfg, attr, (unsigned)((rows + warps - 1) / warps), fly::kFoldThreads, st, true);
-    e = cudaLaunchKernelEx(&cfg, fly::fold_partials, (const fly::Partial*)h->lm_partials, grid, h->lm_folded, (int)rows,
-                           exponent_scale(a->temperature));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fly::fold_partials, (const fly::Partial*)h->lm_partials, grid, h->lm_folded, (int)rows,
+                                             exponent_scale(a->temperature));
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->last_launches++;
-    parts = h->lm_folded;
-    per_row = 1;
   }
-  fly::ScanParams sp = scan_params(h, a, parts, per_row);
+  fly::ScanParams sp = scan_params(h, a, wide ? h->lm_partials : h->lm_folded, wide ? grid : 1);
   sp.status = h->lm_status;  // a step whose GEMM kernel gave up is marked row by row, in stream order
-  e = launch_scan(sp, false, st);
+  cudaError_t e;
+  if (wide) {
+    const int warps = a->K + 1 <= 32 ? a->K + 1 : (a->K + 2) / 2;  // (two at least: the second writes what the first does not)
+    fill_launch(&cfg, attr, (unsigned)a->B, 32u * (unsigned)warps, st, true);
+    e = cudaLaunchKernelEx(&cfg, fly::scan_wide, sp);
+  } else {
+    e = launch_scan(sp, false, st);
+  }
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches++;
   return FLY_OK;

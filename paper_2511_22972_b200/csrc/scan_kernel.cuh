@@ -182,6 +182,11 @@ struct ScanShared {
   int pend, len, corr;  // carried state as it is honoured
   int failed;           // a wait ran out before
 };
+struct WideShared : ScanShared {
+  int greedy[kMaxRows];
+  float H[kMaxRows];
+  uint32_t flag[kMaxRows];
+};
 
 // What a thread reads for its row, all at once.
 struct ScanLoads {
@@ -342,11 +347,18 @@ __device__ __forceinline__ void finish_round(const ScanParams& p, int b, const i
   }
 }
 
+// What finish_round wants of row r.  A step that runs while a wait's run-out is on record has no usable statistics: nothing is accepted.
+__device__ __forceinline__ void round_row(const ScanParams& p, const ScanShared& sm, bool failed, int r, int& bits, int& draft, int& y) {
+  bits = r > p.K ? 0 : failed ? 1 : sm.bits[r];
+  draft = r <= p.K ? sm.draft[r] : 0;
+  y = r > p.K || (failed && !p.target_tokens) ? 0 : sm.y[r];
+}
+
 // The block verifies sequence b (or folds row b if that is all that is asked for).  Called by all kScanThreads threads.
 template <bool TAGGED>
 __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const ScanLoads& q, int64_t own_row, int own_slot,
                                               const Partial& own, ScanShared& sm) {
-  const int K = p.K, K1 = p.K + 1;
+  const int K1 = p.K + 1;
   const int tid = (int)threadIdx.x;
   const int i = tid >> p.lanes_log2, l = tid & ((1 << p.lanes_log2) - 1);
   const int64_t row = (int64_t)b * K1 + i;
@@ -386,17 +398,12 @@ __device__ __forceinline__ void scan_sequence(const ScanParams& p, int b, const 
   // A step that runs while a wait's run-out is on record has no usable statistics: its rows are flagged, nothing is accepted.
   const bool failed = sm.failed != 0;
   if (tid < 32) {
-    auto row_at = [&](int r, int& bits, int& draft, int& y) {
-      bits = r >= K1 ? 0 : failed ? 1 : sm.bits[r];
-      draft = r < K1 ? sm.draft[r] : 0;
-      y = r >= K1 || (failed && !p.target_tokens) ? 0 : sm.y[r];
-    };
     int bits[2], draft[2], y[2];
-    row_at(tid, bits[0], draft[0], y[0]);
+    round_row(p, sm, failed, tid, bits[0], draft[0], y[0]);
     if (__builtin_expect(K1 <= 32, 1)) {
       finish_round<uint32_t>(p, b, {bits[0]}, {draft[0]}, {y[0]}, sm.pend, sm.len, sm.corr);
     } else {
-      row_at(tid + 32, bits[1], draft[1], y[1]);
+      round_row(p, sm, failed, tid + 32, bits[1], draft[1], y[1]);
       finish_round<uint64_t>(p, b, bits, draft, y, sm.pend, sm.len, sm.corr);
     }
   }
@@ -478,27 +485,96 @@ __device__ __forceinline__ void scan_warp(const ScanParams& p, int b, int64_t ow
   }
 }
 
-// Folds the n partial states in[row * n ..] of every row into out[row]; one warp per row.  The fused LM-head kernel
-// leaves one partial state per row and CTA; folding them with 32 lanes in parallel keeps the acceptance scan short.
+// Folds the n partial states at src (the fused LM-head kernel leaves one per row and CTA) by a warp, with kWideParts loads of a lane in
+// flight and without a chain of merges.
+constexpr int kWideParts = 5;
+__device__ __forceinline__ Partial fold_row(const Partial* src, int n, float scale) {
+  const int lane = (int)threadIdx.x & 31;
+  Partial acc = empty_partial();
+  for (int j0 = lane; j0 < n; j0 += 32 * kWideParts) {
+    Partial v[kWideParts + 1];
+#pragma unroll
+    for (int t = 0; t < kWideParts; ++t) v[t] = j0 + 32 * t < n ? as_partial(ld_part(src + j0 + 32 * t)) : empty_partial();
+    v[kWideParts] = acc;
+    fold_array(v, acc, scale);
+  }
+  return fold_lanes(acc, 5, scale);
+}
+
+// Folds the n partial states in[row * n ..] of every row into out[row]; one warp per row.
 constexpr int kFoldThreads = 128;
 __global__ void __launch_bounds__(kFoldThreads) fold_partials(const Partial* __restrict__ in, int n, Partial* __restrict__ out,
                                                               int rows, float scale) {
-  const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * (kFoldThreads / 32) + (threadIdx.x >> 5);
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the producer grid has completed
   asm volatile("griddepcontrol.launch_dependents;");
   if (row >= rows) return;
-  const Partial* src = in + (int64_t)row * n;
-  Partial acc = empty_partial();
-  for (int j0 = 0; j0 < n; j0 += 128) {  // four independent loads in flight per lane
-    int4 q[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) if (j0 + t * 32 + lane < n) q[t] = ld_part(src + j0 + t * 32 + lane);
-#pragma unroll
-    for (int t = 0; t < 4; ++t) if (j0 + t * 32 + lane < n) merge_partial(acc, as_partial(q[t]), scale);
+  const Partial acc = fold_row(in + (int64_t)row * n, n, scale);
+  if ((threadIdx.x & 31) == 0) out[row] = acc;
+}
+
+// The scan after a kernel that leaves many partial states per row: a warp per row folds them, the block's first warp ends the
+// round.  One block of 32 * (K + 1) threads, or half as many with two rows per warp, per sequence.  (The scan below has a block of 256 threads
+// for all rows, and a chain of merges for what is more; us a step of the fused path with it / with this: 36 positions x 512 x 4096 7.55 /
+// 7.21, 32 x 1496 x 12000 12.9 / 12.2, 144 x 2048 x 4096 13.2 / 12.7.)
+constexpr int kWideThreads = 1024;
+__global__ void __launch_bounds__(kWideThreads) scan_wide(const __grid_constant__ ScanParams p) {
+  __shared__ WideShared sm;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the producer grid has completed
+  asm volatile("griddepcontrol.launch_dependents;");
+  const int b = (int)blockIdx.x, K1 = p.K + 1, lane = (int)threadIdx.x & 31, warps = (int)blockDim.x >> 5;
+  int pend = 0, len = 0, corr = -1, failed = 0;
+  if (threadIdx.x == 0) {
+    if (p.status) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(failed) : "l"(p.status) : "memory");
+    if (p.carry && p.state_in) {
+      pend = p.state_in[b * 3 + 0];
+      len = p.state_in[b * 3 + 1];
+      corr = p.state_in[b * 3 + 2];
+    }
   }
-  acc = fold_lanes(acc, 5, scale);
-  if (lane == 0) out[row] = acc;
+  for (int i = (int)threadIdx.x >> 5; i < K1; i += warps) {
+    const int64_t row = (int64_t)b * K1 + i;
+    int draft = 0, target = 0;
+    if (lane == 0 && i < p.K) draft = p.draft[(int64_t)b * p.K + i];
+    if (lane == 0 && p.target_tokens) target = p.target_tokens[row];
+    const Partial acc = fold_row(p.partials + row * p.row_pitch, p.splits, p.scale);
+    if (lane == 0) {
+      RowOutcome o = row_outcome(p, acc, i < p.K, draft, target);
+      if (i == 0) {
+        const bool bad = bad_state(p, pend, len, corr);
+        if (bad) o.flag |= kFlagBadState;
+        sm.pend = bad ? 0 : pend;
+        sm.len = bad ? 0 : len;
+        sm.corr = bad ? -1 : corr;
+        sm.failed = failed;
+      }
+      sm.y[i] = o.y;
+      sm.bits[i] = o.bits;
+      sm.draft[i] = draft;
+      sm.greedy[i] = o.greedy;
+      sm.H[i] = o.H;
+      sm.flag[i] = o.flag;
+    }
+  }
+  __syncthreads();
+  const bool lost = sm.failed != 0;
+  if (threadIdx.x < 32) {
+    int bits[2], draft[2], y[2];
+    round_row(p, sm, lost, lane, bits[0], draft[0], y[0]);
+    if (K1 <= 32) {
+      finish_round<uint32_t>(p, b, {bits[0]}, {draft[0]}, {y[0]}, sm.pend, sm.len, sm.corr);
+    } else {
+      round_row(p, sm, lost, lane + 32, bits[1], draft[1], y[1]);
+      finish_round<uint64_t>(p, b, bits, draft, y, sm.pend, sm.len, sm.corr);
+    }
+  } else {
+    for (int i = (int)threadIdx.x - 32; i < K1; i += (int)blockDim.x - 32) {
+      const int64_t row = (int64_t)b * K1 + i;
+      if (p.target_argmax) p.target_argmax[row] = lost ? 0 : sm.greedy[i];
+      if (p.entropy) p.entropy[row] = sm.H[i];
+      if (p.row_flags) p.row_flags[row] = lost ? sm.flag[i] | kFlagStepFailed : sm.flag[i];
+    }
+  }
 }
 
 // Stand-alone launch: one block per sequence, after the kernel (or the all-gather) that leaves the partial states.
