@@ -199,7 +199,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, in
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, code));
 }
 
-// 32 lanes x 16 columns of fp32: thread = lane, register i = column col0 + i.
+// 32 lanes x 16 columns of fp32: thread = lane, register i = column col0 + i.  The registers are there after tmem_wait.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -207,7 +207,13 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                 "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
 }
 
 // Named barriers: 1 and 2 for the two epilogue groups (128 threads each), 3 for all epilogue threads.
@@ -256,16 +262,20 @@ __device__ __forceinline__ void fold16(Stream& st, float (&x)[16], int v0, float
     st.idx = v0 + first;
   }
   const float nr = -st.mx * scale;
-  float S0 = 0.f, S1 = 0.f, u0 = 0.f, u1 = 0.f;
+  const f2 nr2 = pack2(nr, nr), sc2 = pack2(scale, scale);
+  f2 S2 = pack2(0.f, 0.f), u2 = S2;
 #pragma unroll
   for (int e = 0; e < 16; e += 2) {
-    const float t0 = fmaf(x[e], scale, nr), t1 = fmaf(x[e + 1], scale, nr);
-    const float e0 = ex2_approx(t0), e1 = ex2_approx(t1);
-    S0 += e0;
-    u0 = fmaf(e0, t0, u0);
-    S1 += e1;
-    u1 = fmaf(e1, t1, u1);
+    const f2 t2 = fma2(pack2(x[e], x[e + 1]), sc2, nr2);
+    float t0, t1;
+    unpack2(t2, t0, t1);
+    const f2 e2 = pack2(ex2_approx(t0), ex2_approx(t1));
+    S2 = add2(S2, e2);
+    u2 = fma2(e2, t2, u2);
   }
+  float S0, S1, u0, u1;
+  unpack2(S2, S0, S1);
+  unpack2(u2, u0, u1);
   st.S += S0 + S1;
   st.u += u0 + u1;
 }
@@ -482,13 +492,21 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
       // an accumulator of which this group turns no block is handed back at once
       if (last0 < 0) { tc_fence_before(); mbar_arrive_remote(map_to_cta(slot_empty(slot0), 0)); }
       if (nh == 2 && last1 < 0) { tc_fence_before(); mbar_arrive_remote(map_to_cta(slot_empty(slot1), 0)); }
+      // A block's registers are asked for as soon as those of the block before have gone to shared memory (us a step, asked for when
+      // they are needed / so: 288 positions x 1024 x 50264 35.8 / 34.7, x 4096 x 32000 67.9 / 67.4, 144 x 2048 x 4096 12.7 / 12.5; 36 x 512 x
+      // 4096 7.21 / 7.30).
+      uint32_t r[16];
+      auto ask = [&](int k) {  // for the group's k-th block
+        const int c = 2 * k + group, h = c >= half_chunks ? 1 : 0;
+        tmem_ld16(tmem + lane_base + (uint32_t)((h ? slot1 : slot0) * kHalfN + (c - h * half_chunks) * kChunk), r);
+      };
+      if (my_chunks > 0) ask(0);
 #pragma unroll
       for (int k = 0; k < kGroupChunks; ++k) {
         if (k < my_chunks) {
           const int c = 2 * k + group;
           const int h = c >= half_chunks ? 1 : 0;  // which accumulator the block belongs to
-          uint32_t r[16];
-          tmem_ld16(tmem + lane_base + (uint32_t)((h ? slot1 : slot0) * kHalfN + (c - h * half_chunks) * kChunk), r);
+          tmem_wait(r);
           if (k == (h ? last1 : last0)) {  // last read of this accumulator by this thread: hand its slot back
             tc_fence_before();
             mbar_arrive_remote(map_to_cta(slot_empty(h ? slot1 : slot0), 0));
@@ -496,6 +514,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
           group_bar(group);  // the group is done reading the previous block
 #pragma unroll
           for (int i = 0; i < 16; ++i) turn[i * kTurnRow + q * 32 + lane] = __uint_as_float(r[i]);
+          if (k + 1 < my_chunks) ask(k + 1);
           group_bar(group);
           float x[16];
           const float4* src = reinterpret_cast<const float4*>(turn + pos_i * kTurnRow + eighth * 16);

@@ -42,33 +42,6 @@ constexpr int kReduceBlocksPerSM = 4;  // __launch_bounds__ below: <= 64 registe
 constexpr int kDepth = 2;              // slices in flight per warp (3 and 4 measured: no faster)
 constexpr int kMaxPend = 8;            // pieces of a block at most; it holds them back and writes them out at its end
 
-// ---- packed fp32 pairs ------------------------------------------------------------------------
-using f2 = unsigned long long;  // two fp32 values in one 64-bit register: {lo, hi}
-
-__device__ __forceinline__ f2 pack2(float lo, float hi) {
-  f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f2 v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-  f2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f2 add2(f2 a, f2 b) {
-  f2 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-  f2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 // Per-warp streaming state.  S2/u2 are per-lane pairs of accumulators, everything else is warp-uniform.
 struct WarpAcc {
   float cur_max;  // raw running maximum (warp-uniform)
