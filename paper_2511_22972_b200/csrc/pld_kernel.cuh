@@ -12,8 +12,11 @@
 // What bounds it is latency: a 128 KB context is 20 ns of HBM bandwidth but a chain of dependent reads
 // (length, tokens, earlier tokens at a hit, continuation).  A sequence is therefore spread over a cluster
 // of up to 8 blocks of 256 threads, 16 tokens per thread and round with all four loads in flight, and the
-// blocks' best[] meet in distributed shared memory.  32 contexts of 16 - 32 k tokens (3.1 MB), in a CUDA
-// graph: 5.6 us per call; one block per sequence and a pass per n, 4-byte loads: 59 us.
+// blocks' best[] meet in the first block's shared memory.  What is left is short: the tokens of the first round are asked for with
+// the last tokens and do not wait for them, and the look-back exists once and not per token, since a launch also waits for
+// its code.  us a call in a row of calls, before both / after: 32 contexts of 16 - 32 k tokens 5.8 / 3.9, 64 of 8 - 16 k 5.25 / 3.8, 4 of
+// 50 - 100 k 5.4 / 4.1, 64 of 1 - 2 k 2.9 / 2.4, one of 300 2.35 / 2.26.  (Blocks of 512 or 1024 threads, up to 7 loads in flight, without a
+// cluster: 32 contexts of 16 - 32 k 4.3 - 5.3.)
 #pragma once
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -45,8 +48,11 @@ __global__ void __launch_bounds__(kThreads) pld_draft_kernel(const Params p) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   const int ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-  __shared__ int best[kMaxNgram + 1];
+  __shared__ int best[kMaxNgram + 1];   // of the block; in the first block of the cluster, of all of them
+  __shared__ int suffix[kMaxNgram];     // the last tokens, the last one first
   if (threadIdx.x <= kMaxNgram) best[threadIdx.x] = kNone;
+  // Nothing is written to another block's best[] before that block has reached this point.
+  if (ranks > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the previous kernel in the stream may have written the tokens
   asm volatile("griddepcontrol.launch_dependents;");
   const int b = (int)blockIdx.x / ranks;
@@ -55,79 +61,82 @@ __global__ void __launch_bounds__(kThreads) pld_draft_kernel(const Params p) {
   // Such a sequence proposes nothing (count 0, match_pos -1), as an empty one does.
   const int Lraw = p.lengths[b];
   const int L = (Lraw < 0 || (int64_t)Lraw > p.stride) ? 0 : Lraw;
+
+  // Candidates are the tokens t = 0 .. L-2 (the continuation starts at t + 1 <= L - 1), read as 16-byte segments of the row, counted
+  // from the aligned address at or below its start (token t is element t + head of them); the up to three tokens before
+  // the first whole segment and after the last are read one by one, by eight threads.
+  const int n_tok = L - 1;
+  const int head = (int)((reinterpret_cast<uintptr_t>(tok) >> 2) & 3);
+  const int4* seg = reinterpret_cast<const int4*>(tok - head);
+  const int seg0 = head > 0 ? 1 : 0, seg1 = n_tok > 0 ? (head + n_tok) / 4 : 0;
+  constexpr int kStep = kThreads * kVecs;
+  int4 v[kVecs];
+  // (Ordinary loads: the kernel before may have been writing the tokens while this one was already resident, so they are
+  // not read-only for its life, which the non-coherent path would require.)
+  auto fetch = [&](int s) {
+#pragma unroll
+    for (int j = 0; j < kVecs; ++j)
+      if (s + j * kThreads >= seg0 && s + j * kThreads < seg1) v[j] = seg[s + j * kThreads];
+  };
+  // The first round, the last tokens and the single ones are asked for together: one round trip after the length.
+  const int tid = (int)threadIdx.x;
+  int s = rank * kStep + tid;
+  fetch(s);
+  if (tid < kMaxNgram) suffix[tid] = tid < L ? tok[L - 1 - tid] : 0;
+  const int t1 = tid < 4 ? tid : seg1 * 4 - head + tid - 4;
+  const bool single = rank == 0 && tid < 8 && t1 >= 0 && t1 < n_tok && (tid >= 4 || t1 < 4 - head);
+  int x1 = 0;
+  if (single) x1 = tok[t1];
   __syncthreads();
-
-  if (L > 1) {
-    const int last = tok[L - 1];
-    // Longest suffix a thread has recorded so far: its positions ascend, so what it recorded is its earliest.
-    int seen = 0;
-    // Position t holds the last token: the match ends before e = t + 1.  Look back as far as the query goes.
-    auto hit = [&](int t) {
+  const int last = suffix[0];
+  unsigned hits = single && x1 == last ? 1u : 0u;  // bit 0: that token; then four per segment
+  while (true) {
+#pragma unroll
+    for (int j = 0; j < kVecs; ++j)
+      if (s + j * kThreads >= seg0 && s + j * kThreads < seg1)
+        hits |= (v[j].x == last ? 2u << (4 * j) : 0u) | (v[j].y == last ? 4u << (4 * j) : 0u) | (v[j].z == last ? 8u << (4 * j) : 0u) |
+                (v[j].w == last ? 16u << (4 * j) : 0u);
+    // Position t holds the last token: the match ends before e = t + 1.  Look back as far as the query goes.  (One copy of this code:
+    // a launch fetches it anew, and sixteen copies took longer than the reads they made.)
+    for (; hits != 0; hits &= hits - 1) {
+      const int bit = __ffs((int)hits) - 2, t = bit < 0 ? t1 : (s + (bit >> 2) * kThreads) * 4 - head + (bit & 3);
       int m = 1;
-      while (m < p.max_ngram && m <= t && tok[t - m] == tok[L - 1 - m]) ++m;
-      for (; seen < m; ++seen) atomicMin(&best[seen + 1], t + 1);
-    };
-    // 16-byte segments of the row, counted from the aligned address at or below its start; token t is element
-    // t + head of them.  Segments that reach outside [0, L) are read token by token.
-    const int head = (int)((reinterpret_cast<uintptr_t>(tok) >> 2) & 3);
-    const int4* seg = reinterpret_cast<const int4*>(tok - head);
-    const int n_tok = L - 1;  // candidates t = 0 .. L-2 (the continuation starts at t + 1 <= L - 1)
-    const int n_seg = (head + n_tok + 3) / 4;
-    constexpr int kStep = kThreads * kVecs;
-    // (Ordinary loads: the kernel before may have been writing the tokens while this one was already resident, so they are
-    // not read-only for its life, which the non-coherent path would require.)
-    for (int s0 = rank * kStep; s0 < n_seg && seen < p.max_ngram; s0 += ranks * kStep) {
-      int4 v[kVecs];
-#pragma unroll
-      for (int j = 0; j < kVecs; ++j) {
-        const int s = s0 + j * kThreads + (int)threadIdx.x;
-        const int t = s * 4 - head;
-        v[j] = make_int4(~last, ~last, ~last, ~last);
-        if (t >= 0 && t + 3 < n_tok) {
-          v[j] = seg[s];
-        } else if (s < n_seg) {
-          if (t >= 0 && t < n_tok) v[j].x = tok[t];
-          if (t + 1 >= 0 && t + 1 < n_tok) v[j].y = tok[t + 1];
-          if (t + 2 >= 0 && t + 2 < n_tok) v[j].z = tok[t + 2];
-          if (t + 3 >= 0 && t + 3 < n_tok) v[j].w = tok[t + 3];
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kVecs; ++j) {
-        const int t = (s0 + j * kThreads + (int)threadIdx.x) * 4 - head;
-        if (v[j].x == last) hit(t);
-        if (v[j].y == last) hit(t + 1);
-        if (v[j].z == last) hit(t + 2);
-        if (v[j].w == last) hit(t + 3);
-      }
+      while (m < p.max_ngram && m <= t && tok[t - m] == suffix[m]) ++m;
+      for (; m > 0; --m)
+        if (t + 1 < best[m]) atomicMin(&best[m], t + 1);
     }
+    s += ranks * kStep;
+    // (a block's positions ascend: once it has a match of the longest query, it has its earliest)
+    if (s - tid >= seg1 || __syncthreads_or(best[p.max_ngram] != kNone)) break;
+    fetch(s);
   }
-  if (ranks > 1) cluster.sync();
-  else __syncthreads();
+  __syncthreads();
+  if (ranks > 1) {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank > 0 && threadIdx.x >= 1 && threadIdx.x <= kMaxNgram && best[threadIdx.x] != kNone)
+      atomicMin(cluster.map_shared_rank(best + threadIdx.x, 0), best[threadIdx.x]);
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (rank > 0) return;  // nobody looks into this block's shared memory
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
 
-  if (rank == 0) {
-    // every thread takes the same decision from the cluster's best[]
-    int end = 0, ngram = 0;
-    if (L > 1) {
-      const int lane = (int)threadIdx.x & 31;
-      int e = kNone;  // lane n: the earliest match of n tokens over all blocks
-      if (lane >= p.min_ngram && lane <= p.max_ngram)
-        for (int r = 0; r < ranks; ++r) e = min(e, r == 0 ? best[lane] : *cluster.map_shared_rank(best + lane, r));
-      const unsigned found = __ballot_sync(0xffffffffu, e != kNone);
-      if (found) {
-        ngram = 31 - __clz((int)found);
-        end = __shfl_sync(0xffffffffu, e, ngram);
-      }
-    }
-    const int cnt = ngram > 0 ? min(p.K, L - end) : 0;
-    for (int i = threadIdx.x; i < p.K; i += kThreads) p.draft[(int64_t)b * p.K + i] = i < cnt ? tok[end + i] : -1;
-    if (threadIdx.x == 0) {
-      p.count[b] = cnt;
-      if (p.match_pos) p.match_pos[b] = ngram > 0 ? end - ngram : -1;
-      if (p.match_ngram) p.match_ngram[b] = ngram;
-    }
+  // every thread takes the same decision
+  int end = 0, ngram = 0;
+  const int lane = (int)threadIdx.x & 31;
+  const int e = lane >= p.min_ngram && lane <= p.max_ngram ? best[lane] : kNone;  // lane n: the earliest match of n tokens
+  const unsigned found = __ballot_sync(0xffffffffu, e != kNone);
+  if (found) {
+    ngram = 31 - __clz((int)found);
+    end = __shfl_sync(0xffffffffu, e, ngram);
   }
-  if (ranks > 1) cluster.sync();  // rank 0 has read every block's best[]
+  const int cnt = ngram > 0 ? min(p.K, L - end) : 0;
+  for (int i = threadIdx.x; i < p.K; i += kThreads) p.draft[(int64_t)b * p.K + i] = i < cnt ? tok[end + i] : -1;
+  if (threadIdx.x == 0) {
+    p.count[b] = cnt;
+    if (p.match_pos) p.match_pos[b] = ngram > 0 ? end - ngram : -1;
+    if (p.match_ngram) p.match_ngram[b] = ngram;
+  }
 }
 
 }  // namespace pld

@@ -118,3 +118,22 @@ def test_contexts_written_by_the_kernel_before_in_the_stream():
         for b, (prop, p, n) in enumerate(want[i % len(steps)]):
             assert (count[b].item(), pos[b].item(), ng[b].item()) == (len(prop), p, n) and draft[b, :len(prop)].tolist() == prop, (i, b)
     fv.close()
+
+
+@pytest.mark.parametrize("width", [9, 4097, 8195, 32771, 70001])
+def test_rows_at_every_alignment_and_lengths_around_a_round(width):
+    # rows start 4, 8 and 12 bytes off a 16-byte boundary; contexts end just before, at and after what a block or a cluster of
+    # blocks tests at a time; the repeat lies at the very start, across a boundary, or nowhere
+    rng = random.Random(width)
+    seqs = []
+    for L in [1, 2, 3, 4, 5, 6, 7, 8, 9] + [width - d for d in (0, 1, 2, 3, 4, 5)] + [width // 2 + d for d in (0, 1, 2)]:
+        L = max(1, min(L, width))
+        s = [rng.randrange(10 ** 6) + 10 for _ in range(L)]
+        n = min(rng.randrange(0, 6), L // 2)
+        at = rng.choice([0, 1, 2, 3, max(0, L // 2 - n), max(0, L - 2 * n - 1), min(L, 4096) - n])
+        if n > 0 and 0 <= at and at + n <= L - n:
+            s[at:at + n] = s[L - n:]
+        seqs.append(s)
+    seqs.append([rng.randrange(3) for _ in range(width)])
+    for K, mx, mn in [(15, 3, 1), (5, 8, 2)]:
+        run(seqs, K, mx, mn, pad_to=width)
