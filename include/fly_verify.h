@@ -254,16 +254,19 @@ fly_status_t fly_pld_draft(int32_t device, int32_t B, const int32_t* tokens, int
  * The first call on each device looks up the device address of the built-in
  * array (which also makes the CUDA runtime load the library's device code).
  * Make that first call outside any stream capture; later calls only enqueue
- * work on `cuda_stream` (a small kernel that clears the scratch, then the step's kernel).
+ * work on `cuda_stream` (the step's kernel; while the stream is being captured, or with inputs_ready, a small kernel that
+ * clears the scratch before it).
  *
  * All calls on a device share the one array, and it keeps whatever the last
- * call left there.  Counters and partial states are cleared on the stream at the
- * start of every call, so stale contents never leak into a result.  But two calls whose work
+ * calls left there.  They take turns at its parts, and each clears the counters and partial states of the part whose turn is next
+ * (captured calls and calls with inputs_ready have a part of their own, cleared at the start of each), so stale contents
+ * never leak into a result.  But two calls whose work
  * overlaps on the GPU (different streams, or several host threads) write the same
  * scratch and corrupt each other: serialise them, e.g. keep them on one stream. */
 #define FLY_STATIC_MAX_BATCH 1024
 #define FLY_STATIC_MAX_PIECES 16384
-#define FLY_STATIC_SCRATCH_BYTES (FLY_STATIC_MAX_BATCH * 4 + FLY_STATIC_MAX_PIECES * 16) /* 260 KiB */
+#define FLY_STATIC_PARTS 5
+#define FLY_STATIC_SCRATCH_BYTES (FLY_STATIC_PARTS * (FLY_STATIC_MAX_BATCH * 4 + FLY_STATIC_MAX_PIECES * 16)) /* 5 x 260 KiB */
 fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t logits_dtype,
                                    const fly_verify_args_t* args, void* cuda_stream);
 
@@ -304,7 +307,7 @@ fly_status_t fly_verify_set_option(fly_verify_t* handle, fly_option_t option, in
  * cleared), else FLY_OK.  While a record is pending, every further step of the same path
  * marks all of its rows with row_flags bit 4 (fused steps give up early), so the failure is
  * also visible in stream order without a host synchronisation.  fly_verify_run_static keeps
- * no record: bit 4 marks the rows, and every call clears its scratch. */
+ * no record: bit 4 marks the rows, and the scratch of every call is cleared before it. */
 fly_status_t fly_verify_device_status(fly_verify_t* handle, void* cuda_stream);
 
 /* Self-test of that mechanism, safe to run anywhere: enqueues a one-thread kernel that waits, with a

@@ -332,7 +332,7 @@ float exponent_scale(double temperature) {
 template <typename T>
 cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, int V, int64_t rows, int forced, int cap,
                           fly::Partial* partials, cudaStream_t st, fly::ScanParams* tail, double temperature,
-                          bool inputs_ready) {
+                          bool inputs_ready, uint4* clear, int clear_words) {
   constexpr int kE = fly::Seg<T>::kElems;
   const bool vec = vector_path_ok<T>(logits, V);
   const int64_t n = vec ? V / kE : V;
@@ -343,7 +343,7 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   g.n = n; g.span = pl.span; g.Q = pl.Q; g.total = rows * pl.span;
   g.pieces = pl.Q < (1 << 30) ? pl.pieces : 0; g.V = V; g.row_stride = row_stride;
   g.scale = exponent_scale(temperature); g.wait_first = inputs_ready ? 0 : 1;
-  g.rows = (int)rows;
+  g.rows = (int)rows; g.clear = clear; g.clear_words = clear_words;
   static_assert(fly::kReduceWarps == 8, "rows per block x warps per row");
   g.warps_log2 = 3 - pl.rows_log2;
   tail->splits = pl.slots;
@@ -380,11 +380,12 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
 // The current device must be the one the pointers belong to.
 cudaError_t launch_reduce_any(fly_dtype_t dt, int sm_count, const void* logits, int64_t row_stride, int V,
                               int64_t rows, int forced, int cap, fly::Partial* partials, cudaStream_t st,
-                              fly::ScanParams* tail, double temperature, bool inputs_ready) {
+                              fly::ScanParams* tail, double temperature, bool inputs_ready, uint4* clear = nullptr, int clear_words = 0) {
   if (dt == FLY_BF16)
     return launch_reduce<__nv_bfloat16>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature,
-                                        inputs_ready);
-  return launch_reduce<float>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature, inputs_ready);
+                                        inputs_ready, clear, clear_words);
+  return launch_reduce<float>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature, inputs_ready, clear,
+                              clear_words);
 }
 
 // tagged: the parts are in the self-validating form that the row reduction leaves.
@@ -982,15 +983,18 @@ static __device__ __align__(256) unsigned char g_fly_static_scratch[FLY_STATIC_S
 namespace {
 
 constexpr int kStaticMaxDevices = 64;
+constexpr size_t kStaticPartBytes = FLY_STATIC_SCRATCH_BYTES / FLY_STATIC_PARTS;  // arrival counters, then slots
+static_assert(kStaticPartBytes == FLY_STATIC_MAX_BATCH * 4 + FLY_STATIC_MAX_PIECES * 16 && kStaticPartBytes % 256 == 0, "");
 struct StaticSlot {
-  void* base = nullptr;  // device address of g_fly_static_scratch on this device
+  unsigned char* base = nullptr;  // device address of g_fly_static_scratch on this device
   int sm_count = 0;
+  unsigned calls = 0;             // that took their turn at the first FLY_STATIC_PARTS - 1 parts
 };
 StaticSlot g_static_slots[kStaticMaxDevices];
 std::mutex g_static_mu;
 
-// Once per device, with that device current.
-cudaError_t static_scratch_for(int device, StaticSlot* out) {
+// With the device current; looked up once per device.
+cudaError_t static_scratch_for(int device, bool takes_turn, StaticSlot* out) {
   std::lock_guard<std::mutex> lock(g_static_mu);
   StaticSlot& s = g_static_slots[device];
   if (!s.base) {
@@ -1002,9 +1006,10 @@ cudaError_t static_scratch_for(int device, StaticSlot* out) {
     if (e != cudaSuccess) return e;
     s.sm_count = sms > 0 ? sms : 148;
     if ((e = set_reduce_attrs()) != cudaSuccess) return e;
-    s.base = p;
+    s.base = static_cast<unsigned char*>(p);
   }
   *out = s;
+  if (takes_turn) s.calls = (s.calls + 1) % (FLY_STATIC_PARTS - 1);
   return cudaSuccess;
 }
 
@@ -1030,32 +1035,46 @@ fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t lo
 
   DeviceGuard g(device);
   if (!g.ok) return FLY_ERR_CUDA;
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  // Counters and slots must start empty, whatever an earlier call left behind.  Calls take turns at the parts of the scratch, and each
+  // empties the part of the next one while its first logits are on their way: a kernel that empties a part before each call
+  // costs the chain of launches a link (104 rows of 128256 bf16 9.2 us a step in a row of steps, 8.4 so).  Not so the calls that a
+  // graph is made of, which are replayed in any order, and those that write nothing before their end (inputs_ready): they
+  // have a part of their own, which such a kernel empties.
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
+    (void)cudaGetLastError();  // (the legacy stream while another one is being captured: the launch says so)
+    capture = cudaStreamCaptureStatusActive;
+  }
+  const bool takes_turn = a->inputs_ready == 0 && capture == cudaStreamCaptureStatusNone;
   StaticSlot slot;
-  if (static_scratch_for(device, &slot) != cudaSuccess) return FLY_ERR_CUDA;
-  unsigned int* tickets = static_cast<unsigned int*>(slot.base);
-  fly::Partial* partials =
-      reinterpret_cast<fly::Partial*>(static_cast<unsigned char*>(slot.base) + FLY_STATIC_MAX_BATCH * 4);
+  if (static_scratch_for(device, takes_turn, &slot) != cudaSuccess) return FLY_ERR_CUDA;
+  const unsigned turns = FLY_STATIC_PARTS - 1;
+  unsigned char* const part = slot.base + (takes_turn ? slot.calls : turns) * kStaticPartBytes;
+  unsigned char* const next = slot.base + (slot.calls + 1) % turns * kStaticPartBytes;
+  unsigned int* tickets = reinterpret_cast<unsigned int*>(part);
+  fly::Partial* partials = reinterpret_cast<fly::Partial*>(part + FLY_STATIC_MAX_BATCH * 4);
   h.sm_count = slot.sm_count;
 
-  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const int64_t stride = a->row_stride ? a->row_stride : vocab;
   const int64_t room = FLY_STATIC_MAX_PIECES / rows;  // Partial slots per row that fit, >= 1
   const int cap = (int)(room < kMaxSplits ? room : kMaxSplits);
 
   fly::ScanParams p = scan_params(&h, a, partials, 1);
   p.tickets = tickets;
-
-  // Counters and slots must start empty, whatever an earlier call left behind.  A kernel in the stream's chain of
-  // programmatic dependents and not a memset, which would break the chain: the reduction's launch latency stays hidden.
-  const int slot_words = (int)(rows * cap), ticket_words = (a->B + 3) / 4;
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[1];
-  fill_launch(&cfg, attr, (unsigned)((slot_words + fly::kClearThreads - 1) / fly::kClearThreads), fly::kClearThreads, st, true);
-  cudaError_t e = cudaLaunchKernelEx(&cfg, fly::clear_scratch, reinterpret_cast<uint4*>(tickets), ticket_words,
-                                     reinterpret_cast<uint4*>(partials), slot_words);
-  if (e != cudaSuccess) return FLY_ERR_CUDA;
+  cudaError_t e = cudaSuccess;
+  if (!takes_turn) {
+    // A kernel in the stream's chain of programmatic dependents and not a memset, which would break the chain.
+    const int slot_words = (int)(rows * cap), ticket_words = (a->B + 3) / 4;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    fill_launch(&cfg, attr, (unsigned)((slot_words + fly::kClearThreads - 1) / fly::kClearThreads), fly::kClearThreads, st, true);
+    e = cudaLaunchKernelEx(&cfg, fly::clear_scratch, reinterpret_cast<uint4*>(tickets), ticket_words, reinterpret_cast<uint4*>(partials),
+                           slot_words);
+    if (e != cudaSuccess) return FLY_ERR_CUDA;
+  }
   e = launch_reduce_any(logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, a->temperature,
-                        a->inputs_ready != 0);
+                        a->inputs_ready != 0, takes_turn ? reinterpret_cast<uint4*>(next) : nullptr, (int)(kStaticPartBytes / 16));
   return e == cudaSuccess ? FLY_OK : FLY_ERR_CUDA;
 }
 

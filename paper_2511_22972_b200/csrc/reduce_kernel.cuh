@@ -320,6 +320,8 @@ struct ReducePlan {
   float scale;     // log2(e) / temperature
   int warps_log2;  // SHORT: warps that share a row
   int rows;        // SHORT: all rows
+  uint4* clear;    // not null (wait_first == 1): scratch of the next call, which this one empties (counted in 16-byte words)
+  int clear_words;
   int wait_first;  // 1: wait for the previous kernel in the stream before the first read (plain stream
                    //    order); 0: the logits are known to be complete, wait only before the first write
 };
@@ -545,6 +547,9 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     for (int d = 0; d < kDepth; ++d) issue(d);
     fetch_leftover(row, u1);
   }
+  if (g.clear != nullptr)  // (while the first slices are on their way)
+    for (int i = (int)(blockIdx.x * kReduceThreads + threadIdx.x); i < g.clear_words; i += (int)gridDim.x * kReduceThreads)
+      g.clear[i] = make_uint4(0, 0, 0, 0);
 
   // The acceptance scan at the end of the step reads draft tokens and carried state, which nothing has
   // touched yet: pull them into L2 now so that the last block does not wait on DRAM for them.
