@@ -134,10 +134,8 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Tiled TMA load into THIS CTA's shared memory; the bytes are reported to `bar`, a shared::cluster
 // address that may lie in the other CTA of the pair.  No multicast.
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
@@ -216,8 +214,9 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&r)[16]) {
                : "memory");
 }
 
-// Named barriers: 1 and 2 for the two epilogue groups (128 threads each), 3 for all epilogue threads.
+// Named barriers: 1 and 2 for the two epilogue groups (128 threads each), 3 for all epilogue threads, 4 for the whole CTA.
 __device__ __forceinline__ void group_bar(int group) { asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory"); }
+__device__ __forceinline__ void role_bar() { asm volatile("bar.sync 4, %0;" ::"n"(kThreads) : "memory"); }
 __device__ __forceinline__ void epi_all_bar() { asm volatile("bar.sync 3, 256;" ::: "memory"); }
 
 // ---- descriptors ---------------------------------------------------------------
@@ -298,7 +297,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   auto slot_full = [&](int i) { return bar0 + 8u * (2 * kMaxStages + i); };
   auto slot_empty = [&](int i) { return bar0 + 8u * (2 * kMaxStages + kSlots + i); };
   const uint32_t drain_bar = bar0 + 8u * (2 * kMaxStages + 2 * kSlots);  // used only on the give-up path
-  volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(gbase + kOffMisc);  // [0] tmem base, [1], [2] go flags of the epilogue groups
+  volatile uint32_t* misc = reinterpret_cast<volatile uint32_t*>(gbase + kOffMisc);  // [0] tmem base, [1], [2] go flags of the epilogue groups, [3] a role gave up
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();  // 0: leader of the pair (issues the MMAs, owns the "full" barriers)
@@ -314,6 +313,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
       mbar_init(slot_empty(i), 2 * kEpiThreads);   // the epilogue threads of both CTAs arrive on the leader's
     }
     mbar_init(drain_bar, 1);
+    misc[3] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {  // warp 0 of both CTAs together allocate all of tensor memory (one CTA per SM)
@@ -324,7 +324,8 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync();  // both CTAs' barriers exist before anything is sent to them
+  cluster_arrive();
+  cluster_wait();  // both CTAs' barriers exist before anything is sent to them
   tc_fence_after();
   const uint32_t tmem = misc[0];
 
@@ -348,6 +349,20 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   asm volatile("griddepcontrol.launch_dependents;");
 
   bool failed = false;  // a bounded wait of this thread's role ran out
+  // Where a role has done what the partner CTA takes part in: its last MMA, remote arrival and tensor-memory read.  After a failed wait
+  // give stragglers (TMA copies still in flight towards this CTA's shared memory) time to land first.
+  auto role_done = [&]() {
+    if (failed) misc[3] = 1;
+    tc_fence_before();
+    __syncwarp();
+    role_bar();
+    if (misc[3] != 0) {
+      const unsigned long long t0 = global_ns();
+      while (global_ns() - t0 < 2000000ull) {}
+    }
+    __syncwarp();
+    cluster_arrive();
+  };
   const uint32_t full_leader = map_to_cta(full(0), 0);  // the "full" barriers as both CTAs address them
   const uint32_t half_bytes = (uint32_t)(p.box * kBytesPos);  // one accumulator's hidden tile of this CTA
   const uint32_t h_bytes = p.n1 > 0 ? 2 * half_bytes : half_bytes;
@@ -536,7 +551,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
     // once (a lane per eighth and a fold by shuffles for every 32 positions took 3.3 us of the end of a step of 288; us a step,
     // before / after: 288 positions x 1024 x 50264 38.5 / 36.2, x 2048 x 10000 25.3 / 23.0, 36 x 512 x 4096 8.0 / 7.55).
     // The weight ring is free by now: every MMA that read it has completed (slot_full of the last tile).
-    epi_all_bar();
+    role_done();
     Partial* buf = reinterpret_cast<Partial*>(gbase + kOffW);
 #pragma unroll
     for (int k = 0; k < kGroupChunks; ++k) {
@@ -555,15 +570,11 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
     }
   }
 
-  // Common exit.  After a failed wait give stragglers (TMA copies still in flight towards this
-  // CTA's shared memory) time to land before the shared memory is handed back.
-  if (__syncthreads_or(failed)) {
-    const unsigned long long t0 = global_ns();
-    while (global_ns() - t0 < 2000000ull) {}
-  }
-  tc_fence_before();
-  __syncthreads();
-  cluster_sync();  // neither CTA leaves while its partner may still signal its barriers or read its operands
+  if (warp >= kEpiWarps) role_done();
+
+  // Common exit.  Neither CTA leaves, nor gives tensor memory back, while its partner may still signal its barriers, read its
+  // operands or read tensor memory; that has been over since role_done, so the merge above ran meanwhile.
+  cluster_wait();
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
