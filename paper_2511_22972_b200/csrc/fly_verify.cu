@@ -64,10 +64,11 @@ struct fly_verify {
   int lm_pairs = 0;                     // CTA pairs that can be resident at once
   int weight_vd = 0;                    // 0: weight [hidden, V]; 1: weight [V, hidden]
   PFN_cuTensorMapEncodeTiled encode_tiled = nullptr;
-  CUtensorMap map_w, map_h;             // cached for (map_w_ptr, map_h_ptr, map_h_rows)
+  CUtensorMap map_w, map_h;             // cached for (map_w_ptr, map_w_rows, map_h_ptr, map_h_rows)
   const void* map_w_ptr = nullptr;
   const void* map_h_ptr = nullptr;
   int64_t map_h_rows = 0;
+  int map_w_rows = 0;                   // entries per tile that map_w is for
   void* st_hidden = nullptr;            // staging of fly_verify_run_host
   size_t st_hidden_bytes = 0;
   // staging for fly_verify_run_host (allocated on first use)
@@ -307,6 +308,16 @@ cudaError_t set_reduce_attrs() {
   return e != cudaSuccess ? e : set_all(float());
 }
 
+// The same of the fused kernel.
+cudaError_t set_lm_attrs() {
+  cudaFuncAttributes have;
+  cudaError_t e = cudaFuncGetAttributes(&have, fly::lmhead::lmhead_verify_kernel<2>);
+  if (e != cudaSuccess || have.maxDynamicSharedSizeBytes >= fly::lmhead::kSmemBytes) return e;
+  e = cudaFuncSetAttribute(fly::lmhead::lmhead_verify_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, fly::lmhead::kSmemBytes);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(fly::lmhead::lmhead_verify_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     fly::lmhead::kSmemBytes);
+}
+
 // Lanes (as a power of two) that share a row's parts in the acceptance scan: one per part as far as a block has threads
 // for all rows of a sequence.
 int lanes_for(int64_t parts, int rows) {
@@ -436,6 +447,21 @@ bool encode_map(fly_verify* h, CUtensorMap* map, const void* ptr, uint64_t inner
   return r == CUDA_SUCCESS;
 }
 
+// Vocabulary entries per tile of a CTA pair for a weight stored [V, D] and up to 144 positions, where the weight stream is the work: 256,
+// or as few as give every pair as many tiles.  Where all pairs are busy most of the time they take in all that HBM has and an uneven
+// last round costs little; narrow tiles are for rounds that would be less than 80 % full, and small vocabularies whose few
+// tiles (of 128 then, at least) would leave pairs out: a CTA takes in 64 bytes a cycle at most.  us a step, 256 / so: 36 positions x 4096
+// x 20000 35.7 / 30.5, 64 x 3000 x 40000 54.3 / 46.1, 96 x 4096 x 20000 39.9 / 34.2, 144 x 4096 x 20000 42.2 / 39.4, 36 x 4096 x 30000 42.8 / 42.0, x
+// 8192 x 4096 23.3 / 19.8, 144 x 4096 x 12000 25.1 / 24.5; not for 36 x 4096 x 32000 45.3 / 44.8 but 144 x 4096 x 32000 49.7 / 51.3; nor, with
+// more partial states to fold, for one round of more than half of the pairs and few slices: 36 x 1504 x 12000 11.95 / 12.24.
+int lm_tile(int V, int num_kb, int pairs) {
+  namespace L = fly::lmhead;
+  const int tiles = (V + L::kPairV - 1) / L::kPairV, rounds = (tiles + pairs - 1) / pairs, even = rounds * pairs;
+  if (5 * tiles > 4 * even || (rounds == 1 && 2 * tiles > pairs && num_kb < 48)) return L::kPairV;
+  const int fewest = ((V + even - 1) / even + 15) / 16 * 16;  // (CTAs hold whole groups of eight entries)
+  return fewest < 128 ? 128 : fewest;
+}
+
 // Fused LM-head step: one GEMM + row-statistics launch per block of up to 288
 // positions, then the acceptance scan over the per-CTA partial states.
 fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t st) {
@@ -444,11 +470,14 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
   const int64_t rows = (int64_t)a->B * (a->K + 1);
   if ((reinterpret_cast<uintptr_t>(a->hidden) & 15u) || (reinterpret_cast<uintptr_t>(a->weight) & 15u))
     return FLY_ERR_UNSUPPORTED;  // TMA needs 16-byte aligned bases
-  if (h->map_w_ptr != a->weight) {
-    const bool ok = h->weight_vd ? encode_map(h, &h->map_w, a->weight, (uint64_t)D, (uint64_t)V, (uint64_t)D * 2, L::kBlockV)
+  const int num_kb = (D + L::kBlockK - 1) / L::kBlockK;
+  const int tile_v = h->weight_vd && rows <= L::kHalfN ? lm_tile(V, num_kb, h->lm_pairs) : L::kPairV;
+  if (h->map_w_ptr != a->weight || h->map_w_rows != tile_v) {
+    const bool ok = h->weight_vd ? encode_map(h, &h->map_w, a->weight, (uint64_t)D, (uint64_t)V, (uint64_t)D * 2, (uint32_t)tile_v / 2)
                                  : encode_map(h, &h->map_w, a->weight, (uint64_t)V, (uint64_t)D, (uint64_t)V * 2, 64);
     if (!ok) return FLY_ERR_CUDA;
     h->map_w_ptr = a->weight;
+    h->map_w_rows = tile_v;
   }
   // One accumulator takes up to 144 positions; more are shared evenly between two, so that both issuers have the same to do.
   auto first_half = [](int positions) {
@@ -461,7 +490,7 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     h->map_h_ptr = a->hidden;
     h->map_h_rows = rows;
   }
-  const int num_tiles = (V + L::kPairV - 1) / L::kPairV;  // one tile = 256 vocabulary entries = one CTA pair
+  const int num_tiles = (V + tile_v - 1) / tile_v;  // one tile = one CTA pair
   const int grid = 2 * (num_tiles < h->lm_pairs ? num_tiles : h->lm_pairs);
   for (int64_t row0 = 0; row0 < rows; row0 += L::kMaxPos) {
     L::Params p;
@@ -470,21 +499,30 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     p.n0 = first_half(p.R);
     p.n1 = r16 - p.n0;
     p.box = box;
-    p.stages = L::kRingBytes / (L::kBytesW + (p.n1 > 0 ? 2 : 1) * box * L::kBytesPos);
-    // A weight stored [D, V] is read 128 bytes of a row at a time, the next stage's 64 rows far away: a deeper ring spreads
-    // the requests over more DRAM pages than it gains (36 positions, D = 4096, V = 50264: 6 / 7 / 8 / 10 stages 79.4 / 79.3 /
-    // 80.8 / 82.8 us).  Stored [V, D] the next stage is the next 128 bytes (80.2 / 79.4 / 78.8 / 77.8; at D = 8192 and
-    // V = 128256 344 / 339 / 335 / 328).
-    const int deepest = h->weight_vd ? L::kMaxStages : 7;
+    p.tile_v = tile_v;
+    p.w_bytes = h->weight_vd ? tile_v / 2 * L::kBlockK * 2 : L::kBytesW;
+    // Two slices per stage where the ring holds five such stages (up to 64 positions, more with narrow tiles).  us a step, one / two:
+    // stored [V, D]: 36 positions x 512 x 4096 7.25 / 6.9, x 8192 x 4096 25.4 / 19.8 (tiles of 128), 12 x 1024 x 32000 16.3 / 15.4, 32 x
+    // 2752 x 50264 47.0 / 45.5, 36 x 2048 x 128256 80.4 / 79.3; in shorter rings 96 x 4096 x 32000 46.9 / 47.7,
+    // 288 x 4096 x 32000 68.9 / 69.3.
+    // A weight stored [D, V] is read 128 bytes of a row at a time, the next slice's 64 rows far away: a deeper ring spreads
+    // the requests over more DRAM pages than it gains (36 positions, D = 4096, V = 50264: 6 / 7 / 8 / 10 slices 79.4 / 79.3 /
+    // 80.8 / 82.8 us), unless its rows are whole lines (seven single / five double stages: 36 x 8192 x 4096 25.7 / 22.7, x 4096 x 20000 37.4 /
+    // 35.8, 12 x 1024 x 32000 16.6 / 16.0; off lines 32 x 2760 x 50264 49.6 / 51.0).
+    const int slice = p.w_bytes + (p.n1 > 0 ? 2 : 1) * box * L::kBytesPos;
+    const bool enough = num_kb >= 16 || p.n0 > 16;  // (2 x 640 x 128256 31.0 / 31.5)
+    const int slices = (h->weight_vd || V % 64 == 0) && enough && L::kRingBytes / (2 * slice) >= 5 ? 2 : 1;
+    const int deepest = h->weight_vd ? L::kMaxStages : slices == 2 ? 5 : 7;
+    p.stages = L::kRingBytes / (slices * slice);
     if (p.stages > deepest) p.stages = deepest;
     // The ring's worth of the first weight tile is asked for in L2 before the wait for the previous kernel.  us a step in a row of
     // steps, without / with: 12 positions, D = 1024, V = 32000 17.54 / 17.11; 2 x 640 x 128256 31.66 / 31.2; 4 x 4096 x 32000 49.7 /
     // 49.0; 32 x 2752 x 50264 47.3 / 46.6.  Only where the weight's rows are whole lines: others gain nothing or lose
     // (32 x 2760 x 50264 51.5 / 51.5 - 52.5, x 2752 x 50000, stored [D, V], 46.4 / 46.6).
-    p.ahead = (h->weight_vd ? D : V) % 64 == 0 ? p.stages : 0;
+    p.ahead = (h->weight_vd ? D : V) % 64 == 0 ? p.stages * slices : 0;
     p.V = V; p.D = D;
     p.num_tiles = num_tiles;
-    p.num_kb = (D + L::kBlockK - 1) / L::kBlockK;
+    p.num_kb = num_kb;
     p.row0 = (int)row0;
     p.w_kmajor = h->weight_vd;
     p.scale = exponent_scale(a->temperature);
@@ -495,7 +533,7 @@ fly_status_t run_fused(fly_verify* h, const fly_verify_args_t* a, cudaStream_t s
     cudaLaunchAttribute attr[1];
     fill_launch(&cfg, attr, (unsigned)grid, L::kThreads, st, true);
     cfg.dynamicSmemBytes = L::kSmemBytes;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, L::lmhead_verify_kernel, h->map_w, h->map_h, p);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, slices == 2 ? L::lmhead_verify_kernel<2> : L::lmhead_verify_kernel<1>, h->map_w, h->map_h, p);
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->last_launches++;
   }
@@ -617,9 +655,7 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
   h->scratch_bytes = bytes;
   if (c->hidden > 0) {
     e = cudaMalloc(&h->lm_partials, (size_t)h->max_rows * h->sm_count * sizeof(fly::Partial));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(fly::lmhead::lmhead_verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               fly::lmhead::kSmemBytes);
+    if (e == cudaSuccess) e = set_lm_attrs();
     if (e == cudaSuccess) {
       // how many pairs (clusters of two CTAs, one CTA per SM) fit on the device at once
       cudaLaunchConfig_t lc;
@@ -633,7 +669,7 @@ fly_status_t fly_verify_create(const fly_verify_config_t* c, fly_verify_t** out)
       lc.attrs = at;
       lc.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, fly::lmhead::lmhead_verify_kernel, &lc) != cudaSuccess || n < 1) {
+      if (cudaOccupancyMaxActiveClusters(&n, fly::lmhead::lmhead_verify_kernel<1>, &lc) != cudaSuccess || n < 1) {
         (void)cudaGetLastError();
         n = h->sm_count / 2;
       }

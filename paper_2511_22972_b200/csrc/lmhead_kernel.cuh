@@ -7,7 +7,8 @@
 // its N dimension ("swap-AB"):  D[v, p] = sum_d weight[d, v] * hidden[p, d].
 // Two CTAs on neighbouring SMs work as one pair (tcgen05 cta_group::2) on a tile
 // of 256 vocabulary entries x up to 288 positions:
-//   A = weight tile.  Each CTA holds ITS 128 vocabulary entries x 64 hidden dims.
+//   A = weight tile.  Each CTA holds ITS 128 vocabulary entries x 64 hidden dims (fewer entries where that shares the
+//       vocabulary evenly: the accumulators' other rows are then of whatever lies behind, and not looked at).
 //       weight is [D, V] with V contiguous, so A is MN-major; TMA lays it down as
 //       two boxes of 64 entries (128 bytes) x 64 dims with the 128-byte swizzle.
 //   B = hidden tile, K-major, 128-byte swizzle.  The pair shares it: each CTA
@@ -70,9 +71,10 @@ constexpr int kBytesW = kBlockK * kBlockV * 2;      // 16 KB per stage
 constexpr int kBytesWBox = kBlockK * 64 * 2;        // one TMA box: 64 entries x 64 dims
 constexpr int kBoxPos = kHalfN / 2;                 // positions per TMA box at most: this CTA's half of one accumulator
 constexpr int kBytesPos = kBlockK * 2;              // one position's 64 dims
-// Operand ring: one stage = one 64-dim slice of the weight tile and of the hidden tile.  A stage takes as much shared
-// memory as its positions need, and the ring as many stages as fit: 6 at 288 positions, 12 at 16.  With few positions
-// the weight stream is the work, and what is in flight bounds it.
+// Operand ring: one stage = one or two 64-dim slices of the weight tile and of the hidden tile.  A stage takes as much shared
+// memory as its entries and positions need, and the ring as many stages as fit: 6 at 288 positions.  With few positions
+// the weight stream is the work, and what is in flight bounds it, or, where few CTAs share a small vocabulary, what a
+// stage costs its issuer (a wait, four MMAs and a commit, about 230 cycles): two slices per stage save one of two.
 constexpr int kRingBytes = 6 * (kBytesW + 2 * kBoxPos * kBytesPos);
 constexpr int kMaxStages = 12;
 constexpr int kChunk = 16;                          // positions turned through shared memory at a time
@@ -106,10 +108,12 @@ struct Params {
   int box;        // positions per TMA box of the hidden tile: n0 / 2, or more
   int stages;     // of the operand ring
   int V, D;
-  int num_tiles;  // ceil(V / 256): tiles of the CTA pairs
+  int tile_v;     // vocabulary entries per tile of a pair (256, or less of them in use: a multiple of 16), half of them per CTA
+  int num_tiles;  // ceil(V / tile_v)
+  int w_bytes;    // of the weight tile of a CTA and stage
   int num_kb;     // ceil(D / 64)
   int row0;       // first row of this launch in hidden / partials
-  int ahead;      // stages of the first weight tile asked for in L2 before the wait for the previous kernel
+  int ahead;      // slices of the first weight tile asked for in L2 before the wait for the previous kernel
   int w_kmajor;   // 0: weight is [D, V] (vocabulary contiguous, MN-major A); 1: weight is [V, D] (K-major A)
   float scale;    // log2(e) / temperature: logit -> base-2 exponent
   float floor;    // logits at or below it are masked
@@ -279,6 +283,8 @@ __device__ __forceinline__ void fold16(Stream& st, float (&x)[16], int v0, float
   st.u += u0 + u1;
 }
 
+// SLICES: 64-dim slices per stage of the operand ring.
+template <int SLICES>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_h,
                      const Params p) {
@@ -332,7 +338,7 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   const int my_tiles = pair < p.num_tiles ? (p.num_tiles - 1 - pair) / npairs + 1 : 0;
   // A prefetch reads nothing for the program: the kernel before may still be writing the weight.
   if (warp == kWarpW && my_tiles > 0 && elect_lane()) {
-    const int v0 = pair * kPairV + (int)rank * kBlockV;
+    const int v0 = pair * p.tile_v + (int)rank * (p.tile_v >> 1);
     for (int kb = 0; kb < min(p.ahead, p.num_kb); ++kb) {
       if (p.w_kmajor) {
         tma_prefetch_2d(&map_w, kb * kBlockK, v0);
@@ -366,7 +372,8 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
   const uint32_t full_leader = map_to_cta(full(0), 0);  // the "full" barriers as both CTAs address them
   const uint32_t half_bytes = (uint32_t)(p.box * kBytesPos);  // one accumulator's hidden tile of this CTA
   const uint32_t h_bytes = p.n1 > 0 ? 2 * half_bytes : half_bytes;
-  const uint32_t off_h = (uint32_t)(kOffW + p.stages * kBytesW);
+  const uint32_t w_stage = (uint32_t)(SLICES * p.w_bytes), h_stage = SLICES * h_bytes;
+  const uint32_t off_h = (uint32_t)kOffW + (uint32_t)p.stages * w_stage;
 
   if (warp == kWarpW) {
     // ---------------- weight producer: this CTA's 128 vocabulary entries ----------------
@@ -374,18 +381,22 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
     uint32_t ph = 0;
     const bool lead = elect_lane();
     for (int t = 0; t < my_tiles && !failed; ++t) {
-      const int v0 = (pair + t * npairs) * kPairV + (int)rank * kBlockV;
-      for (int kb = 0; kb < p.num_kb; ++kb) {
+      const int v0 = (pair + t * npairs) * p.tile_v + (int)rank * (p.tile_v >> 1);
+      for (int kb = 0; kb < p.num_kb; kb += SLICES) {
         if (!mbar_wait_warp(empty(s), ph ^ 1, p.status, kErrTimeoutProducer)) { failed = true; break; }
         const uint32_t bar = full_leader + 8u * s;
-        const uint32_t dst = base + kOffW + s * kBytesW;
         if (lead) {
-          if (rank == 0) mbar_expect_tx(full(s), 2 * kBytesW);  // both CTAs' bytes
-          if (p.w_kmajor) {  // [V, D]: one box of 128 entries x 64 dims, each entry's 64 dims contiguous
-            tma_load_2d(dst, &map_w, kb * kBlockK, v0, bar);
-          } else {           // [D, V]: two boxes of 64 entries x 64 dims, each dim's 64 entries contiguous
-            tma_load_2d(dst, &map_w, v0, kb * kBlockK, bar);
-            tma_load_2d(dst + kBytesWBox, &map_w, v0 + 64, kb * kBlockK, bar);
+          if (rank == 0) mbar_expect_tx(full(s), 2u * (uint32_t)(min(SLICES, p.num_kb - kb) * p.w_bytes));  // both CTAs' bytes
+#pragma unroll
+          for (int j = 0; j < SLICES; ++j) {
+            if (j > 0 && kb + j >= p.num_kb) break;
+            const uint32_t dst = base + kOffW + s * w_stage + j * p.w_bytes;
+            if (p.w_kmajor) {  // [V, D]: one box of the CTA's entries x 64 dims, each entry's 64 dims contiguous
+              tma_load_2d(dst, &map_w, (kb + j) * kBlockK, v0, bar);
+            } else {           // [D, V]: two boxes of 64 entries x 64 dims, each dim's 64 entries contiguous
+              tma_load_2d(dst, &map_w, v0, (kb + j) * kBlockK, bar);
+              tma_load_2d(dst + kBytesWBox, &map_w, v0 + 64, (kb + j) * kBlockK, bar);
+            }
           }
         }
         __syncwarp();
@@ -400,14 +411,18 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
     const int y0 = p.row0 + (int)rank * (p.n0 / 2);
     const int y1 = p.row0 + p.n0 + (int)rank * (p.n1 / 2);
     for (int t = 0; t < my_tiles && !failed; ++t) {
-      for (int kb = 0; kb < p.num_kb; ++kb) {
+      for (int kb = 0; kb < p.num_kb; kb += SLICES) {
         if (!mbar_wait_warp(empty(s), ph ^ 1, p.status, kErrTimeoutProducer)) { failed = true; break; }
         const uint32_t bar = full_leader + 8u * s;
-        const uint32_t dst = base + off_h + s * h_bytes;
         if (lead) {
-          if (rank == 0) mbar_expect_tx(full(s), 2 * h_bytes);
-          tma_load_2d(dst, &map_h, kb * kBlockK, y0, bar);
-          if (p.n1 > 0) tma_load_2d(dst + half_bytes, &map_h, kb * kBlockK, y1, bar);
+          if (rank == 0) mbar_expect_tx(full(s), 2u * (uint32_t)min(SLICES, p.num_kb - kb) * h_bytes);
+#pragma unroll
+          for (int j = 0; j < SLICES; ++j) {
+            if (j > 0 && kb + j >= p.num_kb) break;
+            const uint32_t dst = base + off_h + s * h_stage + j * h_bytes;
+            tma_load_2d(dst, &map_h, (kb + j) * kBlockK, y0, bar);
+            if (p.n1 > 0) tma_load_2d(dst + half_bytes, &map_h, (kb + j) * kBlockK, y1, bar);
+          }
         }
         __syncwarp();
         if (++s == p.stages) { s = 0; ph ^= 1; }
@@ -438,16 +453,22 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
         const uint32_t d_tmem = tmem + (uint32_t)(slot * kHalfN);
         if (!mbar_wait_warp(slot_empty(slot), ((use / kSlots) & 1) ^ 1, p.status, kErrTimeoutMma)) { failed = true; break; }
         tc_fence_after();
-        for (int kb = 0; kb < p.num_kb; ++kb) {
+        for (int kb = 0; kb < p.num_kb; kb += SLICES) {
           // TMA-written operands need no tcgen05 fence: the barrier wait orders them before the MMAs
           if (!mbar_wait_warp(full(st), ph, p.status, kErrTimeoutMma)) { failed = true; break; }
-          const uint32_t a_lo = a_lo0 + (uint32_t)st * (kBytesW >> 4);
-          const uint32_t b_lo = b_lo0 + (uint32_t)st * (h_bytes >> 4);
+          uint32_t a_lo = a_lo0 + (uint32_t)st * (w_stage >> 4);
+          uint32_t b_lo = b_lo0 + (uint32_t)st * (h_stage >> 4);
           if (lead) {
 #pragma unroll
-            for (int ks = 0; ks < kBlockK / kMmaK; ++ks) {
-              const uint32_t acc = ks == 0 ? (uint32_t)(kb != 0) : 1u;
-              mma_bf16(d_tmem, a_lo + ks * a_step, b_lo + ks * ((kMmaK * 2) >> 4), kDescHi, idesc, acc);
+            for (int j = 0; j < SLICES; ++j) {
+              if (j > 0 && kb + j >= p.num_kb) break;
+#pragma unroll
+              for (int ks = 0; ks < kBlockK / kMmaK; ++ks) {
+                const uint32_t acc = ks == 0 ? (uint32_t)(kb + j != 0) : 1u;
+                mma_bf16(d_tmem, a_lo + ks * a_step, b_lo + ks * ((kMmaK * 2) >> 4), kDescHi, idesc, acc);
+              }
+              a_lo += (uint32_t)p.w_bytes >> 4;
+              b_lo += h_bytes >> 4;
             }
             // the stage may be refilled, in both CTAs, once these MMAs have read it
             mma_commit_pair(empty(st));
@@ -502,8 +523,8 @@ lmhead_verify_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
       const bool go = misc[1 + group] != 0;  // one thread per group waits, the group takes the same decision
       if (!go) { failed = true; break; }
       tc_fence_after();
-      const int v0 = (pair + t * npairs) * kPairV + (int)rank * kBlockV + eighth * 16;
-      const int limit = p.V - v0;  // entries of this eighth that exist
+      const int v0 = (pair + t * npairs) * p.tile_v + (int)rank * (p.tile_v >> 1) + eighth * 16;
+      const int limit = min(p.V - v0, (p.tile_v >> 1) - eighth * 16);  // entries of this eighth that exist
       // an accumulator of which this group turns no block is handed back at once
       if (last0 < 0) { tc_fence_before(); mbar_arrive_remote(map_to_cta(slot_empty(slot0), 0)); }
       if (nh == 2 && last1 < 0) { tc_fence_before(); mbar_arrive_remote(map_to_cta(slot_empty(slot1), 0)); }
