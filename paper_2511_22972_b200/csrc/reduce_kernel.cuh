@@ -462,6 +462,10 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
   __shared__ float leftover[SHORT ? kReduceWarps : 1][32];  // VEC: what the segments of the current row leave over (last warp)
   const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
 
+  // The next kernel in the stream may get scheduled early if it asks for that; it waits for this grid's completion before it
+  // touches anything this grid writes.  With inputs_ready that is what the pace of a queue of small steps hangs on: at once.
+  if (g.wait_first == 0) asm volatile("griddepcontrol.launch_dependents;");
+
   int row, u0, u1, slot;  // the current piece: units [u0, u1) of `row`, stored in the row's slot `slot`
   int64_t left, take;     // flat units of this block not yet assigned to a piece; flat units the current piece takes
   if (SHORT) {
@@ -537,10 +541,10 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
   // The grid is launched as a programmatic dependent of the previous kernel in the stream.  Plain
   // stream order: wait for that kernel to complete (and its writes to be visible) before anything is
   // read.  With inputs_ready the reads start at once and the wait comes before the first write.
-  if (g.wait_first != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-  // Let the next kernel in the stream get scheduled early if it asks for that; it waits for this
-  // grid's completion before it touches anything this grid writes.
-  asm volatile("griddepcontrol.launch_dependents;");
+  if (g.wait_first != 0) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+  }
 
   if constexpr (VEC) {
 #pragma unroll
