@@ -329,7 +329,7 @@ PyObject* py_pld_draft(PyObject*, PyObject* const* v, Py_ssize_t n) {
     const int64_t B = tokens.size(0);
     if (tokens.is_cuda()) {
       // Straight from torch's allocator: through the dispatcher each of the four takes 0.5 us longer, and the call as long as
-      // the kernel (32 contexts of 32768 tokens: 7.0 us a call, 5.5 so).
+      // the kernel (32 contexts of 32768 tokens: 6.9 us a call, 5.6 so).
       const c10::DeviceGuard guard(tokens.device());
       c10::Allocator* const allocator = at::detail::getCUDAHooks().getCUDADeviceAllocator();
       auto empty = [&](at::IntArrayRef shape) {
