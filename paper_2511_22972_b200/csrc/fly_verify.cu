@@ -52,6 +52,7 @@ struct fly_verify {
   int forced_splits = 0;
   int scan_mode = 0;   // 0: fused tail, 1: separate kernel
   int last_launches = 0;
+  bool host_logits = false;  // the step's logits are host memory, read in place
   int last_cuda_error = 0;
   // fused LM-head path (cfg.hidden > 0)
   fly::Partial* lm_partials = nullptr;  // [max_rows * sm_count]: one partial state per row and CTA
@@ -343,7 +344,7 @@ float exponent_scale(double temperature) {
 template <typename T>
 cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, int V, int64_t rows, int forced, int cap,
                           fly::Partial* partials, cudaStream_t st, fly::ScanParams* tail, double temperature,
-                          bool inputs_ready, uint4* clear, int clear_words) {
+                          bool inputs_ready, bool host_logits, uint4* clear, int clear_words) {
   constexpr int kE = fly::Seg<T>::kElems;
   const bool vec = vector_path_ok<T>(logits, V);
   const int64_t n = vec ? V / kE : V;
@@ -353,7 +354,7 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   fly::ReducePlan g;
   g.n = n; g.span = pl.span; g.Q = pl.Q; g.total = rows * pl.span;
   g.pieces = pl.Q < (1 << 30) ? pl.pieces : 0; g.V = V; g.row_stride = row_stride;
-  g.scale = exponent_scale(temperature); g.wait_first = inputs_ready ? 0 : 1;
+  g.scale = exponent_scale(temperature); g.wait_first = inputs_ready ? 0 : host_logits ? 2 : 1;
   g.rows = (int)rows; g.clear = clear; g.clear_words = clear_words;
   static_assert(fly::kReduceWarps == 8, "rows per block x warps per row");
   g.warps_log2 = 3 - pl.rows_log2;
@@ -391,12 +392,12 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
 // The current device must be the one the pointers belong to.
 cudaError_t launch_reduce_any(fly_dtype_t dt, int sm_count, const void* logits, int64_t row_stride, int V,
                               int64_t rows, int forced, int cap, fly::Partial* partials, cudaStream_t st,
-                              fly::ScanParams* tail, double temperature, bool inputs_ready, uint4* clear = nullptr, int clear_words = 0) {
+                              fly::ScanParams* tail, double temperature, bool inputs_ready, bool host_logits = false, uint4* clear = nullptr, int clear_words = 0) {
   if (dt == FLY_BF16)
     return launch_reduce<__nv_bfloat16>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature,
-                                        inputs_ready, clear, clear_words);
-  return launch_reduce<float>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature, inputs_ready, clear,
-                              clear_words);
+                                        inputs_ready, host_logits, clear, clear_words);
+  return launch_reduce<float>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature, inputs_ready, host_logits,
+                              clear, clear_words);
 }
 
 // tagged: the parts are in the self-validating form that the row reduction leaves.
@@ -893,7 +894,7 @@ fly_status_t fly_verify_run(fly_verify_t* h, const fly_verify_args_t* a, void* c
   p.tickets = fused_tail ? h->tickets : nullptr;
   p.status = h->state_status;
   e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, a->logits, stride, V, rows, h->forced_splits,
-                                    kMaxSplits, h->partials, st, &p, a->temperature, a->inputs_ready != 0);
+                                    kMaxSplits, h->partials, st, &p, a->temperature, a->inputs_ready != 0, h->host_logits);
   if (e != cudaSuccess) return cuda_fail(h, e);
   h->last_launches++;
   if (!fused_tail) {
@@ -990,7 +991,9 @@ fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, vo
   d.entropy = reinterpret_cast<float*>(dv + o_entropy);
   d.row_flags = reinterpret_cast<uint32_t*>(dv + o_flags);
   d.target_tokens = a->target_tokens ? dv + o_target : nullptr;
+  h->host_logits = direct != nullptr;  // (nothing precedes them, and over the bus a read ahead is a read more)
   s = fly_verify_run(h, &d, cuda_stream);
+  h->host_logits = false;
   if (s != FLY_OK) return s;
 
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(h, e);
@@ -1110,7 +1113,7 @@ fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t lo
     if (e != cudaSuccess) return FLY_ERR_CUDA;
   }
   e = launch_reduce_any(logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, a->temperature,
-                        a->inputs_ready != 0, takes_turn ? reinterpret_cast<uint4*>(next) : nullptr, (int)(kStaticPartBytes / 16));
+                        a->inputs_ready != 0, false, takes_turn ? reinterpret_cast<uint4*>(next) : nullptr, (int)(kStaticPartBytes / 16));
   return e == cudaSuccess ? FLY_OK : FLY_ERR_CUDA;
 }
 

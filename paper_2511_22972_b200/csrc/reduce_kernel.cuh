@@ -323,7 +323,8 @@ struct ReducePlan {
   uint4* clear;    // not null (wait_first == 1): scratch of the next call, which this one empties (counted in 16-byte words)
   int clear_words;
   int wait_first;  // 1: wait for the previous kernel in the stream before the first read (plain stream
-                   //    order); 0: the logits are known to be complete, wait only before the first write
+                   //    order); 0: the logits are known to be complete, wait only before the first write;
+                   //    2: as 1, and nothing is asked for ahead of the wait
 };
 
 // Lanes -> warp -> block; warp 0 ends up with the piece's Partial (lane l with that of warp l's group of 2^warps_log2
@@ -536,7 +537,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
   };
   if constexpr (VEC) {
     open_piece(row, u0, u1);
-    if (g.wait_first != 0) ask_ahead();
+    if (g.wait_first == 1) ask_ahead();
   }
   // The grid is launched as a programmatic dependent of the previous kernel in the stream.  Plain
   // stream order: wait for that kernel to complete (and its writes to be visible) before anything is
