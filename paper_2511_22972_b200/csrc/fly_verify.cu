@@ -1081,7 +1081,7 @@ fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t lo
   // graph is made of, which are replayed in any order, and those that write nothing before their end (inputs_ready): they
   // have a part of their own, which such a kernel empties.
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
+  if (a->inputs_ready == 0 && cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
     (void)cudaGetLastError();  // (the legacy stream while another one is being captured: the launch says so)
     capture = cudaStreamCaptureStatusActive;
   }
