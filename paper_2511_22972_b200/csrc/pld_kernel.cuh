@@ -48,10 +48,11 @@ __global__ void __launch_bounds__(kThreads) pld_draft_kernel(const Params p) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   const int ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-  __shared__ int best[kMaxNgram + 1];   // of the block; in the first block of the cluster, of all of them
+  __shared__ int best[kMaxNgram + 1];   // of the block: its own matches alone, by which it also ends its rounds
+  __shared__ int others[kMaxNgram + 1]; // in the first block of the cluster: of the others, which may end before it does
   __shared__ int suffix[kMaxNgram];     // the last tokens, the last one first
-  if (threadIdx.x <= kMaxNgram) best[threadIdx.x] = kNone;
-  // Nothing is written to another block's best[] before that block has reached this point.
+  if (threadIdx.x <= kMaxNgram) best[threadIdx.x] = others[threadIdx.x] = kNone;
+  // Nothing is written to another block's others[] before that block has reached this point.
   if (ranks > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the previous kernel in the stream may have written the tokens
   asm volatile("griddepcontrol.launch_dependents;");
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(kThreads) pld_draft_kernel(const Params p) {
   if (ranks > 1) {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (rank > 0 && threadIdx.x >= 1 && threadIdx.x <= kMaxNgram && best[threadIdx.x] != kNone)
-      atomicMin(cluster.map_shared_rank(best + threadIdx.x, 0), best[threadIdx.x]);
+      atomicMin(cluster.map_shared_rank(others + threadIdx.x, 0), best[threadIdx.x]);
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     if (rank > 0) return;  // nobody looks into this block's shared memory
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(kThreads) pld_draft_kernel(const Params p) {
   // every thread takes the same decision
   int end = 0, ngram = 0;
   const int lane = (int)threadIdx.x & 31;
-  const int e = lane >= p.min_ngram && lane <= p.max_ngram ? best[lane] : kNone;  // lane n: the earliest match of n tokens
+  const int e = lane >= p.min_ngram && lane <= p.max_ngram ? min(best[lane], others[lane]) : kNone;  // lane n: the earliest match of n tokens
   const unsigned found = __ballot_sync(0xffffffffu, e != kNone);
   if (found) {
     ngram = 31 - __clz((int)found);

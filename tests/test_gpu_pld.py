@@ -137,3 +137,31 @@ def test_rows_at_every_alignment_and_lengths_around_a_round(width):
     seqs.append([rng.randrange(3) for _ in range(width)])
     for K, mx, mn in [(15, 3, 1), (5, 8, 2)]:
         run(seqs, K, mx, mn, pad_to=width)
+
+
+@pytest.mark.parametrize("slow,at", [((0,), 34000), ((0, 32768), 66000)])
+def test_the_first_block_goes_on_when_others_end_first(slow, at):
+    # The first block of a cluster is held up by look-backs one token short of a match, all over one or two of its rounds; the other
+    # blocks have a match in a later round and end before it gets to its own, earlier one.
+    query, L, B = [9] + [5] * 7, 100000, 64
+    seqs = []
+    for i in range(4):
+        s = list(range(10, 10 + L))
+        for lo in slow:
+            s[lo:lo + 4096] = [5] * 4096
+        for e in (at + 100 * i, *range(at + 3000, at + 3000 + 7 * 4096, 4096)):
+            s[e:e + 8] = query
+        s[L - 8 - i:] = query                     # (the last tokens at every alignment)
+        seqs.append(s)
+    want = [oracle_pld(s, 15, 8, 1) for s in seqs]
+    assert [(p, n) for _, p, n in want] == [(at + 100 * i, 8) for i in range(4)]
+    tok = torch.full((B, L + 1), -7, dtype=torch.int32)
+    for b in range(B):
+        tok[b, :len(seqs[b % 4])] = torch.tensor(seqs[b % 4], dtype=torch.int32)
+    lengths = torch.tensor([len(seqs[b % 4]) for b in range(B)], dtype=torch.int32, device=DEV)
+    tok, st = tok.to(DEV), torch.cuda.current_stream().cuda_stream
+    got = [Bd.pld_draft(tok, lengths, 15, 8, 1, stream=st) for _ in range(20)]
+    torch.cuda.synchronize()
+    for draft, count, pos, ng in got:
+        assert pos.tolist() == [want[b % 4][1] for b in range(B)] and ng.tolist() == [8] * B and count.tolist() == [15] * B
+        assert draft.tolist() == [want[b % 4][0] for b in range(B)]
