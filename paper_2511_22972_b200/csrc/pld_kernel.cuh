@@ -107,8 +107,10 @@ __global__ void __launch_bounds__(kThreads) pld_draft_kernel(const Params p) {
         if (t + 1 < best[m]) atomicMin(&best[m], t + 1);
     }
     s += ranks * kStep;
-    // (a block's positions ascend: once it has a match of the longest query, it has its earliest)
-    if (s - tid >= seg1 || __syncthreads_or(best[p.max_ngram] != kNone)) break;
+    // The block is done with a match of the longest query that ends before its next round begins.  (Not with any: the tokens behind the last
+    // segment are tested in the first round, and what they end may have an earlier match in rounds to come.)
+    const int next = s - tid;  // the round's first segment
+    if (next >= seg1 || __syncthreads_or(best[p.max_ngram] <= next * 4 - head)) break;
     fetch(s);
   }
   __syncthreads();

@@ -165,3 +165,24 @@ def test_the_first_block_goes_on_when_others_end_first(slow, at):
     for draft, count, pos, ng in got:
         assert pos.tolist() == [want[b % 4][1] for b in range(B)] and ng.tolist() == [8] * B and count.tolist() == [15] * B
         assert draft.tolist() == [want[b % 4][0] for b in range(B)]
+
+
+@pytest.mark.parametrize("L", [32800, 40000, 65560, 131072])
+@pytest.mark.parametrize("pad", [0, 1, 2, 3])
+def test_contexts_that_end_in_a_run_of_one_token(L, pad):
+    # The tokens behind the last whole 16-byte segment are tested first and match the longest query; the earliest match lies in a
+    # later round of the first block of the cluster, or in one of another block.
+    seqs, cases = [], []
+    for mx in (1, 3, 8):
+        for at in (32770, 36850, 45000, 65540, 69620):
+            if at + mx > L - 16:
+                continue
+            n = L - len(seqs) % 4                 # (the last tokens at every alignment)
+            s = list(range(10, 10 + n))
+            s[at:at + mx] = [7] * mx
+            s[n - mx - 3:] = [7] * (mx + 3)
+            seqs.append(s)
+            cases.append((mx, at))
+    for mx in (1, 3, 8):
+        run([s for s, c in zip(seqs, cases) if c[0] == mx], 8, mx, 1, pad_to=(L + 3) // 4 * 4 + pad)
+    assert all(oracle_pld(s, 8, mx, 1)[1:] == (at, mx) for s, (mx, at) in zip(seqs, cases))
