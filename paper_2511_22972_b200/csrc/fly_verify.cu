@@ -344,7 +344,7 @@ float exponent_scale(double temperature) {
 template <typename T>
 cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, int V, int64_t rows, int forced, int cap,
                           fly::Partial* partials, cudaStream_t st, fly::ScanParams* tail, double temperature,
-                          bool inputs_ready, bool host_logits, uint4* clear, int clear_words) {
+                          bool inputs_ready, bool host_logits, uint4* clear) {
   constexpr int kE = fly::Seg<T>::kElems;
   const bool vec = vector_path_ok<T>(logits, V);
   const int64_t n = vec ? V / kE : V;
@@ -352,10 +352,10 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
   const int64_t stride_units = (int64_t)fly::kReduceWarps * kReduceUnroll * 32;
   const FlatPlan pl = plan_flat(sm_count, rows, n, (int)sizeof(T), vec, min_units, stride_units, cap, inputs_ready, forced);
   fly::ReducePlan g;
-  g.n = n; g.span = pl.span; g.Q = pl.Q; g.total = rows * pl.span;
+  g.n = n; g.span = pl.span; g.Q = pl.Q;
   g.pieces = pl.Q < (1 << 30) ? pl.pieces : 0; g.V = V; g.row_stride = row_stride;
   g.scale = exponent_scale(temperature); g.wait_first = inputs_ready ? 0 : host_logits ? 2 : 1;
-  g.rows = (int)rows; g.clear = clear; g.clear_words = clear_words;
+  g.rows = (int)rows; g.clear = clear;
   static_assert(fly::kReduceWarps == 8, "rows per block x warps per row");
   g.warps_log2 = 3 - pl.rows_log2;
   tail->splits = pl.slots;
@@ -392,12 +392,12 @@ cudaError_t launch_reduce(int sm_count, const void* logits, int64_t row_stride, 
 // The current device must be the one the pointers belong to.
 cudaError_t launch_reduce_any(fly_dtype_t dt, int sm_count, const void* logits, int64_t row_stride, int V,
                               int64_t rows, int forced, int cap, fly::Partial* partials, cudaStream_t st,
-                              fly::ScanParams* tail, double temperature, bool inputs_ready, bool host_logits = false, uint4* clear = nullptr, int clear_words = 0) {
+                              fly::ScanParams* tail, double temperature, bool inputs_ready, bool host_logits = false, uint4* clear = nullptr) {
   if (dt == FLY_BF16)
     return launch_reduce<__nv_bfloat16>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature,
-                                        inputs_ready, host_logits, clear, clear_words);
+                                        inputs_ready, host_logits, clear);
   return launch_reduce<float>(sm_count, logits, row_stride, V, rows, forced, cap, partials, st, tail, temperature, inputs_ready, host_logits,
-                              clear, clear_words);
+                              clear);
 }
 
 // tagged: the parts are in the self-validating form that the row reduction leaves.
@@ -1023,7 +1023,7 @@ namespace {
 
 constexpr int kStaticMaxDevices = 64;
 constexpr size_t kStaticPartBytes = FLY_STATIC_SCRATCH_BYTES / FLY_STATIC_PARTS;  // arrival counters, then slots
-static_assert(kStaticPartBytes == FLY_STATIC_MAX_BATCH * 4 + FLY_STATIC_MAX_PIECES * 16 && kStaticPartBytes % 256 == 0, "");
+static_assert(kStaticPartBytes == FLY_STATIC_MAX_BATCH * 4 + FLY_STATIC_MAX_PIECES * 16 && kStaticPartBytes % 256 == 0 && kStaticPartBytes == fly::kClearWords * 16, "");
 struct StaticSlot {
   unsigned char* base = nullptr;  // device address of g_fly_static_scratch on this device
   int sm_count = 0;
@@ -1113,7 +1113,7 @@ fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t lo
     if (e != cudaSuccess) return FLY_ERR_CUDA;
   }
   e = launch_reduce_any(logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, a->temperature,
-                        a->inputs_ready != 0, false, takes_turn ? reinterpret_cast<uint4*>(next) : nullptr, (int)(kStaticPartBytes / 16));
+                        a->inputs_ready != 0, false, takes_turn ? reinterpret_cast<uint4*>(next) : nullptr);
   return e == cudaSuccess ? FLY_OK : FLY_ERR_CUDA;
 }
 

@@ -308,24 +308,27 @@ __device__ __forceinline__ void reduce_piece_scalar(WarpAcc& a, const T* __restr
     warp_slice_scalar<T, UNROLL>(a, rp, e0, e_end, lane, floor);
 }
 
-// Geometry of one launch (see the head of this file).
+constexpr int kClearWords = 16640;  // 16-byte words of a part of the static entry point's scratch
+
+// Geometry of one launch (see the head of this file).  The size matters: what a launch costs the host depends on the sizes and offsets of the
+// kernel's arguments, in no order that a rule was found for.  us a step in a row of steps with inputs_ready, 9 rows of 32000 fp32 (median of five
+// processes, which differ by 0.1), by the bytes of this struct, with the 216 of ScanParams: 56 3.28, 64 3.30, 80 3.72; 56 and 208 3.59.
 struct ReducePlan {
   int64_t n;       // units per row
   int64_t span;    // units a row takes in the flat index space (>= n)
   int64_t Q;       // units per block
-  int64_t total;   // rows * span
   int pieces;      // > 0: span = pieces * Q, block b is piece b % pieces of row b / pieces (32-bit arithmetic)
   int V;
   int64_t row_stride;  // elements
   float scale;     // log2(e) / temperature
   int warps_log2;  // SHORT: warps that share a row
-  int rows;        // SHORT: all rows
-  uint4* clear;    // not null (wait_first == 1): scratch of the next call, which this one empties (counted in 16-byte words)
-  int clear_words;
+  int rows;
   int wait_first;  // 1: wait for the previous kernel in the stream before the first read (plain stream
                    //    order); 0: the logits are known to be complete, wait only before the first write;
                    //    2: as 1, and nothing is asked for ahead of the wait
+  uint4* clear;    // not null (wait_first == 1): kClearWords of scratch of the next call, which this one empties
 };
+static_assert(sizeof(ReducePlan) == 64 && sizeof(ScanParams) == 216, "measure what a launch costs the host");
 
 // Lanes -> warp -> block; warp 0 ends up with the piece's Partial (lane l with that of warp l's group of 2^warps_log2
 // warps).  sm: kReduceWarps Partials of
@@ -483,7 +486,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     left = take = g.Q;
   } else {
     const int64_t f0 = (int64_t)blockIdx.x * g.Q;
-    const int64_t f_end = min(f0 + g.Q, g.total);
+    const int64_t f_end = min(f0 + g.Q, (int64_t)g.rows * g.span);
     row = (int)(f0 / g.span);
     u0 = (int)(f0 - (int64_t)row * g.span);
     slot = (int)((int64_t)blockIdx.x - ((int64_t)row * g.span) / g.Q);     // pieces of the row that earlier blocks hold
@@ -553,7 +556,7 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     fetch_leftover(row, u1);
   }
   if (g.clear != nullptr)  // (while the first slices are on their way)
-    for (int i = (int)(blockIdx.x * kReduceThreads + threadIdx.x); i < g.clear_words; i += (int)gridDim.x * kReduceThreads)
+    for (int i = (int)(blockIdx.x * kReduceThreads + threadIdx.x); i < kClearWords; i += (int)gridDim.x * kReduceThreads)
       g.clear[i] = make_uint4(0, 0, 0, 0);
 
   // The acceptance scan at the end of the step reads draft tokens and carried state, which nothing has
