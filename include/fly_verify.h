@@ -258,11 +258,12 @@ fly_status_t fly_pld_draft(int32_t device, int32_t B, const int32_t* tokens, int
  * clears the scratch before it).
  *
  * All calls on a device share the one array, and it keeps whatever the last
- * calls left there.  They take turns at its parts, and each clears the counters and partial states of the part whose turn is next
- * (captured calls and calls with inputs_ready have a part of their own, cleared at the start of each), so stale contents
- * never leak into a result.  But two calls whose work
- * overlaps on the GPU (different streams, or several host threads) write the same
- * scratch and corrupt each other: serialise them, e.g. keep them on one stream. */
+ * calls left there.  They take turns at its parts in the order in which they are launched, and each clears the counters and partial states
+ * of the part whose turn is next (captured calls and calls with inputs_ready have a part of their own, cleared at the start of each);
+ * a call that returns an error has taken no turn.  So stale contents never leak into a result, and several host threads may enqueue
+ * their calls on one stream.  But two calls whose work
+ * overlaps on the GPU (different streams) write the same scratch and corrupt each other: serialise them, e.g. keep them on
+ * one stream. */
 #define FLY_STATIC_MAX_BATCH 1024
 #define FLY_STATIC_MAX_PIECES 16384
 #define FLY_STATIC_PARTS 5

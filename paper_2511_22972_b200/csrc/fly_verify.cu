@@ -17,6 +17,7 @@
 #include "pld_kernel.cuh"
 #include "reduce_kernel.cuh"
 #include "scan_kernel.cuh"
+#include "static_turns.h"
 
 namespace {
 
@@ -1027,13 +1028,13 @@ static_assert(kStaticPartBytes == FLY_STATIC_MAX_BATCH * 4 + FLY_STATIC_MAX_PIEC
 struct StaticSlot {
   unsigned char* base = nullptr;  // device address of g_fly_static_scratch on this device
   int sm_count = 0;
-  unsigned calls = 0;             // that took their turn at the first FLY_STATIC_PARTS - 1 parts
+  fly::Turns<FLY_STATIC_PARTS - 1> turns;  // at the first parts
 };
 StaticSlot g_static_slots[kStaticMaxDevices];
 std::mutex g_static_mu;
 
 // With the device current; looked up once per device.
-cudaError_t static_scratch_for(int device, bool takes_turn, StaticSlot* out) {
+cudaError_t static_slot_for(int device, StaticSlot** out) {
   std::lock_guard<std::mutex> lock(g_static_mu);
   StaticSlot& s = g_static_slots[device];
   if (!s.base) {
@@ -1047,8 +1048,7 @@ cudaError_t static_scratch_for(int device, bool takes_turn, StaticSlot* out) {
     if ((e = set_reduce_attrs()) != cudaSuccess) return e;
     s.base = static_cast<unsigned char*>(p);
   }
-  *out = s;
-  if (takes_turn) s.calls = (s.calls + 1) % (FLY_STATIC_PARTS - 1);
+  *out = &s;
   return cudaSuccess;
 }
 
@@ -1086,35 +1086,38 @@ fly_status_t fly_verify_run_static(int32_t device, int32_t vocab, fly_dtype_t lo
     capture = cudaStreamCaptureStatusActive;
   }
   const bool takes_turn = a->inputs_ready == 0 && capture == cudaStreamCaptureStatusNone;
-  StaticSlot slot;
-  if (static_scratch_for(device, takes_turn, &slot) != cudaSuccess) return FLY_ERR_CUDA;
-  const unsigned turns = FLY_STATIC_PARTS - 1;
-  unsigned char* const part = slot.base + (takes_turn ? slot.calls : turns) * kStaticPartBytes;
-  unsigned char* const next = slot.base + (slot.calls + 1) % turns * kStaticPartBytes;
-  unsigned int* tickets = reinterpret_cast<unsigned int*>(part);
-  fly::Partial* partials = reinterpret_cast<fly::Partial*>(part + FLY_STATIC_MAX_BATCH * 4);
-  h.sm_count = slot.sm_count;
+  StaticSlot* slot;
+  if (static_slot_for(device, &slot) != cudaSuccess) return FLY_ERR_CUDA;
+  h.sm_count = slot->sm_count;
 
   const int64_t stride = a->row_stride ? a->row_stride : vocab;
   const int64_t room = FLY_STATIC_MAX_PIECES / rows;  // Partial slots per row that fit, >= 1
   const int cap = (int)(room < kMaxSplits ? room : kMaxSplits);
-
-  fly::ScanParams p = scan_params(&h, a, partials, 1);
-  p.tickets = tickets;
-  cudaError_t e = cudaSuccess;
-  if (!takes_turn) {
+  fly::ScanParams p = scan_params(&h, a, nullptr, 1);
+  auto launch = [&](unsigned char* part, unsigned char* next) {
+    fly::Partial* const partials = reinterpret_cast<fly::Partial*>(part + FLY_STATIC_MAX_BATCH * 4);
+    p.tickets = reinterpret_cast<unsigned int*>(part);
+    return launch_reduce_any(logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, a->temperature,
+                             a->inputs_ready != 0, false, reinterpret_cast<uint4*>(next));
+  };
+  bool ok;
+  if (takes_turn) {
+    ok = slot->turns.take([&](unsigned part, unsigned next) {
+      return launch(slot->base + part * kStaticPartBytes, slot->base + next * kStaticPartBytes) == cudaSuccess;
+    });
+  } else {
     // A kernel in the stream's chain of programmatic dependents and not a memset, which would break the chain.
+    std::lock_guard<std::mutex> lock(slot->turns.mu);  // (nobody's clearing comes between this one and its step)
+    unsigned char* const part = slot->base + (FLY_STATIC_PARTS - 1) * kStaticPartBytes;
     const int slot_words = (int)(rows * cap), ticket_words = (a->B + 3) / 4;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     fill_launch(&cfg, attr, (unsigned)((slot_words + fly::kClearThreads - 1) / fly::kClearThreads), fly::kClearThreads, st, true);
-    e = cudaLaunchKernelEx(&cfg, fly::clear_scratch, reinterpret_cast<uint4*>(tickets), ticket_words, reinterpret_cast<uint4*>(partials),
-                           slot_words);
-    if (e != cudaSuccess) return FLY_ERR_CUDA;
+    ok = cudaLaunchKernelEx(&cfg, fly::clear_scratch, reinterpret_cast<uint4*>(part), ticket_words,
+                            reinterpret_cast<uint4*>(part + FLY_STATIC_MAX_BATCH * 4), slot_words) == cudaSuccess &&
+         launch(part, nullptr) == cudaSuccess;
   }
-  e = launch_reduce_any(logits_dtype, h.sm_count, a->logits, stride, vocab, rows, 0, cap, partials, st, &p, a->temperature,
-                        a->inputs_ready != 0, false, takes_turn ? reinterpret_cast<uint4*>(next) : nullptr);
-  return e == cudaSuccess ? FLY_OK : FLY_ERR_CUDA;
+  return ok ? FLY_OK : FLY_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -65,3 +65,42 @@ def test_calls_take_turns():
             check(i, "plain")
             check((i + 2) % len(steps), "after it")
             check(1, "captured") if i % 3 == 0 else None
+
+
+def test_two_host_threads_on_one_stream():
+    import threading
+    shapes = [(4, 25, 32064, "bf16"), (300, 3, 1000, "f32")]
+    stream, steps, failed = torch.cuda.Stream(), [], []
+    for n, (B, K, V, dtype) in enumerate(shapes):
+        w = S.shrink(S.LLAMA3, B=B, K=K, V=V, dtype=dtype)
+        logits, draft = draw(w, step=n, guard=False)
+        outs = [VerifyBuffers(B, K, DEV) for _ in range(400)]
+        args = [Bd.static_args(B, K, draft, o.accept_len, o.out_tokens, logits=logits, theta=1.0, W=2, state_out=o.state,
+                               rollback=o.rollback, target_argmax=o.target_argmax, entropy=o.entropy, row_flags=o.row_flags,
+                               inputs_ready=i % 7 == 3) for i, o in enumerate(outs)]
+        fv, want = FlyVerify(B, K, V, dtype), VerifyBuffers(B, K, DEV)
+        fv.run(Bd.static_args(B, K, draft, want.accept_len, want.out_tokens, logits=logits, theta=1.0, W=2, state_out=want.state,
+                              rollback=want.rollback, target_argmax=want.target_argmax, entropy=want.entropy,
+                              row_flags=want.row_flags), torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        fv.close()
+        steps.append((args, outs, want, V, dtype))
+
+    def work(args, V, dtype):
+        try:
+            for a in args:
+                Bd.run_static(a, V, dtype, 0, stream.cuda_stream)
+        except Exception as e:
+            failed.append(e)
+    threads = [threading.Thread(target=work, args=(args, V, dtype)) for args, _, _, V, dtype in steps]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed
+    for (_, outs, want, _, _), shape in zip(steps, shapes):
+        for i, got in enumerate(outs):
+            for f in FIELDS:
+                a, b = getattr(got, f), getattr(want, f)
+                assert torch.equal(a, b) if f != "entropy" else torch.allclose(a, b, rtol=0, atol=1e-5), (shape, i, f)
