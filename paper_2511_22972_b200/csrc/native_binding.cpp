@@ -12,10 +12,13 @@
 // one copy of it in the process.
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <ATen/Context.h>
 #include <ATen/EmptyTensor.h>
 #include <ATen/detail/CUDAHooksInterface.h>
 #include <ATen/ops/empty.h>
+#include <ATen/record_function.h>
 #include <c10/core/DeviceGuard.h>
+#include <c10/core/impl/LocalDispatchKeySet.h>
 
 #include "fly_verify.h"
 
@@ -122,6 +125,12 @@ struct Unlocked {
   PyThreadState* state = PyEval_SaveThread();
   ~Unlocked() { PyEval_RestoreThread(state); }
 };
+
+// Whether at::empty is nothing but an allocation here: no dispatch mode, tracing or transform in this thread, no profiler, no fill.
+bool plain_empty() {
+  return (c10::impl::tls_local_dispatch_key_set().included_ - c10::default_included_set).empty() && !at::hasCallbacks() &&
+         !(at::globalContext().deterministicAlgorithms() && at::globalContext().deterministicFillUninitializedMemory());
+}
 
 PyObject* status(fly_status_t s) { return PyLong_FromLong((long)s); }
 
@@ -327,7 +336,7 @@ PyObject* py_pld_draft(PyObject*, PyObject* const* v, Py_ssize_t n) {
   {
     Unlocked unlocked;
     const int64_t B = tokens.size(0);
-    if (tokens.is_cuda()) {
+    if (tokens.is_cuda() && plain_empty()) {
       // Straight from torch's allocator: through the dispatcher each of the four takes 0.5 us longer, and the call as long as
       // the kernel (32 contexts of 32768 tokens: 6.9 us a call, 5.6 so).
       const c10::DeviceGuard guard(tokens.device());

@@ -186,3 +186,26 @@ def test_contexts_that_end_in_a_run_of_one_token(L, pad):
     for mx in (1, 3, 8):
         run([s for s, c in zip(seqs, cases) if c[0] == mx], 8, mx, 1, pad_to=(L + 3) // 4 * 4 + pad)
     assert all(oracle_pld(s, 8, mx, 1)[1:] == (at, mx) for s, (mx, at) in zip(seqs, cases))
+
+
+def test_the_allocation_of_the_results_is_seen_by_modes_and_the_profiler():
+    from torch.profiler import ProfilerActivity, profile
+    from torch.utils._python_dispatch import TorchDispatchMode
+
+    class Log(TorchDispatchMode):
+        seen = []
+
+        def __torch_dispatch__(self, func, types, args=(), kwargs=None):
+            self.seen.append(str(func))
+            return func(*args, **(kwargs or {}))
+    tok = torch.randint(0, 9, (3, 100), dtype=torch.int32, device=DEV)
+    lengths, st = torch.full((3,), 100, dtype=torch.int32, device=DEV), torch.cuda.current_stream().cuda_stream
+    want = Bd.pld_draft(tok, lengths, 5, 3, 1, stream=st)
+    with Log() as log:
+        logged = Bd.pld_draft(tok, lengths, 5, 3, 1, stream=st)
+    assert log.seen.count("aten.empty.memory_format") == 4, log.seen
+    with profile(activities=[ProfilerActivity.CPU]) as prof:
+        profiled = Bd.pld_draft(tok, lengths, 5, 3, 1, stream=st)
+    assert sum(e.name == "aten::empty" for e in prof.events()) == 4
+    for got in (logged, profiled):
+        assert all(torch.equal(a, b) and a.stride() == b.stride() for a, b in zip(got, want))
