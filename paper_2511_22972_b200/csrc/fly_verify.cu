@@ -53,7 +53,6 @@ struct fly_verify {
   int forced_splits = 0;
   int scan_mode = 0;   // 0: fused tail, 1: separate kernel
   int last_launches = 0;
-  bool host_logits = false;  // the step's logits are host memory, read in place
   int last_cuda_error = 0;
   // fused LM-head path (cfg.hidden > 0)
   fly::Partial* lm_partials = nullptr;  // [max_rows * sm_count]: one partial state per row and CTA
@@ -600,6 +599,41 @@ fly::ScanParams scan_params(const fly_verify* h, const fly_verify_args_t* a, fly
   return p;
 }
 
+// host_logits: the logits are host memory that is read in place (nothing precedes them, and over the bus a read ahead is a read more).
+fly_status_t run_step(fly_verify_t* h, const fly_verify_args_t* a, void* cuda_stream, bool host_logits) {
+  fly_status_t s = check_args(h, a);
+  if (s != FLY_OK) return s;
+  if (!a->logits && h->cfg.hidden <= 0) return FLY_ERR_INVALID_ARG;  // the handle was created without a hidden size
+  DeviceGuard g(h->cfg.device);
+  if (!g.ok) return FLY_ERR_CUDA;
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  const int V = h->cfg.vocab;
+  const int64_t rows = (int64_t)a->B * (a->K + 1);
+  const int64_t stride = a->row_stride ? a->row_stride : V;
+  h->last_launches = 0;
+  cudaError_t e = scratch_ready(h, st);
+  if (e != cudaSuccess) return cuda_fail(h, e);
+  if (!a->logits) return run_fused(h, a, st);
+
+  fly::ScanParams p = scan_params(h, a, h->partials, 1);
+  // The acceptance scan runs as the tail of the reduction (the block that completes a sequence verifies it) unless
+  // the handle asks for a kernel of its own.  Measured in plain stream order the two cost the same; the tail also
+  // lets consecutive steps overlap (inputs_ready) and keeps a step at one launch.
+  const bool fused_tail = h->scan_mode == 0;
+  p.tickets = fused_tail ? h->tickets : nullptr;
+  p.status = h->state_status;
+  e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, a->logits, stride, V, rows, h->forced_splits,
+                                    kMaxSplits, h->partials, st, &p, a->temperature, a->inputs_ready != 0, host_logits);
+  if (e != cudaSuccess) return cuda_fail(h, e);
+  h->last_launches++;
+  if (!fused_tail) {
+    e = launch_scan(p, true, st);
+    if (e != cudaSuccess) return cuda_fail(h, e);
+    h->last_launches++;
+  }
+  return FLY_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -873,37 +907,7 @@ int32_t fly_verify_last_launch_count(const fly_verify_t* h) { return h ? h->last
 int32_t fly_verify_last_cuda_error(const fly_verify_t* h) { return h ? h->last_cuda_error : 0; }
 
 fly_status_t fly_verify_run(fly_verify_t* h, const fly_verify_args_t* a, void* cuda_stream) {
-  fly_status_t s = check_args(h, a);
-  if (s != FLY_OK) return s;
-  if (!a->logits && h->cfg.hidden <= 0) return FLY_ERR_INVALID_ARG;  // the handle was created without a hidden size
-  DeviceGuard g(h->cfg.device);
-  if (!g.ok) return FLY_ERR_CUDA;
-  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const int V = h->cfg.vocab;
-  const int64_t rows = (int64_t)a->B * (a->K + 1);
-  const int64_t stride = a->row_stride ? a->row_stride : V;
-  h->last_launches = 0;
-  cudaError_t e = scratch_ready(h, st);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  if (!a->logits) return run_fused(h, a, st);
-
-  fly::ScanParams p = scan_params(h, a, h->partials, 1);
-  // The acceptance scan runs as the tail of the reduction (the block that completes a sequence verifies it) unless
-  // the handle asks for a kernel of its own.  Measured in plain stream order the two cost the same; the tail also
-  // lets consecutive steps overlap (inputs_ready) and keeps a step at one launch.
-  const bool fused_tail = h->scan_mode == 0;
-  p.tickets = fused_tail ? h->tickets : nullptr;
-  p.status = h->state_status;
-  e = launch_reduce_any(h->cfg.logits_dtype, h->sm_count, a->logits, stride, V, rows, h->forced_splits,
-                                    kMaxSplits, h->partials, st, &p, a->temperature, a->inputs_ready != 0, h->host_logits);
-  if (e != cudaSuccess) return cuda_fail(h, e);
-  h->last_launches++;
-  if (!fused_tail) {
-    e = launch_scan(p, true, st);
-    if (e != cudaSuccess) return cuda_fail(h, e);
-    h->last_launches++;
-  }
-  return FLY_OK;
+  return run_step(h, a, cuda_stream, false);
 }
 
 fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, void* cuda_stream) {
@@ -992,9 +996,7 @@ fly_status_t fly_verify_run_host(fly_verify_t* h, const fly_verify_args_t* a, vo
   d.entropy = reinterpret_cast<float*>(dv + o_entropy);
   d.row_flags = reinterpret_cast<uint32_t*>(dv + o_flags);
   d.target_tokens = a->target_tokens ? dv + o_target : nullptr;
-  h->host_logits = direct != nullptr;  // (nothing precedes them, and over the bus a read ahead is a read more)
-  s = fly_verify_run(h, &d, cuda_stream);
-  h->host_logits = false;
+  s = run_step(h, &d, cuda_stream, direct != nullptr);
   if (s != FLY_OK) return s;
 
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(h, e);
