@@ -317,6 +317,7 @@ struct ReducePlan {
   int64_t n;       // units per row
   int64_t span;    // units a row takes in the flat index space (>= n)
   int64_t Q;       // units per block
+  uint4* clear;    // not null (wait_first == 1): kClearWords of scratch of the next call, which this one empties
   int pieces;      // > 0: span = pieces * Q, block b is piece b % pieces of row b / pieces (32-bit arithmetic)
   int V;
   int64_t row_stride;  // elements
@@ -326,7 +327,6 @@ struct ReducePlan {
   int wait_first;  // 1: wait for the previous kernel in the stream before the first read (plain stream
                    //    order); 0: the logits are known to be complete, wait only before the first write;
                    //    2: as 1, and nothing is asked for ahead of the wait
-  uint4* clear;    // not null (wait_first == 1): kClearWords of scratch of the next call, which this one empties
 };
 static_assert(sizeof(ReducePlan) == 64 && sizeof(ScanParams) == 216, "measure what a launch costs the host");
 
@@ -555,7 +555,9 @@ reduce_rows_flat(const T* __restrict__ logits, const __grid_constant__ ReducePla
     for (int d = 0; d < kDepth; ++d) issue(d);
     fetch_leftover(row, u1);
   }
-  if (g.clear != nullptr)  // (while the first slices are on their way)
+  // (While the first slices are on their way.  Unrolled, its code costs the steps that do not clear: 9 rows of 32000 fp32 3.98 us, 3.94 so.)
+  if (g.clear != nullptr)
+#pragma unroll 1
     for (int i = (int)(blockIdx.x * kReduceThreads + threadIdx.x); i < kClearWords; i += (int)gridDim.x * kReduceThreads)
       g.clear[i] = make_uint4(0, 0, 0, 0);
 
