@@ -12,10 +12,10 @@
 // What bounds it is latency: a 128 KB context is 20 ns of HBM bandwidth but a chain of dependent reads
 // (length, tokens, earlier tokens at a hit, continuation).  A sequence is therefore spread over a cluster
 // of up to 8 blocks of 256 threads, 16 tokens per thread and round with all four loads in flight, and the
-// blocks' best[] meet in the first block's shared memory.  What is left is short: the tokens of the first round are asked for with
+// blocks' findings meet in the first block's shared memory.  What is left is short: the tokens of the first round are asked for with
 // the last tokens and do not wait for them, and the look-back exists once and not per token, since a launch also waits for
-// its code.  us a call in a row of calls, before both / after: 32 contexts of 16 - 32 k tokens 5.8 / 3.9, 64 of 8 - 16 k 5.25 / 3.8, 4 of
-// 50 - 100 k 5.4 / 4.1, 64 of 1 - 2 k 2.9 / 2.4, one of 300 2.35 / 2.26.  (Blocks of 512 or 1024 threads, up to 7 loads in flight, without a
+// its code.  us a call in a CUDA graph, before both / after, on two boxes that agree to 0.04: 32 contexts of 16 - 32 k tokens 4.29 / 3.44, 64 of
+// 8 - 16 k 4.35 / 3.39, 4 of 50 - 100 k 5.13 / 3.80, 16 of 64 - 128 k 6.27 / 5.37, 64 of 1 - 2 k 2.77 / 2.57, one of 300 2.06 / 1.81.  (Blocks of 512 or 1024 threads, up to 7 loads in flight, without a
 // cluster: 32 contexts of 16 - 32 k 4.3 - 5.3.)
 #pragma once
 #include <cooperative_groups.h>
